@@ -48,6 +48,20 @@ static bool tuned_shape(const ssm_problem_t& p) {
   return p.io_dtype == SSM_BF16 && p.N == 16 && p.D % 8 == 0 && !(p.flags & SSM_FLAG_COMPLEX) &&
          !(static_bc && (p.flags & SSM_FLAG_ZOH_BBAR));   // non-selective B / C: tuned with the default B-bar rule only
 }
+// Checkpoint states are tiled by groups of 32 channels whenever a channel's states are whole 16-byte quads.
+static bool ckpt_tiled(const ssm_problem_t& p) { return p.N % 4 == 0 && !(p.flags & SSM_FLAG_COMPLEX); }
+// Problems the lane-per-channel kernels run (ssm_lane.cuh): what the tuned kernels do not take.
+bool lane_shape(const ssm_problem_t& p) {
+  if (p.flags & (SSM_FLAG_COMPLEX | SSM_FLAG_ZOH_BBAR | SSM_FLAG_STATIC_B | SSM_FLAG_STATIC_C)) return false;
+  return !tuned_shape(p);
+}
+// Time segments of a lane launch.  A chain already spreads over up to 64 warps of a cluster, so the launch itself is
+// split (summary pass, carry, full pass) only for a handful of chains and then into segments of at least 2048 steps.
+static int lane_segments(const ssm_problem_t& p) {
+  const long long chains = (long long)p.batch * ((p.D + 31) / 32);
+  const long long want = (8LL * kNumSMs + 64 * chains - 1) / (64 * chains);
+  return (int)std::max<long long>(1, std::min<long long>(want, p.L / 2048));
+}
 // Workers the hand-off slots of a workspace allow for `chains` chains: none while every chain can have a warp of its
 // own in the first round (one warp per SM sub-partition); else at least two rounds (a kernel may share chains between
 // more warps than there are chains) and at most 12 resident warps per SM.
@@ -133,6 +147,8 @@ Plan make_plan(const ssm_problem_t& p) {
   int nseg = 1;
   if (p.flags & SSM_FLAG_COMPLEX) {
     // the complex path does not split time
+  } else if (lane_shape(p)) {
+    nseg = lane_segments(p);
   } else if (tuned_shape(p)) {
     // one warp per chain of fwd_fast_channels_per_warp() channels; a split costs half a forward sweep more, so only
     // when fewer than half of the sub-partitions would have a warp, and then into two rounds of chains
@@ -259,7 +275,7 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
   w.dA_part = take(parts * p.D * p.N * sizeof(float));
   w.dD_part = take(parts * p.D * sizeof(float));
   w.dbias_part = take(parts * p.D * sizeof(float));
-  w.ckpt = take((size_t)p.batch * pl.nck * ckpt_floats_per_step(tuned_shape(p), p.D, p.N) * sizeof(float));
+  w.ckpt = take((size_t)p.batch * pl.nck * ckpt_floats_per_step(ckpt_tiled(p), p.D, p.N) * sizeof(float));
   if (pl.nseg > 1) {
     const size_t st = parts * p.D * p.N * sizeof(float);
     w.seg_local = take(st);
@@ -350,7 +366,7 @@ size_t ssm_scan_saved_state_bytes(const ssm_problem_t* p) {
   ssm_problem_t wide;
   if (widen_route(*p, &wide)) return ssm_scan_saved_state_bytes(&wide);
   const size_t nck = (size_t)(p->L + kCkptSteps - 1) / kCkptSteps;
-  return (size_t)p->batch * nck * ckpt_floats_per_step(tuned_shape(*p), p->D, p->N) * sizeof(float);
+  return (size_t)p->batch * nck * ckpt_floats_per_step(ckpt_tiled(*p), p->D, p->N) * sizeof(float);
 }
 
 int32_t ssm_scan_checkpoint_steps(void) { return kCkptSteps; }
@@ -497,7 +513,7 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.h_start = h_start;
   fp.h_last = h_last;
   fp.ckpt = save ? static_cast<float*>(saved_states) : nullptr;
-  fp.ckpt_tiled = tuned_shape(*p) ? 1 : 0;
+  fp.ckpt_tiled = ckpt_tiled(*p) ? 1 : 0;
   if (launch_fwd(*p, pl, fp, kFwdFull, s) != cudaSuccess) return SSM_ERR_CUDA;
   return SSM_OK;
 }
@@ -667,7 +683,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
       return SSM_ERR_CUDA;
     fp.h_start = h_start;
     fp.ckpt = reinterpret_cast<float*>(ws + w.ckpt);
-    fp.ckpt_tiled = tuned_shape(*p) ? 1 : 0;
+    fp.ckpt_tiled = ckpt_tiled(*p) ? 1 : 0;
     if (launch_fwd(*p, pl_fwd, fp, kFwdCkptOnly, s) != cudaSuccess) return SSM_ERR_CUDA;
     ckpt = fp.ckpt;
   }
@@ -682,7 +698,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   bp.Dskip = has_d ? D_skip : nullptr;
   bp.dout = dout;
   bp.ckpt = ckpt;
-  bp.ckpt_tiled = tuned_shape(*p) ? 1 : 0;
+  bp.ckpt_tiled = ckpt_tiled(*p) ? 1 : 0;
   bp.dx = dx;
   bp.ddelta = ddelta;
   bp.dz = has_z ? dz : nullptr;

@@ -1,0 +1,471 @@
+// Forward selective scan, one lane per channel, for everything the tuned bf16 / N = 16 kernel does not take and for the
+// problems with too few chains to fill the GPU (mathematics and modes as in ssm_fwd.cu; layout and time split: ssm_lane.cuh).
+//
+// A lane owns one channel and 16 of its states at a time as packed float2 pairs, so the readout sum over n stays in the
+// thread.  With N > 16 the groups of 16 states of a batch run one after the other, their state parked in shared memory;
+// everything that belongs to the channel (step size, input, gate, rounding) is done once.
+//
+// Bound: instruction issue (80 warp instructions per warp and step, 0.4 issued per cycle by a lone warp of a
+// sub-partition) and, with one exponential per state, the special-function unit (16 ex2 = 128 cycles per warp and step),
+// so the registers are capped for three warps per sub-partition and a chain is split in time until they are there.
+// Measured against the generic kernel with its summary and carry launches: float32 (2, 2048, 1536), N = 16: 262 -> 76 us;
+// bf16 (3, 1237, 1001), N = 16: 268 -> 51 us; bf16 (1, 2048, 5120), N = 64: 1204 -> 362 us; float32 (1, 256, 64):
+// 126 -> 8 us.
+#include <type_traits>
+
+#include "ssm_lane.cuh"
+
+namespace ssm {
+
+namespace {
+
+namespace cg = cooperative_groups;
+
+// shared memory of a block, in floats: per warp, the tiles of two batches (x, delta, z; B, C widened), the output tile,
+// the state, the sum of delta; per chain, A * log2(e), the chain's totals over this block (for the other blocks of the
+// cluster) and its sum of delta
+template <typename IO, int NG>
+struct FwdLaneSmem {
+  static constexpr int NP = 16 * NG;              // padded states
+  static constexpr int kTile = kLB * 32 * (int)sizeof(IO) / 4;
+  static constexpr int kBuf = 3 * kTile + 2 * kLB * NP;   // one batch: x | delta | z | B | C
+  static constexpr int kIO = 2 * kBuf + kTile;    // floats per warp
+  static constexpr int kState = NP * 32;          // floats per warp
+  static constexpr int kChain = 2 * kState + 32;  // floats per chain
+  static constexpr size_t bytes(int warps, int chains) {
+    return sizeof(float) * ((size_t)warps * (kIO + kState + 32) + (size_t)chains * kChain);
+  }
+};
+
+template <typename IO, int NG, bool VEC>
+__global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const FwdParams p, const LaneSplit sp, const int N, const int mode) {
+  using SM = FwdLaneSmem<IO, NG>;
+  constexpr int NP = SM::NP;
+  const bool full = mode == kFwdFull, summary = mode == kFwdSummary;
+  extern __shared__ __align__(16) float smem[];
+  const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
+  const int W = sp.warps, CL = sp.cluster;
+  constexpr int nwarps = kLaneWarps;
+  const int sub = bwarp / W, warp = bwarp % W;   // sub: which chain of the block
+  float* const sIO = smem + (size_t)bwarp * SM::kIO;
+  float* const sE = smem + (size_t)nwarps * SM::kIO + (size_t)sub * W * SM::kState;         // [W][NP][32]
+  float* const sDs = smem + (size_t)nwarps * (SM::kIO + SM::kState) + sub * W * 32;         // [W][32]
+  float* const sA = smem + (size_t)nwarps * (SM::kIO + SM::kState + 32) + (size_t)sub * SM::kChain;   // [NP][32]
+  float* const sTot = sA + SM::kState;                                                      // [NP][32]
+  float* const sTotDs = sTot + SM::kState;                                                  // [32]
+  float* const sH = sE + (size_t)warp * SM::kState;                 // this warp's states
+
+  const IO* __restrict__ gx = static_cast<const IO*>(p.x);
+  const IO* __restrict__ gd = static_cast<const IO*>(p.delta);
+  const IO* __restrict__ gz = static_cast<const IO*>(p.z);
+  const IO* __restrict__ gB = static_cast<const IO*>(p.B);
+  const IO* __restrict__ gC = static_cast<const IO*>(p.C);
+  IO* __restrict__ gout = static_cast<IO*>(p.out);
+
+  const int D = p.D;
+  const int groups = (D + 31) / 32;
+  const int rank = (int)(blockIdx.x % (unsigned)CL);
+  const int chains = p.batch * p.nseg * groups;
+  const int chain_id = (int)(blockIdx.x / (unsigned)CL) * (nwarps / W) + sub;
+  const int chain = min(chain_id, chains - 1);
+  const int grp = chain % groups;
+  const int bs = chain / groups;
+  const int seg = bs % p.nseg, b = bs / p.nseg;
+  const int c_own = grp * 32 + lane;
+  const bool valid = c_own < D;
+  const int c_ld = valid ? c_own : D - 1;       // lanes past the last channel read it along and store nothing
+  const int seg_t0 = seg * p.seg_steps;
+  const int seg_end = min(p.L, seg_t0 + p.seg_steps);
+  const int piece0 = (rank * W + warp) * sp.piece;
+  const int t_begin = chain_id < chains ? min(seg_end, seg_t0 + piece0) : seg_end;   // (a spare warp has no steps)
+  const int t_end = min(seg_end, t_begin + sp.piece);
+  const bool split = W * CL > 1;
+  const bool bvec = (reinterpret_cast<uintptr_t>(p.B) & (4 * sizeof(IO) - 1)) == 0;
+  const bool cvec = (reinterpret_cast<uintptr_t>(p.C) & (4 * sizeof(IO) - 1)) == 0;
+  const bool has_z = full && gz != nullptr;
+  const int cols = min(32, D - grp * 32);
+
+  // One batch in flight from global memory.  read: with z and C.
+  LaneRows<IO, VEC> rx, rd, rz;
+  LaneQuad<IO> qB[NG], qC[NG];
+  const size_t row_b = (size_t)b * p.L;
+  if (!has_z) rz.zero();
+  auto prefetch = [&](int t0, bool read) {
+    const size_t base = (row_b + t0) * D + grp * 32, baseBC = (row_b + t0) * N;
+    const int last = t_end - 1 - t0;
+    rd.load(gd + base, D, lane, last, cols);
+    rx.load(gx + base, D, lane, last, cols);
+    if (read && has_z) rz.load(gz + base, D, lane, last, cols);
+#pragma unroll
+    for (int i = 0; i < NG; ++i) {
+      const int v = lane + 32 * i, n = 4 * (v % (4 * NG));
+      const unsigned o = (unsigned)(min(v / (4 * NG), last) * N + n);
+      qB[i].load(gB + baseBC + o, N - n, bvec && N >= 4);
+      if (read) qC[i].load(gC + baseBC + o, N - n, cvec && N >= 4);
+    }
+  };
+  // The first batch is requested before anything else is set up.  What leaves the last piece of the launch is wanted by
+  // the summary mode only.
+  const bool live_piece = t_begin < t_end;
+  const bool first_sweep = (split || summary) && (summary || rank * W + warp < W * CL - 1);
+  if (live_piece) prefetch(t_begin, full && !first_sweep);
+
+  for (int n = warp; n < NP; n += W) sA[n * 32 + lane] = n < N ? p.A[(size_t)c_ld * N + n] * kLog2e : 0.f;
+  __syncthreads();
+  float2 A2[8];
+  float2 h[8];
+  // which groups of 16 have their A in arithmetic progression (padded states continue it as long as they decay)
+  unsigned ap_mask = 0;
+  if (sizeof(IO) == 2 && !p.general_A) {
+#pragma unroll 1
+    for (int g = 0; g < NG; ++g) {
+      const float* a = sA + g * 512 + lane;
+      const int live = min(16, N - 16 * g);
+      const float a0 = a[0], step = live > 1 ? a[32] - a0 : 0.f;
+      const float tol = 1e-6f * fabsf(a[32 * (live - 1)]);
+      bool ok = live == 16 || step <= 0.f;
+      for (int k = 2; k < live; ++k) ok = ok && fabsf(a[32 * k] - (a0 + (float)k * step)) <= tol;
+      if (__all_sync(0xffffffffu, ok)) ap_mask |= 1u << g;
+    }
+  }
+  if constexpr (NG == 1) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) A2[k] = make_float2(sA[(2 * k) * 32 + lane], sA[(2 * k + 1) * 32 + lane]);
+  }
+  const float bias = p.delta_bias != nullptr ? p.delta_bias[c_ld] : 0.f;
+  const float Dk = (full && p.Dskip != nullptr) ? p.Dskip[c_ld] : 0.f;
+  const float gate_off = has_z ? 0.f : 1.f;
+  float dsum = 0.f;
+
+  auto load_h = [&](int g) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      h[k] = make_float2(sH[(g * 16 + 2 * k) * 32 + lane], sH[(g * 16 + 2 * k + 1) * 32 + lane]);
+  };
+  auto store_h = [&](int g) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      sH[(g * 16 + 2 * k) * 32 + lane] = h[k].x;
+      sH[(g * 16 + 2 * k + 1) * 32 + lane] = h[k].y;
+    }
+  };
+
+  // One sweep over the warp's piece, whose first batch has been requested.  READ: with readout, gate and output; else the
+  // state only.
+  auto sweep = [&](auto read_tag, bool write_ckpt) {
+    constexpr bool READ = decltype(read_tag)::value;
+    if (!live_piece) return;
+    int buf = 0;
+#pragma unroll 1
+    for (int t0 = t_begin; t0 < t_end; t0 += kLB, buf ^= 1) {
+      float* const sBuf = sIO + buf * SM::kBuf;
+      IO* const tx = reinterpret_cast<IO*>(sBuf);
+      IO* const td = reinterpret_cast<IO*>(sBuf + SM::kTile);
+      IO* const tz = reinterpret_cast<IO*>(sBuf + 2 * SM::kTile);
+      IO* const to = reinterpret_cast<IO*>(sIO + 2 * SM::kBuf);
+      float* const fB = sBuf + 3 * SM::kTile;
+      float* const fC = fB + kLB * NP;
+      const int live = t_end - t0;
+      rd.put(td, lane);
+      rx.put(tx, lane);
+      if constexpr (READ) rz.put(tz, lane);
+#pragma unroll
+      for (int i = 0; i < NG; ++i) {
+        const int v = lane + 32 * i;
+        *reinterpret_cast<float4*>(fB + 4 * v) = qB[i].widen();
+        if constexpr (READ) *reinterpret_cast<float4*>(fC + 4 * v) = qC[i].widen();
+      }
+      if constexpr (VEC) {
+        __syncwarp();
+        if (t0 + kLB < t_end) prefetch(t0 + kLB, READ);
+      }
+      float dt[kLB], u[kLB], zf[READ ? kLB : 1], y[READ ? kLB : 1];
+#pragma unroll
+      for (int t = 0; t < kLB; ++t) {
+        dt[t] = rd.get(td, t, lane) + bias;
+        u[t] = rx.get(tx, t, lane);
+        if constexpr (READ) {
+          zf[t] = rz.get(tz, t, lane);
+          y[t] = Dk * u[t];
+        }
+      }
+      if constexpr (!VEC) {
+        if (t0 + kLB < t_end) prefetch(t0 + kLB, READ);
+        __syncwarp();
+      }
+      if (p.softplus) {
+#pragma unroll
+        for (int t = 0; t < kLB; ++t) dt[t] = lane_softplus<IO>(dt[t]);
+      }
+      if (live < kLB) {   // rows past the end are identity steps
+#pragma unroll
+        for (int t = 0; t < kLB; ++t) dt[t] = t < live ? dt[t] : 0.f;
+      }
+      if (!READ) {
+#pragma unroll
+        for (int t = 0; t < kLB; ++t) dsum += dt[t];
+      }
+
+#pragma unroll 1
+      for (int g = 0; g < NG; ++g) {
+        if constexpr (NG > 1) load_h(g);
+        if (write_ckpt) {
+          const int kc = t0 / kCkptSteps;
+          if (SSM_IN_RANGE(kc < p.nck, p.abort)) {
+            if (N >= 4) {   // (lanes past the last channel fill the padding of the tiled layout)
+              float* dst = p.ckpt + ckpt_offset(1, b, p.nck, kc, D, N, c_own, 16 * g);
+#pragma unroll
+              for (int k = 0; k < 4; ++k)
+                if (16 * g + 4 * k < N)
+                  *reinterpret_cast<float4*>(dst + 128 * k) = make_float4(h[2 * k].x, h[2 * k].y, h[2 * k + 1].x, h[2 * k + 1].y);
+            } else if (valid) {
+              float* dst = p.ckpt + ckpt_offset(0, b, p.nck, kc, D, N, c_own, 0);
+              dst[0] = h[0].x;
+              if (N > 1) dst[1] = h[0].y;
+            }
+          }
+        }
+        // Decays, input terms and C of a step do not depend on the state: they are prepared one step ahead of the
+        // recurrence that consumes them.
+        auto run = [&](auto ap_tag) {
+          constexpr bool AP = decltype(ap_tag)::value;
+          constexpr int GB = AP ? kLB : 4;   // steps whose exponentials are in flight together
+          float a0s = 0.f, rs = 0.f;
+          if constexpr (AP) {
+            a0s = sA[(16 * g) * 32 + lane];
+            rs = N - 16 * g > 1 ? sA[(16 * g + 1) * 32 + lane] - a0s : 0.f;
+          } else if constexpr (NG > 1) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              A2[k] = make_float2(sA[(16 * g + 2 * k) * 32 + lane], sA[(16 * g + 2 * k + 1) * 32 + lane]);
+          }
+#pragma unroll
+          for (int gb = 0; gb < kLB / GB; ++gb) {
+            float e0[AP ? GB : 1], e1[AP ? GB : 1];
+            float2 af[AP ? 1 : GB][AP ? 1 : 8];
+#pragma unroll
+            for (int t = 0; t < GB; ++t) {
+              const float dtt = dt[gb * GB + t];
+              if constexpr (AP) {
+                e0[t] = ex2_approx(dtt * a0s);
+                e1[t] = ex2_approx(dtt * rs);
+              } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                  const float2 e = f2mul(f2dup(dtt), A2[k]);
+                  af[t][k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+                }
+              }
+            }
+            float2 aN[2][8], bxN[2][8], CvN[2][READ ? 8 : 1];
+            auto front = [&](int t, float2 (&a)[8], float2 (&bx)[8], float2 (&Cv)[READ ? 8 : 1]) {
+              const int ts = gb * GB + t;
+              load16(fB + ts * NP + 16 * g, bx);
+              if constexpr (READ) load16(fC + ts * NP + 16 * g, Cv);
+              if constexpr (AP) {
+                const float a0 = e0[t], rr = e1[t], r2 = rr * rr, r4 = r2 * r2, r8 = r4 * r4;
+                a[0] = make_float2(a0, a0 * rr);
+                a[1] = f2mul(a[0], f2dup(r2));
+                a[2] = f2mul(a[0], f2dup(r4));
+                a[3] = f2mul(a[1], f2dup(r4));
+#pragma unroll
+                for (int k = 0; k < 4; ++k) a[4 + k] = f2mul(a[k], f2dup(r8));
+              } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) a[k] = af[t][k];
+              }
+              const float2 du2 = f2dup(dt[ts] * u[ts]);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) bx[k] = f2mul(du2, bx[k]);
+            };
+            front(0, aN[0], bxN[0], CvN[0]);
+#pragma unroll
+            for (int t = 0; t < GB; ++t) {
+              if (t + 1 < GB) front(t + 1, aN[(t + 1) & 1], bxN[(t + 1) & 1], CvN[(t + 1) & 1]);
+              float2 yv = make_float2(0.f, 0.f), yw = yv;
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                h[k] = f2fma(aN[t & 1][k], h[k], bxN[t & 1][k]);
+                if constexpr (READ) {
+                  if (k & 1) yw = f2fma(CvN[t & 1][k], h[k], yw);
+                  else yv = f2fma(CvN[t & 1][k], h[k], yv);
+                }
+              }
+              if constexpr (READ) y[gb * GB + t] += (yv.x + yw.x) + (yv.y + yw.y);
+            }
+          }
+        };
+        if (ap_mask >> g & 1) run(std::true_type{});
+        else run(std::false_type{});
+        if constexpr (NG > 1) store_h(g);
+      }
+      if constexpr (READ) {
+        IO* const bo = gout + (row_b + t0) * D + grp * 32;
+#pragma unroll
+        for (int t = 0; t < kLB; ++t) {
+          // without z its rows are zero: silu(0) = 0, and gate_off = 1 takes its place
+          const float v = y[t] * fmaf(zf[t], sigmoid_fast(zf[t]), gate_off);
+          LaneOut<IO, VEC>::put(to, bo, D, t, lane, valid && t < live, v);
+        }
+        if constexpr (VEC) {
+          __syncwarp();
+          LaneOut<IO, VEC>::flush(to, bo, D, lane, live, cols);
+        }
+      }
+    }
+  };
+
+  // ---- first sweep and the fold over the pieces (only if the chain or the launch is split)
+  const size_t seg_row = ((size_t)b * p.nseg + seg) * D;
+  if (split || summary) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) h[k] = make_float2(0.f, 0.f);
+    if constexpr (NG > 1) {
+      for (int g = 0; g < NG; ++g) store_h(g);
+    }
+    if (first_sweep) sweep(std::false_type{}, false);
+    if (first_sweep && live_piece && !summary) prefetch(t_begin, full);
+    if constexpr (NG == 1) store_h(0);
+    sDs[warp * 32 + lane] = dsum;
+    __syncthreads();
+    // exclusive fold over the block's pieces from a zero inflow, and the block's totals
+    for (int n = warp; n < NP; n += W) {
+      const float a2 = sA[n * 32 + lane];
+      float pre = 0.f, ds = 0.f;
+      for (int w = 0; w < W; ++w) {
+        float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
+        const float e = *at, d = sDs[w * 32 + lane];
+        *at = pre;
+        pre = fmaf(ex2_approx(a2 * d), pre, e);
+        ds += d;
+      }
+      sTot[n * 32 + lane] = pre;
+      if (n == 0) sTotDs[lane] = ds;
+    }
+    if (CL > 1) cg::this_cluster().sync();
+    else __syncthreads();
+    // add the inflow of the block: the segment's start state behind the totals of the blocks before it
+    for (int n = warp; n < NP; n += W) {
+      const float a2 = sA[n * 32 + lane];
+      float H = (p.h_start != nullptr && n < N) ? p.h_start[(seg_row + c_ld) * N + n] : 0.f;
+      float ds_all = 0.f, rt[kLaneMaxCluster - 1], rds[kLaneMaxCluster - 1];
+#pragma unroll
+      for (int r = 0; r < kLaneMaxCluster - 1; ++r) {   // (all requested before the first is used)
+        if (r < rank) {
+          rt[r] = cg::this_cluster().map_shared_rank(sTot, r)[n * 32 + lane];
+          rds[r] = cg::this_cluster().map_shared_rank(sTotDs, r)[lane];
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < kLaneMaxCluster - 1; ++r) {
+        if (r < rank) {
+          H = fmaf(ex2_approx(a2 * rds[r]), H, rt[r]);
+          ds_all += rds[r];
+        }
+      }
+      if (summary && rank == CL - 1 && valid && n < N && chain_id < chains) {
+        const float d = sTotDs[lane];
+        p.seg_end[(seg_row + c_own) * N + n] = fmaf(ex2_approx(a2 * d), H, sTot[n * 32 + lane]);
+        if (n == 0) p.seg_dsum[seg_row + c_own] = ds_all + d;
+      }
+      float cum = 0.f;
+      for (int w = 0; w < W; ++w) {
+        float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
+        *at = fmaf(ex2_approx(a2 * cum), H, *at);
+        cum += sDs[w * 32 + lane];
+      }
+    }
+    if (CL > 1) cg::this_cluster().sync();   // (also: no block leaves while another still reads its totals)
+    else __syncthreads();
+    if constexpr (NG == 1) load_h(0);
+  } else {
+    for (int n = 0; n < NP; ++n)
+      sH[n * 32 + lane] = (p.h_start != nullptr && n < N) ? p.h_start[(seg_row + c_ld) * N + n] : 0.f;
+    if constexpr (NG == 1) load_h(0);
+  }
+  if (summary) return;
+
+  // ---- the sweep proper
+  if (full) sweep(std::true_type{}, p.ckpt != nullptr);
+  else sweep(std::false_type{}, true);
+  if (full && p.h_last != nullptr && valid && t_begin < t_end && t_end == p.L) {
+    if constexpr (NG == 1) store_h(0);
+    for (int n = 0; n < N; ++n) p.h_last[((size_t)b * D + c_own) * N + n] = sH[n * 32 + lane];
+  }
+}
+
+template <typename IO, int NG, bool VEC>
+cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int mode, cudaStream_t s) {
+  auto kern = ssm_fwd_lane_kernel<IO, NG, VEC>;
+  const int steps = plan.nseg > 1 ? plan.seg_steps : p.L;
+  const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
+  const LaneSplit sp = choose_lane_split(chains, steps, 0.75f, NG > 2 ? 2 : 3);
+  const int per_block = kLaneWarps / sp.warps;
+  const size_t smem = FwdLaneSmem<IO, NG>::bytes(kLaneWarps, per_block);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)((chains + per_block - 1) / per_block * sp.cluster));
+  cfg.blockDim = dim3(32 * kLaneWarps);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = sp.cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = sp.cluster > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, p, sp, N, mode);
+}
+
+template <typename IO, int NG>
+cudaError_t launch_fwd_lane_vec(const Plan& plan, const FwdParams& p, int N, int mode, cudaStream_t s) {
+  // 16-byte row pieces need aligned rows and at least one whole vector of channels
+  bool vec = (size_t)p.D * sizeof(IO) % 16 == 0;
+  for (const void* q : {p.x, p.delta, p.z, (const void*)p.out}) vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
+  return vec ? launch_fwd_lane_n<IO, NG, true>(plan, p, N, mode, s) : launch_fwd_lane_n<IO, NG, false>(plan, p, N, mode, s);
+}
+
+template <typename IO>
+cudaError_t launch_fwd_lane_io(const Plan& plan, const FwdParams& p, int N, int mode, cudaStream_t s) {
+  if (N <= 16) return launch_fwd_lane_vec<IO, 1>(plan, p, N, mode, s);
+  if (N <= 32) return launch_fwd_lane_vec<IO, 2>(plan, p, N, mode, s);
+  return launch_fwd_lane_vec<IO, 4>(plan, p, N, mode, s);
+}
+
+}  // namespace
+
+LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm) {
+  // run time of 1, 2, 3 warps on a sub-partition relative to one (measured on these kernels)
+  static const float slow[4] = {1.0f, 1.0f, 1.5f, 2.1f};
+  LaneSplit best{1, 1, (steps + kLB - 1) / kLB * kLB};
+  float best_t = 0.f;
+  for (int cl = 1; cl <= kLaneMaxCluster; cl *= 2) {
+    for (int w = cl > 1 ? kLaneWarps : 1; w <= kLaneWarps; w *= 2) {
+      const int pieces = cl * w;
+      const int piece = ((steps + pieces - 1) / pieces + kLB - 1) / kLB * kLB;
+      if (pieces > 1 && (long long)piece * (pieces - w) >= steps) continue;   // the last block would be idle
+      const long long blocks = (chains * w + kLaneWarps - 1) / kLaneWarps * cl;
+      const long long per = (blocks + kNumSMs - 1) / kNumSMs;     // blocks on the fullest SM
+      const long long waves = (per + blocks_per_sm - 1) / blocks_per_sm;
+      float t = (float)piece * (pieces > 1 ? 1.f + extra : 1.f) * slow[per < blocks_per_sm ? per : blocks_per_sm] * (float)waves;
+      if (pieces > 1) t += 8.f + (cl > 1 ? 8.f + (float)cl : 0.f);   // the fold, in steps
+      if (best_t == 0.f || t < best_t) {
+        best_t = t;
+        best = LaneSplit{w, cl, piece};
+      }
+    }
+  }
+  return best;
+}
+
+bool fwd_lane_applicable(const ssm_problem_t& prob, const FwdParams& p) {
+  return !p.zoh && !p.static_B && !p.static_C;
+}
+
+cudaError_t launch_fwd_lane(const ssm_problem_t& prob, const Plan& plan, const FwdParams& p, int mode, cudaStream_t s) {
+  if (prob.io_dtype == SSM_BF16) return launch_fwd_lane_io<__nv_bfloat16>(plan, p, prob.N, mode, s);
+  return launch_fwd_lane_io<float>(plan, p, prob.N, mode, s);
+}
+
+}  // namespace ssm

@@ -1,0 +1,196 @@
+// Pieces shared by the lane-per-channel kernels (ssm_fwd_lane.cu, ssm_bwd_lane.cu): element loads and stores of either io
+// dtype at any alignment, the staging of B and C, and the split of a chain over the warps of a cluster.
+//
+// These kernels take what the tuned bf16 / N = 16 kernels do not: float32 io, any D and any pointer alignment, any
+// N (states are handled 16 at a time; N < 16 is padded with states that stay zero).  x, delta, z, dout go straight from
+// global memory to the lane that owns the channel (a warp's 32 lanes read one contiguous row piece, so no alignment
+// beyond the element's is needed), one batch of 8 steps ahead of its use; only B and C, which every lane needs, pass
+// through shared memory.
+//
+// A chain is 32 adjacent channels of one batch entry (of one time segment of the launch, if the launch is split in
+// time).  When the chains alone cannot fill the GPU a chain is cut in time between the W warps of a block and the blocks
+// of a cluster: every warp sweeps its piece from a zero state, the (decay, end state) pairs are folded through
+// (distributed) shared memory, and every warp sweeps its piece again from the true state.  That costs what the summary
+// launch of a time split costs, but no carry launch and no round trip through global memory, and pieces may be as short
+// as one batch.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
+#include "ssm_common.cuh"
+
+namespace ssm {
+
+constexpr int kLB = kCkptSteps;   // steps per batch of the lane kernels (= checkpoint spacing)
+constexpr int kLaneChannels = 32; // channels per chain
+
+// How a launch cuts its chains: `cluster` blocks of `warps` warps share a chain, each warp takes `piece` steps.  Blocks
+// always have kLaneWarps warps (a warp's place in its block decides its SM sub-partition, so smaller blocks would pile up
+// on one): with warps < kLaneWarps a block holds several chains.
+constexpr int kLaneWarps = 4, kLaneMaxCluster = 8;
+struct LaneSplit {
+  int warps, cluster, piece;
+};
+// Split with the shortest estimated run.  `extra`: cost of the first sweep over a piece relative to the second.
+LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm);
+
+#ifdef __CUDACC__
+template <typename IO>
+struct LaneRaw;
+template <>
+struct LaneRaw<float> {
+  using T = float;
+  static __device__ __forceinline__ T load(const float* p) { return __ldg(p); }
+  static __device__ __forceinline__ float widen(T v) { return v; }
+};
+template <>
+struct LaneRaw<__nv_bfloat16> {
+  using T = unsigned short;
+  static __device__ __forceinline__ T load(const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const unsigned short*>(p)); }
+  static __device__ __forceinline__ float widen(T v) { return __uint_as_float((uint32_t)v << 16); }
+};
+
+// Four adjacent elements of a B / C row, still in the io dtype.  `n` of them exist; vec: the row pieces are aligned to
+// four elements.
+template <typename IO>
+struct LaneQuad;
+template <>
+struct LaneQuad<float> {
+  float4 v;
+  __device__ __forceinline__ void load(const float* p, int n, bool vec) {
+    v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (n >= 4 && vec) {
+      v = __ldg(reinterpret_cast<const float4*>(p));
+    } else {
+      if (n > 0) v.x = __ldg(p);
+      if (n > 1) v.y = __ldg(p + 1);
+      if (n > 2) v.z = __ldg(p + 2);
+      if (n > 3) v.w = __ldg(p + 3);
+    }
+  }
+  __device__ __forceinline__ float4 widen() const { return v; }
+};
+template <>
+struct LaneQuad<__nv_bfloat16> {
+  uint2 v;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p, int n, bool vec) {
+    v = make_uint2(0u, 0u);
+    if (n >= 4 && vec) {
+      v = __ldg(reinterpret_cast<const uint2*>(p));
+    } else {
+      const unsigned short* q = reinterpret_cast<const unsigned short*>(p);
+      if (n > 0) v.x = __ldg(q);
+      if (n > 1) v.x |= (uint32_t)__ldg(q + 1) << 16;
+      if (n > 2) v.y = __ldg(q + 2);
+      if (n > 3) v.y |= (uint32_t)__ldg(q + 3) << 16;
+    }
+  }
+  __device__ __forceinline__ float4 widen() const { return make_float4(bf16lo(v.x), bf16hi(v.x), bf16lo(v.y), bf16hi(v.y)); }
+};
+
+// The warp index, in a form the compiler can see is the same in all lanes
+// (a warp reduction lands in a uniform register, so addresses built on it cost no vector instructions)
+__device__ __forceinline__ int uniform_warp() { return __reduce_max_sync(0xffffffffu, (int)(threadIdx.x >> 5)); }
+
+template <typename T>
+__device__ __forceinline__ T* at_bytes(T* base, unsigned bytes) {
+  using C = typename std::conditional<std::is_const<T>::value, const char, char>::type;
+  return reinterpret_cast<T*>(reinterpret_cast<C*>(base) + bytes);
+}
+
+// A batch of 8 rows of 32 channels of one tensor, in flight from global memory.  VEC (rows are 16-byte aligned): the warp
+// reads it with 16-byte loads, 8 / EPV x 32 lanes of them per row, and passes it through shared memory to the lanes that
+// own the channels; otherwise every lane reads its own channel row by row.
+template <typename IO, bool VEC>
+struct LaneRows {
+  static constexpr int EPV = 16 / (int)sizeof(IO);   // elements of a 16-byte vector
+  static constexpr int VPR = 32 / EPV;               // vectors of a row piece
+  static constexpr int NV = kLB * VPR / 32;          // vectors per lane
+  using RawT = typename LaneRaw<IO>::T;
+  uint4 v[VEC ? NV : 1];
+  RawT r[VEC ? 1 : kLB];
+  // base: first row of the batch and first channel of the group; `last`: last row that exists (rows past it repeat it);
+  // `cols`: channels of the group that exist (lanes past them read existing ones)
+  __device__ __forceinline__ void load(const IO* base, int D, int lane, int last, int cols) {
+    if constexpr (VEC) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        const int q = lane + 32 * i, row = min(q / VPR, last), col = min(q % VPR * EPV, cols - EPV);
+        v[i] = __ldg(reinterpret_cast<const uint4*>(base + (size_t)row * D + col));
+      }
+    } else {
+      const IO* p = base + min(lane, cols - 1);
+      if (last >= kLB - 1) {
+#pragma unroll
+        for (int t = 0; t < kLB; ++t) r[t] = LaneRaw<IO>::load(at_bytes(p, (unsigned)t * (unsigned)D * (unsigned)sizeof(IO)));
+      } else {
+#pragma unroll
+        for (int t = 0; t < kLB; ++t)
+          r[t] = LaneRaw<IO>::load(at_bytes(p, (unsigned)min(t, last) * (unsigned)D * (unsigned)sizeof(IO)));
+      }
+    }
+  }
+  __device__ __forceinline__ void zero() {
+    if constexpr (VEC) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) v[i] = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+#pragma unroll
+      for (int t = 0; t < kLB; ++t) r[t] = RawT(0);
+    }
+  }
+  // into the tile [kLB][32] (VEC only)
+  __device__ __forceinline__ void put(IO* tile, int lane) const {
+    if constexpr (VEC) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) reinterpret_cast<uint4*>(tile)[lane + 32 * i] = v[i];
+    }
+  }
+  // this lane's value of row t
+  __device__ __forceinline__ float get(const IO* tile, int t, int lane) const {
+    if constexpr (VEC) return LaneRaw<IO>::widen(reinterpret_cast<const RawT*>(tile)[t * 32 + lane]);
+    else return LaneRaw<IO>::widen(r[t]);
+  }
+};
+// The way back: results of a batch, collected in a tile (VEC) and written with 16-byte stores, or written one by one.
+template <typename IO, bool VEC>
+struct LaneOut {
+  using R = LaneRows<IO, VEC>;
+  static __device__ __forceinline__ void put(IO* tile, IO* base, int D, int t, int lane, bool ok, float v) {
+    if constexpr (VEC) tile[t * 32 + lane] = float_to_io<IO>(v);
+    else if (ok) *at_bytes(base + lane, (unsigned)t * (unsigned)D * (unsigned)sizeof(IO)) = float_to_io<IO>(v);
+  }
+  // after a __syncwarp
+  static __device__ __forceinline__ void flush(const IO* tile, IO* base, int D, int lane, int live, int cols) {
+    if constexpr (VEC) {
+#pragma unroll
+      for (int i = 0; i < R::NV; ++i) {
+        const int q = lane + 32 * i, row = q / R::VPR, col = q % R::VPR * R::EPV;
+        if (row < live && col < cols)
+          *reinterpret_cast<uint4*>(base + (size_t)row * D + col) = reinterpret_cast<const uint4*>(tile)[q];
+      }
+    }
+  }
+};
+
+// step size from the staged value: float32 io keeps the precise logarithm
+template <typename IO>
+__device__ __forceinline__ float lane_softplus(float v) {
+  if constexpr (sizeof(IO) == 4) return softplus_precise(v);
+  else return softplus_fast(v);
+}
+
+// 16 floats of a shared-memory row as packed pairs
+__device__ __forceinline__ void load16(const float* row, float2 (&v)[8]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float4 a = *reinterpret_cast<const float4*>(row + 4 * k);
+    v[2 * k] = make_float2(a.x, a.y);
+    v[2 * k + 1] = make_float2(a.z, a.w);
+  }
+}
+#endif
+
+}  // namespace ssm
