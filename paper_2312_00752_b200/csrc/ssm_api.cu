@@ -3,6 +3,7 @@
 #include <algorithm>
 
 #include "ssm_common.cuh"
+#include "ssm_lane.cuh"
 
 namespace ssm {
 
@@ -25,6 +26,7 @@ int fwd_states_per_thread();
 int fwd_fast_channels_per_warp();
 int bwd_fast_channels_per_warp();
 bool bwd_fast_applicable(const ssm_problem_t& prob, const BwdParams& p);
+bool bwd_lane_applicable(const BwdParams& p);
 // ssm_repack.cu
 enum { kRepackBf16 = 0, kRepackF32 = 1, kRepackA = 2 };
 constexpr int kRepackMax = 6;
@@ -170,7 +172,36 @@ Plan make_plan(const ssm_problem_t& p) {
   seg_steps = (seg_steps + kSegAlign - 1) / kSegAlign * kSegAlign;
   pl.seg_steps = seg_steps;
   pl.nseg = (p.L + seg_steps - 1) / seg_steps;
+  pl.split = LaneSplit{1, 1, seg_steps};
   return pl;
+}
+
+// Time split of the lane backward kernel: inside clusters (one launch, for little work) or into segments of the launch
+// with a pre-pass of its own (which runs at twice the occupancy).  Costs in steps of a lone warp of the main kernel:
+// segments are chosen to fill whole waves of two blocks per SM; two warps on a sub-partition take 1.45 times as long each;
+// the pre-pass is a quarter of the work spread over all sub-partitions, its two launches 15 steps.
+static void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl) {
+  const long long chains = (long long)p.batch * pl->bwd_groups;
+  auto align8 = [](long long v) { return (int)((v + kCkptSteps - 1) / kCkptSteps * kCkptSteps); };
+  pl->nseg = 1;
+  pl->seg_steps = (p.L + kSegAlign - 1) / kSegAlign * kSegAlign;
+  float best;
+  pl->split = choose_lane_split(chains, p.L, 0.3f, 2, teams, &best);
+  const long long wave = 2LL * kNumSMs * teams;   // pieces the GPU holds
+  const float prepass = 15.f + 0.22f * (float)chains * (float)(kLaneWarps / teams) * (float)p.L / (4.f * kNumSMs);
+  for (int half = 1; half <= 12; ++half) {        // half waves: one block per SM, then whole waves
+    if (half > 1 && half % 2) continue;
+    const long long most = std::min<long long>(std::min<long long>(half * wave / 2 / chains, p.L / 64), 65535);
+    if (most < 2) continue;
+    const int seg = align8((p.L + most - 1) / most), nseg = (p.L + seg - 1) / seg;
+    const float t = (float)seg * (half == 1 ? 1.f : 1.45f * (float)(half / 2)) + prepass;
+    if (t < best) {
+      best = t;
+      pl->nseg = nseg;
+      pl->seg_steps = seg;
+      pl->split = LaneSplit{1, 1, seg};
+    }
+  }
 }
 
 static long long generic_bwd_warps(int N) {   // warps of a block of the generic backward kernel
@@ -183,6 +214,13 @@ static long long generic_bwd_warps(int N) {   // warps of a block of the generic
 // it pays when the chains alone leave the SM sub-partitions with too few warps.  Segments are at least 256 steps.
 Plan make_bwd_plan(const ssm_problem_t& p) {
   Plan pl = make_plan(p);
+  if (lane_shape(p)) {
+    const int ng = p.N <= 16 ? 1 : (p.N <= 32 ? 2 : 4);   // warps of a team
+    pl.bwd_ch = kLaneChannels;
+    pl.bwd_groups = (p.D + kLaneChannels - 1) / kLaneChannels;
+    plan_lane_bwd(p, kLaneWarps / ng, &pl);
+    return pl;
+  }
   if (tuned_shape(p)) {
     // the tuned kernel's chains (and the channel groups of its dB / dC partial sums) are narrower than the generic ones
     pl.bwd_ch = bwd_fast_channels_per_warp();
@@ -209,6 +247,7 @@ Plan make_bwd_plan(const ssm_problem_t& p) {
   }
   int seg_steps = (p.L + nseg - 1) / nseg;
   seg_steps = (seg_steps + kSegAlign - 1) / kSegAlign * kSegAlign;
+  pl.split = LaneSplit{1, 1, seg_steps};
   pl.seg_steps = seg_steps;
   pl.nseg = (p.L + seg_steps - 1) / seg_steps;
   return pl;
@@ -270,21 +309,21 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
     return at;
   };
   const size_t bln = (size_t)p.batch * p.L * p.N;
-  const size_t parts = (size_t)p.batch * pl.nseg;
+  const size_t segs = (size_t)p.batch * pl.nseg, parts = segs * pl.split.cluster;
   w.dBC_part = take((size_t)pl.bwd_groups * 2 * bln * sizeof(float));
   w.dA_part = take(parts * p.D * p.N * sizeof(float));
   w.dD_part = take(parts * p.D * sizeof(float));
   w.dbias_part = take(parts * p.D * sizeof(float));
   w.ckpt = take((size_t)p.batch * pl.nck * ckpt_floats_per_step(ckpt_tiled(p), p.D, p.N) * sizeof(float));
   if (pl.nseg > 1) {
-    const size_t st = parts * p.D * p.N * sizeof(float);
+    const size_t st = segs * p.D * p.N * sizeof(float);
     w.seg_local = take(st);
     w.mu_in = take(st);
-    w.seg_dsum = take(parts * p.D * sizeof(float));
+    w.seg_dsum = take(segs * p.D * sizeof(float));
   }
   w.fwd = take(fwd_layout(p, pl_fwd).total);   // the forward sweep that rebuilds checkpoints uses the forward split
   // (batch, segment, channel group) chains of the tuned kernel; SSM_FLAG_TEST_WITHHOLD forces chains to be shared
-  const long long chains = (long long)parts * pl.bwd_groups;
+  const long long chains = (long long)segs * pl.bwd_groups;
   w.max_workers = !tuned_shape(p) ? 0 : (p.flags & SSM_FLAG_TEST_WITHHOLD) ? (int)std::max<long long>(1, (2 * chains + 2) / 3)
                                                                             : shared_workers(chains);
   w.flags = take((size_t)2 * (w.max_workers + 1) * sizeof(int));   // backward kernel | adjoint pre-pass
@@ -757,8 +796,8 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
     if (launch_carry(cp, s) != cudaSuccess) return SSM_ERR_CUDA;
     bp.mu_in = cp.carried;
   }
-  // the generic kernel (taken when a pointer is not 16-byte aligned) writes one partial sum per 32 channels
-  if (!bwd_fast_applicable(*p, bp)) bp.groups = (p->D + bwd_channels_per_block(p->N) - 1) / bwd_channels_per_block(p->N);
+  // the generic kernel (ZOH or parameter B / C off the tuned shapes) writes one partial sum per block of its own width
+  if (!bwd_fast_applicable(*p, bp) && !bwd_lane_applicable(bp)) bp.groups = (p->D + bwd_channels_per_block(p->N) - 1) / bwd_channels_per_block(p->N);
   if (launch_bwd(*p, pl, bp, kBwdFull, s) != cudaSuccess) return SSM_ERR_CUDA;
 
   ReduceParams rp{};
@@ -777,7 +816,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   rp.dbias = ddelta_bias;
   rp.bln = (long long)p->batch * p->L * p->N;
   rp.groups = bp.groups;
-  rp.parts = p->batch * pl.nseg;
+  rp.parts = p->batch * pl.nseg * pl.split.cluster;
   rp.D = p->D;
   rp.N = p->N;
   if (launch_bwd_reduce(*p, rp, s) != cudaSuccess) return SSM_ERR_CUDA;

@@ -22,6 +22,11 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kNumSMs = 148;
 
 // ---------------------------------------------------------------------------------------------- plan (host)
+// How a launch of the lane-per-channel kernels cuts its chains (ssm_lane.cuh): `cluster` blocks share a chain, `warps`
+// warps (or teams of warps) of each of them, and each takes `piece` steps.
+struct LaneSplit {
+  int warps, cluster, piece;
+};
 struct Plan {
   int nseg;        // time segments per sequence (1: a thread sweeps the whole sequence)
   int seg_steps;   // steps per segment (multiple of kSegAlign; the last segment may be shorter)
@@ -30,6 +35,7 @@ struct Plan {
   int fwd_ch;      // channels per block, forward
   int bwd_ch;      // channels per block, backward (= channel-group size of the dB/dC partial sums)
   int bwd_groups;  // ceil(D / bwd_ch)
+  LaneSplit split; // lane-per-channel kernels only (of the direction the plan is for)
 };
 Plan make_plan(const ssm_problem_t& p);
 
@@ -124,13 +130,13 @@ struct BwdParams {
   void* ddelta;
   void* dz;               // null: not produced
   float* dBC_part;        // [groups][2][batch*L*N] float partial sums over the channels of one block
-  float* dA_part;         // [batch*nseg][D][N]
-  float* dD_part;         // [batch*nseg][D]
+  float* dA_part;         // [batch*nseg*cluster][D][N] (cluster: 1 but for the lane kernel, which has one sum per block)
+  float* dD_part;         // [batch*nseg*cluster][D]
   int batch, L, D, nseg, seg_steps, nck, groups;
   int general_A;          // 1: never take the arithmetic-progression fast path
   const float* delta_bias;  // as in FwdParams
   int softplus;
-  float* dbias_part;      // [batch*nseg][D] sums of the pre-activation gradient; null: not wanted
+  float* dbias_part;      // like dD_part: sums of the pre-activation gradient; null: not wanted
   float* dh0;             // [batch][D][N] gradient of the initial state (the adjoint mu that leaves the first step);
                           // null: not wanted
   int zoh;                // as in FwdParams

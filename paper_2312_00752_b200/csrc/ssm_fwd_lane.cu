@@ -399,7 +399,7 @@ cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int m
   auto kern = ssm_fwd_lane_kernel<IO, NG, VEC>;
   const int steps = plan.nseg > 1 ? plan.seg_steps : p.L;
   const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
-  const LaneSplit sp = choose_lane_split(chains, steps, 0.75f, NG > 2 ? 2 : 3);
+  const LaneSplit sp = choose_lane_split(chains, steps, 0.75f, NG > 2 ? 2 : 3, kLaneWarps);
   const int per_block = kLaneWarps / sp.warps;
   const size_t smem = FwdLaneSmem<IO, NG>::bytes(kLaneWarps, per_block);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
@@ -435,17 +435,17 @@ cudaError_t launch_fwd_lane_io(const Plan& plan, const FwdParams& p, int N, int 
 
 }  // namespace
 
-LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm) {
+LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm, int teams, float* cost) {
   // run time of 1, 2, 3 warps on a sub-partition relative to one (measured on these kernels)
   static const float slow[4] = {1.0f, 1.0f, 1.5f, 2.1f};
   LaneSplit best{1, 1, (steps + kLB - 1) / kLB * kLB};
   float best_t = 0.f;
   for (int cl = 1; cl <= kLaneMaxCluster; cl *= 2) {
-    for (int w = cl > 1 ? kLaneWarps : 1; w <= kLaneWarps; w *= 2) {
+    for (int w = cl > 1 ? teams : 1; w <= teams; w *= 2) {
       const int pieces = cl * w;
       const int piece = ((steps + pieces - 1) / pieces + kLB - 1) / kLB * kLB;
       if (pieces > 1 && (long long)piece * (pieces - w) >= steps) continue;   // the last block would be idle
-      const long long blocks = (chains * w + kLaneWarps - 1) / kLaneWarps * cl;
+      const long long blocks = (chains * w + teams - 1) / teams * cl;
       const long long per = (blocks + kNumSMs - 1) / kNumSMs;     // blocks on the fullest SM
       const long long waves = (per + blocks_per_sm - 1) / blocks_per_sm;
       float t = (float)piece * (pieces > 1 ? 1.f + extra : 1.f) * slow[per < blocks_per_sm ? per : blocks_per_sm] * (float)waves;
@@ -456,6 +456,7 @@ LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks
       }
     }
   }
+  if (cost != nullptr) *cost = best_t;
   return best;
 }
 

@@ -26,15 +26,13 @@ namespace ssm {
 constexpr int kLB = kCkptSteps;   // steps per batch of the lane kernels (= checkpoint spacing)
 constexpr int kLaneChannels = 32; // channels per chain
 
-// How a launch cuts its chains: `cluster` blocks of `warps` warps share a chain, each warp takes `piece` steps.  Blocks
-// always have kLaneWarps warps (a warp's place in its block decides its SM sub-partition, so smaller blocks would pile up
-// on one): with warps < kLaneWarps a block holds several chains.
+// Blocks always have kLaneWarps warps (a warp's place in its block decides its SM sub-partition, so smaller blocks would
+// pile up on one); with fewer warps on a chain than that a block holds several chains.
 constexpr int kLaneWarps = 4, kLaneMaxCluster = 8;
-struct LaneSplit {
-  int warps, cluster, piece;
-};
-// Split with the shortest estimated run.  `extra`: cost of the first sweep over a piece relative to the second.
-LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm);
+// Split with the shortest estimated run.  `extra`: cost of the first sweep over a piece relative to the second; `teams`:
+// pieces a block holds (a piece is swept by one warp, or by a team of warps that share its states); `cost`: the estimate,
+// in steps of a lone warp.
+LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm, int teams, float* cost = nullptr);
 
 #ifdef __CUDACC__
 template <typename IO>

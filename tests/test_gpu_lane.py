@@ -23,6 +23,8 @@ pytestmark = pytest.mark.gpu
     (5, 40, 2048, 16, "f32"),      # more chains than SM sub-partitions: several chains per block, no split
     (1, 4133, 20, 16, "f32"),      # the launch itself split in time (summary and carry)
     (1, 4100, 33, 64, "bf16"),
+    (2, 707, 1001, 16, "bf16"),    # backward split into segments with a pre-pass: odd rows, ragged last segment
+    (1, 650, 1300, 32, "f32"),
 ])
 def test_edges(batch, L, D, N, io):
     cfg = synth.ScanConfig("lane", 21, batch, L, D, N, io, 1e-3, 1e-1)
