@@ -2,6 +2,8 @@
 
 Every step of the selective scan runs in the CUDA kernels of libssm_scan.so; torch is used for device memory and
 streams.  There is no CPU or eager fallback: if the library is missing or fails to load, importing a symbol raises.
+The calls that launch kernels marshal their arguments in a compiled module (csrc/marshal.cpp); queries, and the call on
+host buffers, go through ctypes.
 """
 from __future__ import annotations
 
@@ -49,6 +51,7 @@ class SsmScanError(RuntimeError):
 
 
 _lib = None
+_library_path = None   # of the loaded library
 
 
 def library_path() -> str:
@@ -57,7 +60,7 @@ def library_path() -> str:
 
 def load_library() -> ctypes.CDLL:
     """dlopen libssm_scan.so (building it first if nvcc is present and the sources are newer)."""
-    global _lib
+    global _lib, _library_path
     if _lib is not None:
         return _lib
     path = os.environ.get("SSM_SCAN_LIBRARY")    # e.g. the bounds-checking build (build.DEBUG_LIB_PATH)
@@ -68,6 +71,7 @@ def load_library() -> ctypes.CDLL:
     if not os.path.exists(path):
         raise SsmScanError(f"{path} is missing and nvcc is not available to build it; there is no fallback path")
     lib = ctypes.CDLL(path)
+    _library_path = path
     P = ctypes.POINTER(ssm_problem_t)
     vp, sz = ctypes.c_void_p, ctypes.c_size_t
     for name in ("ssm_scan_fwd_workspace_bytes", "ssm_scan_bwd_workspace_bytes", "ssm_scan_saved_state_bytes",
@@ -158,23 +162,22 @@ def _dev_ptr(t, name, shape=None, dtype=None):
     return ctypes.c_void_p(t.data_ptr())
 
 
-_workspaces: dict = {}
+_marshal_module = None
 
 
-def _workspace(nbytes: int, device, stream_ptr: int) -> torch.Tensor | None:
-    """Grow-only scratch buffer per (device, stream): calls on different streams never share scratch memory."""
-    if nbytes == 0:
-        return None
-    key = (str(device), int(stream_ptr))
-    ws = _workspaces.get(key)
-    if ws is None or ws.numel() < nbytes:
-        if ws is not None:
-            # kernels already enqueued on that stream may still use the old buffer: the caching allocator must not hand
-            # its memory to other work before they are done
-            ws.record_stream(torch.cuda.ExternalStream(int(stream_ptr), device=device))
-        ws = torch.empty(nbytes, dtype=torch.uint8, device=device)
-        _workspaces[key] = ws
-    return ws
+def _native():
+    """The compiled marshalling module, bound to the loaded library."""
+    global _marshal_module
+    if _marshal_module is None:
+        load_library()
+        if _build.marshal_is_stale() and shutil.which(os.environ.get("CXX", "g++")):
+            _build.build_marshal()
+        if not os.path.exists(_build.MARSHAL_PATH):
+            raise SsmScanError(f"{_build.MARSHAL_PATH} is missing and there is no compiler to build it; there is no fallback path")
+        from . import _marshal
+        _marshal.init(_library_path, SsmScanError, torch.OutOfMemoryError)
+        _marshal_module = _marshal
+    return _marshal_module
 
 
 def plan(problem: ssm_problem_t) -> dict:
@@ -221,32 +224,9 @@ def ssm_scan_fwd(x, delta, A, B, C, D_skip=None, z=None, *, save_states=False, g
     if a float32 tensor `h_last` (batch, D, N) is passed it receives the state after the last step
     (ssm_scan_fwd_state).
     """
-    lib = load_library()
-    prob = make_problem(x, B, z is not None, D_skip is not None, save_states, general_A, zoh, static_B, static_C,
-                        complex_state)
-    batch, L, D, N = prob.batch, prob.L, prob.D, prob.N
-    io = x.dtype
-    c2 = (2,) if complex_state else ()
-    bshape, bdt = ((D, N), torch.float32) if static_B else ((batch, L, N) + c2, io)   # static: a parameter like A
-    cshape, cdt = ((D, N), torch.float32) if static_C else ((batch, L, N) + c2, io)
-    if out is None:
-        out = torch.empty_like(x)
-    if save_states and saved_states is None:
-        saved_states = torch.empty(saved_state_bytes(prob) // 4, dtype=torch.float32, device=x.device)
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    need = fwd_workspace_bytes(prob)
-    ws = workspace if workspace is not None else _workspace(need, x.device, stream_ptr)
-    code = lib.ssm_scan_fwd_state(
-        ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io), _dev_ptr(delta, "delta", (batch, L, D), io),
-        _dev_ptr(A, "A", (D, N) + c2, torch.float32), _dev_ptr(B, "B", bshape, bdt),
-        _dev_ptr(C, "C", cshape, cdt), _dev_ptr(D_skip, "D_skip", (D,), torch.float32),
-        _dev_ptr(z, "z", (batch, L, D), io), _dev_ptr(h0, "h0", (batch, D, N) + c2, torch.float32),
-        _dev_ptr(out, "out", (batch, L, D), io), _dev_ptr(h_last, "h_last", (batch, D, N) + c2, torch.float32),
-        _dev_ptr(saved_states if save_states else None, "saved_states"),
-        _dev_ptr(ws, "workspace"), ctypes.c_size_t(0 if ws is None else ws.numel() * ws.element_size()),
-        ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_scan_fwd_state")
-    return (out, saved_states) if save_states else out
+    return (_marshal_module or _native()).fwd(
+        x, delta, None, A, B, C, D_skip, z, h0, out, h_last, saved_states, workspace, stream, save_states, general_A, zoh,
+        static_B, static_C, complex_state, False, 0)
 
 
 def ssm_scan_fwd_fused_dt(x, delta_pre, delta_bias, A, B, C, D_skip=None, z=None, *, softplus=True, save_states=False,
@@ -254,32 +234,9 @@ def ssm_scan_fwd_fused_dt(x, delta_pre, delta_bias, A, B, C, D_skip=None, z=None
                           static_C=False):
     """Forward with the step-size activation fused: delta = softplus(delta_pre + delta_bias) (or the plain sum with
     softplus=False), in float32.  Otherwise as ssm_scan_fwd (static_B / static_C: B / C float32 (D, N))."""
-    lib = load_library()
-    prob = make_problem(x, B, z is not None, D_skip is not None, save_states, False, zoh, static_B, static_C)
-    if softplus:
-        prob.flags |= SSM_FLAG_DELTA_SOFTPLUS
-    batch, L, D, N = prob.batch, prob.L, prob.D, prob.N
-    io = x.dtype
-    bshape, bdt = ((D, N), torch.float32) if static_B else ((batch, L, N), io)
-    cshape, cdt = ((D, N), torch.float32) if static_C else ((batch, L, N), io)
-    if out is None:
-        out = torch.empty_like(x)
-    if save_states and saved_states is None:
-        saved_states = torch.empty(saved_state_bytes(prob) // 4, dtype=torch.float32, device=x.device)
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    ws = _workspace(fwd_workspace_bytes(prob), x.device, stream_ptr)
-    code = lib.ssm_scan_fwd_fused_dt(
-        ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io), _dev_ptr(delta_pre, "delta_pre", (batch, L, D), io),
-        _dev_ptr(delta_bias, "delta_bias", (D,), torch.float32), _dev_ptr(A, "A", (D, N), torch.float32),
-        _dev_ptr(B, "B", bshape, bdt), _dev_ptr(C, "C", cshape, cdt),
-        _dev_ptr(D_skip, "D_skip", (D,), torch.float32), _dev_ptr(z, "z", (batch, L, D), io),
-        _dev_ptr(h0, "h0", (batch, D, N), torch.float32), _dev_ptr(out, "out", (batch, L, D), io),
-        _dev_ptr(h_last, "h_last", (batch, D, N), torch.float32),
-        _dev_ptr(saved_states if save_states else None, "saved_states"),
-        _dev_ptr(ws, "workspace"), ctypes.c_size_t(0 if ws is None else ws.numel() * ws.element_size()),
-        ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_scan_fwd_fused_dt")
-    return (out, saved_states) if save_states else out
+    return (_marshal_module or _native()).fwd(
+        x, delta_pre, delta_bias, A, B, C, D_skip, z, h0, out, h_last, saved_states, None, stream, save_states, False, zoh,
+        static_B, static_C, False, softplus, 1)
 
 
 def ssm_scan_bwd_fused_dt(x, delta_pre, delta_bias, A, B, C, D_skip, z, dout, saved_states=None, *, softplus=True,
@@ -287,80 +244,17 @@ def ssm_scan_bwd_fused_dt(x, delta_pre, delta_bias, A, B, C, D_skip, z, dout, sa
                           static_C=False):
     """Backward of ssm_scan_fwd_fused_dt.  Returns the dict of ssm_scan_bwd with `ddelta` the gradient of delta_pre
     and an extra `ddelta_bias` (D,) float32.  h0, dh_last, want_dh0 as in ssm_scan_bwd (ssm_scan_bwd_fused_dt_state)."""
-    lib = load_library()
-    prob = make_problem(x, B, z is not None, D_skip is not None, False, False, zoh, static_B, static_C)
-    if softplus:
-        prob.flags |= SSM_FLAG_DELTA_SOFTPLUS
-    batch, L, D, N = prob.batch, prob.L, prob.D, prob.N
-    io = x.dtype
-    bshape, bdt = ((D, N), torch.float32) if static_B else ((batch, L, N), io)
-    cshape, cdt = ((D, N), torch.float32) if static_C else ((batch, L, N), io)
-    o = {"dx": torch.empty_like(x), "ddelta": torch.empty_like(x),
-         "ddelta_bias": torch.empty((D,), dtype=torch.float32, device=x.device),
-         "dA": torch.empty((D, N), dtype=torch.float32, device=x.device), "dB": torch.empty_like(B),
-         "dC": torch.empty_like(C),
-         "dD": torch.empty((D,), dtype=torch.float32, device=x.device) if D_skip is not None else None,
-         "dz": torch.empty_like(x) if z is not None else None}
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    ws = _workspace(bwd_workspace_bytes(prob), x.device, stream_ptr)
-    if h0 is not None or dh_last is not None or want_dh0:
-        f32 = torch.float32
-        if want_dh0:
-            o["dh0"] = torch.empty((batch, D, N), dtype=f32, device=x.device)
-        code = lib.ssm_scan_bwd_fused_dt_state(
-            ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io), _dev_ptr(delta_pre, "delta_pre", (batch, L, D), io),
-            _dev_ptr(delta_bias, "delta_bias", (D,), f32), _dev_ptr(A, "A", (D, N), f32),
-            _dev_ptr(B, "B", bshape, bdt), _dev_ptr(C, "C", cshape, cdt), _dev_ptr(D_skip, "D_skip", (D,), f32),
-            _dev_ptr(z, "z", (batch, L, D), io), _dev_ptr(dout, "dout", (batch, L, D), io),
-            _dev_ptr(h0, "h0", (batch, D, N), f32), _dev_ptr(dh_last, "dh_last", (batch, D, N), f32),
-            _dev_ptr(saved_states, "saved_states"), _dev_ptr(o["dx"], "dx"), _dev_ptr(o["ddelta"], "ddelta"),
-            _dev_ptr(o["ddelta_bias"], "ddelta_bias"), _dev_ptr(o["dA"], "dA"), _dev_ptr(o["dB"], "dB"),
-            _dev_ptr(o["dC"], "dC"), _dev_ptr(o["dD"], "dD"), _dev_ptr(o["dz"], "dz"), _dev_ptr(o.get("dh0"), "dh0"),
-            _dev_ptr(ws, "workspace"), ctypes.c_size_t(0 if ws is None else ws.numel() * ws.element_size()),
-            ctypes.c_void_p(stream_ptr))
-        _check(code, "ssm_scan_bwd_fused_dt_state")
-        return o
-    code = lib.ssm_scan_bwd_fused_dt(
-        ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io), _dev_ptr(delta_pre, "delta_pre", (batch, L, D), io),
-        _dev_ptr(delta_bias, "delta_bias", (D,), torch.float32), _dev_ptr(A, "A", (D, N), torch.float32),
-        _dev_ptr(B, "B", bshape, bdt), _dev_ptr(C, "C", cshape, cdt),
-        _dev_ptr(D_skip, "D_skip", (D,), torch.float32), _dev_ptr(z, "z", (batch, L, D), io),
-        _dev_ptr(dout, "dout", (batch, L, D), io), _dev_ptr(saved_states, "saved_states"),
-        _dev_ptr(o["dx"], "dx"), _dev_ptr(o["ddelta"], "ddelta"), _dev_ptr(o["ddelta_bias"], "ddelta_bias"),
-        _dev_ptr(o["dA"], "dA"), _dev_ptr(o["dB"], "dB"), _dev_ptr(o["dC"], "dC"), _dev_ptr(o["dD"], "dD"),
-        _dev_ptr(o["dz"], "dz"),
-        _dev_ptr(ws, "workspace"), ctypes.c_size_t(0 if ws is None else ws.numel() * ws.element_size()),
-        ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_scan_bwd_fused_dt")
-    return o
+    return (_marshal_module or _native()).bwd(
+        x, delta_pre, delta_bias, A, B, C, D_skip, z, dout, saved_states, h0, dh_last, None, stream, {}, False, zoh,
+        static_B, static_C, False, softplus, True, want_dh0, 0)
 
 
 def ssm_step(x, delta, A, B, C, D_skip, z, h, *, zoh=False, out=None, stream=None, static_B=False, static_C=False,
              complex_state=False):
     """One recurrent step: x, delta, z (batch, D), B, C (batch, N) io dtype; h (batch, D, N) float32 is updated in
     place.  Returns out (batch, D).  complex_state: A (D, N, 2), B, C (batch, N, 2), h (batch, D, N, 2)."""
-    lib = load_library()
-    batch, D = x.shape
-    N = B.shape[-2] if complex_state else B.shape[-1]
-    c2 = (2,) if complex_state else ()
-    prob = ssm_problem_t(batch, 1, D, N, _io_dtype(x),
-                         (SSM_FLAG_HAS_Z if z is not None else 0) | (SSM_FLAG_HAS_DSKIP if D_skip is not None else 0)
-                         | (SSM_FLAG_ZOH_BBAR if zoh else 0) | (SSM_FLAG_STATIC_B if static_B else 0)
-                         | (SSM_FLAG_STATIC_C if static_C else 0) | (SSM_FLAG_COMPLEX if complex_state else 0))
-    io = x.dtype
-    if out is None:
-        out = torch.empty_like(x)
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    code = lib.ssm_step(
-        ctypes.byref(prob), _dev_ptr(x, "x", (batch, D), io), _dev_ptr(delta, "delta", (batch, D), io),
-        _dev_ptr(A, "A", (D, N) + c2, torch.float32),
-        _dev_ptr(B, "B", (D, N) if static_B else (batch, N) + c2, torch.float32 if static_B else io),
-        _dev_ptr(C, "C", (D, N) if static_C else (batch, N) + c2, torch.float32 if static_C else io),
-        _dev_ptr(D_skip, "D_skip", (D,), torch.float32), _dev_ptr(z, "z", (batch, D), io),
-        _dev_ptr(h, "h", (batch, D, N) + c2, torch.float32), _dev_ptr(out, "out", (batch, D), io),
-        ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_step")
-    return out
+    return (_marshal_module or _native()).step(x, delta, A, B, C, D_skip, z, h, out, stream, zoh, static_B, static_C,
+                                               complex_state)
 
 
 def check_status(problem: ssm_problem_t, workspace: torch.Tensor, stream=None) -> None:
@@ -372,8 +266,10 @@ def check_status(problem: ssm_problem_t, workspace: torch.Tensor, stream=None) -
 
 def last_bwd_workspace(device, stream=None):
     """The cached workspace tensor the binding used for calls on (device, stream), or None."""
+    device = torch.device(device)
+    index = device.index if device.index is not None else torch.cuda.current_device()
     stream_ptr = (stream if stream is not None else torch.cuda.current_stream(device)).cuda_stream
-    return _workspaces.get((str(device), int(stream_ptr)))
+    return _native().workspace(index, int(stream_ptr))
 
 
 def ssm_scan_fwd_static(x, delta, A, B, C, D_skip=None, z=None, *, save_states=False, general_A=False, out=None,
@@ -382,23 +278,9 @@ def ssm_scan_fwd_static(x, delta, A, B, C, D_skip=None, z=None, *, save_states=F
     when `out` (and `saved_states`, if asked for) are passed in.  The scratch memory is the fixed array inside the
     library (SSM_STATIC_SCRATCH_BYTES); a problem that needs more raises SsmScanError (SSM_ERR_WORKSPACE).  Calls that
     may overlap on the GPU must be ordered by the caller, because they share that array."""
-    lib = load_library()
-    prob = make_problem(x, B, z is not None, D_skip is not None, save_states, general_A)
-    batch, L, D, N = prob.batch, prob.L, prob.D, prob.N
-    io = x.dtype
-    if out is None:
-        out = torch.empty_like(x)
-    if save_states and saved_states is None:
-        saved_states = torch.empty(saved_state_bytes(prob) // 4, dtype=torch.float32, device=x.device)
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    code = lib.ssm_scan_fwd_static(
-        ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io), _dev_ptr(delta, "delta", (batch, L, D), io),
-        _dev_ptr(A, "A", (D, N), torch.float32), _dev_ptr(B, "B", (batch, L, N), io),
-        _dev_ptr(C, "C", (batch, L, N), io), _dev_ptr(D_skip, "D_skip", (D,), torch.float32),
-        _dev_ptr(z, "z", (batch, L, D), io), _dev_ptr(out, "out", (batch, L, D), io),
-        _dev_ptr(saved_states if save_states else None, "saved_states"), ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_scan_fwd_static")
-    return (out, saved_states) if save_states else out
+    return (_marshal_module or _native()).fwd(
+        x, delta, None, A, B, C, D_skip, z, None, out, None, saved_states, None, stream, save_states, general_A, False, False,
+        False, False, False, 2)
 
 
 def ssm_scan_bwd(x, delta, A, B, C, D_skip, z, dout, saved_states=None, *, general_A=False, zoh=False, workspace=None,
@@ -414,63 +296,9 @@ def ssm_scan_bwd(x, delta, A, B, C, D_skip, z, dout, saved_states=None, *, gener
     float32 (D, N) gradient.  With complex_state every complex array (A, B, C, their gradients, h0, dh_last, dh0) has a
     trailing dimension 2 of (re, im) pairs, and a gradient pair is (dL/dRe, dL/dIm).
     """
-    lib = load_library()
-    prob = make_problem(x, B, z is not None, D_skip is not None, False, general_A, zoh, static_B, static_C, complex_state)
-    prob.flags |= int(extra_flags)
-    batch, L, D, N = prob.batch, prob.L, prob.D, prob.N
-    io = x.dtype
-    c2 = (2,) if complex_state else ()
-    bshape, bdt = ((D, N), torch.float32) if static_B else ((batch, L, N) + c2, io)
-    cshape, cdt = ((D, N), torch.float32) if static_C else ((batch, L, N) + c2, io)
-    o = dict(outputs or {})
-    o.setdefault("dx", torch.empty_like(x))
-    o.setdefault("ddelta", torch.empty_like(x))
-    o.setdefault("dA", torch.empty((D, N) + c2, dtype=torch.float32, device=x.device))
-    o.setdefault("dB", torch.empty_like(B))
-    o.setdefault("dC", torch.empty_like(C))
-    if D_skip is not None:
-        o.setdefault("dD", torch.empty((D,), dtype=torch.float32, device=x.device))
-    else:
-        o["dD"] = None
-    if z is not None:
-        o.setdefault("dz", torch.empty_like(x))
-    else:
-        o["dz"] = None
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    need = bwd_workspace_bytes(prob)
-    ws = workspace if workspace is not None else _workspace(need, x.device, stream_ptr)
-    if h0 is not None or dh_last is not None or want_dh0:
-        f32 = torch.float32
-        if want_dh0:
-            o.setdefault("dh0", torch.empty((batch, D, N) + c2, dtype=f32, device=x.device))
-        code = lib.ssm_scan_bwd_state(
-            ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io), _dev_ptr(delta, "delta", (batch, L, D), io),
-            _dev_ptr(A, "A", (D, N) + c2, f32), _dev_ptr(B, "B", bshape, bdt), _dev_ptr(C, "C", cshape, cdt),
-            _dev_ptr(D_skip, "D_skip", (D,), f32), _dev_ptr(z, "z", (batch, L, D), io),
-            _dev_ptr(dout, "dout", (batch, L, D), io), _dev_ptr(h0, "h0", (batch, D, N) + c2, f32),
-            _dev_ptr(dh_last, "dh_last", (batch, D, N) + c2, f32), _dev_ptr(saved_states, "saved_states"),
-            _dev_ptr(o["dx"], "dx", (batch, L, D), io), _dev_ptr(o["ddelta"], "ddelta", (batch, L, D), io),
-            _dev_ptr(o["dA"], "dA", (D, N) + c2, f32), _dev_ptr(o["dB"], "dB", bshape, bdt),
-            _dev_ptr(o["dC"], "dC", cshape, cdt), _dev_ptr(o["dD"], "dD", (D,), f32),
-            _dev_ptr(o["dz"], "dz", (batch, L, D), io), _dev_ptr(o.get("dh0"), "dh0", (batch, D, N) + c2, f32),
-            _dev_ptr(ws, "workspace"), ctypes.c_size_t(0 if ws is None else ws.numel() * ws.element_size()),
-            ctypes.c_void_p(stream_ptr))
-        _check(code, "ssm_scan_bwd_state")
-        return o
-    code = lib.ssm_scan_bwd(
-        ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io), _dev_ptr(delta, "delta", (batch, L, D), io),
-        _dev_ptr(A, "A", (D, N) + c2, torch.float32), _dev_ptr(B, "B", bshape, bdt),
-        _dev_ptr(C, "C", cshape, cdt), _dev_ptr(D_skip, "D_skip", (D,), torch.float32),
-        _dev_ptr(z, "z", (batch, L, D), io), _dev_ptr(dout, "dout", (batch, L, D), io),
-        _dev_ptr(saved_states, "saved_states"),
-        _dev_ptr(o["dx"], "dx", (batch, L, D), io), _dev_ptr(o["ddelta"], "ddelta", (batch, L, D), io),
-        _dev_ptr(o["dA"], "dA", (D, N) + c2, torch.float32), _dev_ptr(o["dB"], "dB", bshape, bdt),
-        _dev_ptr(o["dC"], "dC", cshape, cdt), _dev_ptr(o["dD"], "dD", (D,), torch.float32),
-        _dev_ptr(o["dz"], "dz", (batch, L, D), io),
-        _dev_ptr(ws, "workspace"), ctypes.c_size_t(0 if ws is None else ws.numel() * ws.element_size()),
-        ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_scan_bwd")
-    return o
+    return (_marshal_module or _native()).bwd(
+        x, delta, None, A, B, C, D_skip, z, dout, saved_states, h0, dh_last, workspace, stream, dict(outputs or {}), general_A,
+        zoh, static_B, static_C, complex_state, False, False, want_dh0, int(extra_flags))
 
 
 def _host_ptr(t, name, shape, dtype):
@@ -534,46 +362,10 @@ def make_conv_problem(x: torch.Tensor, w: torch.Tensor, silu: bool, has_bias: bo
 def ssm_conv1d_fwd(x, w, bias=None, *, silu=True, x_prev=None, out=None, stream=None):
     """y = silu(causal depthwise conv1d(x; w) + bias), see include/ssm_conv1d.h.  x (batch, L, D) io dtype; w (D, W)
     float32 with the last tap on the current step; bias (D) float32 or None; x_prev (batch, W-1, D) io dtype or None."""
-    lib = load_library()
-    prob = make_conv_problem(x, w, silu, bias is not None)
-    batch, L, D, W = prob.batch, prob.L, prob.D, prob.width
-    io = x.dtype
-    if out is None:
-        out = torch.empty_like(x)
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    code = lib.ssm_conv1d_fwd(ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io),
-                              _dev_ptr(w, "w", (D, W), torch.float32), _dev_ptr(bias, "bias", (D,), torch.float32),
-                              _dev_ptr(x_prev, "x_prev", (batch, W - 1, D), io), _dev_ptr(out, "y", (batch, L, D), io),
-                              ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_conv1d_fwd")
-    return out
+    return (_marshal_module or _native()).conv_fwd(x, w, bias, x_prev, out, stream, silu)
 
 
 def ssm_conv1d_bwd(x, w, bias, dy, *, silu=True, x_prev=None, want_dx_prev=False, outputs=None, stream=None):
     """Gradients of sum(dy * y) of ssm_conv1d_fwd: dict with dx (io dtype), dw (D, W) and dbias (D) float32 (dbias None
     without bias), and dx_prev (batch, W-1, D) if asked for."""
-    lib = load_library()
-    prob = make_conv_problem(x, w, silu, bias is not None)
-    batch, L, D, W = prob.batch, prob.L, prob.D, prob.width
-    io = x.dtype
-    o = dict(outputs or {})
-    o.setdefault("dx", torch.empty_like(x))
-    o.setdefault("dw", torch.empty((D, W), dtype=torch.float32, device=x.device))
-    if bias is not None:
-        o.setdefault("dbias", torch.empty((D,), dtype=torch.float32, device=x.device))
-    else:
-        o["dbias"] = None
-    if want_dx_prev and W > 1:
-        o.setdefault("dx_prev", torch.empty((batch, W - 1, D), dtype=io, device=x.device))
-    stream_ptr = (stream if stream is not None else torch.cuda.current_stream(x.device)).cuda_stream
-    ws = _workspace(int(lib.ssm_conv1d_bwd_workspace_bytes(ctypes.byref(prob))), x.device, stream_ptr)
-    code = lib.ssm_conv1d_bwd(ctypes.byref(prob), _dev_ptr(x, "x", (batch, L, D), io),
-                              _dev_ptr(w, "w", (D, W), torch.float32), _dev_ptr(bias, "bias", (D,), torch.float32),
-                              _dev_ptr(x_prev, "x_prev", (batch, W - 1, D), io), _dev_ptr(dy, "dy", (batch, L, D), io),
-                              _dev_ptr(o["dx"], "dx", (batch, L, D), io), _dev_ptr(o["dw"], "dw", (D, W), torch.float32),
-                              _dev_ptr(o["dbias"], "dbias", (D,), torch.float32),
-                              _dev_ptr(o.get("dx_prev"), "dx_prev", (batch, W - 1, D), io),
-                              _dev_ptr(ws, "workspace"), ctypes.c_size_t(0 if ws is None else ws.numel() * ws.element_size()),
-                              ctypes.c_void_p(stream_ptr))
-    _check(code, "ssm_conv1d_bwd")
-    return o
+    return (_marshal_module or _native()).conv_bwd(x, w, bias, x_prev, dy, stream, dict(outputs or {}), silu, want_dx_prev)

@@ -1,9 +1,13 @@
-"""Compiles the CUDA sources in csrc/ into libssm_scan.so next to this file (sm_100a only, in-tree)."""
+"""Compiles the CUDA sources in csrc/ into libssm_scan.so next to this file (sm_100a only, in-tree), and the binding's
+argument marshalling (csrc/marshal.cpp, against torch's headers) into _marshal.so."""
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
+import shutil
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
@@ -14,6 +18,9 @@ DEBUG_LIB_PATH = os.path.join(_HERE, "libssm_scan_debug.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "--use_fast_math", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-cudart", "static"]
+
+MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
+MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
 
 
 def sources():
@@ -64,3 +71,30 @@ def _build(lib_path: str, obj_suffix: str, extra_flags, verbose: bool) -> str:
 if __name__ == "__main__":
     import sys
     print(build_library(force=True, verbose="-v" in sys.argv))
+
+
+def marshal_is_stale() -> bool:
+    if not os.path.exists(MARSHAL_PATH):
+        return True
+    t = os.path.getmtime(MARSHAL_PATH)
+    return any(os.path.getmtime(d) > t for d in [MARSHAL_SOURCE, *glob.glob(os.path.join(INCLUDE, "*.h"))])
+
+
+def build_marshal(force: bool = False) -> str:
+    """g++ -shared of the marshalling module; returns its path.  Raises if the compiler fails."""
+    if not force and not marshal_is_stale():
+        return MARSHAL_PATH
+    torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
+    include = os.path.join(torch_dir, "include")
+    cuda = os.path.dirname(os.path.dirname(shutil.which(os.environ.get("NVCC", "nvcc")) or "/usr/local/cuda/bin/nvcc"))
+    tmp = MARSHAL_PATH + f".tmp{os.getpid()}"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", INCLUDE,
+           "-I", include, "-I", os.path.join(include, "torch", "csrc", "api", "include"),
+           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), MARSHAL_SOURCE, "-o", tmp,
+           "-L", os.path.join(torch_dir, "lib"), "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-lc10_cuda", "-lc10", "-ldl"]
+    pr = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
+    if pr.returncode != 0:
+        print(pr.stdout)
+        raise RuntimeError(f"{cmd[0]} failed on {MARSHAL_SOURCE}")
+    os.replace(tmp, MARSHAL_PATH)
+    return MARSHAL_PATH

@@ -270,6 +270,8 @@ static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
     off += align_up(bytes);
     return at;
   };
+  // (the flags follow the status word, so that one memset clears both)
+  if (w.max_workers > 0) w.flags = take((size_t)(w.max_workers + 1) * sizeof(int));
   if (pl.nseg > 1) {
     const size_t st = (size_t)p.batch * pl.nseg * p.D * p.N * sizeof(float);
     w.seg_end = take(st);
@@ -277,18 +279,24 @@ static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
     w.seg_dsum = take((size_t)p.batch * pl.nseg * p.D * sizeof(float));
   }
   if (w.max_workers > 0) {
-    w.flags = take((size_t)(w.max_workers + 1) * sizeof(int));
     w.handoff = take((size_t)(w.max_workers + 1) * fwd_handoff_bytes_per_worker());
   }
   w.total = off;
   return w;
 }
-// Points the forward parameters at the scheduling words of a forward workspace and clears them.
+// Points the forward parameters at the scheduling words of a forward workspace and clears them; a status word at the head
+// of that workspace is cleared with them.
 static cudaError_t attach_fwd_sched(const ssm_problem_t& p, const Plan& pl, char* ws, int* abort_word, FwdParams& fp,
-                                    cudaStream_t s) {
+                                    cudaStream_t s, bool clear_status = false) {
   const FwdWorkspace w = fwd_layout(p, pl);
   fp.abort = abort_word;
   fp.max_workers = w.max_workers;
+  if (clear_status) {
+    if (w.total == 0) return cudaSuccess;
+    fp.flags = reinterpret_cast<int*>(ws + w.flags);
+    fp.handoff = reinterpret_cast<float4*>(ws + w.handoff);
+    return cudaMemsetAsync(ws, 0, w.max_workers > 0 ? w.flags + (size_t)(w.max_workers + 1) * sizeof(int) : sizeof(int), s);
+  }
   if (w.max_workers == 0) return cudaSuccess;
   fp.flags = reinterpret_cast<int*>(ws + w.flags);
   fp.handoff = reinterpret_cast<float4*>(ws + w.handoff);
@@ -310,6 +318,12 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
   };
   const size_t bln = (size_t)p.batch * p.L * p.N;
   const size_t segs = (size_t)p.batch * pl.nseg, parts = segs * pl.split.cluster;
+  // (batch, segment, channel group) chains of the tuned kernel; SSM_FLAG_TEST_WITHHOLD forces chains to be shared
+  const long long chains = (long long)segs * pl.bwd_groups;
+  w.max_workers = !tuned_shape(p) ? 0 : (p.flags & SSM_FLAG_TEST_WITHHOLD) ? (int)std::max<long long>(1, (2 * chains + 2) / 3)
+                                                                            : shared_workers(chains);
+  // (behind the status word, so that one memset clears both: backward kernel | adjoint pre-pass)
+  w.flags = take((size_t)2 * (w.max_workers + 1) * sizeof(int));
   w.dBC_part = take((size_t)pl.bwd_groups * 2 * bln * sizeof(float));
   w.dA_part = take(parts * p.D * p.N * sizeof(float));
   w.dD_part = take(parts * p.D * sizeof(float));
@@ -322,11 +336,6 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
     w.seg_dsum = take(segs * p.D * sizeof(float));
   }
   w.fwd = take(fwd_layout(p, pl_fwd).total);   // the forward sweep that rebuilds checkpoints uses the forward split
-  // (batch, segment, channel group) chains of the tuned kernel; SSM_FLAG_TEST_WITHHOLD forces chains to be shared
-  const long long chains = (long long)segs * pl.bwd_groups;
-  w.max_workers = !tuned_shape(p) ? 0 : (p.flags & SSM_FLAG_TEST_WITHHOLD) ? (int)std::max<long long>(1, (2 * chains + 2) / 3)
-                                                                            : shared_workers(chains);
-  w.flags = take((size_t)2 * (w.max_workers + 1) * sizeof(int));   // backward kernel | adjoint pre-pass
   w.handoff = take((size_t)(w.max_workers + 1) *
                    bwd_handoff_bytes_per_worker(p.flags & SSM_FLAG_STATIC_B, p.flags & SSM_FLAG_STATIC_C));
   if (p.flags & SSM_FLAG_STATIC_B) w.dBs_part = take(parts * p.D * p.N * sizeof(float));
@@ -537,11 +546,9 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.static_C = (p->flags & SSM_FLAG_STATIC_C) ? 1 : 0;
   fp.delta_bias = delta_bias;
   fp.softplus = (p->flags & SSM_FLAG_DELTA_SOFTPLUS) ? 1 : 0;
-  if (fwd_layout(*p, pl).total > 0) {
-    if (cudaMemsetAsync(workspace, 0, kStatusBytes, s) != cudaSuccess) return SSM_ERR_CUDA;
-    if (attach_fwd_sched(*p, pl, static_cast<char*>(workspace), static_cast<int*>(workspace), fp, s) != cudaSuccess)
-      return SSM_ERR_CUDA;
-  }
+  if (fwd_layout(*p, pl).total > 0 &&
+      attach_fwd_sched(*p, pl, static_cast<char*>(workspace), static_cast<int*>(workspace), fp, s, true) != cudaSuccess)
+    return SSM_ERR_CUDA;
   const float* h_start = nullptr;
   if (run_segment_starts(*p, pl, fp, static_cast<char*>(workspace), h0, &h_start, s) != cudaSuccess) return SSM_ERR_CUDA;
   if (fp.max_workers > 0 && pl.nseg > 1) {
@@ -692,7 +699,17 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
 
-  if (cudaMemsetAsync(ws, 0, kStatusBytes, s) != cudaSuccess) return SSM_ERR_CUDA;
+  // the status word, and the hand-off flags of the tuned kernels (the lane kernel clears the status word itself)
+  bool clear = true;
+#ifndef SSM_DEBUG_BOUNDS
+  BwdParams in{};
+  in.x = x;
+  in.delta = delta;
+  in.z = has_z ? z : nullptr;
+  in.dout = dout;
+  clear = !lane_shape(*p) || !bwd_lane_applicable(in);
+#endif
+  if (clear && cudaMemsetAsync(ws, 0, w.flags + (size_t)2 * (w.max_workers + 1) * sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
   // checkpoint states: the caller's, or rebuilt here with one more forward sweep
   const float* ckpt = static_cast<const float*>(saved_states);
   if (ckpt == nullptr) {
@@ -767,8 +784,6 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   bp.flags = reinterpret_cast<int*>(ws + w.flags);
   bp.handoff = reinterpret_cast<float4*>(ws + w.handoff);
   bp.max_workers = w.max_workers;
-  // the hand-off flags of the tuned kernel start at zero (the status word was cleared above)
-  if (cudaMemsetAsync(ws + w.flags, 0, w.handoff - w.flags, s) != cudaSuccess) return SSM_ERR_CUDA;
 
   if (pl.nseg == 2 && dh_last == nullptr && (bp.seg_local = reinterpret_cast<float*>(ws + w.mu_in),
                                               bp.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum),

@@ -403,7 +403,8 @@ static cudaError_t launch_bwd_n(const Plan& plan, const BwdParams& p, int mode, 
     return cudaGetLastError();
   }
   constexpr size_t smem = bwd_smem_bytes<IO, N>();
-  cudaError_t e = cudaFuncSetAttribute(ssm_bwd_kernel<IO, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  KernelLimits lim;
+  const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(ssm_bwd_kernel<IO, N>), kBwdThreads, smem, &lim);
   if (e != cudaSuccess) return e;
   ssm_bwd_kernel<IO, N><<<grid, kBwdThreads, smem, s>>>(p);
   return cudaGetLastError();

@@ -536,6 +536,9 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   const bool cvec = N >= 4 && (reinterpret_cast<uintptr_t>(p.C) & (4 * sizeof(IO) - 1)) == 0;
   const size_t row_b = (size_t)b * p.L;
   const int t_last = live_piece ? t_begin + (t_end - t_begin - 1) / kLB * kLB : t_begin;   // first step of the last block
+#ifndef SSM_DEBUG_BOUNDS
+  if (blockIdx.x == 0 && threadIdx.x == 0) *p.abort = 0;   // the status word of the workspace: nothing here can give up
+#endif
   auto team_sync = [&] {
     if constexpr (NG == 1) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * NG) : "memory");
@@ -877,7 +880,8 @@ cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int m
   const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
   const LaneSplit sp = plan.split;
   const int per_block = SM::kTeams / sp.warps;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SM::bytes(SM::kTeams));
+  KernelLimits lim;
+  const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), 32 * kLaneWarps, SM::bytes(SM::kTeams), &lim);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)((chains + per_block - 1) / per_block * sp.cluster));

@@ -292,18 +292,14 @@ template <bool SP, bool SC>
 cudaError_t launch_local(const Plan& plan, const BwdParams& p, cudaStream_t s) {
   const size_t smem = sizeof(LocalWarpSmem<SP, SC>) * kLWarps;
   auto kern = ssm_bwd_local_warp_kernel<SP, SC>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  KernelLimits lim;
+  cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), kLWarps * 32, smem, &lim);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kLWarps * 32, smem)) != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorLaunchOutOfResources;
   WarpSched sc{};
   sc.chains = p.batch * (plan.nseg - 1) * ((p.D + 31) / 32);
   sc.tiles = (plan.seg_steps + kLT - 1) / kLT;
   const bool can_share = p.abort != nullptr && p.flags != nullptr && p.handoff != nullptr && p.max_workers > 0;
-  sc.workers = warp_workers(sc.chains, sms, per_sm * kLWarps, can_share ? p.max_workers : 0);
+  sc.workers = warp_workers(sc.chains, lim.sms, lim.per_sm * kLWarps, can_share ? p.max_workers : 0);
   const long long total = (long long)sc.chains * sc.tiles;
   sc.quota = (int)((total + sc.workers - 1) / sc.workers);
   sc.spin_limit = 1 << 22;
@@ -315,7 +311,7 @@ cudaError_t launch_local(const Plan& plan, const BwdParams& p, cudaStream_t s) {
     // no ragged tile or channel group anywhere: the instantiation without range tests (same launch shape)
     if (p.L % kLT == 0 && plan.seg_steps % kLT == 0 && p.D % 32 == 0) {
       auto whole = ssm_bwd_local_warp_kernel<SP, SC, true>;
-      if ((e = cudaFuncSetAttribute(whole, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+      if ((e = kernel_limits(reinterpret_cast<const void*>(whole), kLWarps * 32, smem, &lim)) != cudaSuccess) return e;
       whole<<<grid, kLWarps * 32, smem, s>>>(p, sc);
       return cudaGetLastError();
     }

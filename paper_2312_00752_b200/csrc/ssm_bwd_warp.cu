@@ -889,13 +889,10 @@ cudaError_t launch_bwd_variant(const Plan& plan, const BwdParams& p, cudaStream_
   constexpr int CW = Lane<S, CPT>::CW;
   const size_t smem = sizeof(BwdWarpSmem<S, CPT, SP>) * kBwdWarps;
   auto kern = ssm_bwd_warp_kernel<S, CPT, SP, ZOH, BC>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  KernelLimits lim;
+  cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), kBwdWarps * 32, smem, &lim);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBwdWarps * 32, smem)) != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorLaunchOutOfResources;
+  const int sms = lim.sms, per_sm = lim.per_sm;
   WarpSched sc{};
   sc.chains = p.batch * plan.nseg * ((p.D + CW - 1) / CW);
   sc.tiles = (plan.seg_steps + kBT - 1) / kBT;
@@ -917,7 +914,7 @@ cudaError_t launch_bwd_variant(const Plan& plan, const BwdParams& p, cudaStream_
     // no ragged tile or channel group anywhere: the instantiation without range tests (same launch shape)
     if (p.L % kBT == 0 && plan.seg_steps % kBT == 0 && p.D % CW == 0) {
       auto whole = ssm_bwd_warp_kernel<S, CPT, SP, ZOH, BC, true>;
-      if ((e = cudaFuncSetAttribute(whole, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+      if ((e = kernel_limits(reinterpret_cast<const void*>(whole), kBwdWarps * 32, smem, &lim)) != cudaSuccess) return e;
       whole<<<grid, kBwdWarps * 32, smem, s>>>(p, sc);
       return cudaGetLastError();
     }

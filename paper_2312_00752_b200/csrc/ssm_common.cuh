@@ -168,6 +168,13 @@ struct ReduceParams {
   float* dCs;
 };
 
+// SMs of the current device and blocks of a kernel that fit one of them, with `smem` bytes of dynamic shared memory, which
+// the kernel is allowed to use from then on.  Asked of the runtime once per thread, kernel and device (ssm_launch.cu).
+struct KernelLimits {
+  int sms, per_sm;
+};
+cudaError_t kernel_limits(const void* kernel, int threads, size_t smem, KernelLimits* out);
+
 cudaError_t launch_fwd(const ssm_problem_t& prob, const Plan& plan, const FwdParams& p, int mode, cudaStream_t s);
 cudaError_t launch_carry(const CarryParams& p, cudaStream_t s);
 cudaError_t launch_bwd(const ssm_problem_t& prob, const Plan& plan, const BwdParams& p, int mode, cudaStream_t s);

@@ -430,7 +430,8 @@ cudaError_t launch_cbwd_n(const CplxParams& p, cudaStream_t s) {
   using G = CGeom<N>;
   const dim3 grid((p.D + G::CH - 1) / G::CH, p.batch);
   constexpr size_t smem = cbwd_smem_bytes<IO, N>();
-  cudaError_t e = cudaFuncSetAttribute(ssm_cbwd_kernel<IO, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  KernelLimits lim;
+  cudaError_t e = kernel_limits(reinterpret_cast<const void*>(ssm_cbwd_kernel<IO, N>), G::THREADS, smem, &lim);
   if (e != cudaSuccess) return e;
   ssm_cbwd_kernel<IO, N><<<grid, G::THREADS, smem, s>>>(p);
   return cudaGetLastError();

@@ -541,12 +541,10 @@ template <typename Kernel>
 cudaError_t launch_conv_kernel(Kernel kernel, ConvParams p, int W, int channels_per_thread, int* chunks_out, cudaStream_t s) {
   const int vecs = (p.D + channels_per_thread - 1) / channels_per_thread;
   const int gx = (vecs + kConvThreads - 1) / kConvThreads;
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kConvThreads, 0)) != cudaSuccess) return e;
-  p.steps = choose_steps((long long)gx * p.batch, p.L, W, (long long)sms * (per_sm > 0 ? per_sm : 1));
+  KernelLimits lim;
+  const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kernel), kConvThreads, 0, &lim);
+  if (e != cudaSuccess) return e;
+  p.steps = choose_steps((long long)gx * p.batch, p.L, W, (long long)lim.sms * lim.per_sm);
   const int chunks = (p.L + p.steps - 1) / p.steps;
   if (chunks_out != nullptr) *chunks_out = chunks;
   dim3 grid(gx, chunks, p.batch);

@@ -402,7 +402,8 @@ cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int m
   const LaneSplit sp = choose_lane_split(chains, steps, 0.75f, NG > 2 ? 2 : 3, kLaneWarps);
   const int per_block = kLaneWarps / sp.warps;
   const size_t smem = FwdLaneSmem<IO, NG>::bytes(kLaneWarps, per_block);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  KernelLimits lim;
+  const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), 32 * kLaneWarps, FwdLaneSmem<IO, NG>::bytes(kLaneWarps, kLaneWarps), &lim);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)((chains + per_block - 1) / per_block * sp.cluster));

@@ -514,26 +514,25 @@ constexpr int kFwdS = 16;  // a lane per channel, 32-channel chains
 namespace {
 
 template <int S, int MODE, bool SP, bool ZOH, int BC, int NST>
-cudaError_t fwd_occupancy(int* per_sm, size_t* smem_bytes) {
+cudaError_t fwd_occupancy(int* sms, int* per_sm, size_t* smem_bytes) {
   constexpr int CW = 2 * S;   // channels per chain
   const size_t smem = sizeof(FwdWarpSmem<CW, MODE == kFwdFull, SP && ZOH, BC, NST>) * kWarpsPerBlock;
   auto kern = ssm_fwd_warp_kernel<S, MODE, SP, ZOH, BC, NST>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
+  KernelLimits lim{};
+  const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), kWarpsPerBlock * 32, smem, &lim);
   *smem_bytes = smem;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, kern, kWarpsPerBlock * 32, smem);
+  *per_sm = lim.per_sm;
+  *sms = lim.sms;
+  return e;
 }
 
 template <int S, int MODE, bool SP, bool ZOH, int BC>
 cudaError_t launch_variant_w(const Plan& plan, const FwdParams& p, cudaStream_t s) {
   constexpr int CW = 2 * S;   // channels per chain
-  int dev = 0, sms = 0, per_sm = 0;
+  int sms = 0, per_sm = 0;
   size_t smem = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = fwd_occupancy<S, MODE, SP, ZOH, BC, 3>(&per_sm, &smem)) != cudaSuccess) return e;
-  if (per_sm < 1) return cudaErrorLaunchOutOfResources;
+  if ((e = fwd_occupancy<S, MODE, SP, ZOH, BC, 3>(&sms, &per_sm, &smem)) != cudaSuccess) return e;
   WarpSched sc{};
   sc.chains = p.batch * plan.nseg * ((p.D + CW - 1) / CW);
   sc.tiles = (plan.seg_steps + kWT - 1) / kWT;
@@ -545,7 +544,7 @@ cudaError_t launch_variant_w(const Plan& plan, const FwdParams& p, cudaStream_t 
   if constexpr (!ZOH && MODE != kFwdSummary && BC == 0) {
     int per_sm2 = 0;
     size_t smem2 = 0;
-    if ((e = fwd_occupancy<S, MODE, SP, ZOH, BC, 2>(&per_sm2, &smem2)) != cudaSuccess) return e;
+    if ((e = fwd_occupancy<S, MODE, SP, ZOH, BC, 2>(&sms, &per_sm2, &smem2)) != cudaSuccess) return e;
     if (per_sm2 > per_sm && warp_run_estimate(sc.chains, sms, per_sm2 * kWarpsPerBlock, max_workers) <
                                 0.93f * warp_run_estimate(sc.chains, sms, per_sm * kWarpsPerBlock, max_workers)) {
       two_stage = true;
@@ -566,7 +565,8 @@ cudaError_t launch_variant_w(const Plan& plan, const FwdParams& p, cudaStream_t 
     // shape as the ones the occupancy was taken from)
     if (p.L % kWT == 0 && plan.seg_steps % kWT == 0 && p.D % CW == 0) {
       auto go = [&](auto kern) {
-        const cudaError_t ea = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        KernelLimits lim;
+        const cudaError_t ea = kernel_limits(reinterpret_cast<const void*>(kern), kWarpsPerBlock * 32, smem, &lim);
         if (ea != cudaSuccess) return ea;
         kern<<<grid, kWarpsPerBlock * 32, smem, s>>>(p, sc);
         return cudaGetLastError();
