@@ -52,10 +52,61 @@ static bool tuned_shape(const ssm_problem_t& p) {
 }
 // Checkpoint states are tiled by groups of 32 channels whenever a channel's states are whole 16-byte quads.
 static bool ckpt_tiled(const ssm_problem_t& p) { return p.N % 4 == 0 && !(p.flags & SSM_FLAG_COMPLEX); }
-// Problems the lane-per-channel kernels run (ssm_lane.cuh): what the tuned kernels do not take.
-bool lane_shape(const ssm_problem_t& p) {
+// Time segments of the tuned forward: one warp per chain of 32 channels; a split costs half a forward sweep more, so only
+// when fewer than half of the sub-partitions would have a warp, and then into two rounds of chains.
+static int tuned_fwd_segments(const ssm_problem_t& p) {
+  const int cw = fwd_fast_channels_per_warp();
+  const long long chains = (long long)p.batch * ((p.D + cw - 1) / cw), sub_partitions = 4LL * kNumSMs;
+  if (2 * chains >= sub_partitions) return 1;
+  const long long want = (2 * sub_partitions + chains - 1) / chains;
+  return (int)std::min<long long>(std::min<long long>(want, std::max(1, p.L / 256)), 65535);
+}
+// Time segments of the tuned backward: its kernel wants two warps per sub-partition (a lone warp cannot cover its own
+// latencies), i.e. two rounds of chains; the adjoint pre-pass that a split costs is about a tenth of the backward work.
+static int tuned_bwd_segments(const ssm_problem_t& p) {
+  const int cw = bwd_fast_channels_per_warp();
+  const long long chains = (long long)p.batch * ((p.D + cw - 1) / cw), resident = 4LL * kNumSMs;
+  if (chains >= 2 * resident) return 1;
+  const long long want = (2 * resident + chains - 1) / chains;
+  return (int)std::min<long long>(std::min<long long>(want, std::max(1, p.L / 256)), 65535);
+}
+// The lane-per-channel kernels (ssm_lane.cuh) run what the tuned kernels do not take, and of the shapes both take those
+// with so few chains that the split inside a cluster is faster: below, both sides' run times are estimated in cycles (a
+// lone tuned warp takes 178 cycles per forward step, a lone lane warp about 205; 890 and 1037 backward; the rest is measured
+// launch and fold overhead).  Measured at batch 1, D = 1536, L = 333, forward, A trained and step size fused: 56 us with
+// the tuned kernel (one warp walks the 333 steps of each chain), 17 us with the lane kernel; the lines meet near
+// chains * L = 2^18 .. 2^20.
+static bool lane_shape(const ssm_problem_t& p) {
   if (p.flags & (SSM_FLAG_COMPLEX | SSM_FLAG_ZOH_BBAR | SSM_FLAG_STATIC_B | SSM_FLAG_STATIC_C)) return false;
-  return !tuned_shape(p);
+  return !(tuned_shape(p) && (p.flags & SSM_FLAG_TEST_WITHHOLD));   // (the hook withholds the tuned kernel's flags)
+}
+static void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl, float* cost);
+bool lane_fwd(const ssm_problem_t& p) {
+  if (!lane_shape(p)) return false;
+  if (!tuned_shape(p)) return true;
+  const long long chains = (long long)p.batch * ((p.D + kLaneChannels - 1) / kLaneChannels);
+  const int nseg = tuned_fwd_segments(p);
+  if (2 * chains >= 4 * kNumSMs) return false;
+  const float steps = (float)((p.L + nseg - 1) / nseg), share = (float)(chains * nseg) / (8.f * kNumSMs);
+  const float tuned = nseg == 1 ? 178.f * steps + 8e3f
+                                : 273.f * steps * (chains * nseg > 4 * kNumSMs ? 1.8f : 1.f) * std::max(1.f, share) + 20e3f;
+  float lane = 0.f;
+  choose_lane_split(chains, p.L, 0.75f, 25.f, 3, kLaneWarps, &lane);
+  return 205.f * lane + 6e3f < tuned;
+}
+bool lane_bwd(const ssm_problem_t& p) {
+  if (!lane_shape(p)) return false;
+  if (!tuned_shape(p)) return true;
+  const long long chains = (long long)p.batch * ((p.D + kLaneChannels - 1) / kLaneChannels);
+  const int nseg = tuned_bwd_segments(p);
+  if (2 * chains >= 4 * kNumSMs) return false;
+  const float steps = (float)((p.L + nseg - 1) / nseg), share = (float)(chains * nseg) / (8.f * kNumSMs);
+  const float tuned = nseg == 1 ? 890.f * steps + 16e3f : (1048.f + 190.f) * steps * std::max(1.f, share) + 40e3f;
+  Plan pl{};
+  pl.bwd_groups = (p.D + kLaneChannels - 1) / kLaneChannels;
+  float lane = 0.f;
+  plan_lane_bwd(p, kLaneWarps, &pl, &lane);
+  return 1037.f * lane + 20e3f < tuned;
 }
 // Time segments of a lane launch.  A chain already spreads over up to 64 warps of a cluster, so the launch itself is
 // split (summary pass, carry, full pass) only for a handful of chains and then into segments of at least 2048 steps.
@@ -82,10 +133,12 @@ constexpr int kWideN = 16;
 static bool widen_route(const ssm_problem_t& p, ssm_problem_t* wide) {
   if (p.io_dtype != SSM_BF16 || p.N >= kWideN || p.D % 8 != 0 || (p.flags & SSM_FLAG_COMPLEX)) return false;
   if ((long long)p.batch * p.L > 0x7fffffffLL || (long long)p.batch * p.D > 0x7fffffffLL) return false;
-  if (wide) {
-    *wide = p;
-    wide->N = kWideN;
-  }
+  ssm_problem_t w = p;
+  w.N = kWideN;
+  // (where both directions would take the lane kernels, these run the problem as it is; the layout of the checkpoint
+  // states must not depend on the direction)
+  if (lane_fwd(w) && lane_bwd(w)) return false;
+  if (wide) *wide = w;
   return true;
 }
 // Buffers of the widened arrays, placed behind the wide problem's own workspace (whose head holds the status word).
@@ -149,18 +202,10 @@ Plan make_plan(const ssm_problem_t& p) {
   int nseg = 1;
   if (p.flags & SSM_FLAG_COMPLEX) {
     // the complex path does not split time
-  } else if (lane_shape(p)) {
+  } else if (lane_fwd(p)) {
     nseg = lane_segments(p);
   } else if (tuned_shape(p)) {
-    // one warp per chain of fwd_fast_channels_per_warp() channels; a split costs half a forward sweep more, so only
-    // when fewer than half of the sub-partitions would have a warp, and then into two rounds of chains
-    const int cw = fwd_fast_channels_per_warp();
-    const long long chains = (long long)p.batch * ((p.D + cw - 1) / cw);
-    if (2 * chains < sub_partitions) {
-      const long long want = (2 * sub_partitions + chains - 1) / chains;
-      const long long max_by_len = std::max(1, p.L / 256);
-      nseg = (int)std::min<long long>(std::min(want, max_by_len), 65535);
-    }
+    nseg = tuned_fwd_segments(p);
   } else if (warps < sub_partitions * 3) {
     // generic kernels: a warp is latency-bound, so aim for 6 warps per sub-partition although a split costs half a
     // sweep more (measured 2 to 2.5 times faster than one or two warps per sub-partition)
@@ -179,16 +224,16 @@ Plan make_plan(const ssm_problem_t& p) {
 // Time split of the lane backward kernel: inside clusters (one launch, for little work) or into segments of the launch
 // with a pre-pass of its own (which runs at twice the occupancy).  Costs in steps of a lone warp of the main kernel:
 // segments are chosen to fill whole waves of two blocks per SM; two warps on a sub-partition take 1.45 times as long each;
-// the pre-pass is a quarter of the work spread over all sub-partitions, its two launches 15 steps.
-static void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl) {
+// the pre-pass is a quarter of the work spread over all sub-partitions, its two launches 25 steps.
+static void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl, float* cost) {
   const long long chains = (long long)p.batch * pl->bwd_groups;
   auto align8 = [](long long v) { return (int)((v + kCkptSteps - 1) / kCkptSteps * kCkptSteps); };
   pl->nseg = 1;
   pl->seg_steps = (p.L + kSegAlign - 1) / kSegAlign * kSegAlign;
   float best;
-  pl->split = choose_lane_split(chains, p.L, 0.3f, 2, teams, &best);
+  pl->split = choose_lane_split(chains, p.L, 0.3f, 8.f, 2, teams, &best);
   const long long wave = 2LL * kNumSMs * teams;   // pieces the GPU holds
-  const float prepass = 15.f + 0.22f * (float)chains * (float)(kLaneWarps / teams) * (float)p.L / (4.f * kNumSMs);
+  const float prepass = 25.f + 0.22f * (float)chains * (float)(kLaneWarps / teams) * (float)p.L / (4.f * kNumSMs);
   for (int half = 1; half <= 12; ++half) {        // half waves: one block per SM, then whole waves
     if (half > 1 && half % 2) continue;
     const long long most = std::min<long long>(std::min<long long>(half * wave / 2 / chains, p.L / 64), 65535);
@@ -202,6 +247,7 @@ static void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl) {
       pl->split = LaneSplit{1, 1, seg};
     }
   }
+  *cost = best;
 }
 
 static long long generic_bwd_warps(int N) {   // warps of a block of the generic backward kernel
@@ -214,11 +260,12 @@ static long long generic_bwd_warps(int N) {   // warps of a block of the generic
 // it pays when the chains alone leave the SM sub-partitions with too few warps.  Segments are at least 256 steps.
 Plan make_bwd_plan(const ssm_problem_t& p) {
   Plan pl = make_plan(p);
-  if (lane_shape(p)) {
+  if (lane_bwd(p)) {
     const int ng = p.N <= 16 ? 1 : (p.N <= 32 ? 2 : 4);   // warps of a team
     pl.bwd_ch = kLaneChannels;
     pl.bwd_groups = (p.D + kLaneChannels - 1) / kLaneChannels;
-    plan_lane_bwd(p, kLaneWarps / ng, &pl);
+    float cost;
+    plan_lane_bwd(p, kLaneWarps / ng, &pl, &cost);
     return pl;
   }
   if (tuned_shape(p)) {
@@ -232,13 +279,7 @@ Plan make_bwd_plan(const ssm_problem_t& p) {
   if (p.flags & SSM_FLAG_COMPLEX) {
     // the complex path does not split time
   } else if (tuned_shape(p)) {
-    // the tuned kernel wants two warps per SM sub-partition (a lone warp cannot cover its own latencies), i.e. two
-    // rounds of chains; the adjoint pre-pass that a split costs is about a tenth of the backward work
-    if (chains < 2 * resident) {
-      const long long want = (2 * resident + chains - 1) / chains;
-      const long long max_by_len = std::max(1, p.L / 256);
-      nseg = (int)std::min<long long>(std::min(want, max_by_len), 65535);
-    }
+    nseg = tuned_bwd_segments(p);
   } else if (chains * generic_bwd_warps(p.N) < 4 * resident) {
     // generic kernel: latency-bound warps, so aim for 8 per sub-partition (measured against 2: 1.1 to 1.5 times faster)
     const long long want = (8 * resident + chains * generic_bwd_warps(p.N) - 1) / (chains * generic_bwd_warps(p.N));
@@ -262,7 +303,7 @@ struct FwdWorkspace {
 static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
   FwdWorkspace w{};
   const int cw = fwd_fast_channels_per_warp();
-  w.max_workers = tuned_shape(p) ? shared_workers((long long)p.batch * pl.nseg * ((p.D + cw - 1) / cw)) : 0;
+  w.max_workers = tuned_shape(p) && !lane_fwd(p) ? shared_workers((long long)p.batch * pl.nseg * ((p.D + cw - 1) / cw)) : 0;
   if (pl.nseg == 1 && w.max_workers == 0) return w;
   size_t off = kStatusBytes;
   auto take = [&](size_t bytes) {
@@ -320,7 +361,7 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
   const size_t segs = (size_t)p.batch * pl.nseg, parts = segs * pl.split.cluster;
   // (batch, segment, channel group) chains of the tuned kernel; SSM_FLAG_TEST_WITHHOLD forces chains to be shared
   const long long chains = (long long)segs * pl.bwd_groups;
-  w.max_workers = !tuned_shape(p) ? 0 : (p.flags & SSM_FLAG_TEST_WITHHOLD) ? (int)std::max<long long>(1, (2 * chains + 2) / 3)
+  w.max_workers = !tuned_shape(p) || lane_bwd(p) ? 0 : (p.flags & SSM_FLAG_TEST_WITHHOLD) ? (int)std::max<long long>(1, (2 * chains + 2) / 3)
                                                                             : shared_workers(chains);
   // (behind the status word, so that one memset clears both: backward kernel | adjoint pre-pass)
   w.flags = take((size_t)2 * (w.max_workers + 1) * sizeof(int));
@@ -454,7 +495,7 @@ ssm_status_t ssm_scan_plan(const ssm_problem_t* p, int32_t* n_segments, int32_t*
   if (n_segments) *n_segments = pl.nseg;
   if (segment_steps) *segment_steps = pl.seg_steps;
   if (channels_per_block) *channels_per_block = pl.fwd_ch;
-  if (states_per_thread) *states_per_thread = tuned_shape(*p) ? fwd_states_per_thread() : (p->N < 4 ? p->N : 4);
+  if (states_per_thread) *states_per_thread = lane_fwd(*p) ? 16 : tuned_shape(*p) ? fwd_states_per_thread() : (p->N < 4 ? p->N : 4);
   return SSM_OK;
 }
 
@@ -707,7 +748,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   in.delta = delta;
   in.z = has_z ? z : nullptr;
   in.dout = dout;
-  clear = !lane_shape(*p) || !bwd_lane_applicable(in);
+  clear = !lane_bwd(*p) || !bwd_lane_applicable(in);
 #endif
   if (clear && cudaMemsetAsync(ws, 0, w.flags + (size_t)2 * (w.max_workers + 1) * sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
   // checkpoint states: the caller's, or rebuilt here with one more forward sweep

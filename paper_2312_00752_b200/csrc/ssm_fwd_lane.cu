@@ -399,7 +399,7 @@ cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int m
   auto kern = ssm_fwd_lane_kernel<IO, NG, VEC>;
   const int steps = plan.nseg > 1 ? plan.seg_steps : p.L;
   const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
-  const LaneSplit sp = choose_lane_split(chains, steps, 0.75f, NG > 2 ? 2 : 3, kLaneWarps);
+  const LaneSplit sp = choose_lane_split(chains, steps, 0.75f, 25.f, NG > 2 ? 2 : 3, kLaneWarps);
   const int per_block = kLaneWarps / sp.warps;
   const size_t smem = FwdLaneSmem<IO, NG>::bytes(kLaneWarps, per_block);
   KernelLimits lim;
@@ -436,7 +436,7 @@ cudaError_t launch_fwd_lane_io(const Plan& plan, const FwdParams& p, int N, int 
 
 }  // namespace
 
-LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm, int teams, float* cost) {
+LaneSplit choose_lane_split(long long chains, int steps, float extra, float fixed, int blocks_per_sm, int teams, float* cost) {
   // run time of 1, 2, 3 warps on a sub-partition relative to one (measured on these kernels)
   static const float slow[4] = {1.0f, 1.0f, 1.5f, 2.1f};
   LaneSplit best{1, 1, (steps + kLB - 1) / kLB * kLB};
@@ -449,8 +449,8 @@ LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks
       const long long blocks = (chains * w + teams - 1) / teams * cl;
       const long long per = (blocks + kNumSMs - 1) / kNumSMs;     // blocks on the fullest SM
       const long long waves = (per + blocks_per_sm - 1) / blocks_per_sm;
-      float t = (float)piece * (pieces > 1 ? 1.f + extra : 1.f) * slow[per < blocks_per_sm ? per : blocks_per_sm] * (float)waves;
-      if (pieces > 1) t += 8.f + (cl > 1 ? 8.f + (float)cl : 0.f);   // the fold, in steps
+      const float block = (float)piece * (pieces > 1 ? 1.f + extra : 1.f) + (pieces > 1 ? fixed : 0.5f * fixed) + (cl > 1 ? 0.3f * fixed : 0.f);
+      const float t = block * slow[per < blocks_per_sm ? per : blocks_per_sm] * (float)waves;
       if (best_t == 0.f || t < best_t) {
         best_t = t;
         best = LaneSplit{w, cl, piece};

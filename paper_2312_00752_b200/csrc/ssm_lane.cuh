@@ -29,10 +29,11 @@ constexpr int kLaneChannels = 32; // channels per chain
 // Blocks always have kLaneWarps warps (a warp's place in its block decides its SM sub-partition, so smaller blocks would
 // pile up on one); with fewer warps on a chain than that a block holds several chains.
 constexpr int kLaneWarps = 4, kLaneMaxCluster = 8;
-// Split with the shortest estimated run.  `extra`: cost of the first sweep over a piece relative to the second; `teams`:
+// Split with the shortest estimated run.  `extra`: cost of the first sweep over a piece relative to the second; `fixed`: what a
+// block costs besides its steps (set-up and fold, in steps); `teams`:
 // pieces a block holds (a piece is swept by one warp, or by a team of warps that share its states); `cost`: the estimate,
 // in steps of a lone warp.
-LaneSplit choose_lane_split(long long chains, int steps, float extra, int blocks_per_sm, int teams, float* cost = nullptr);
+LaneSplit choose_lane_split(long long chains, int steps, float extra, float fixed, int blocks_per_sm, int teams, float* cost = nullptr);
 
 #ifdef __CUDACC__
 template <typename IO>
