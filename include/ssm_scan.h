@@ -31,10 +31,10 @@
  *   - Calls enqueue work on `stream` and return without synchronising.  Argument errors are detected before
  *     anything is launched and reported by the return value; nothing is written in that case.  A failed kernel
  *     launch is reported as SSM_ERR_CUDA.
- *   - N must be 1, 2, 4, 8, 16 (the state sizes Table 10 ablates), 32 or 64 (larger states on the generic kernels;
- *     the tuned kernels are N = 16; bf16 problems with N < 16 and D % 8 == 0 run on them too, with A, B, C and the
- *     state arrays widened inside the workspace by columns that stay zero).  All io pointers must be
- *     aligned to the element size; 16-byte aligned pointers together with D % 8 == 0 select the vector path.
+ *   - N must be 1, 2, 4, 8, 16 (the state sizes Table 10 ablates), 32 or 64.  (bf16 with N = 16 and D % 8 == 0 has kernels
+ *     of its own; larger bf16 problems with N < 16 and D % 8 == 0 run on them too, with A, B, C and the state arrays
+ *     widened inside the workspace by columns that stay zero.)  All io pointers must be aligned to the element size;
+ *     16-byte aligned pointers together with rows that are multiples of 16 bytes select the vector path.
  *   - Results are bitwise reproducible for fixed inputs, shape, flags and library build: every reduction (over n,
  *     over channels for dB/dC, over batch and time for dA/dD) has a fixed order and no floating-point atomics
  *     are used.
@@ -90,7 +90,7 @@ enum {
                                  s = 2 Re(sum_n C h) + D_skip x (the N states stand for N conjugate pairs); a gradient
                                  of a complex quantity holds (dL/dRe, dL/dIm).  N <= 32.  Not combined with
                                  SSM_FLAG_ZOH_BBAR, SSM_FLAG_STATIC_B / _C, the *_fused_dt calls or
-                                 ssm_scan_fwd_bwd_host (SSM_ERR_UNSUPPORTED).  Plain kernels, no time split.      */
+                                 ssm_scan_fwd_bwd_host (SSM_ERR_UNSUPPORTED).                                     */
   SSM_FLAG_TEST_WITHHOLD = 16u /* test hook for the bounded waits: the tuned backward kernel shares channel groups
                                  between neighbouring warps whatever the shape, never publishes a hand-off flag and
                                  polls only 1000 times, so every warp that continues a group gives up and
@@ -109,8 +109,8 @@ SSM_API size_t ssm_scan_fwd_workspace_bytes(const ssm_problem_t* p);
 SSM_API size_t ssm_scan_bwd_workspace_bytes(const ssm_problem_t* p);
 
 /* Bytes of the `saved_states` buffer: float32 states h at the start of every block of ssm_scan_checkpoint_steps()
- * time steps.  The buffer is opaque: its layout is the library's ([batch][ceil(L / steps)][D][N], or for bf16 io with
- * N = 16 and D % 8 == 0 a layout tiled by groups of 32 channels, D rounded up to a multiple of 32) and depends on the
+ * time steps.  The buffer is opaque: its layout is the library's (tiled by groups of 32 channels, D rounded up to a
+ * multiple of 32, where a channel's states are whole 16-byte quads, else [batch][ceil(L / steps)][D][N]) and depends on the
  * problem (dimensions, dtype, SSM_FLAG_COMPLEX, the STATIC / ZOH flags); a buffer written by a forward call is valid
  * for backward calls with the same ssm_problem_t only. */
 SSM_API size_t ssm_scan_saved_state_bytes(const ssm_problem_t* p);

@@ -80,7 +80,6 @@ static bool lane_shape(const ssm_problem_t& p) {
   if (p.flags & (SSM_FLAG_COMPLEX | SSM_FLAG_ZOH_BBAR | SSM_FLAG_STATIC_B | SSM_FLAG_STATIC_C)) return false;
   return !(tuned_shape(p) && (p.flags & SSM_FLAG_TEST_WITHHOLD));   // (the hook withholds the tuned kernel's flags)
 }
-static void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl, float* cost);
 bool lane_fwd(const ssm_problem_t& p) {
   if (!lane_shape(p)) return false;
   if (!tuned_shape(p)) return true;
@@ -225,7 +224,7 @@ Plan make_plan(const ssm_problem_t& p) {
 // with a pre-pass of its own (which runs at twice the occupancy).  Costs in steps of a lone warp of the main kernel:
 // segments are chosen to fill whole waves of two blocks per SM; two warps on a sub-partition take 1.45 times as long each;
 // the pre-pass is a quarter of the work spread over all sub-partitions, its two launches 25 steps.
-static void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl, float* cost) {
+void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl, float* cost) {
   const long long chains = (long long)p.batch * pl->bwd_groups;
   auto align8 = [](long long v) { return (int)((v + kCkptSteps - 1) / kCkptSteps * kCkptSteps); };
   pl->nseg = 1;
@@ -371,10 +370,11 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
   w.dbias_part = take(parts * p.D * sizeof(float));
   w.ckpt = take((size_t)p.batch * pl.nck * ckpt_floats_per_step(ckpt_tiled(p), p.D, p.N) * sizeof(float));
   if (pl.nseg > 1) {
-    const size_t st = segs * p.D * p.N * sizeof(float);
-    w.seg_local = take(st);
-    w.mu_in = take(st);
-    w.seg_dsum = take(segs * p.D * sizeof(float));
+    // (the lane kernels keep whole groups of 32 channels and of 16 states)
+    const size_t d32 = (size_t)((p.D + 31) / 32) * 32, n16 = (size_t)((p.N + 15) / 16) * 16;
+    w.seg_local = take(segs * d32 * n16 * sizeof(float));
+    if (!lane_bwd(p)) w.mu_in = take(segs * p.D * p.N * sizeof(float));
+    w.seg_dsum = take(segs * d32 * sizeof(float));
   }
   w.fwd = take(fwd_layout(p, pl_fwd).total);   // the forward sweep that rebuilds checkpoints uses the forward split
   w.handoff = take((size_t)(w.max_workers + 1) *
@@ -743,12 +743,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   // the status word, and the hand-off flags of the tuned kernels (the lane kernel clears the status word itself)
   bool clear = true;
 #ifndef SSM_DEBUG_BOUNDS
-  BwdParams in{};
-  in.x = x;
-  in.delta = delta;
-  in.z = has_z ? z : nullptr;
-  in.dout = dout;
-  clear = !lane_bwd(*p) || !bwd_lane_applicable(in);
+  clear = !lane_bwd(*p);
 #endif
   if (clear && cudaMemsetAsync(ws, 0, w.flags + (size_t)2 * (w.max_workers + 1) * sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
   // checkpoint states: the caller's, or rebuilt here with one more forward sweep
@@ -826,7 +821,15 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   bp.handoff = reinterpret_cast<float4*>(ws + w.handoff);
   bp.max_workers = w.max_workers;
 
-  if (pl.nseg == 2 && dh_last == nullptr && (bp.seg_local = reinterpret_cast<float*>(ws + w.mu_in),
+  BwdParams carried = bp;
+  if (pl.nseg > 1) carried.mu_in = nullptr;   // (the main kernel's inflow is then in the workspace)
+  const bool lane = bwd_lane_applicable(bp) && (lane_bwd(*p) || !bwd_fast_applicable(*p, carried));
+  if (lane && pl.nseg > 1) {
+    // the lane kernel folds the segments' results itself
+    bp.seg_local = reinterpret_cast<float*>(ws + w.seg_local);
+    bp.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum);
+    if (launch_bwd_lane(*p, pl, bp, kBwdLocal, s) != cudaSuccess) return SSM_ERR_CUDA;
+  } else if (pl.nseg == 2 && dh_last == nullptr && (bp.seg_local = reinterpret_cast<float*>(ws + w.mu_in),
                                               bp.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum),
                                               bwd_local_fast_applicable(*p, bp))) {
     // two segments and nothing flowing in from outside: the adjoint leaving segment 1 IS the inflow of segment 0, so
@@ -853,8 +856,8 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
     bp.mu_in = cp.carried;
   }
   // the generic kernel (ZOH or parameter B / C off the tuned shapes) writes one partial sum per block of its own width
-  if (!bwd_fast_applicable(*p, bp) && !bwd_lane_applicable(bp)) bp.groups = (p->D + bwd_channels_per_block(p->N) - 1) / bwd_channels_per_block(p->N);
-  if (launch_bwd(*p, pl, bp, kBwdFull, s) != cudaSuccess) return SSM_ERR_CUDA;
+  if (!lane && !bwd_fast_applicable(*p, bp)) bp.groups = (p->D + bwd_channels_per_block(p->N) - 1) / bwd_channels_per_block(p->N);
+  if ((lane ? launch_bwd_lane(*p, pl, bp, kBwdFull, s) : launch_bwd(*p, pl, bp, kBwdFull, s)) != cudaSuccess) return SSM_ERR_CUDA;
 
   ReduceParams rp{};
   rp.dBC_part = bp.dBC_part;

@@ -59,24 +59,25 @@ __device__ __forceinline__ void cp_async16_bytes(void* dst, const void* src, int
 // Raw rows: the 32 channels of a block of 8 steps of x, delta, z, dout, copied asynchronously.  Rows that are not 16-byte
 // aligned go word by word, the words of the 8 rows dealt out over the lanes; a bf16 row piece that starts at an odd element
 // is copied from the word it starts in and read with a shift of one element.  Blocks are 8 rows apart, an even number of
-// elements, so what a lane copies of a block is at the same offsets in every block and in all four tensors (which
-// bwd_lane_applicable wants aligned to a word).
-template <typename IO, bool VEC>
+// elements, so what a lane copies of a block is at the same offsets in every block and in all four tensors.  If one of the
+// tensors is not even aligned to a word, elements are copied one by one.
+enum { kElements = 0, kWords = 1, kVectors = 2 };   // how rows are copied
+template <typename IO, int ROWS>
 struct RawRows {
+  static constexpr bool VEC = ROWS == kVectors;
   static constexpr int kPitch = BwdLaneSmem<IO, 1, VEC>::kPitch;
-  static constexpr int kWords = sizeof(IO) == 4 ? 32 : 17;    // words of a row (not VEC)
-  static constexpr int kCopies = VEC ? LaneRows<IO, true>::NV : (kLB * kWords + 31) / 32;
+  static constexpr int kRowWords = sizeof(IO) == 4 ? 32 : 17; // words of a row (not VEC)
+  static constexpr int kCopies = VEC ? LaneRows<IO, true>::NV : (kLB * kRowWords + 31) / 32;
   unsigned off[kCopies];   // bytes from the first element of the block's rows (plus 2 if a row may start half a word in)
   unsigned dst[kCopies];   // bytes in the tile | row << 16 (a row past the block: nothing to copy) | half a word << 12
-  int shift[2];            // elements by which rows of even / odd number are shifted in the tile
+  int shift_even, shift_odd;   // elements by which rows of even / odd number are shifted in the tile
   static constexpr unsigned kBack = VEC ? 0u : 2u;
   // first: element index (in the tensor) of the first row's first channel
+  __device__ __forceinline__ int shift(int t) const { return ROWS == kWords && sizeof(IO) == 2 ? ((t & 1) ? shift_odd : shift_even) : 0; }
   __device__ __forceinline__ void setup(size_t first, int D, int lane, int cols) {
-    shift[0] = shift[1] = 0;
-    if constexpr (!VEC && sizeof(IO) == 2) {
-      shift[0] = (int)(first & 1);
-      shift[1] = (int)((first + D) & 1);
-    }
+    shift_even = (int)(first & 1);
+    shift_odd = (int)((first + D) & 1);
+    if constexpr (ROWS == kElements) return;
 #pragma unroll
     for (int i = 0; i < kCopies; ++i) {
       const int q = lane + 32 * i;
@@ -87,13 +88,19 @@ struct RawRows {
         dst[i] = (unsigned)q * 16u | (unsigned)(col < cols ? row : kLB) << 16;
       } else {
         // (the last word of a row piece may be half: what lies behind the row may lie behind the tensor)
-        const int row = q / kWords, w = q % kWords, sh = shift[row & 1], bytes = (cols + sh) * (int)sizeof(IO) - w * 4;
+        const int row = q / kRowWords, w = q % kRowWords, sh = shift(row), bytes = (cols + sh) * (int)sizeof(IO) - w * 4;
         off[i] = (unsigned)(row * D - sh) * (unsigned)sizeof(IO) + (unsigned)w * 4u + kBack;
         dst[i] = (unsigned)(row * kPitch + w * 4) | (bytes == 2 ? 1u << 12 : 0u) | (unsigned)(bytes > 0 ? row : kLB) << 16;
       }
     }
   }
-  __device__ __forceinline__ void issue(unsigned char* tile, const IO* base, int live) const {
+  __device__ __forceinline__ void issue(unsigned char* tile, const IO* base, int D, int lane, int cols, int live) const {
+    if constexpr (ROWS == kElements) {
+#pragma unroll 1
+      for (int t = 0; t < live; ++t)
+        if (lane < cols) reinterpret_cast<IO*>(tile + t * kPitch)[lane] = base[(size_t)t * D + lane];
+      return;
+    }
     const IO* const from = reinterpret_cast<const IO*>(reinterpret_cast<const char*>(base) - kBack);
 #pragma unroll
     for (int i = 0; i < kCopies; ++i) {
@@ -106,7 +113,7 @@ struct RawRows {
   }
   __device__ __forceinline__ float get(const unsigned char* tile, int t, int lane) const {
     using RawT = typename LaneRaw<IO>::T;
-    return LaneRaw<IO>::widen(reinterpret_cast<const RawT*>(tile + t * kPitch)[lane + (VEC ? 0 : shift[t & 1])]);
+    return LaneRaw<IO>::widen(reinterpret_cast<const RawT*>(tile + t * kPitch)[lane + shift(t)]);
   }
 };
 
@@ -120,9 +127,13 @@ struct LaneChain {
   float Dk, dD, dbias;
 };
 
-template <bool AP>
+// the decays of a lane's 8 rows (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1)
+template <bool AP, bool CPLX>
 __device__ __forceinline__ void lane_decays(float dt, const float2 (&A2)[4], float2 (&a)[4]) {
-  if constexpr (AP) {
+  if constexpr (CPLX) {
+    cexp_pair(dt, A2[0], A2[2], a[0], a[2]);
+    cexp_pair(dt, A2[1], A2[3], a[1], a[3]);
+  } else if constexpr (AP) {
     const float a0 = ex2_approx(dt * A2[0].x), r = ex2_approx(dt * (A2[0].y - A2[0].x)), r2 = r * r, r4 = r2 * r2;
     a[0] = make_float2(a0, a0 * r);
     a[1] = f2mul(a[0], f2dup(r2));
@@ -134,6 +145,47 @@ __device__ __forceinline__ void lane_decays(float dt, const float2 (&A2)[4], flo
       const float2 e = f2mul(f2dup(dt), A2[k]);
       a[k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
     }
+  }
+}
+// a u + v and a u for the lane's rows, and (conj a) u
+template <bool CPLX>
+__device__ __forceinline__ void lane_mul_add(const float2 (&a)[4], const float2 (&u)[4], const float2 (&v)[4], float2 (&out)[4]) {
+  if constexpr (CPLX) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float2 ur = u[k], ui = u[k + 2];
+      out[k] = f2fma(f2neg(a[k + 2]), ui, f2fma(a[k], ur, v[k]));
+      out[k + 2] = f2fma(a[k + 2], ur, f2fma(a[k], ui, v[k + 2]));
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k] = f2fma(a[k], u[k], v[k]);
+  }
+}
+template <bool CPLX>
+__device__ __forceinline__ void lane_mul_conj(const float2 (&a)[4], const float2 (&u)[4], float2 (&out)[4]) {
+  if constexpr (CPLX) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float2 ur = u[k], ui = u[k + 2];
+      out[k] = f2fma(a[k + 2], ui, f2mul(a[k], ur));
+      out[k + 2] = f2fma(f2neg(a[k + 2]), ur, f2mul(a[k], ui));
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k] = f2mul(a[k], u[k]);
+  }
+}
+// sum over the lane's rows of w A, in units of 1 / ln 2 (A as staged)
+template <bool CPLX>
+__device__ __forceinline__ float lane_dot_a(const float2 (&w)[4], const float2 (&A2)[4], float2 part) {
+  // part: the sum over pairs 0, 1 (real parts) on entry
+  if constexpr (CPLX) {
+    const float2 im = f2fma(w[3], A2[3], f2mul(w[2], A2[2]));
+    return fmaf(im.x + im.y, kTurn / kLn2, part.x + part.y);
+  } else {
+    const float2 all = f2fma(w[3], A2[3], f2fma(w[2], A2[2], part));
+    return all.x + all.y;
   }
 }
 __device__ __forceinline__ void load8(const float* row, float2 (&v)[4]) {
@@ -158,7 +210,7 @@ __device__ __forceinline__ float3 finish_step(LaneChain& lc, float4 v1, float4 v
 // One block of 8 steps of one group of 16 states.  t1 / t2: per-step values; fB / fC: rows of 16 states; ck: the states
 // before the block; part_dB / part_dC: first row of this block in the partial sums (stride N); emit(t, y, lb, wa, v1, v2)
 // takes the sums over the 16 states for the lane's own channel.
-template <bool AP, typename Emit>
+template <bool AP, bool CPLX, typename Emit>
 __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, const float4* t2, const float* fB, const float* fC,
                                            const float4* ck, float4* red, float* part_dB, float* part_dC, int N, int n_live,
                                            int live, int lane, Emit&& emit) {
@@ -183,12 +235,16 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
       for (int q = 0; q < 2; ++q) {
         const float dt = q ? v.y : v.x, u = q ? v.w : v.z;
         float2 a[4];
-        lane_decays<AP>(dt, lc.A2[q], a);
+        lane_decays<AP, CPLX>(dt, lc.A2[q], a);
         const float2 du2 = f2dup(dt * u);
+        float2 bx[4], hn[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) bx[k] = f2mul(du2, Bv[k]);
+        lane_mul_add<CPLX>(a, h[q], bx, hn);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          h[q][k] = f2fma(a[k], h[q][k], f2mul(du2, Bv[k]));
-          if (t & 1) hist[t >> 1][q][k] = h[q][k];
+          h[q][k] = hn[k];
+          if (t & 1) hist[t >> 1][q][k] = hn[k];
         }
       }
     }
@@ -208,19 +264,21 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
       for (int q = 0; q < 2; ++q) {
         const float dt = q ? v1o.y : v1o.x, u = q ? v1o.w : v1o.z, ds = q ? v2o.y : v2o.x;
         float2 a[4];
-        lane_decays<AP>(dt, lc.A2[q], a);
-        const float2 ds2 = f2dup(ds), du2 = f2dup(dt * u);
-        float2 yv = make_float2(0.f, 0.f), lb = yv;
+        lane_decays<AP, CPLX>(dt, lc.A2[q], a);
+        // (complex: the staged C is its conjugate and the readout twice a real part, so lam = 2 ds conj(C) + mu; the
+        // imaginary rows of dC come out with the other sign)
+        const float2 ds2 = f2dup(CPLX ? 2.f * ds : ds), du2 = f2dup(dt * u);
+        float2 yv = make_float2(0.f, 0.f), lb = yv, lam[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const float2 hc = hist[m][q][k];
-          const float2 lam = f2fma(Cv[k], ds2, lc.mu[q][k]);
+          lam[k] = f2fma(Cv[k], ds2, lc.mu[q][k]);
           dCt[k] = q == 0 ? f2mul(ds2, hc) : f2fma(ds2, hc, dCt[k]);
-          dBt[k] = q == 0 ? f2mul(lam, du2) : f2fma(lam, du2, dBt[k]);
-          lb = f2fma(lam, Bv[k], lb);
+          dBt[k] = q == 0 ? f2mul(lam[k], du2) : f2fma(lam[k], du2, dBt[k]);
+          lb = f2fma(lam[k], Bv[k], lb);
           yv = f2fma(Cv[k], hc, yv);
-          lc.mu[q][k] = f2mul(a[k], lam);
         }
+        lane_mul_conj<CPLX>(a, lam, lc.mu[q]);
         yo[q] = yv.x + yv.y;
         lo[q] = lb.x + lb.y;
       }
@@ -244,36 +302,39 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
       for (int q = 0; q < 2; ++q) {
         const float dt = q ? v1e.y : v1e.x, u = q ? v1e.w : v1e.z, ds = q ? v2e.y : v2e.x;
         float2 a[4];
-        lane_decays<AP>(dt, lc.A2[q], a);
-        const float2 ds2 = f2dup(ds), du2 = f2dup(dt * u), dte2 = f2dup(dt), dto2 = f2dup(q ? v1o.y : v1o.x);
-        float2 yv = make_float2(0.f, 0.f), lb = yv, wea = yv, woa = yv;
+        lane_decays<AP, CPLX>(dt, lc.A2[q], a);
+        const float2 ds2 = f2dup(CPLX ? 2.f * ds : ds), du2 = f2dup(dt * u), dte2 = f2dup(dt), dto2 = f2dup(q ? v1o.y : v1o.x);
+        float2 yv = make_float2(0.f, 0.f), lb = yv, hpp[4], he[4], bx[4], w1[4], lam[4], w0[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          float2 hpp;   // the state before the even step: the history entry before, or the checkpoint
+          // the state before the even step: the history entry before, or the checkpoint
           if (m > 0) {
-            hpp = hist[m > 0 ? m - 1 : 0][q][k];
+            hpp[k] = hist[m > 0 ? m - 1 : 0][q][k];
           } else {
             const float4 v = ck[(2 * q + (k >> 1)) * 32 + lane];
-            hpp = (k & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+            hpp[k] = (k & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
           }
-          const float2 he = f2fma(a[k], hpp, f2mul(du2, Bv[k]));
-          const float2 w1 = f2mul(lc.mu[q][k], he);
-          woa = f2fma(w1, lc.A2[q][k], woa);
-          lc.dA[q][k] = f2fma(w1, dto2, lc.dA[q][k]);
-          const float2 lam = f2fma(Cv[k], ds2, lc.mu[q][k]);
-          dCt[k] = q == 0 ? f2mul(ds2, he) : f2fma(ds2, he, dCt[k]);
-          dBt[k] = q == 0 ? f2mul(lam, du2) : f2fma(lam, du2, dBt[k]);
-          lb = f2fma(lam, Bv[k], lb);
-          yv = f2fma(Cv[k], he, yv);
-          lc.mu[q][k] = f2mul(a[k], lam);
-          const float2 w0 = f2mul(lc.mu[q][k], hpp);
-          wea = f2fma(w0, lc.A2[q][k], wea);
-          lc.dA[q][k] = f2fma(w0, dte2, lc.dA[q][k]);
+          bx[k] = f2mul(du2, Bv[k]);
         }
+        lane_mul_add<CPLX>(a, hpp, bx, he);
+        lane_mul_conj<CPLX>(he, lc.mu[q], w1);   // the odd step's w = conj(h_{t-1}) mu_t
+        wo[q] = lane_dot_a<CPLX>(w1, lc.A2[q], f2fma(w1[1], lc.A2[q][1], f2mul(w1[0], lc.A2[q][0])));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          lc.dA[q][k] = f2fma(w1[k], dto2, lc.dA[q][k]);
+          lam[k] = f2fma(Cv[k], ds2, lc.mu[q][k]);
+          dCt[k] = q == 0 ? f2mul(ds2, he[k]) : f2fma(ds2, he[k], dCt[k]);
+          dBt[k] = q == 0 ? f2mul(lam[k], du2) : f2fma(lam[k], du2, dBt[k]);
+          lb = f2fma(lam[k], Bv[k], lb);
+          yv = f2fma(Cv[k], he[k], yv);
+        }
+        lane_mul_conj<CPLX>(a, lam, lc.mu[q]);
+        lane_mul_conj<CPLX>(hpp, lc.mu[q], w0);
+        we[q] = lane_dot_a<CPLX>(w0, lc.A2[q], f2fma(w0[1], lc.A2[q][1], f2mul(w0[0], lc.A2[q][0])));
+#pragma unroll
+        for (int k = 0; k < 4; ++k) lc.dA[q][k] = f2fma(w0[k], dte2, lc.dA[q][k]);
         ye[q] = yv.x + yv.y;
         le[q] = lb.x + lb.y;
-        we[q] = wea.x + wea.y;
-        wo[q] = woa.x + woa.y;
       }
       float4* rrow = red + (te & 3) * 128 + lane * 4;
 #pragma unroll
@@ -287,8 +348,8 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
     we[0] += __shfl_xor_sync(0xffffffffu, we[1], 1);
     wo[0] += __shfl_xor_sync(0xffffffffu, wo[1], 1);
     __syncwarp();   // all lanes have read the two rows of t2: their slots may take results
-    emit(to, yo[0], lo[0], wo[0], v1o, v2o);
-    emit(te, ye[0], le[0], we[0], v1e, v2e);
+    emit(to, CPLX ? 2.f * yo[0] : yo[0], lo[0], wo[0], v1o, v2o);
+    emit(te, CPLX ? 2.f * ye[0] : ye[0], le[0], we[0], v1e, v2e);
     if (m % 2 == 0) {
       // dB / dC of steps 2m .. 2m + 3: every lane sums one float4 of one step over the 16 lane pairs, ascending
       __syncwarp();
@@ -303,7 +364,14 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
         lo = gg == 0 ? make_float2(x.x, x.y) : __fadd2_rn(lo, make_float2(x.x, x.y));
         hi = gg == 0 ? make_float2(x.z, x.w) : __fadd2_rn(hi, make_float2(x.z, x.w));
       }
-      const float4 acc = make_float4(lo.x, lo.y, hi.x, hi.y);
+      float4 acc = make_float4(lo.x, lo.y, hi.x, hi.y);
+      if constexpr (CPLX) {
+        // four real or four imaginary rows to four columns: the lanes of a half exchange two values each
+        const bool im = o & 1;
+        if (im && which) acc = make_float4(-acc.x, -acc.y, -acc.z, -acc.w);
+        const float gx = __shfl_xor_sync(0xffffffffu, im ? acc.x : acc.z, 1), gy = __shfl_xor_sync(0xffffffffu, im ? acc.y : acc.w, 1);
+        acc = im ? make_float4(gx, acc.z, gy, acc.w) : make_float4(acc.x, gx, acc.y, gy);
+      }
       const int row = 2 * m + s;
       if (row < live && n0 < n_live) {
         float* dst = (which ? part_dC : part_dB) + (size_t)row * N + n0;
@@ -321,7 +389,7 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
 
 // The lam / mu recurrence alone over steps [t_begin, t_end) of one chain, last to first, from mu (a lane per channel, states
 // 16 gi ..): what it leaves and the sum of delta.  a_log2: A * log2(e) of the 16 states [16][32]; tiles: 2048 floats.
-template <typename IO, bool VEC>
+template <typename IO, bool VEC, bool CPLX>
 __device__ __forceinline__ void adjoint_sweep(const BwdParams& p, int N, int gi, size_t row_b, int t_begin, int t_end, int c0, int lane,
                                               const float* a_log2, bool ap, float bias, bool cvec, float* tiles, float2 (&mu)[8],
                                               float& dsum) {
@@ -362,7 +430,7 @@ __device__ __forceinline__ void adjoint_sweep(const BwdParams& p, int N, int gi,
       rd.put(td, lane);
       rz.put(tz, lane);
       rg.put(tg, lane);
-      *reinterpret_cast<float4*>(tC + 4 * lane) = qC.widen();
+      put_quad<CPLX>(tC, lane, qC.widen(), -1.f);
       float dt[kLB], ds[kLB];
       if constexpr (VEC) {
         __syncwarp();
@@ -394,7 +462,13 @@ __device__ __forceinline__ void adjoint_sweep(const BwdParams& p, int N, int gi,
       // decays and C ds of a step are prepared one step ahead of the recurrence that consumes them
       float2 aN[2][8], cN[2][8];
       auto front = [&](int t, float2 (&a)[8], float2 (&cd)[8]) {
-        if constexpr (AP) {
+        if constexpr (CPLX) {
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            const int k = (kk & 1) + 4 * (kk >> 1);
+            cexp_pair(dt[t], A2[k], A2[k + 2], a[k], a[k + 2]);
+          }
+        } else if constexpr (AP) {
           const float a0 = ex2_approx(dt[t] * A2[0].x), r = ex2_approx(dt[t] * (A2[0].y - A2[0].x)), r2 = r * r, r4 = r2 * r2,
                       r8 = r4 * r4;
           a[0] = make_float2(a0, a0 * r);
@@ -416,13 +490,24 @@ __device__ __forceinline__ void adjoint_sweep(const BwdParams& p, int N, int gi,
 #pragma unroll
       for (int t = kLB - 1; t >= 0; --t) {
         if (t > 0) front(t - 1, aN[(t - 1) & 1], cN[(t - 1) & 1]);
-        const float2 ds2 = f2dup(ds[t]);
+        const float2 ds2 = f2dup(CPLX ? 2.f * ds[t] : ds[t]);
+        if constexpr (CPLX) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) mu[k] = f2mul(aN[t & 1][k], f2fma(cN[t & 1][k], ds2, mu[k]));
+          for (int kk = 0; kk < 4; ++kk) {
+            const int k = (kk & 1) + 4 * (kk >> 1);
+            const float2 ar = aN[t & 1][k], ai = aN[t & 1][k + 2];
+            const float2 lr = f2fma(cN[t & 1][k], ds2, mu[k]), li = f2fma(cN[t & 1][k + 2], ds2, mu[k + 2]);
+            mu[k] = f2fma(ai, li, f2mul(ar, lr));
+            mu[k + 2] = f2fma(f2neg(ai), lr, f2mul(ar, li));
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) mu[k] = f2mul(aN[t & 1][k], f2fma(cN[t & 1][k], ds2, mu[k]));
+        }
       }
     }
   };
-  if constexpr (sizeof(IO) == 2) {
+  if constexpr (sizeof(IO) == 2 && !CPLX) {
     if (ap) run(std::true_type{});
     else run(std::false_type{});
   } else {
@@ -442,10 +527,11 @@ __device__ __forceinline__ bool lane_progression(const float* a_log2, int N, int
   return __all_sync(0xffffffffu, ap);
 }
 
-// First pass of a launch split in time: one warp per (chain, group of 16 states), the adjoint that leaves the segment.
-// Latency-bound, so capped for four warps per sub-partition.
-template <typename IO, bool VEC>
-__global__ void __launch_bounds__(kLaneWarps * 32, 4) ssm_bwd_lane_local_kernel(const BwdParams p, const int N, const int ng) {
+// First pass of a launch split in time: one warp per (chain, group of 16 states), the adjoint that leaves the segment (the
+// main kernel folds what leaves the segments behind its own).
+// Latency-bound, so capped for four warps per sub-partition (float32 rows in flight take more registers: three).
+template <typename IO, bool VEC, bool CPLX>
+__global__ void __launch_bounds__(kLaneWarps * 32, sizeof(IO) == 4 ? 3 : 4) ssm_bwd_lane_local_kernel(const BwdParams p, const int N, const int ng) {
   __shared__ __align__(16) float s_tiles[kLaneWarps][2048];
   __shared__ float s_A[kLaneWarps][16 * 32];
   const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
@@ -457,26 +543,33 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 4) ssm_bwd_lane_local_kernel(
   const int c_own = grp * 32 + lane, c_ld = min(c_own, D - 1);
   const int t_begin = seg * p.seg_steps, t_end = min(p.L, t_begin + p.seg_steps);
   float* const sA = s_A[bwarp];
-  for (int n = 0; n < 16; ++n) sA[n * 32 + lane] = 16 * gi + n < N ? p.A[(size_t)c_ld * N + 16 * gi + n] * kLog2e : 0.f;
+  for (int n = 0; n < 16; ++n) {
+    const int col = lane_col<CPLX>(16 * gi + n);
+    sA[n * 32 + lane] = col < N ? p.A[(size_t)c_ld * N + col] * lane_a_scale<CPLX>(n) : 0.f;
+  }
   const float bias = p.delta_bias != nullptr ? p.delta_bias[c_ld] : 0.f;
   const bool cvec = N >= 4 && (reinterpret_cast<uintptr_t>(p.C) & (4 * sizeof(IO) - 1)) == 0;
-  const bool ap = lane_progression<IO>(sA, N, gi, p.general_A, lane);
+  const bool ap = !CPLX && lane_progression<IO>(sA, N, gi, p.general_A, lane);
   float2 mu[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) mu[k] = make_float2(0.f, 0.f);
   float dsum = 0.f;
-  adjoint_sweep<IO, VEC>(p, N, gi, (size_t)b * p.L, t_begin, t_end, grp * 32, lane, sA, ap, bias, cvec, s_tiles[bwarp], mu, dsum);
-  if (c_own < D) {
-    const size_t row = ((size_t)b * p.nseg + seg) * D + c_own;
+  adjoint_sweep<IO, VEC, CPLX>(p, N, gi, (size_t)b * p.L, t_begin, t_end, grp * 32, lane, sA, ap, bias, cvec, s_tiles[bwarp], mu, dsum);
+  // [batch][segment][channel group][row][32], rows as in shared memory
+  const size_t at = ((size_t)b * p.nseg + seg) * groups + grp;
+  float* const dst = p.seg_local + (at * ng + gi) * 512 + lane;
 #pragma unroll
-    for (int n = 0; n < 16; ++n)
-      if (16 * gi + n < N) p.seg_local[row * N + 16 * gi + n] = (n & 1) ? mu[n >> 1].y : mu[n >> 1].x;
-    if (gi == 0) p.seg_dsum[row] = dsum;
+  for (int k = 0; k < 8; ++k) {
+    dst[64 * k] = mu[k].x;
+    dst[64 * k + 32] = mu[k].y;
   }
+  if (gi == 0) p.seg_dsum[at * 32 + lane] = dsum;
 }
 
-template <typename IO, int NG, bool VEC>
+// CPLX: complex states, as in ssm_fwd_lane.cu
+template <typename IO, int NG, int ROWS, bool CPLX>
 __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const BwdParams p, const LaneSplit sp, const int N) {
+  constexpr bool VEC = ROWS == kVectors;
   using SM = BwdLaneSmem<IO, NG, VEC>;
   constexpr int NP = SM::NP, kTeams = SM::kTeams;
   extern __shared__ __align__(16) unsigned char smem[];
@@ -544,7 +637,10 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * NG) : "memory");
   };
 
-  for (int n = tw * NG + gi; n < NP; n += W * NG) sA[n * 32 + lane] = n < N ? p.A[(size_t)c_ld * N + n] * kLog2e : 0.f;
+  for (int n = tw * NG + gi; n < NP; n += W * NG) {
+    const int col = lane_col<CPLX>(n);
+    sA[n * 32 + lane] = col < N ? p.A[(size_t)c_ld * N + col] * lane_a_scale<CPLX>(n) : 0.f;
+  }
   const float bias = p.delta_bias != nullptr ? p.delta_bias[c_ld] : 0.f;
   // four of the 16 states of row lane / 4 of a block of B or C; rows past the end are zero
   auto quad = [&](LaneQuad<IO>& q, const IO* src, int t0, bool vec) {
@@ -552,10 +648,9 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
     q.load(src + (row_b + t0 + r) * N + n, t0 + r < t_end ? N - n : 0, vec);
   };
   __syncthreads();
-  const bool ap = lane_progression<IO>(sA + gi * 512, N, gi, p.general_A, lane);
+  const bool ap = !CPLX && lane_progression<IO>(sA + gi * 512, N, gi, p.general_A, lane);
 
   const bool split = W * CL > 1;
-  const size_t seg_row = ((size_t)b * p.nseg + seg) * D;
   // ---- first sweep: the adjoint that leaves the piece with nothing flowing in (a lane per channel, 16 states)
   float dsum = 0.f;
   if (split) {
@@ -563,7 +658,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
 #pragma unroll
     for (int k = 0; k < 8; ++k) mu[k] = make_float2(0.f, 0.f);
     if (live_piece && rank * W + tw > 0) {   // (nobody wants what leaves the first piece)
-      adjoint_sweep<IO, VEC>(p, N, gi, row_b, t_begin, t_end, grp * 32, lane, sA + gi * 512, ap, bias, cvec,
+      adjoint_sweep<IO, VEC, CPLX>(p, N, gi, row_b, t_begin, t_end, grp * 32, lane, sA + gi * 512, ap, bias, cvec,
                              reinterpret_cast<float*>(red), mu, dsum);
       __syncwarp();
     }
@@ -577,26 +672,27 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   }
 
   // ---- rows of the main sweep: each warp of the team copies its share of the four tensors
-  RawRows<IO, VEC> rr;
+  RawRows<IO, ROWS> rr;
   rr.setup((row_b + t_begin) * D + grp * 32, D, lane, cols);
   auto issue_rows = [&](int t0) {
     const size_t base = (row_b + t0) * D + grp * 32;
     const int live = min(kLB, t_end - t0);
-    if (0 % NG == gi) rr.issue(rX, gx + base, live);
-    if (1 % NG == gi) rr.issue(rD, gd + base, live);
-    if (2 % NG == gi && has_z) rr.issue(rZ, gz + base, live);
-    if (3 % NG == gi) rr.issue(rG, gg + base, live);
+    if (0 % NG == gi) rr.issue(rX, gx + base, D, lane, cols, live);
+    if (1 % NG == gi) rr.issue(rD, gd + base, D, lane, cols, live);
+    if (2 % NG == gi && has_z) rr.issue(rZ, gz + base, D, lane, cols, live);
+    if (3 % NG == gi) rr.issue(rG, gg + base, D, lane, cols, live);
   };
   // the states before a block, for the lane's two channels and 8 states: vectors [2 q + k][lane]
   const bool ck_vec = p.ckpt_tiled && (reinterpret_cast<uintptr_t>(p.ckpt) & 15) == 0;
   const int n_own = 16 * gi + 8 * (lane & 1);   // first of the lane's states
-  const float* const ck_own = p.ckpt + ckpt_offset(1, b, p.nck, 0, D, N, grp * 32, 0) + (size_t)(n_own >> 2) * 128;
-  const size_t ck_step = ckpt_floats_per_step(1, D, N);
+  const int NC = lane_ckpt_rows<CPLX>(N);
+  const float* const ck_own = p.ckpt + ckpt_offset(1, b, p.nck, 0, D, NC, grp * 32, 0) + (size_t)(n_own >> 2) * 128;
+  const size_t ck_step = ckpt_floats_per_step(1, D, NC);
   int ck_bytes[2][2];   // 16, or 0 where the channel or the states do not exist
 #pragma unroll
   for (int q = 0; q < 2; ++q)
 #pragma unroll
-    for (int k = 0; k < 2; ++k) ck_bytes[q][k] = (lane ^ q) < cols && n_own + 4 * k < N ? 16 : 0;
+    for (int k = 0; k < 2; ++k) ck_bytes[q][k] = (lane ^ q) < cols && n_own + 4 * k < NC ? 16 : 0;
   auto issue_ckpt = [&](int t0, float4* dst) {
     const int kc = t0 / kCkptSteps;
     const float* const src = ck_own + (size_t)kc * ck_step;
@@ -611,7 +707,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
 #pragma unroll 1
           for (int i = 0; i < 4; ++i) {
             const int n = n_own + 4 * k + i;
-            const float x = (lane ^ q) < cols && n < N ? p.ckpt[ckpt_offset(p.ckpt_tiled, b, p.nck, kc, D, N, grp * 32 + (lane ^ q), n)] : 0.f;
+            const float x = (lane ^ q) < cols && n < NC ? p.ckpt[ckpt_offset(p.ckpt_tiled, b, p.nck, kc, D, NC, grp * 32 + (lane ^ q), n)] : 0.f;
             reinterpret_cast<float*>(at)[i] = x;
           }
         }
@@ -633,45 +729,104 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   lc.dD = lc.dbias = 0.f;
   if (split) {
     __syncthreads();
+    // (a complex adjoint: rows n and n + 4)
+    constexpr int kRow2 = 4 * 32;
     for (int n = tw * NG + gi; n < NP; n += W * NG) {
-      const float a2 = sA[n * 32 + lane];
-      float pre = 0.f, ds = 0.f;
+      if (CPLX && (n & 4)) continue;
+      const float a2 = sA[n * 32 + lane], ai = CPLX ? sA[n * 32 + kRow2 + lane] : 0.f;
+      float2 pre = make_float2(0.f, 0.f);
+      float ds = 0.f;
       for (int w = W - 1; w >= 0; --w) {
         float* const at = leaving(w, n) + lane;
-        const float l = *at, d = sDs[w * 32 + lane];
-        *at = pre;
-        pre = fmaf(ex2_approx(a2 * d), pre, l);
+        const float d = sDs[w * 32 + lane];
+        const float2 l = make_float2(*at, CPLX ? at[kRow2] : 0.f);
+        *at = pre.x;
+        if (CPLX) at[kRow2] = pre.y;
+        const float2 q = CPLX ? cexp_apply<true>(d, a2, ai, pre) : make_float2(ex2_approx(a2 * d) * pre.x, 0.f);
+        pre = make_float2(q.x + l.x, q.y + l.y);
         ds += d;
       }
-      sTot[n * 32 + lane] = pre;
+      sTot[n * 32 + lane] = pre.x;
+      if (CPLX) sTot[n * 32 + kRow2 + lane] = pre.y;
       if (n == 0) sTotDs[lane] = ds;
     }
     if (CL > 1) cg::this_cluster().sync();
     else __syncthreads();
     for (int n = tw * NG + gi; n < NP; n += W * NG) {
-      const float a2 = sA[n * 32 + lane];
-      float M = (p.mu_in != nullptr && n < N) ? p.mu_in[(seg_row + c_ld) * N + n] : 0.f;
-      float rt[kLaneMaxCluster], rds[kLaneMaxCluster];
+      if (CPLX && (n & 4)) continue;
+      const int col = lane_col<CPLX>(n);
+      const float a2 = sA[n * 32 + lane], ai = CPLX ? sA[n * 32 + kRow2 + lane] : 0.f;
+      auto step = [&](float d, float2 v) {
+        return CPLX ? cexp_apply<true>(d, a2, ai, v) : make_float2(ex2_approx(a2 * d) * v.x, 0.f);
+      };
+      float2 M = make_float2(0.f, 0.f);
+      if (p.mu_in != nullptr && col < N) {
+        M.x = p.mu_in[((size_t)b * D + c_ld) * N + col];
+        if (CPLX) M.y = p.mu_in[((size_t)b * D + c_ld) * N + col + 1];
+      }
+      float2 rt[kLaneMaxCluster];
+      float rds[kLaneMaxCluster];
 #pragma unroll
       for (int r = kLaneMaxCluster - 1; r > 0; --r) {   // (all requested before the first is used)
         if (r > rank && r < CL) {
-          rt[r] = cg::this_cluster().map_shared_rank(sTot, r)[n * 32 + lane];
+          const float* const tot = cg::this_cluster().map_shared_rank(sTot, r) + n * 32 + lane;
+          rt[r] = make_float2(tot[0], CPLX ? tot[kRow2] : 0.f);
           rds[r] = cg::this_cluster().map_shared_rank(sTotDs, r)[lane];
         }
       }
 #pragma unroll
       for (int r = kLaneMaxCluster - 1; r > 0; --r) {
-        if (r > rank && r < CL) M = fmaf(ex2_approx(a2 * rds[r]), M, rt[r]);
+        if (r > rank && r < CL) {
+          const float2 q = step(rds[r], M);
+          M = make_float2(q.x + rt[r].x, q.y + rt[r].y);
+        }
       }
       float cum = 0.f;
       for (int w = W - 1; w >= 0; --w) {
         float* const at = leaving(w, n) + lane;
-        *at = fmaf(ex2_approx(a2 * cum), M, *at);
+        const float2 q = step(cum, M);
+        *at += q.x;
+        if (CPLX) at[kRow2] += q.y;
         cum += sDs[w * 32 + lane];
       }
     }
     if (CL > 1) cg::this_cluster().sync();   // (also: no block leaves while another still reads its totals)
     else __syncthreads();
+  }
+  // a launch split into segments: fold what leaves the segments behind this one, last to first
+  const bool behind = p.nseg > 1 && seg < p.nseg - 1;
+  if (behind) {
+    float M[16];
+#pragma unroll
+    for (int n = 0; n < 16; ++n) {
+      const int col = lane_col<CPLX>(16 * gi + n);
+      M[n] = p.mu_in != nullptr && col < N ? p.mu_in[((size_t)b * D + c_ld) * N + col] : 0.f;
+    }
+    const float* const a = sA + gi * 512 + lane;
+#pragma unroll 1
+    for (int sg = p.nseg - 1; sg > seg; --sg) {
+      const size_t at = ((size_t)b * p.nseg + sg) * groups + grp;
+      const float* const src = p.seg_local + (at * NG + gi) * 512 + lane;
+      const float ds = p.seg_dsum[at * 32 + lane];
+      float l[16];
+#pragma unroll
+      for (int n = 0; n < 16; ++n) l[n] = src[32 * n];
+#pragma unroll
+      for (int n = 0; n < 16; ++n) {
+        if constexpr (CPLX) {
+          if (n & 4) continue;
+          const float2 q = cexp_apply<true>(ds, a[32 * n], a[32 * n + 128], make_float2(M[n], M[n + 4]));
+          M[n] = q.x + l[n];
+          M[n + 4] = q.y + l[n + 4];
+        } else {
+          M[n] = fmaf(ex2_approx(a[32 * n] * ds), M[n], l[n]);
+        }
+      }
+    }
+    float* const to = leaving(tw, 16 * gi) + lane;
+#pragma unroll
+    for (int n = 0; n < 16; ++n) to[32 * n] = M[n];
+    __syncwarp();
   }
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
@@ -681,8 +836,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
     for (int k = 0; k < 8; ++k) {
       const int n = 16 * gi + 8 * (lane & 1) + k;
       float m = 0.f;
-      if (split) m = ok ? leaving(tw, n)[cl] : 0.f;
-      else if (p.mu_in != nullptr && ok && n < N) m = p.mu_in[(seg_row + grp * 32 + cl) * N + n];
+      if (split || behind) m = ok ? leaving(tw, n)[cl] : 0.f;
+      else if (p.mu_in != nullptr && ok && lane_col<CPLX>(n) < N) m = p.mu_in[((size_t)b * D + grp * 32 + cl) * N + lane_col<CPLX>(n)];
       reinterpret_cast<float*>(lc.mu[q])[k] = m;
       reinterpret_cast<float*>(lc.A2[q])[k] = sA[n * 32 + cl];
       reinterpret_cast<float*>(lc.dA[q])[k] = 0.f;
@@ -716,8 +871,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
       const int live = min(kLB, t_end - t0);
       const size_t row0 = row_b + t0, base = row0 * D + grp * 32;
       cp_async_wait_all();
-      *reinterpret_cast<float4*>(fB + 4 * lane) = qB.widen();
-      *reinterpret_cast<float4*>(fC + 4 * lane) = qC.widen();
+      put_quad<CPLX>(fB, lane, qB.widen(), 1.f);
+      put_quad<CPLX>(fC, lane, qC.widen(), -1.f);   // (complex: conj C)
       team_sync();   // the rows of all warps of the team have landed
       // per-step values of the rows, each warp its share: step size, input, gate terms.  (Not unrolled further: the body of a
       // block is near the size of the instruction cache.)
@@ -755,7 +910,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
       cp_async_commit();
       auto put = [&](int t, float3 r) { t2[t * 32 + out_slot(t, lane)] = make_float4(r.x, r.y, r.z, 0.f); };
       float* const part_dB = p.dBC_part + (size_t)grp * 2 * bln + row0 * N + 16 * gi;
-      lane_block<AP>(lc, t1, t2, fB, fC, ck + st * 128, red, part_dB, part_dB + bln, N, N - 16 * gi, live, lane,
+      lane_block<AP, CPLX>(lc, t1, t2, fB, fC, ck + st * 128, red, part_dB, part_dB + bln, N, N - 16 * gi, live, lane,
                      [&](int t, float y, float lb, float wa, float4 v1, float4 v2) {
                        if constexpr (NG == 1) put(t, finish_step(lc, v1, v2, y, lb, wa, t < live));
                        else ex[t * 32 + lane] = make_float4(y, lb, wa, 0.f);
@@ -815,7 +970,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
     }
   };
   if (live_piece) {
-    if constexpr (sizeof(IO) == 2) {
+    if constexpr (sizeof(IO) == 2 && !CPLX) {
       if (ap) sweep(std::true_type{});
       else sweep(std::false_type{});
     } else {
@@ -842,7 +997,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int n = 16 * gi + 8 * (lane & 1) + k;
-          if (c < D && n < N) p.dh0[((size_t)b * D + c) * N + n] = reinterpret_cast<float*>(lc.mu[q])[k];
+          const int col = lane_col<CPLX>(n);
+          if (c < D && col < N) p.dh0[((size_t)b * D + c) * N + col] = reinterpret_cast<float*>(lc.mu[q])[k];
         }
       }
     }
@@ -850,10 +1006,11 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   __syncthreads();
   if (valid && chain_id < chains) {
     const size_t part = ((size_t)b * p.nseg + seg) * CL + rank;
-    for (int n = tw * NG + gi; n < N; n += W * NG) {
+    for (int n = tw * NG + gi; n < NP; n += W * NG) {
+      const int col = lane_col<CPLX>(n);
       float v = 0.f;
       for (int w = 0; w < W; ++w) v += leaving(w, n)[lane];
-      p.dA_part[(part * D + c_own) * N + n] = v;
+      if (col < N) p.dA_part[(part * D + c_own) * N + col] = v;
     }
     if (tw == 0 && gi == 0) {
       float dD = 0.f, db = 0.f;
@@ -867,14 +1024,15 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   }
 }
 
-template <typename IO, int NG, bool VEC>
+template <typename IO, int NG, int ROWS, bool CPLX>
 cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int mode, cudaStream_t s) {
+  constexpr bool VEC = ROWS == kVectors;
   using SM = BwdLaneSmem<IO, NG, VEC>;
-  auto kern = ssm_bwd_lane_kernel<IO, NG, VEC>;
+  auto kern = ssm_bwd_lane_kernel<IO, NG, ROWS, CPLX>;
   if (mode == kBwdLocal) {
     const long long items = (long long)p.batch * (plan.nseg - 1) * ((p.D + 31) / 32) * NG;
     if (items > 0)
-      ssm_bwd_lane_local_kernel<IO, VEC><<<(unsigned)((items + kLaneWarps - 1) / kLaneWarps), kLaneWarps * 32, 0, s>>>(p, N, NG);
+      ssm_bwd_lane_local_kernel<IO, VEC, CPLX><<<(unsigned)((items + kLaneWarps - 1) / kLaneWarps), kLaneWarps * 32, 0, s>>>(p, N, NG);
     return cudaGetLastError();
   }
   const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
@@ -897,33 +1055,34 @@ cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int m
   return cudaLaunchKernelEx(&cfg, kern, p, sp, N);
 }
 
-template <typename IO, int NG>
+template <typename IO, int NG, bool CPLX>
 cudaError_t launch_bwd_lane_vec(const Plan& plan, const BwdParams& p, int N, int mode, cudaStream_t s) {
-  bool vec = (size_t)p.D * sizeof(IO) % 16 == 0;
-  for (const void* q : {p.x, p.delta, p.z, p.dout, (const void*)p.dx, (const void*)p.ddelta, (const void*)p.dz})
-    vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
-  return vec ? launch_bwd_lane_n<IO, NG, true>(plan, p, N, mode, s) : launch_bwd_lane_n<IO, NG, false>(plan, p, N, mode, s);
+  uintptr_t in = 0, out = 0;
+  for (const void* q : {p.x, p.delta, p.z, p.dout}) in |= reinterpret_cast<uintptr_t>(q);
+  for (const void* q : {p.dx, p.ddelta, p.dz}) out |= reinterpret_cast<uintptr_t>(q);
+  if ((size_t)p.D * sizeof(IO) % 16 == 0 && ((in | out) & 15) == 0) return launch_bwd_lane_n<IO, NG, kVectors, CPLX>(plan, p, N, mode, s);
+  if constexpr (sizeof(IO) == 2) {
+    if (in & 3) return launch_bwd_lane_n<IO, NG, kElements, CPLX>(plan, p, N, mode, s);
+  }
+  return launch_bwd_lane_n<IO, NG, kWords, CPLX>(plan, p, N, mode, s);
 }
 
-template <typename IO>
+template <typename IO, bool CPLX>
 cudaError_t launch_bwd_lane_io(const Plan& plan, const BwdParams& p, int N, int mode, cudaStream_t s) {
-  if (N <= 16) return launch_bwd_lane_vec<IO, 1>(plan, p, N, mode, s);
-  if (N <= 32) return launch_bwd_lane_vec<IO, 2>(plan, p, N, mode, s);
-  return launch_bwd_lane_vec<IO, 4>(plan, p, N, mode, s);
+  if (N <= 16) return launch_bwd_lane_vec<IO, 1, CPLX>(plan, p, N, mode, s);
+  if (N <= 32) return launch_bwd_lane_vec<IO, 2, CPLX>(plan, p, N, mode, s);
+  return launch_bwd_lane_vec<IO, 4, CPLX>(plan, p, N, mode, s);
 }
 
 }  // namespace
 
-bool bwd_lane_applicable(const BwdParams& p) {
-  if (p.zoh || p.static_B || p.static_C) return false;
-  for (const void* q : {p.x, p.delta, p.z, p.dout})
-    if (reinterpret_cast<uintptr_t>(q) & 3) return false;
-  return true;
-}
+bool bwd_lane_applicable(const BwdParams& p) { return !p.zoh && !p.static_B && !p.static_C; }
 
 cudaError_t launch_bwd_lane(const ssm_problem_t& prob, const Plan& plan, const BwdParams& p, int mode, cudaStream_t s) {
-  if (prob.io_dtype == SSM_BF16) return launch_bwd_lane_io<__nv_bfloat16>(plan, p, prob.N, mode, s);
-  return launch_bwd_lane_io<float>(plan, p, prob.N, mode, s);
+  const bool bf = prob.io_dtype == SSM_BF16;
+  if (prob.flags & SSM_FLAG_COMPLEX)
+    return bf ? launch_bwd_lane_io<__nv_bfloat16, true>(plan, p, 2 * prob.N, mode, s) : launch_bwd_lane_io<float, true>(plan, p, 2 * prob.N, mode, s);
+  return bf ? launch_bwd_lane_io<__nv_bfloat16, false>(plan, p, prob.N, mode, s) : launch_bwd_lane_io<float, false>(plan, p, prob.N, mode, s);
 }
 
 }  // namespace ssm

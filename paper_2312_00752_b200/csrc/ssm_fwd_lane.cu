@@ -37,7 +37,8 @@ struct FwdLaneSmem {
   }
 };
 
-template <typename IO, int NG, bool VEC>
+// CPLX: complex states (N is then the number of columns, twice that of states; layout of the rows: lane_col)
+template <typename IO, int NG, bool VEC, bool CPLX>
 __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const FwdParams p, const LaneSplit sp, const int N, const int mode) {
   using SM = FwdLaneSmem<IO, NG>;
   constexpr int NP = SM::NP;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   const bool cvec = (reinterpret_cast<uintptr_t>(p.C) & (4 * sizeof(IO) - 1)) == 0;
   const bool has_z = full && gz != nullptr;
   const int cols = min(32, D - grp * 32);
+  const int NC = lane_ckpt_rows<CPLX>(N);
 
   // One batch in flight from global memory.  read: with z and C.
   LaneRows<IO, VEC> rx, rd, rz;
@@ -110,13 +112,16 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   const bool first_sweep = (split || summary) && (summary || rank * W + warp < W * CL - 1);
   if (live_piece) prefetch(t_begin, full && !first_sweep);
 
-  for (int n = warp; n < NP; n += W) sA[n * 32 + lane] = n < N ? p.A[(size_t)c_ld * N + n] * kLog2e : 0.f;
+  for (int n = warp; n < NP; n += W) {
+    const int col = lane_col<CPLX>(n);
+    sA[n * 32 + lane] = col < N ? p.A[(size_t)c_ld * N + col] * lane_a_scale<CPLX>(n) : 0.f;
+  }
   __syncthreads();
   float2 A2[8];
   float2 h[8];
   // which groups of 16 have their A in arithmetic progression (padded states continue it as long as they decay)
   unsigned ap_mask = 0;
-  if (sizeof(IO) == 2 && !p.general_A) {
+  if (sizeof(IO) == 2 && !CPLX && !p.general_A) {
 #pragma unroll 1
     for (int g = 0; g < NG; ++g) {
       const float* a = sA + g * 512 + lane;
@@ -172,8 +177,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
       for (int i = 0; i < NG; ++i) {
         const int v = lane + 32 * i;
-        *reinterpret_cast<float4*>(fB + 4 * v) = qB[i].widen();
-        if constexpr (READ) *reinterpret_cast<float4*>(fC + 4 * v) = qC[i].widen();
+        put_quad<CPLX>(fB, v, qB[i].widen(), 1.f);
+        if constexpr (READ) put_quad<CPLX>(fC, v, qC[i].widen(), -1.f);   // (complex: conj C, what the real part of C h wants)
       }
       if constexpr (VEC) {
         __syncwarp();
@@ -186,7 +191,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
         u[t] = rx.get(tx, t, lane);
         if constexpr (READ) {
           zf[t] = rz.get(tz, t, lane);
-          y[t] = Dk * u[t];
+          y[t] = CPLX ? 0.f : Dk * u[t];
         }
       }
       if constexpr (!VEC) {
@@ -212,11 +217,11 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
         if (write_ckpt) {
           const int kc = t0 / kCkptSteps;
           if (SSM_IN_RANGE(kc < p.nck, p.abort)) {
-            if (N >= 4) {   // (lanes past the last channel fill the padding of the tiled layout)
-              float* dst = p.ckpt + ckpt_offset(1, b, p.nck, kc, D, N, c_own, 16 * g);
+            if (NC >= 4) {   // (lanes past the last channel fill the padding of the tiled layout)
+              float* dst = p.ckpt + ckpt_offset(1, b, p.nck, kc, D, NC, c_own, 16 * g);
 #pragma unroll
               for (int k = 0; k < 4; ++k)
-                if (16 * g + 4 * k < N)
+                if (16 * g + 4 * k < NC)
                   *reinterpret_cast<float4*>(dst + 128 * k) = make_float4(h[2 * k].x, h[2 * k].y, h[2 * k + 1].x, h[2 * k + 1].y);
             } else if (valid) {
               float* dst = p.ckpt + ckpt_offset(0, b, p.nck, kc, D, N, c_own, 0);
@@ -242,7 +247,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
           for (int gb = 0; gb < kLB / GB; ++gb) {
             float e0[AP ? GB : 1], e1[AP ? GB : 1];
-            float2 af[AP ? 1 : GB][AP ? 1 : 8];
+            float2 af[AP ? 1 : GB][AP ? 1 : 8];   // (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1, 4, 5)
 #pragma unroll
             for (int t = 0; t < GB; ++t) {
               const float dtt = dt[gb * GB + t];
@@ -250,10 +255,18 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
                 e0[t] = ex2_approx(dtt * a0s);
                 e1[t] = ex2_approx(dtt * rs);
               } else {
+                if constexpr (CPLX) {
 #pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                  const float2 e = f2mul(f2dup(dtt), A2[k]);
-                  af[t][k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+                  for (int kk = 0; kk < 4; ++kk) {
+                    const int k = (kk & 1) + 4 * (kk >> 1);
+                    cexp_pair(dtt, A2[k], A2[k + 2], af[t][k], af[t][k + 2]);
+                  }
+                } else {
+#pragma unroll
+                  for (int k = 0; k < 8; ++k) {
+                    const float2 e = f2mul(f2dup(dtt), A2[k]);
+                    af[t][k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+                  }
                 }
               }
             }
@@ -283,9 +296,18 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
             for (int t = 0; t < GB; ++t) {
               if (t + 1 < GB) front(t + 1, aN[(t + 1) & 1], bxN[(t + 1) & 1], CvN[(t + 1) & 1]);
               float2 yv = make_float2(0.f, 0.f), yw = yv;
+              if constexpr (CPLX) {
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                  const int k = (kk & 1) + 4 * (kk >> 1);
+                  const float2 ar = aN[t & 1][k], ai = aN[t & 1][k + 2], hr = h[k], hi = h[k + 2];
+                  h[k] = f2fma(f2neg(ai), hi, f2fma(ar, hr, bxN[t & 1][k]));
+                  h[k + 2] = f2fma(ai, hr, f2fma(ar, hi, bxN[t & 1][k + 2]));
+                }
+              }
 #pragma unroll
               for (int k = 0; k < 8; ++k) {
-                h[k] = f2fma(aN[t & 1][k], h[k], bxN[t & 1][k]);
+                if constexpr (!CPLX) h[k] = f2fma(aN[t & 1][k], h[k], bxN[t & 1][k]);
                 if constexpr (READ) {
                   if (k & 1) yw = f2fma(CvN[t & 1][k], h[k], yw);
                   else yv = f2fma(CvN[t & 1][k], h[k], yv);
@@ -295,8 +317,12 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
             }
           }
         };
-        if (ap_mask >> g & 1) run(std::true_type{});
-        else run(std::false_type{});
+        if constexpr (sizeof(IO) == 2 && !CPLX) {
+          if (ap_mask >> g & 1) run(std::true_type{});
+          else run(std::false_type{});
+        } else {
+          run(std::false_type{});
+        }
         if constexpr (NG > 1) store_h(g);
       }
       if constexpr (READ) {
@@ -304,7 +330,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
         for (int t = 0; t < kLB; ++t) {
           // without z its rows are zero: silu(0) = 0, and gate_off = 1 takes its place
-          const float v = y[t] * fmaf(zf[t], sigmoid_fast(zf[t]), gate_off);
+          const float yt = CPLX ? fmaf(Dk, u[t], 2.f * y[t]) : y[t];   // (s = 2 Re(sum C h) + D x)
+          const float v = yt * fmaf(zf[t], sigmoid_fast(zf[t]), gate_off);
           LaneOut<IO, VEC>::put(to, bo, D, t, lane, valid && t < live, v);
         }
         if constexpr (VEC) {
@@ -328,50 +355,71 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
     if constexpr (NG == 1) store_h(0);
     sDs[warp * 32 + lane] = dsum;
     __syncthreads();
-    // exclusive fold over the block's pieces from a zero inflow, and the block's totals
+    // exclusive fold over the block's pieces from a zero inflow, and the block's totals (a complex state: rows n and n + 4)
+    constexpr int kRow2 = 4 * 32;
     for (int n = warp; n < NP; n += W) {
-      const float a2 = sA[n * 32 + lane];
-      float pre = 0.f, ds = 0.f;
+      if (CPLX && (n & 4)) continue;
+      const float a2 = sA[n * 32 + lane], ai = CPLX ? sA[n * 32 + kRow2 + lane] : 0.f;
+      float2 pre = make_float2(0.f, 0.f);
+      float ds = 0.f;
       for (int w = 0; w < W; ++w) {
         float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
-        const float e = *at, d = sDs[w * 32 + lane];
-        *at = pre;
-        pre = fmaf(ex2_approx(a2 * d), pre, e);
+        const float d = sDs[w * 32 + lane];
+        const float2 e = make_float2(*at, CPLX ? at[kRow2] : 0.f);
+        *at = pre.x;
+        if (CPLX) at[kRow2] = pre.y;
+        const float2 q = CPLX ? cexp_apply<false>(d, a2, ai, pre) : make_float2(ex2_approx(a2 * d) * pre.x, 0.f);
+        pre = make_float2(q.x + e.x, q.y + e.y);
         ds += d;
       }
-      sTot[n * 32 + lane] = pre;
+      sTot[n * 32 + lane] = pre.x;
+      if (CPLX) sTot[n * 32 + kRow2 + lane] = pre.y;
       if (n == 0) sTotDs[lane] = ds;
     }
     if (CL > 1) cg::this_cluster().sync();
     else __syncthreads();
     // add the inflow of the block: the segment's start state behind the totals of the blocks before it
     for (int n = warp; n < NP; n += W) {
-      const float a2 = sA[n * 32 + lane];
-      float H = (p.h_start != nullptr && n < N) ? p.h_start[(seg_row + c_ld) * N + n] : 0.f;
-      float ds_all = 0.f, rt[kLaneMaxCluster - 1], rds[kLaneMaxCluster - 1];
+      if (CPLX && (n & 4)) continue;
+      const int col = lane_col<CPLX>(n);
+      const float a2 = sA[n * 32 + lane], ai = CPLX ? sA[n * 32 + kRow2 + lane] : 0.f;
+      auto step = [&](float d, float2 v) {
+        return CPLX ? cexp_apply<false>(d, a2, ai, v) : make_float2(ex2_approx(a2 * d) * v.x, 0.f);
+      };
+      float2 H = make_float2(0.f, 0.f);
+      if (p.h_start != nullptr && col < N) {
+        H.x = p.h_start[(seg_row + c_ld) * N + col];
+        if (CPLX) H.y = p.h_start[(seg_row + c_ld) * N + col + 1];
+      }
+      float2 rt[kLaneMaxCluster - 1];
+      float ds_all = 0.f, rds[kLaneMaxCluster - 1];
 #pragma unroll
       for (int r = 0; r < kLaneMaxCluster - 1; ++r) {   // (all requested before the first is used)
         if (r < rank) {
-          rt[r] = cg::this_cluster().map_shared_rank(sTot, r)[n * 32 + lane];
+          const float* const tot = cg::this_cluster().map_shared_rank(sTot, r) + n * 32 + lane;
+          rt[r] = make_float2(tot[0], CPLX ? tot[kRow2] : 0.f);
           rds[r] = cg::this_cluster().map_shared_rank(sTotDs, r)[lane];
         }
       }
 #pragma unroll
       for (int r = 0; r < kLaneMaxCluster - 1; ++r) {
         if (r < rank) {
-          H = fmaf(ex2_approx(a2 * rds[r]), H, rt[r]);
+          const float2 q = step(rds[r], H);
+          H = make_float2(q.x + rt[r].x, q.y + rt[r].y);
           ds_all += rds[r];
         }
       }
-      if (summary && rank == CL - 1 && valid && n < N && chain_id < chains) {
+      if (summary && rank == CL - 1 && valid && col < N && chain_id < chains) {   // (never complex: no launch is split)
         const float d = sTotDs[lane];
-        p.seg_end[(seg_row + c_own) * N + n] = fmaf(ex2_approx(a2 * d), H, sTot[n * 32 + lane]);
+        p.seg_end[(seg_row + c_own) * N + col] = step(d, H).x + sTot[n * 32 + lane];
         if (n == 0) p.seg_dsum[seg_row + c_own] = ds_all + d;
       }
       float cum = 0.f;
       for (int w = 0; w < W; ++w) {
         float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
-        *at = fmaf(ex2_approx(a2 * cum), H, *at);
+        const float2 q = step(cum, H);
+        *at += q.x;
+        if (CPLX) at[kRow2] += q.y;
         cum += sDs[w * 32 + lane];
       }
     }
@@ -379,8 +427,10 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
     else __syncthreads();
     if constexpr (NG == 1) load_h(0);
   } else {
-    for (int n = 0; n < NP; ++n)
-      sH[n * 32 + lane] = (p.h_start != nullptr && n < N) ? p.h_start[(seg_row + c_ld) * N + n] : 0.f;
+    for (int n = 0; n < NP; ++n) {
+      const int col = lane_col<CPLX>(n);
+      sH[n * 32 + lane] = (p.h_start != nullptr && col < N) ? p.h_start[(seg_row + c_ld) * N + col] : 0.f;
+    }
     if constexpr (NG == 1) load_h(0);
   }
   if (summary) return;
@@ -390,13 +440,16 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   else sweep(std::false_type{}, true);
   if (full && p.h_last != nullptr && valid && t_begin < t_end && t_end == p.L) {
     if constexpr (NG == 1) store_h(0);
-    for (int n = 0; n < N; ++n) p.h_last[((size_t)b * D + c_own) * N + n] = sH[n * 32 + lane];
+    for (int n = 0; n < NP; ++n) {
+      const int col = lane_col<CPLX>(n);
+      if (col < N) p.h_last[((size_t)b * D + c_own) * N + col] = sH[n * 32 + lane];
+    }
   }
 }
 
-template <typename IO, int NG, bool VEC>
+template <typename IO, int NG, bool VEC, bool CPLX>
 cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int mode, cudaStream_t s) {
-  auto kern = ssm_fwd_lane_kernel<IO, NG, VEC>;
+  auto kern = ssm_fwd_lane_kernel<IO, NG, VEC, CPLX>;
   const int steps = plan.nseg > 1 ? plan.seg_steps : p.L;
   const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
   const LaneSplit sp = choose_lane_split(chains, steps, 0.75f, 25.f, NG > 2 ? 2 : 3, kLaneWarps);
@@ -419,19 +472,19 @@ cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int m
   return cudaLaunchKernelEx(&cfg, kern, p, sp, N, mode);
 }
 
-template <typename IO, int NG>
+template <typename IO, int NG, bool CPLX>
 cudaError_t launch_fwd_lane_vec(const Plan& plan, const FwdParams& p, int N, int mode, cudaStream_t s) {
   // 16-byte row pieces need aligned rows and at least one whole vector of channels
   bool vec = (size_t)p.D * sizeof(IO) % 16 == 0;
   for (const void* q : {p.x, p.delta, p.z, (const void*)p.out}) vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
-  return vec ? launch_fwd_lane_n<IO, NG, true>(plan, p, N, mode, s) : launch_fwd_lane_n<IO, NG, false>(plan, p, N, mode, s);
+  return vec ? launch_fwd_lane_n<IO, NG, true, CPLX>(plan, p, N, mode, s) : launch_fwd_lane_n<IO, NG, false, CPLX>(plan, p, N, mode, s);
 }
 
-template <typename IO>
+template <typename IO, bool CPLX>
 cudaError_t launch_fwd_lane_io(const Plan& plan, const FwdParams& p, int N, int mode, cudaStream_t s) {
-  if (N <= 16) return launch_fwd_lane_vec<IO, 1>(plan, p, N, mode, s);
-  if (N <= 32) return launch_fwd_lane_vec<IO, 2>(plan, p, N, mode, s);
-  return launch_fwd_lane_vec<IO, 4>(plan, p, N, mode, s);
+  if (N <= 16) return launch_fwd_lane_vec<IO, 1, CPLX>(plan, p, N, mode, s);
+  if (N <= 32) return launch_fwd_lane_vec<IO, 2, CPLX>(plan, p, N, mode, s);
+  return launch_fwd_lane_vec<IO, 4, CPLX>(plan, p, N, mode, s);
 }
 
 }  // namespace
@@ -466,8 +519,10 @@ bool fwd_lane_applicable(const ssm_problem_t& prob, const FwdParams& p) {
 }
 
 cudaError_t launch_fwd_lane(const ssm_problem_t& prob, const Plan& plan, const FwdParams& p, int mode, cudaStream_t s) {
-  if (prob.io_dtype == SSM_BF16) return launch_fwd_lane_io<__nv_bfloat16>(plan, p, prob.N, mode, s);
-  return launch_fwd_lane_io<float>(plan, p, prob.N, mode, s);
+  const bool bf = prob.io_dtype == SSM_BF16;
+  if (prob.flags & SSM_FLAG_COMPLEX)
+    return bf ? launch_fwd_lane_io<__nv_bfloat16, true>(plan, p, 2 * prob.N, mode, s) : launch_fwd_lane_io<float, true>(plan, p, 2 * prob.N, mode, s);
+  return bf ? launch_fwd_lane_io<__nv_bfloat16, false>(plan, p, prob.N, mode, s) : launch_fwd_lane_io<float, false>(plan, p, prob.N, mode, s);
 }
 
 }  // namespace ssm

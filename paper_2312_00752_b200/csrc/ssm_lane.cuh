@@ -35,6 +35,12 @@ constexpr int kLaneWarps = 4, kLaneMaxCluster = 8;
 // in steps of a lone warp.
 LaneSplit choose_lane_split(long long chains, int steps, float extra, float fixed, int blocks_per_sm, int teams, float* cost = nullptr);
 
+// Time split of the lane backward kernel for a problem whose teams have kLaneWarps / teams warps (ssm_api.cu); pl->bwd_groups
+// is set.
+void plan_lane_bwd(const ssm_problem_t& p, int teams, Plan* pl, float* cost);
+cudaError_t launch_fwd_lane(const ssm_problem_t& prob, const Plan& plan, const FwdParams& p, int mode, cudaStream_t s);
+cudaError_t launch_bwd_lane(const ssm_problem_t& prob, const Plan& plan, const BwdParams& p, int mode, cudaStream_t s);
+
 #ifdef __CUDACC__
 template <typename IO>
 struct LaneRaw;
@@ -179,6 +185,54 @@ template <typename IO>
 __device__ __forceinline__ float lane_softplus(float v) {
   if constexpr (sizeof(IO) == 4) return softplus_precise(v);
   else return softplus_fast(v);
+}
+
+// ---- complex states (SSM_FLAG_COMPLEX) in the lane kernels.  N complex states are 2 N columns of the same arrays; a group
+// of 16 rows holds 8 of them as two halves of 4 real parts and their 4 imaginary parts, so that packed arithmetic works on
+// pairs of real parts and pairs of imaginary parts.  lane_col: the column (re, im interleaved) of row n.
+template <bool CPLX>
+__device__ __forceinline__ int lane_col(int n) {
+  return CPLX ? (n & ~7) + 2 * (n & 3) + ((n >> 2) & 1) : n;
+}
+// rows (and columns) of a channel's checkpoint
+template <bool CPLX>
+__host__ __device__ __forceinline__ int lane_ckpt_rows(int N) { return CPLX && N < 8 ? 8 : N; }
+constexpr float kTurn = 6.2831853071795865f;   // 2 pi
+constexpr float kInvTurn = 0.15915494309189534f;
+// what a row of A is multiplied with when it is staged: real parts for ex2, imaginary parts in turns
+template <bool CPLX>
+__device__ __forceinline__ float lane_a_scale(int n) { return CPLX && (n & 4) ? kInvTurn : kLog2e; }
+// Four columns of B or C (quad v of a batch of rows of 16 NG) into the staged rows; im_sign: of imaginary parts
+template <bool CPLX>
+__device__ __forceinline__ void put_quad(float* rows, int v, float4 q, float im_sign) {
+  if constexpr (CPLX) {
+    // columns 4 v .. 4 v + 3 are two complex states: real parts next to each other, imaginary parts 4 rows on
+    float* const at = rows + (v >> 1) * 8 + (v & 1) * 2;
+    *reinterpret_cast<float2*>(at) = make_float2(q.x, q.z);
+    *reinterpret_cast<float2*>(at + 4) = make_float2(im_sign * q.y, im_sign * q.w);
+  } else {
+    *reinterpret_cast<float4*>(rows + 4 * v) = q;
+  }
+}
+
+// exp(dt A) for a pair of complex states: magnitude by ex2, phase by sin and cos of the angle reduced to half a turn (the
+// reduction is one multiply-add of the unrounded product)
+__device__ __forceinline__ void cexp_pair(float dt, float2 are, float2 aim, float2& ar, float2& ai) {
+  const float2 e = f2mul(f2dup(dt), are);
+  const float2 m = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+  constexpr float kRound = 12582912.f;   // 1.5 * 2^23: adding it rounds to a whole number
+  const float2 k = __fadd2_rn(__fadd2_rn(f2mul(f2dup(dt), aim), f2dup(kRound)), f2dup(-kRound));
+  const float2 r = f2mul(f2fma(f2dup(dt), aim, f2mul(k, f2dup(-1.f))), f2dup(kTurn));
+  ar = f2mul(m, make_float2(__cosf(r.x), __cosf(r.y)));
+  ai = f2mul(m, make_float2(__sinf(r.x), __sinf(r.y)));
+}
+__device__ __forceinline__ float2 f2neg(float2 v) { return make_float2(-v.x, -v.y); }
+// (re, im) <- exp(s A) (re, im) (conjugate: exp(s conj A)), A as staged
+template <bool CONJ>
+__device__ __forceinline__ float2 cexp_apply(float s, float are, float aim, float2 v) {
+  const float m = ex2_approx(s * are), t = s * aim, r = fmaf(s, aim, -rintf(t)) * kTurn;
+  const float c = m * __cosf(r), n = (CONJ ? -m : m) * __sinf(r);
+  return make_float2(fmaf(c, v.x, -n * v.y), fmaf(c, v.y, n * v.x));
 }
 
 // 16 floats of a shared-memory row as packed pairs
