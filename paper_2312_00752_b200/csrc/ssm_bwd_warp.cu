@@ -60,6 +60,7 @@ struct BwdWarpSmem {
   float ds[kBT][CW];             // dout * silu(z)
   float gp[kBT][CW];             // dout * silu'(z)
   float dF[SP ? kBT : 1][CW];    // SP: step sizes after bias and softplus
+  float dS[SP ? kBT : 1][CW];    // SP: derivative of the step size by its pre-activation
   uint32_t ox[kBT][CW / 2];      // dx, ddelta, dz of the tile (bf16 pairs)
   uint32_t od[kBT][CW / 2];
   uint32_t oz[kBT][CW / 2];
@@ -197,8 +198,8 @@ struct ChainRegs {
 // ZS (ZOH only): some |delta A| of the sub-block is too small for the closed form of the input gain.
 template <int S, int CPT, bool SP, bool AP, bool ZOH, bool ZS, int BC>
 __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, CPT, ZOH, BC>& cr, int r0, int nlive, float gate_on,
-                                          bool softplus, const uint32_t* tx, const uint32_t* td, const float* tfB,
-                                          const float* tfC, const float* tds, const float* tgp, const float* tdF,
+                                          const uint32_t* tx, const uint32_t* td, const float* tfB,
+                                          const float* tfC, const float* tds, const float* tgp, const float* tdF, const float* tdS,
                                           const float4* tck, uint32_t* tox, uint32_t* tod, uint32_t* toz, float4* tred,
                                           float* part_dB, float* part_dC, int* abort_word) {
   using LN = Lane<S, CPT>;
@@ -436,10 +437,8 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
       float dd0 = fmaf(u0[0], ZOH ? mb0[0] : lb0[0], wa0[0] * kInvLog2e);
       if constexpr (SP) {
         // the gradient goes to the pre-activation v: d softplus(v) / dv = sigmoid(v); the bias gets the sum over time
-        if (softplus) {
-          dd1 *= sigmoid_from_softplus(dt1[0]);
-          dd0 *= sigmoid_from_softplus(dt0[0]);
-        }
+        dd1 *= tdS[r1 * CW + lane];
+        dd0 *= tdS[r0e * CW + lane];
         if (r0 + 2 * m + 1 < nlive) cr.dbias += dd1;
         if (r0 + 2 * m < nlive) cr.dbias += dd0;
       }
@@ -466,7 +465,7 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
       cr.dD = fmaf(dsm, um, cr.dD);
       float ddm = fmaf(um, ZOH ? (odd ? mb1[0] : mb0[0]) : lbm, wam * kInvLog2e);
       if constexpr (SP) {
-        if (softplus) ddm *= sigmoid_from_softplus(dtm);
+        ddm *= tdS[rm * CW + ln.co];
         if (r0 + 2 * m + (odd ? 1 : 0) < nlive) cr.dbias += ddm;
       }
       reinterpret_cast<__nv_bfloat16*>(tox + rm * WPR)[ln.co] = __float2bfloat16_rn(dxm);
@@ -483,14 +482,15 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
       if (!(which ? SC : SB)) {
         const int jo = n0 / S, v = which * (S / 4) + (n0 % S) / 4;
         const float4* rs_ = tred + s * 32 * V;
-        float4 acc;
+        float2 lo, hi;
 #pragma unroll
         for (int gg = 0; gg < 32 / LPC; ++gg) {
           const int l = gg * LPC + jo;
           const float4 t4 = rs_[l * V + (v ^ ((l / (8 / V)) & (V - 1)))];
-          if (gg == 0) acc = t4;
-          else { acc.x += t4.x; acc.y += t4.y; acc.z += t4.z; acc.w += t4.w; }
+          lo = gg == 0 ? make_float2(t4.x, t4.y) : __fadd2_rn(lo, make_float2(t4.x, t4.y));
+          hi = gg == 0 ? make_float2(t4.z, t4.w) : __fadd2_rn(hi, make_float2(t4.z, t4.w));
         }
+        const float4 acc = make_float4(lo.x, lo.y, hi.x, hi.y);
         const int row = r0 + 2 * m + s;
         if (row < nlive && SSM_IN_RANGE(row < kBT && n0 + 4 <= 16, abort_word))
           *reinterpret_cast<float4*>((which ? part_dC : part_dB) + (size_t)row * 16 + n0) = acc;
@@ -651,6 +651,10 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
     }
     ap = __all_sync(0xffffffffu, ap);
     const int c_own = d_w + ln.co;
+    const float gate_off = has_z ? 0.f : 1.f;
+    // (with 32 channels per warp an element's channel is this lane's own; with 16 it is lane % 16)
+    const int c_el = d_w + lane % CW;
+    const float bias_el = (SP && p.delta_bias != nullptr && c_el < D) ? p.delta_bias[c_el] : 0.f;
     cr.Dk = (p.Dskip != nullptr && c_own < D) ? p.Dskip[c_own] : 0.f;
     cr.dD = 0.f;
     cr.dbias = 0.f;
@@ -733,34 +737,37 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
             }
           }
         }
-        // per-element gate terms of the tile: ds = dout silu(z), gp = dout silu'(z); element e = lane + 32 i
-        constexpr int EPL = kBT * CW / 32;   // elements per lane
-        float zf[EPL], gf[EPL], df[SP ? EPL : 1];
+        // per-element gate terms of the tile: ds = dout silu(z), gp = dout silu'(z); element e = lane + 32 i.  With the
+        // fused step size in two rounds: unrolled eight times, and with the softplus derivative in the unrolled steps, the
+        // body of a tile outgrew the instruction cache (0.39 of a stall per instruction; 476 us for the kernel at batch 8,
+        // L 2048, D 1536, 427 now).
+        constexpr int EPL = kBT * CW / 32, EPR = SP ? EPL / 2 : EPL;   // elements per lane, per round
+#pragma unroll 1
+        for (int i0 = 0; i0 < EPL; i0 += EPR) {
+          float zf[EPR], gf[EPR], df[SP ? EPR : 1];
 #pragma unroll
-        for (int i = 0; i < EPL; ++i) {
-          const int e = lane + 32 * i, r = e / CW, c = e % CW;
-          zf[i] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(sm.z[st][r])[c] << 16);
-          gf[i] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(sm.g[st][r])[c] << 16);
-          if constexpr (SP) df[i] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(sm.d[st][r])[c] << 16);
-        }
-        // (with 32 channels per warp an element's channel is this lane's own; with 16 it is lane % 16)
-        const int c_el = d_w + lane % CW;
-        const float bias_el = (SP && p.delta_bias != nullptr && c_el < D) ? p.delta_bias[c_el] : 0.f;
-#pragma unroll
-        for (int i = 0; i < EPL; ++i) {
-          const int e = lane + 32 * i, r = e / CW, c = e % CW;
-          float dsv = gf[i], gpv = 0.f;
-          if (has_z) {
-            const float sg = sigmoid_fast(zf[i]);
-            dsv = gf[i] * zf[i] * sg;
-            gpv = gf[i] * sg * fmaf(zf[i], 1.f - sg, 1.f);
+          for (int i = 0; i < EPR; ++i) {
+            const int e = lane + 32 * (i0 + i), r = e / CW, c = e % CW;
+            zf[i] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(sm.z[st][r])[c] << 16);
+            gf[i] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(sm.g[st][r])[c] << 16);
+            if constexpr (SP) df[i] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(sm.d[st][r])[c] << 16);
           }
-          sm.ds[r][c] = dsv;
-          sm.gp[r][c] = gpv;
-          if constexpr (SP) {
-            float v = df[i] + bias_el;
-            if (p.softplus) v = softplus_fast(v);
-            sm.dF[r][c] = r < nlive ? v : 0.f;   // rows past the end stay identity steps
+#pragma unroll
+          for (int i = 0; i < EPR; ++i) {
+            const int e = lane + 32 * (i0 + i), r = e / CW, c = e % CW;
+            // without z its tile is zero-filled: silu(0) = 0, and gate_off = 1 takes its place (dz is not wanted then)
+            const float sg = sigmoid_fast(zf[i]), gs = gf[i] * sg;
+            sm.ds[r][c] = fmaf(gs, zf[i], gf[i] * gate_off);
+            sm.gp[r][c] = gs * fmaf(zf[i], 1.f - sg, 1.f);
+            if constexpr (SP) {
+              float v = df[i] + bias_el, step = 1.f;
+              if (p.softplus) {
+                v = softplus_fast(v);
+                step = sigmoid_from_softplus(v);
+              }
+              sm.dF[r][c] = r < nlive ? v : 0.f;   // rows past the end stay identity steps
+              sm.dS[r][c] = step;
+            }
           }
         }
       }
@@ -785,9 +792,9 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
           zs = __any_sync(0xffffffffu, dmin * cr.minA < kZohSmall);
         }
 #define SSM_SUB_BLOCK(ZS_)                                                                                          \
-  sub_block<S, CPT, SP, AP_, ZOH, ZS_, BC>(ln, cr, sb * kSB, nlive, has_z ? 1.f : 0.f, p.softplus != 0, &sm.x[st][0][0], \
+  sub_block<S, CPT, SP, AP_, ZOH, ZS_, BC>(ln, cr, sb * kSB, nlive, has_z ? 1.f : 0.f, &sm.x[st][0][0], \
                                        &sm.d[st][0][0], &sm.fB[0][0], &sm.fC[0][0], &sm.ds[0][0], &sm.gp[0][0],      \
-                                       &sm.dF[0][0], &sm.ck[st][sb][0][0], &sm.ox[0][0], &sm.od[0][0], &sm.oz[0][0], \
+                                       &sm.dF[0][0], &sm.dS[0][0], &sm.ck[st][sb][0][0], &sm.ox[0][0], &sm.od[0][0], &sm.oz[0][0], \
                                        &sm.red[0][0][0], part_dB, part_dC, sc.abort)
         if constexpr (ZOH) {
           if (zs) SSM_SUB_BLOCK(true);

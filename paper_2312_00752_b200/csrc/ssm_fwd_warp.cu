@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MODE == kFwdFull ? 1 : 3)
         }
         // everything of a step that does not depend on the state (B and C of the step, decays, input terms) is
         // prepared one step ahead of the recurrence that consumes it
-        float2 aN[2][H], bxN[2][H], CvN[2][FULL ? H : 1];
+        float2 aN[2][H], bxN[2][H], CvN[3][FULL ? H : 1];
         auto front = [&](int t, float2 (&a)[H], float2 (&bxF)[H], float2 (&CvF)[FULL ? H : 1]) {
           const int r = SSM_TILE_ROW(r0 + gb * GB + t, kWT, sc.abort);
           float2 Bv[H];
@@ -358,19 +358,30 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MODE == kFwdFull ? 1 : 3)
         };
         float ypart[FULL ? GB : 1];
         front(0, aN[0], bxN[0], CvN[0]);
-#pragma unroll
-        for (int t = 0; t < GB; ++t) {
-          if (t + 1 < GB) front(t + 1, aN[(t + 1) & 1], bxN[(t + 1) & 1], CvN[(t + 1) & 1]);
+        // (the readout of a step runs beside the state update of the next one, which does not wait for it)
+        float2 hp[FULL ? H : 1];
+        auto readout = [&](int t, const float2 (&hh)[H]) {
           float2 yv = make_float2(0.f, 0.f), yw = make_float2(0.f, 0.f);
 #pragma unroll
           for (int k = 0; k < H; ++k) {
-            h[k] = f2fma(aN[t & 1][k], h[k], bxN[t & 1][k]);
-            if constexpr (FULL) {
-              if (k & 1) yw = f2fma(CvN[t & 1][k], h[k], yw);
-              else yv = f2fma(CvN[t & 1][k], h[k], yv);
-            }
+            if (k & 1) yw = f2fma(CvN[t % 3][k], hh[k], yw);
+            else yv = f2fma(CvN[t % 3][k], hh[k], yv);
           }
-          if constexpr (FULL) ypart[t] = (yv.x + yw.x) + (yv.y + yw.y);
+          ypart[t] = (yv.x + yw.x) + (yv.y + yw.y);
+        };
+#pragma unroll
+        for (int t = 0; t < GB; ++t) {
+          if (t + 1 < GB) front(t + 1, aN[(t + 1) & 1], bxN[(t + 1) & 1], CvN[(t + 1) % 3]);
+          if constexpr (FULL) {
+#pragma unroll
+            for (int k = 0; k < H; ++k) hp[k] = h[k];
+          }
+#pragma unroll
+          for (int k = 0; k < H; ++k) h[k] = f2fma(aN[t & 1][k], h[k], bxN[t & 1][k]);
+          if constexpr (FULL) {
+            if (t > 0) readout(t - 1, hp);
+            if (t == GB - 1) readout(t, h);
+          }
         }
         if constexpr (FULL) {
 #pragma unroll
