@@ -353,6 +353,7 @@ __global__ void __launch_bounds__(BwdGeom<N>::THREADS) ssm_bwd_local_kernel(cons
 // per-(batch, segment) dA/dD partials, in ascending order, and rounds dB/dC to the io dtype.
 template <typename IO>
 __global__ void __launch_bounds__(256) ssm_bwd_reduce_kernel(const ReduceParams p) {
+  dependency_wait();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < p.bln) {
     float sb = 0.f, sc = 0.f;
@@ -443,9 +444,8 @@ cudaError_t launch_bwd(const ssm_problem_t& prob, const Plan& plan, const BwdPar
 cudaError_t launch_bwd_reduce(const ssm_problem_t& prob, const ReduceParams& p, cudaStream_t s) {
   const long long work = p.bln > (long long)p.D * p.N ? p.bln : (long long)p.D * p.N;
   const unsigned blocks = (unsigned)((work + 255) / 256);
-  if (prob.io_dtype == SSM_BF16) ssm_bwd_reduce_kernel<__nv_bfloat16><<<blocks, 256, 0, s>>>(p);
-  else ssm_bwd_reduce_kernel<float><<<blocks, 256, 0, s>>>(p);
-  return cudaGetLastError();
+  if (prob.io_dtype == SSM_BF16) return launch_dependent(ssm_bwd_reduce_kernel<__nv_bfloat16>, blocks, 256, 0, 1, s, p);
+  return launch_dependent(ssm_bwd_reduce_kernel<float>, blocks, 256, 0, 1, s, p);
 }
 
 }  // namespace ssm

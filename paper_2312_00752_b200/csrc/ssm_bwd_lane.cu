@@ -534,6 +534,7 @@ template <typename IO, bool VEC, bool CPLX>
 __global__ void __launch_bounds__(kLaneWarps * 32, sizeof(IO) == 4 ? 3 : 4) ssm_bwd_lane_local_kernel(const BwdParams p, const int N, const int ng) {
   __shared__ __align__(16) float s_tiles[kLaneWarps][2048];
   __shared__ float s_A[kLaneWarps][16 * 32];
+  dependency_wait();
   const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
   const int D = p.D, groups = (D + 31) / 32, nseg = p.nseg - 1;   // (nobody wants what leaves the first segment)
   const int item = blockIdx.x * kLaneWarps + bwarp;
@@ -573,6 +574,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   using SM = BwdLaneSmem<IO, NG, VEC>;
   constexpr int NP = SM::NP, kTeams = SM::kTeams;
   extern __shared__ __align__(16) unsigned char smem[];
+  dependency_wait();
   const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
   const int W = sp.warps, CL = sp.cluster;      // pieces of a chain in this block, blocks of the chain
   const int team = bwarp / NG, gi = bwarp % NG; // gi: this warp's group of 16 states
@@ -1031,9 +1033,8 @@ cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int m
   auto kern = ssm_bwd_lane_kernel<IO, NG, ROWS, CPLX>;
   if (mode == kBwdLocal) {
     const long long items = (long long)p.batch * (plan.nseg - 1) * ((p.D + 31) / 32) * NG;
-    if (items > 0)
-      ssm_bwd_lane_local_kernel<IO, VEC, CPLX><<<(unsigned)((items + kLaneWarps - 1) / kLaneWarps), kLaneWarps * 32, 0, s>>>(p, N, NG);
-    return cudaGetLastError();
+    if (items <= 0) return cudaSuccess;
+    return launch_dependent(ssm_bwd_lane_local_kernel<IO, VEC, CPLX>, (unsigned)((items + kLaneWarps - 1) / kLaneWarps), kLaneWarps * 32, 0, 1, s, p, N, NG);
   }
   const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
   const LaneSplit sp = plan.split;
@@ -1041,18 +1042,7 @@ cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int m
   KernelLimits lim;
   const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), 32 * kLaneWarps, SM::bytes(SM::kTeams), &lim);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((chains + per_block - 1) / per_block * sp.cluster));
-  cfg.blockDim = dim3(32 * kLaneWarps);
-  cfg.dynamicSmemBytes = SM::bytes(per_block);
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = sp.cluster;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = sp.cluster > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, p, sp, N);
+  return launch_dependent(kern, (unsigned)((chains + per_block - 1) / per_block * sp.cluster), 32 * kLaneWarps, SM::bytes(per_block), sp.cluster, s, p, sp, N);
 }
 
 template <typename IO, int NG, bool CPLX>

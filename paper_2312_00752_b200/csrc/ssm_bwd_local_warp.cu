@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(kLWarps * 32) ssm_bwd_local_warp_kernel(const 
   constexpr int H = 8;   // float2 pairs of states per thread
   using Smem = LocalWarpSmem<SP, SC>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  dependency_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Smem& sm = reinterpret_cast<Smem*>(smem_raw)[warp];
   const int D = p.D;
@@ -312,12 +313,10 @@ cudaError_t launch_local(const Plan& plan, const BwdParams& p, cudaStream_t s) {
     if (p.L % kLT == 0 && plan.seg_steps % kLT == 0 && p.D % 32 == 0) {
       auto whole = ssm_bwd_local_warp_kernel<SP, SC, true>;
       if ((e = kernel_limits(reinterpret_cast<const void*>(whole), kLWarps * 32, smem, &lim)) != cudaSuccess) return e;
-      whole<<<grid, kLWarps * 32, smem, s>>>(p, sc);
-      return cudaGetLastError();
+      return launch_dependent(whole, grid, kLWarps * 32, smem, 1, s, p, sc);
     }
   }
-  kern<<<grid, kLWarps * 32, smem, s>>>(p, sc);
-  return cudaGetLastError();
+  return launch_dependent(kern, grid, kLWarps * 32, smem, 1, s, p, sc);
 }
 
 }  // namespace

@@ -514,6 +514,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
   constexpr bool OWN = LN::OWN;
   using Smem = BwdWarpSmem<S, CPT, SP>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  dependency_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Smem& sm = reinterpret_cast<Smem*>(smem_raw)[warp];
   const LN ln(lane);
@@ -922,12 +923,10 @@ cudaError_t launch_bwd_variant(const Plan& plan, const BwdParams& p, cudaStream_
     if (p.L % kBT == 0 && plan.seg_steps % kBT == 0 && p.D % CW == 0) {
       auto whole = ssm_bwd_warp_kernel<S, CPT, SP, ZOH, BC, true>;
       if ((e = kernel_limits(reinterpret_cast<const void*>(whole), kBwdWarps * 32, smem, &lim)) != cudaSuccess) return e;
-      whole<<<grid, kBwdWarps * 32, smem, s>>>(p, sc);
-      return cudaGetLastError();
+      return launch_dependent(whole, grid, kBwdWarps * 32, smem, 1, s, p, sc);
     }
   }
-  kern<<<grid, kBwdWarps * 32, smem, s>>>(p, sc);
-  return cudaGetLastError();
+  return launch_dependent(kern, grid, kBwdWarps * 32, smem, 1, s, p, sc);
 }
 
 }  // namespace

@@ -20,6 +20,7 @@ constexpr int kCarryRanges = 8;
 
 __global__ void __launch_bounds__(kCarryCols* kCarryRanges) ssm_carry_kernel(const CarryParams p) {
   __shared__ AffinePair s_agg[kCarryRanges][kCarryCols];
+  dependency_wait();
   const int col = blockIdx.x * kCarryCols + threadIdx.x;  // index into D*N
   const int b = blockIdx.y;
   const int r = threadIdx.y;
@@ -58,8 +59,7 @@ __global__ void __launch_bounds__(kCarryCols* kCarryRanges) ssm_carry_kernel(con
 cudaError_t launch_carry(const CarryParams& p, cudaStream_t s) {
   dim3 grid((p.D * p.N + kCarryCols - 1) / kCarryCols, p.batch);
   dim3 block(kCarryCols, kCarryRanges);
-  ssm_carry_kernel<<<grid, block, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_dependent(ssm_carry_kernel, grid, block, 0, 1, s, p);
 }
 
 }  // namespace ssm

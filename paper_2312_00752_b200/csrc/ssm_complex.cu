@@ -61,6 +61,7 @@ __device__ __forceinline__ float2 io2_to_float2(const IO* p) {
 // ---------------------------------------------------------------------------------------------------- one step
 template <typename IO>
 __global__ void __launch_bounds__(128) ssm_cstep_kernel(const CplxStepParams p, int N) {
+  dependency_wait();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)p.batch * p.D) return;
   const int b = (int)(e / p.D), d = (int)(e % p.D);
@@ -266,9 +267,8 @@ cudaError_t complex_step(const ssm_problem_t& prob, const void* x, const void* d
   p.batch = prob.batch;
   p.D = prob.D;
   const unsigned grid = (unsigned)(((long long)prob.batch * prob.D + 127) / 128);
-  if (prob.io_dtype == SSM_BF16) ssm_cstep_kernel<__nv_bfloat16><<<grid, 128, 0, s>>>(p, prob.N);
-  else ssm_cstep_kernel<float><<<grid, 128, 0, s>>>(p, prob.N);
-  return cudaGetLastError();
+  if (prob.io_dtype == SSM_BF16) return launch_dependent(ssm_cstep_kernel<__nv_bfloat16>, grid, 128, 0, 1, s, p, prob.N);
+  return launch_dependent(ssm_cstep_kernel<float>, grid, 128, 0, 1, s, p, prob.N);
 }
 
 }  // namespace ssm

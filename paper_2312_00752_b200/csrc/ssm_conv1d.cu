@@ -95,6 +95,7 @@ __device__ __forceinline__ void load_input_row(const ConvParams& p, int b, int s
 
 template <typename IO, int W, int VEC>
 __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_fwd_kernel(const ConvParams p) {
+  dependency_wait();
   const int c0 = (blockIdx.x * kConvThreads + threadIdx.x) * VEC;
   if (c0 >= p.D) return;
   const int b = blockIdx.z;
@@ -143,6 +144,7 @@ __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_fwd_kernel(const Conv
 
 template <typename IO, int W, int VEC>
 __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_bwd_kernel(const ConvParams p) {
+  dependency_wait();
   const int c0 = (blockIdx.x * kConvThreads + threadIdx.x) * VEC;
   if (c0 >= p.D) return;
   const int b = blockIdx.z;
@@ -314,6 +316,7 @@ __device__ __forceinline__ void load_input_row4(const ConvParams& p, int b, int 
 
 template <typename IO, int W, bool SILU, bool FAST>
 __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_fwd_vec4_kernel(const ConvParams p) {
+  dependency_wait();
   const int c0 = (blockIdx.x * kConvThreads + threadIdx.x) * 4;
   if (c0 >= p.D) return;
   const int b = blockIdx.z;
@@ -372,6 +375,7 @@ __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_fwd_vec4_kernel(const
 
 template <typename IO, int W, bool SILU, bool FAST>
 __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_bwd_vec4_kernel(const ConvParams p) {
+  dependency_wait();
   const int c0 = (blockIdx.x * kConvThreads + threadIdx.x) * 4;
   if (c0 >= p.D) return;
   const int b = blockIdx.z;
@@ -496,6 +500,7 @@ __global__ void __launch_bounds__(kRedOutputs* kRedSlices) ssm_conv1d_reduce_ker
                                                                                    int D, int W, float* __restrict__ dw,
                                                                                    float* __restrict__ dbias) {
   __shared__ float s_sum[kRedSlices][kRedOutputs];
+  dependency_wait();
   const int lane = threadIdx.x % kRedOutputs, slice = threadIdx.x / kRedOutputs;
   const int n = D * (W + 1);
   const int i = blockIdx.x * kRedOutputs + lane;   // index into [D][W + 1]
@@ -548,8 +553,7 @@ cudaError_t launch_conv_kernel(Kernel kernel, ConvParams p, int W, int channels_
   const int chunks = (p.L + p.steps - 1) / p.steps;
   if (chunks_out != nullptr) *chunks_out = chunks;
   dim3 grid(gx, chunks, p.batch);
-  kernel<<<grid, kConvThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  return launch_dependent(kernel, grid, kConvThreads, 0, 1, s, p);
 }
 
 // vector_ok: four channels per thread with packed arithmetic; otherwise the scalar kernels.  The tanh-based sigmoid is
@@ -670,9 +674,10 @@ ssm_status_t ssm_conv1d_bwd(const ssm_conv_problem_t* p, const void* x, const fl
   if (e != cudaSuccess) return SSM_ERR_CUDA;
   const int parts = p->batch * chunks;
   const int n = p->D * (p->width + 1);
-  ssm_conv1d_reduce_kernel<<<(n + kRedOutputs - 1) / kRedOutputs, kRedOutputs * kRedSlices, 0, s>>>(
-      cp.part, parts, p->D, p->width, dw, has_bias ? dbias : nullptr);
-  return cudaGetLastError() == cudaSuccess ? SSM_OK : SSM_ERR_CUDA;
+  return launch_dependent(ssm_conv1d_reduce_kernel, (n + kRedOutputs - 1) / kRedOutputs, kRedOutputs * kRedSlices, 0, 1, s, cp.part, parts,
+                          p->D, p->width, dw, has_bias ? dbias : nullptr) == cudaSuccess
+             ? SSM_OK
+             : SSM_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   constexpr int NP = SM::NP;
   const bool full = mode == kFwdFull, summary = mode == kFwdSummary;
   extern __shared__ __align__(16) float smem[];
+  dependency_wait();
   const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
   const int W = sp.warps, CL = sp.cluster;
   constexpr int nwarps = kLaneWarps;
@@ -458,18 +459,7 @@ cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int m
   KernelLimits lim;
   const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), 32 * kLaneWarps, FwdLaneSmem<IO, NG>::bytes(kLaneWarps, kLaneWarps), &lim);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)((chains + per_block - 1) / per_block * sp.cluster));
-  cfg.blockDim = dim3(32 * kLaneWarps);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = sp.cluster;
-  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = sp.cluster > 1 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, p, sp, N, mode);
+  return launch_dependent(kern, (unsigned)((chains + per_block - 1) / per_block * sp.cluster), 32 * kLaneWarps, smem, sp.cluster, s, p, sp, N, mode);
 }
 
 template <typename IO, int NG, bool CPLX>

@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MODE == kFwdFull ? 1 : 3)
   using Smem = FwdWarpSmem<CW, FULL, SPF, BC, NST>;
   constexpr bool TB = Smem::TB, TC = Smem::TC;   // B / C are inputs [batch][L][16] staged in tiles (else parameters)
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  dependency_wait();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   Smem& sm = reinterpret_cast<Smem*>(smem_raw)[warp];
   const int j = lane % LPC, g = lane / LPC;   // g: this lane's channel of the chain, j: which S states of it
@@ -579,8 +580,7 @@ cudaError_t launch_variant_w(const Plan& plan, const FwdParams& p, cudaStream_t 
         KernelLimits lim;
         const cudaError_t ea = kernel_limits(reinterpret_cast<const void*>(kern), kWarpsPerBlock * 32, smem, &lim);
         if (ea != cudaSuccess) return ea;
-        kern<<<grid, kWarpsPerBlock * 32, smem, s>>>(p, sc);
-        return cudaGetLastError();
+        return launch_dependent(kern, grid, kWarpsPerBlock * 32, smem, 1, s, p, sc);
       };
       if constexpr (!ZOH && MODE != kFwdSummary && BC == 0) {
         if (two_stage) return go(ssm_fwd_warp_kernel<S, MODE, SP, ZOH, BC, 2, true>);
@@ -590,12 +590,10 @@ cudaError_t launch_variant_w(const Plan& plan, const FwdParams& p, cudaStream_t 
   }
   if constexpr (!ZOH && MODE != kFwdSummary && BC == 0) {
     if (two_stage) {
-      ssm_fwd_warp_kernel<S, MODE, SP, ZOH, BC, 2><<<grid, kWarpsPerBlock * 32, smem, s>>>(p, sc);
-      return cudaGetLastError();
+      return launch_dependent(ssm_fwd_warp_kernel<S, MODE, SP, ZOH, BC, 2>, grid, kWarpsPerBlock * 32, smem, 1, s, p, sc);
     }
   }
-  ssm_fwd_warp_kernel<S, MODE, SP, ZOH, BC, 3><<<grid, kWarpsPerBlock * 32, smem, s>>>(p, sc);
-  return cudaGetLastError();
+  return launch_dependent(ssm_fwd_warp_kernel<S, MODE, SP, ZOH, BC, 3>, grid, kWarpsPerBlock * 32, smem, 1, s, p, sc);
 }
 
 template <int S, int MODE, bool SP, bool ZOH>

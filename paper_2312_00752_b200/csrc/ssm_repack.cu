@@ -30,6 +30,7 @@ struct RepackJobs {
 namespace {
 
 __global__ void __launch_bounds__(256) ssm_repack_kernel(const RepackJobs jobs) {
+  dependency_wait();
   const RepackJob jb = jobs.job[blockIdx.y];
   const long long total = (long long)jb.rows * jb.n_dst;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -73,8 +74,7 @@ cudaError_t repack_run(const RepackJobs& jobs, cudaStream_t s) {
   long long most = 1;
   for (int i = 0; i < jobs.count; ++i) most = std::max(most, (long long)jobs.job[i].rows * jobs.job[i].n_dst);
   const unsigned gx = (unsigned)std::min<long long>((most + 255) / 256, 4LL * kNumSMs);
-  ssm_repack_kernel<<<dim3(gx, (unsigned)jobs.count), 256, 0, s>>>(jobs);
-  return cudaGetLastError();
+  return launch_dependent(ssm_repack_kernel, dim3(gx, (unsigned)jobs.count), 256, 0, 1, s, jobs);
 }
 
 }  // namespace ssm

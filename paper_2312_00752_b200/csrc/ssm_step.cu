@@ -41,6 +41,7 @@ __device__ __forceinline__ void load_io_row(const IO* __restrict__ src, float (&
 template <typename IO, int N, bool ZOH, bool SB, bool SC>
 __global__ void __launch_bounds__(128) ssm_step_kernel(const StepParams p) {
   constexpr int S = StepGeom<N>::S, LPC = StepGeom<N>::LPC, CH = StepGeom<N>::CH;
+  dependency_wait();
   const int j = threadIdx.x % LPC;
   const int d = blockIdx.x * CH + threadIdx.x / LPC;
   const int b = blockIdx.y;
@@ -100,34 +101,33 @@ __global__ void __launch_bounds__(128) ssm_step_kernel(const StepParams p) {
 }
 
 template <typename IO, int N>
-static void launch_step_n(const StepParams& p, cudaStream_t s) {
+static cudaError_t launch_step_n(const StepParams& p, cudaStream_t s) {
   const dim3 grid((unsigned)((p.D + StepGeom<N>::CH - 1) / StepGeom<N>::CH), (unsigned)p.batch);
   const int v = (p.zoh ? 1 : 0) | (p.static_B ? 2 : 0) | (p.static_C ? 4 : 0);
   switch (v) {
-    case 0: ssm_step_kernel<IO, N, false, false, false><<<grid, 128, 0, s>>>(p); break;
-    case 1: ssm_step_kernel<IO, N, true, false, false><<<grid, 128, 0, s>>>(p); break;
-    case 2: ssm_step_kernel<IO, N, false, true, false><<<grid, 128, 0, s>>>(p); break;
-    case 3: ssm_step_kernel<IO, N, true, true, false><<<grid, 128, 0, s>>>(p); break;
-    case 4: ssm_step_kernel<IO, N, false, false, true><<<grid, 128, 0, s>>>(p); break;
-    case 5: ssm_step_kernel<IO, N, true, false, true><<<grid, 128, 0, s>>>(p); break;
-    case 6: ssm_step_kernel<IO, N, false, true, true><<<grid, 128, 0, s>>>(p); break;
-    default: ssm_step_kernel<IO, N, true, true, true><<<grid, 128, 0, s>>>(p); break;
+    case 0: return launch_dependent(ssm_step_kernel<IO, N, false, false, false>, grid, 128, 0, 1, s, p);
+    case 1: return launch_dependent(ssm_step_kernel<IO, N, true, false, false>, grid, 128, 0, 1, s, p);
+    case 2: return launch_dependent(ssm_step_kernel<IO, N, false, true, false>, grid, 128, 0, 1, s, p);
+    case 3: return launch_dependent(ssm_step_kernel<IO, N, true, true, false>, grid, 128, 0, 1, s, p);
+    case 4: return launch_dependent(ssm_step_kernel<IO, N, false, false, true>, grid, 128, 0, 1, s, p);
+    case 5: return launch_dependent(ssm_step_kernel<IO, N, true, false, true>, grid, 128, 0, 1, s, p);
+    case 6: return launch_dependent(ssm_step_kernel<IO, N, false, true, true>, grid, 128, 0, 1, s, p);
+    default: return launch_dependent(ssm_step_kernel<IO, N, true, true, true>, grid, 128, 0, 1, s, p);
   }
 }
 
 template <typename IO>
 static cudaError_t launch_step_io(const StepParams& p, cudaStream_t s) {
   switch (p.N) {
-    case 64: launch_step_n<IO, 64>(p, s); break;
-    case 32: launch_step_n<IO, 32>(p, s); break;
-    case 16: launch_step_n<IO, 16>(p, s); break;
-    case 8: launch_step_n<IO, 8>(p, s); break;
-    case 4: launch_step_n<IO, 4>(p, s); break;
-    case 2: launch_step_n<IO, 2>(p, s); break;
-    case 1: launch_step_n<IO, 1>(p, s); break;
+    case 64: return launch_step_n<IO, 64>(p, s);
+    case 32: return launch_step_n<IO, 32>(p, s);
+    case 16: return launch_step_n<IO, 16>(p, s);
+    case 8: return launch_step_n<IO, 8>(p, s);
+    case 4: return launch_step_n<IO, 4>(p, s);
+    case 2: return launch_step_n<IO, 2>(p, s);
+    case 1: return launch_step_n<IO, 1>(p, s);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_step(const ssm_problem_t& prob, const StepParams& p, cudaStream_t s) {
