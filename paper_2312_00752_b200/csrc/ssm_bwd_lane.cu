@@ -578,8 +578,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
   const int W = sp.warps, CL = sp.cluster;      // pieces of a chain in this block, blocks of the chain
   const int team = bwarp / NG, gi = bwarp % NG; // gi: this warp's group of 16 states
-  const int sub = team / W, tw = team % W;      // which chain of the block, which of its pieces here
-  const int per_block = kTeams / W;
+  const int sub = div_pow2(team, W), tw = team - sub * W;      // which chain of the block, which of its pieces here
+  const int per_block = div_pow2(kTeams, W);
   unsigned char* const sTeam = smem + team * SM::kTeam;
   unsigned char* const rX = sTeam;
   unsigned char* const rD = rX + SM::kRaw;
@@ -613,12 +613,12 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   const IO* __restrict__ gC = static_cast<const IO*>(p.C);
 
   const int D = p.D, groups = (D + 31) / 32;
-  const int rank = (int)(blockIdx.x % (unsigned)CL);
+  const int rank = cluster_rank();
   const int nseg = p.nseg, chains = p.batch * nseg * groups;
-  const int chain_id = (int)(blockIdx.x / (unsigned)CL) * per_block + sub;
+  const int chain_id = cluster_index() * per_block + sub;
   const int chain = min(chain_id, chains - 1);
-  const int grp = chain % groups, bs = chain / groups;
-  const int seg = bs % nseg, b = bs / nseg;
+  const int bs = chain / groups, grp = chain - bs * groups;
+  const int b = nseg == 1 ? bs : bs / nseg, seg = bs - b * nseg;
   const int c_own = grp * 32 + lane, cols = min(32, D - grp * 32);
   const bool valid = c_own < D;
   const int c_ld = valid ? c_own : D - 1;
@@ -738,15 +738,24 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
       const float a2 = sA[n * 32 + lane], ai = CPLX ? sA[n * 32 + kRow2 + lane] : 0.f;
       float2 pre = make_float2(0.f, 0.f);
       float ds = 0.f;
-      for (int w = W - 1; w >= 0; --w) {
-        float* const at = leaving(w, n) + lane;
-        const float d = sDs[w * 32 + lane];
-        const float2 l = make_float2(*at, CPLX ? at[kRow2] : 0.f);
-        *at = pre.x;
-        if (CPLX) at[kRow2] = pre.y;
-        const float2 q = CPLX ? cexp_apply<true>(d, a2, ai, pre) : make_float2(ex2_approx(a2 * d) * pre.x, 0.f);
-        pre = make_float2(q.x + l.x, q.y + l.y);
-        ds += d;
+      float2 l[kTeams];
+      float d[kTeams];
+#pragma unroll
+      for (int w = kTeams - 1; w >= 0; --w) {   // (all loaded before the first is used)
+        const float* const at = leaving(w < W ? w : 0, n) + lane;
+        l[w] = make_float2(*at, CPLX ? at[kRow2] : 0.f);
+        d[w] = sDs[(w < W ? w : 0) * 32 + lane];
+      }
+#pragma unroll
+      for (int w = kTeams - 1; w >= 0; --w) {
+        if (w < W) {
+          float* const at = leaving(w, n) + lane;
+          *at = pre.x;
+          if (CPLX) at[kRow2] = pre.y;
+          const float2 q = CPLX ? cexp_apply<true>(d[w], a2, ai, pre) : make_float2(ex2_approx(a2 * d[w]) * pre.x, 0.f);
+          pre = make_float2(q.x + l[w].x, q.y + l[w].y);
+          ds += d[w];
+        }
       }
       sTot[n * 32 + lane] = pre.x;
       if (CPLX) sTot[n * 32 + kRow2 + lane] = pre.y;
@@ -783,13 +792,24 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
           M = make_float2(q.x + rt[r].x, q.y + rt[r].y);
         }
       }
-      float cum = 0.f;
-      for (int w = W - 1; w >= 0; --w) {
-        float* const at = leaving(w, n) + lane;
-        const float2 q = step(cum, M);
-        *at += q.x;
-        if (CPLX) at[kRow2] += q.y;
-        cum += sDs[w * 32 + lane];
+      float2 l[kTeams];
+      float cum[kTeams];
+      float sum = 0.f;
+#pragma unroll
+      for (int w = kTeams - 1; w >= 0; --w) {
+        const float* const at = leaving(w < W ? w : 0, n) + lane;
+        l[w] = make_float2(*at, CPLX ? at[kRow2] : 0.f);
+        cum[w] = sum;
+        if (w < W) sum += sDs[w * 32 + lane];
+      }
+#pragma unroll
+      for (int w = kTeams - 1; w >= 0; --w) {
+        if (w < W) {
+          float* const at = leaving(w, n) + lane;
+          const float2 q = step(cum[w], M);
+          *at = l[w].x + q.x;
+          if (CPLX) at[kRow2] = l[w].y + q.y;
+        }
       }
     }
     if (CL > 1) cg::this_cluster().sync();   // (also: no block leaves while another still reads its totals)

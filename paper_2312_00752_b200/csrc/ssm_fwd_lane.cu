@@ -9,8 +9,8 @@
 // sub-partition) and, with one exponential per state, the special-function unit (16 ex2 = 128 cycles per warp and step),
 // so the registers are capped for three warps per sub-partition and a chain is split in time until they are there.
 // Measured against the generic kernel with its summary and carry launches: float32 (2, 2048, 1536), N = 16: 262 -> 76 us;
-// bf16 (3, 1237, 1001), N = 16: 268 -> 51 us; bf16 (1, 2048, 5120), N = 64: 1204 -> 362 us; float32 (1, 256, 64):
-// 126 -> 8 us.
+// bf16 (3, 1237, 1001), N = 16: 268 -> 51 us; bf16 (1, 2048, 5120), N = 64: 1204 -> 348 us; float32 (1, 256, 64):
+// 126 -> 7 us.
 #include <type_traits>
 
 #include "ssm_lane.cuh"
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
   const int W = sp.warps, CL = sp.cluster;
   constexpr int nwarps = kLaneWarps;
-  const int sub = bwarp / W, warp = bwarp % W;   // sub: which chain of the block
+  const int sub = div_pow2(bwarp, W), warp = bwarp - sub * W;   // sub: which chain of the block
   float* const sIO = smem + (size_t)bwarp * SM::kIO;
   float* const sE = smem + (size_t)nwarps * SM::kIO + (size_t)sub * W * SM::kState;         // [W][NP][32]
   float* const sDs = smem + (size_t)nwarps * (SM::kIO + SM::kState) + sub * W * 32;         // [W][32]
@@ -66,13 +66,12 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 
   const int D = p.D;
   const int groups = (D + 31) / 32;
-  const int rank = (int)(blockIdx.x % (unsigned)CL);
+  const int rank = cluster_rank();
   const int chains = p.batch * p.nseg * groups;
-  const int chain_id = (int)(blockIdx.x / (unsigned)CL) * (nwarps / W) + sub;
+  const int chain_id = cluster_index() * div_pow2(nwarps, W) + sub;
   const int chain = min(chain_id, chains - 1);
-  const int grp = chain % groups;
-  const int bs = chain / groups;
-  const int seg = bs % p.nseg, b = bs / p.nseg;
+  const int bs = chain / groups, grp = chain - bs * groups;
+  const int b = p.nseg == 1 ? bs : bs / p.nseg, seg = bs - b * p.nseg;
   const int c_own = grp * 32 + lane;
   const bool valid = c_own < D;
   const int c_ld = valid ? c_own : D - 1;       // lanes past the last channel read it along and store nothing
@@ -130,7 +129,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
       const float a0 = a[0], step = live > 1 ? a[32] - a0 : 0.f;
       const float tol = 1e-6f * fabsf(a[32 * (live - 1)]);
       bool ok = live == 16 || step <= 0.f;
-      for (int k = 2; k < live; ++k) ok = ok && fabsf(a[32 * k] - (a0 + (float)k * step)) <= tol;
+#pragma unroll
+      for (int k = 2; k < 16; ++k) ok = ok && (k >= live || fabsf(a[32 * k] - (a0 + (float)k * step)) <= tol);
       if (__all_sync(0xffffffffu, ok)) ap_mask |= 1u << g;
     }
   }
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
         // recurrence that consumes them.
         auto run = [&](auto ap_tag) {
           constexpr bool AP = decltype(ap_tag)::value;
-          constexpr int GB = AP ? kLB : 4;   // steps whose exponentials are in flight together
+          constexpr int GB = kLB;
           float a0s = 0.f, rs = 0.f;
           if constexpr (AP) {
             a0s = sA[(16 * g) * 32 + lane];
@@ -248,30 +248,40 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
           for (int gb = 0; gb < kLB / GB; ++gb) {
             float e0[AP ? GB : 1], e1[AP ? GB : 1];
-            float2 af[AP ? 1 : GB][AP ? 1 : 8];   // (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1, 4, 5)
 #pragma unroll
             for (int t = 0; t < GB; ++t) {
               const float dtt = dt[gb * GB + t];
               if constexpr (AP) {
                 e0[t] = ex2_approx(dtt * a0s);
                 e1[t] = ex2_approx(dtt * rs);
-              } else {
-                if constexpr (CPLX) {
-#pragma unroll
-                  for (int kk = 0; kk < 4; ++kk) {
-                    const int k = (kk & 1) + 4 * (kk >> 1);
-                    cexp_pair(dtt, A2[k], A2[k + 2], af[t][k], af[t][k + 2]);
-                  }
-                } else {
-#pragma unroll
-                  for (int k = 0; k < 8; ++k) {
-                    const float2 e = f2mul(f2dup(dtt), A2[k]);
-                    af[t][k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-                  }
-                }
               }
             }
-            float2 aN[2][8], bxN[2][8], CvN[2][READ ? 8 : 1];
+            // general A: the exponentials of a step are taken AH steps ahead of its recurrence, between the multiply-adds of
+            // the steps before it (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1, 4, 5): a batch of
+            // exponentials ahead of a batch of recurrences left the FMA pipe idle during the one and the special-function
+            // unit during the other (bf16 (1, 2048, 5120), N = 64: 394 -> 348 us; complex is fastest two steps ahead)
+            constexpr int AH = CPLX ? 2 : 1, NA = AH + 1;
+            float2 aN[NA][8], bxN[2][8], CvN[2][READ ? 8 : 1];
+            auto exps = [&](int t, float2 (&a)[8]) {
+              const float dtt = dt[gb * GB + t];
+              if constexpr (CPLX) {
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                  const int k = (kk & 1) + 4 * (kk >> 1);
+                  cexp_pair(dtt, A2[k], A2[k + 2], a[k], a[k + 2]);
+                }
+              } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                  const float2 e = f2mul(f2dup(dtt), A2[k]);
+                  a[k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+                }
+              }
+            };
+            if constexpr (!AP) {
+#pragma unroll
+              for (int t = 0; t < AH; ++t) exps(t, aN[t]);
+            }
             auto front = [&](int t, float2 (&a)[8], float2 (&bx)[8], float2 (&Cv)[READ ? 8 : 1]) {
               const int ts = gb * GB + t;
               load16(fB + ts * NP + 16 * g, bx);
@@ -284,9 +294,6 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
                 a[3] = f2mul(a[1], f2dup(r4));
 #pragma unroll
                 for (int k = 0; k < 4; ++k) a[4 + k] = f2mul(a[k], f2dup(r8));
-              } else {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) a[k] = af[t][k];
               }
               const float2 du2 = f2dup(dt[ts] * u[ts]);
 #pragma unroll
@@ -295,20 +302,23 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
             front(0, aN[0], bxN[0], CvN[0]);
 #pragma unroll
             for (int t = 0; t < GB; ++t) {
-              if (t + 1 < GB) front(t + 1, aN[(t + 1) & 1], bxN[(t + 1) & 1], CvN[(t + 1) & 1]);
+              if constexpr (!AP) {
+                if (t + AH < GB) exps(t + AH, aN[(t + AH) % NA]);
+              }
+              if (t + 1 < GB) front(t + 1, aN[(t + 1) % NA], bxN[(t + 1) & 1], CvN[(t + 1) & 1]);
               float2 yv = make_float2(0.f, 0.f), yw = yv;
               if constexpr (CPLX) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk) {
                   const int k = (kk & 1) + 4 * (kk >> 1);
-                  const float2 ar = aN[t & 1][k], ai = aN[t & 1][k + 2], hr = h[k], hi = h[k + 2];
+                  const float2 ar = aN[t % NA][k], ai = aN[t % NA][k + 2], hr = h[k], hi = h[k + 2];
                   h[k] = f2fma(f2neg(ai), hi, f2fma(ar, hr, bxN[t & 1][k]));
                   h[k + 2] = f2fma(ai, hr, f2fma(ar, hi, bxN[t & 1][k + 2]));
                 }
               }
 #pragma unroll
               for (int k = 0; k < 8; ++k) {
-                if constexpr (!CPLX) h[k] = f2fma(aN[t & 1][k], h[k], bxN[t & 1][k]);
+                if constexpr (!CPLX) h[k] = f2fma(aN[t % NA][k], h[k], bxN[t & 1][k]);
                 if constexpr (READ) {
                   if (k & 1) yw = f2fma(CvN[t & 1][k], h[k], yw);
                   else yv = f2fma(CvN[t & 1][k], h[k], yv);
@@ -363,15 +373,24 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
       const float a2 = sA[n * 32 + lane], ai = CPLX ? sA[n * 32 + kRow2 + lane] : 0.f;
       float2 pre = make_float2(0.f, 0.f);
       float ds = 0.f;
-      for (int w = 0; w < W; ++w) {
-        float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
-        const float d = sDs[w * 32 + lane];
-        const float2 e = make_float2(*at, CPLX ? at[kRow2] : 0.f);
-        *at = pre.x;
-        if (CPLX) at[kRow2] = pre.y;
-        const float2 q = CPLX ? cexp_apply<false>(d, a2, ai, pre) : make_float2(ex2_approx(a2 * d) * pre.x, 0.f);
-        pre = make_float2(q.x + e.x, q.y + e.y);
-        ds += d;
+      float2 e[kLaneWarps];
+      float d[kLaneWarps];
+#pragma unroll
+      for (int w = 0; w < kLaneWarps; ++w) {   // (all loaded before the first is used)
+        const float* const at = sE + (size_t)(w < W ? w : 0) * SM::kState + n * 32 + lane;
+        e[w] = make_float2(*at, CPLX ? at[kRow2] : 0.f);
+        d[w] = sDs[(w < W ? w : 0) * 32 + lane];
+      }
+#pragma unroll
+      for (int w = 0; w < kLaneWarps; ++w) {
+        if (w < W) {
+          float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
+          *at = pre.x;
+          if (CPLX) at[kRow2] = pre.y;
+          const float2 q = CPLX ? cexp_apply<false>(d[w], a2, ai, pre) : make_float2(ex2_approx(a2 * d[w]) * pre.x, 0.f);
+          pre = make_float2(q.x + e[w].x, q.y + e[w].y);
+          ds += d[w];
+        }
       }
       sTot[n * 32 + lane] = pre.x;
       if (CPLX) sTot[n * 32 + kRow2 + lane] = pre.y;
@@ -415,13 +434,23 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
         p.seg_end[(seg_row + c_own) * N + col] = step(d, H).x + sTot[n * 32 + lane];
         if (n == 0) p.seg_dsum[seg_row + c_own] = ds_all + d;
       }
-      float cum = 0.f;
-      for (int w = 0; w < W; ++w) {
-        float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
-        const float2 q = step(cum, H);
-        *at += q.x;
-        if (CPLX) at[kRow2] += q.y;
-        cum += sDs[w * 32 + lane];
+      float2 e[kLaneWarps];
+      float cum[kLaneWarps + 1];
+      cum[0] = 0.f;
+#pragma unroll
+      for (int w = 0; w < kLaneWarps; ++w) {
+        const float* const at = sE + (size_t)(w < W ? w : 0) * SM::kState + n * 32 + lane;
+        e[w] = make_float2(*at, CPLX ? at[kRow2] : 0.f);
+        cum[w + 1] = cum[w] + sDs[(w < W ? w : 0) * 32 + lane];
+      }
+#pragma unroll
+      for (int w = 0; w < kLaneWarps; ++w) {
+        if (w < W) {
+          float* const at = sE + (size_t)w * SM::kState + n * 32 + lane;
+          const float2 q = step(cum[w], H);
+          *at = e[w].x + q.x;
+          if (CPLX) at[kRow2] = e[w].y + q.y;
+        }
       }
     }
     if (CL > 1) cg::this_cluster().sync();   // (also: no block leaves while another still reads its totals)
@@ -491,9 +520,11 @@ LaneSplit choose_lane_split(long long chains, int steps, float extra, float fixe
       if (pieces > 1 && (long long)piece * (pieces - w) >= steps) continue;   // the last block would be idle
       const long long blocks = (chains * w + teams - 1) / teams * cl;
       const long long per = (blocks + kNumSMs - 1) / kNumSMs;     // blocks on the fullest SM
-      const long long waves = (per + blocks_per_sm - 1) / blocks_per_sm;
+      // (blocks of a last wave that is not full start as soon as any block ends: between the whole and the exact number)
+      const float exact = (float)blocks / (float)(kNumSMs * blocks_per_sm);
+      const float waves = exact <= 1.f ? 1.f : 0.5f * (exact + (float)((per + blocks_per_sm - 1) / blocks_per_sm));
       const float block = (float)piece * (pieces > 1 ? 1.f + extra : 1.f) + (pieces > 1 ? fixed : 0.5f * fixed) + (cl > 1 ? 0.3f * fixed : 0.f);
-      const float t = block * slow[per < blocks_per_sm ? per : blocks_per_sm] * (float)waves;
+      const float t = block * slow[per < blocks_per_sm ? per : blocks_per_sm] * waves;
       if (best_t == 0.f || t < best_t) {
         best_t = t;
         best = LaneSplit{w, cl, piece};

@@ -187,6 +187,20 @@ __device__ __forceinline__ float lane_softplus(float v) {
   else return softplus_fast(v);
 }
 
+// which cluster this block belongs to (the block itself in a launch without clusters), and its place there
+__device__ __forceinline__ int cluster_index() {
+  unsigned v;
+  asm("mov.u32 %0, %%clusterid.x;" : "=r"(v));
+  return (int)v;
+}
+__device__ __forceinline__ int cluster_rank() {
+  unsigned v;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(v));
+  return (int)v;
+}
+// x / w for w = 1, 2 or 4
+__device__ __forceinline__ int div_pow2(int x, int w) { return x >> (w >> 1); }
+
 // ---- complex states (SSM_FLAG_COMPLEX) in the lane kernels.  N complex states are 2 N columns of the same arrays; a group
 // of 16 rows holds 8 of them as two halves of 4 real parts and their 4 imaginary parts, so that packed arithmetic works on
 // pairs of real parts and pairs of imaginary parts.  lane_col: the column (re, im interleaved) of row n.
