@@ -113,8 +113,8 @@ std::map<std::pair<int, void*>, at::Tensor>& workspaces() {
   static auto* m = new std::map<std::pair<int, void*>, at::Tensor>();
   return *m;
 }
-const at::Tensor* workspace(size_t bytes, const at::Tensor& x, void* stream) {
-  if (bytes == 0) return nullptr;
+at::Tensor workspace(size_t bytes, const at::Tensor& x, void* stream) {
+  if (bytes == 0) return {};
   at::Tensor& ws = workspaces()[{x.device().index(), stream}];
   if (!ws.defined() || (size_t)ws.numel() < bytes) {
     if (ws.defined()) {
@@ -125,10 +125,15 @@ const at::Tensor* workspace(size_t bytes, const at::Tensor& x, void* stream) {
     }
     ws = empty({(int64_t)bytes}, at::kByte, x);
   }
-  return &ws;
+  return ws;   // (a reference of the caller's own: another thread may put a larger one in its place)
 }
 
-void check(ssm_status_t st, const char* what) {
+// Calls a function of the library with the interpreter lock released (a full launch queue blocks), raises its error.
+template <typename F>
+void call(const char* what, F&& f) {
+  PyThreadState* const t = PyEval_SaveThread();
+  const ssm_status_t st = f();
+  PyEval_RestoreThread(t);
   if (st != SSM_OK) raise(std::string(what) + ": " + api.ssm_status_string(st));
 }
 
@@ -226,7 +231,9 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor saved;
     if (save) saved = sgiven != nullptr ? *sgiven : empty({(int64_t)(api.ssm_scan_saved_state_bytes(&pr.p) / 4)}, at::kFloat, x);
     const at::Tensor* ws = tensor(a[12], "workspace");
-    if (ws == nullptr && entry != 2) ws = workspace(api.ssm_scan_fwd_workspace_bytes(&pr.p), x, stream);
+    at::Tensor own;
+    if (ws == nullptr && entry != 2) own = workspace(api.ssm_scan_fwd_workspace_bytes(&pr.p), x, stream);
+    if (own.defined()) ws = &own;
     void* wp = pointer(ws, "workspace");
     const size_t wbytes = ws == nullptr ? 0 : (size_t)ws->numel() * ws->element_size();
     void* px = pointer(&x, "x", pr.rows, pr.io);
@@ -241,12 +248,18 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     auto* pl = static_cast<float*>(pointer(a[10], "h_last", pr.h, at::kFloat));
     void* ps = save ? pointer(&saved, "saved_states") : nullptr;
     if (entry == 2) {
-      check(api.ssm_scan_fwd_static(&pr.p, px, pd, pA, pB, pC, pD, pz, po, ps, stream), "ssm_scan_fwd_static");
+      call("ssm_scan_fwd_static", [&] {
+        return api.ssm_scan_fwd_static(&pr.p, px, pd, pA, pB, pC, pD, pz, po, ps, stream);
+      });
     } else if (entry == 1) {
       auto* pb = static_cast<float*>(pointer(a[2], "delta_bias", {D}, at::kFloat));
-      check(api.ssm_scan_fwd_fused_dt(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, ph, po, pl, ps, wp, wbytes, stream), "ssm_scan_fwd_fused_dt");
+      call("ssm_scan_fwd_fused_dt", [&] {
+        return api.ssm_scan_fwd_fused_dt(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, ph, po, pl, ps, wp, wbytes, stream);
+      });
     } else {
-      check(api.ssm_scan_fwd_state(&pr.p, px, pd, pA, pB, pC, pD, pz, ph, po, pl, ps, wp, wbytes, stream), "ssm_scan_fwd_state");
+      call("ssm_scan_fwd_state", [&] {
+        return api.ssm_scan_fwd_state(&pr.p, px, pd, pA, pB, pC, pD, pz, ph, po, pl, ps, wp, wbytes, stream);
+      });
     }
     if (!save) return wrap(out);
     PyObject* o = wrap(out);
@@ -295,7 +308,9 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     PyObject* o = a[14];
     void* stream = stream_of(a[13], x);
     const at::Tensor* ws = tensor(a[12], "workspace");
-    if (ws == nullptr) ws = workspace(api.ssm_scan_bwd_workspace_bytes(&pr.p), x, stream);
+    at::Tensor own;
+    if (ws == nullptr) own = workspace(api.ssm_scan_bwd_workspace_bytes(&pr.p), x, stream);
+    if (own.defined()) ws = &own;
     void* wp = pointer(ws, "workspace");
     const size_t wbytes = ws == nullptr ? 0 : (size_t)ws->numel() * ws->element_size();
     void* px = pointer(&x, "x", pr.rows, pr.io);
@@ -323,21 +338,25 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (fused) {
       auto* pb = static_cast<float*>(pointer(a[2], "delta_bias", {D}, at::kFloat));
       if (state)
-        check(api.ssm_scan_bwd_fused_dt_state(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, pg, ph, pm, ps, data(dx), data(dd), fdata(dbias),
-                                              fdata(dA), data(dB), data(dC), fdata(dD), data(dz), fdata(dh0), wp, wbytes, stream),
-              "ssm_scan_bwd_fused_dt_state");
+        call("ssm_scan_bwd_fused_dt_state", [&] {
+        return api.ssm_scan_bwd_fused_dt_state(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, pg, ph, pm, ps, data(dx), data(dd), fdata(dbias),
+        fdata(dA), data(dB), data(dC), fdata(dD), data(dz), fdata(dh0), wp, wbytes, stream);
+      });
       else
-        check(api.ssm_scan_bwd_fused_dt(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, pg, ps, data(dx), data(dd), fdata(dbias), fdata(dA),
-                                        data(dB), data(dC), fdata(dD), data(dz), wp, wbytes, stream),
-              "ssm_scan_bwd_fused_dt");
+        call("ssm_scan_bwd_fused_dt", [&] {
+        return api.ssm_scan_bwd_fused_dt(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, pg, ps, data(dx), data(dd), fdata(dbias), fdata(dA),
+        data(dB), data(dC), fdata(dD), data(dz), wp, wbytes, stream);
+      });
     } else if (state) {
-      check(api.ssm_scan_bwd_state(&pr.p, px, pd, pA, pB, pC, pD, pz, pg, ph, pm, ps, data(dx), data(dd), fdata(dA), data(dB), data(dC),
-                                   fdata(dD), data(dz), fdata(dh0), wp, wbytes, stream),
-            "ssm_scan_bwd_state");
+      call("ssm_scan_bwd_state", [&] {
+        return api.ssm_scan_bwd_state(&pr.p, px, pd, pA, pB, pC, pD, pz, pg, ph, pm, ps, data(dx), data(dd), fdata(dA), data(dB), data(dC),
+        fdata(dD), data(dz), fdata(dh0), wp, wbytes, stream);
+      });
     } else {
-      check(api.ssm_scan_bwd(&pr.p, px, pd, pA, pB, pC, pD, pz, pg, ps, data(dx), data(dd), fdata(dA), data(dB), data(dC), fdata(dD),
-                             data(dz), wp, wbytes, stream),
-            "ssm_scan_bwd");
+      call("ssm_scan_bwd", [&] {
+        return api.ssm_scan_bwd(&pr.p, px, pd, pA, pB, pC, pD, pz, pg, ps, data(dx), data(dd), fdata(dA), data(dB), data(dC), fdata(dD),
+        data(dz), wp, wbytes, stream);
+      });
     }
     Py_INCREF(o);
     return o;
@@ -364,7 +383,10 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
     auto* ph = static_cast<float*>(pointer(a[7], "h", pr.h, at::kFloat));
     at::Tensor out = given != nullptr ? *given : empty(pr.rows, pr.io, x);
     void* po = pointer(&out, "out", pr.rows, pr.io);
-    check(api.ssm_step(&pr.p, px, pd, pA, pB, pC, pD, pz, ph, po, stream_of(a[9], x)), "ssm_step");
+    void* stream = stream_of(a[9], x);
+    call("ssm_step", [&] {
+        return api.ssm_step(&pr.p, px, pd, pA, pB, pC, pD, pz, ph, po, stream);
+      });
     return wrap(out);
   });
 }
@@ -394,7 +416,10 @@ PyObject* conv_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const at::Tensor* given = tensor(a[4], "y");
     at::Tensor y = given != nullptr ? *given : empty(x.sizes(), io, x);
     void* py = pointer(&y, "y", x.sizes(), io);
-    check(api.ssm_conv1d_fwd(&p, px, pw, pb, pp, py, stream_of(a[5], x)), "ssm_conv1d_fwd");
+    void* stream = stream_of(a[5], x);
+    call("ssm_conv1d_fwd", [&] {
+        return api.ssm_conv1d_fwd(&p, px, pw, pb, pp, py, stream);
+      });
     return wrap(y);
   });
 }
@@ -421,11 +446,12 @@ PyObject* conv_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (pb != nullptr) db = output(o, "dbias", {D}, at::kFloat, x);
     else no_output(o, "dbias");
     if (truth(a[8]) && W > 1) dp = output(o, "dx_prev", {(int64_t)p.batch, W - 1, D}, io, x);
-    const at::Tensor* ws = workspace(api.ssm_conv1d_bwd_workspace_bytes(&p), x, stream);
-    check(api.ssm_conv1d_bwd(&p, px, pw, pb, pp, pg, dx.data_ptr(), static_cast<float*>(dw.data_ptr()),
-                             db.defined() ? static_cast<float*>(db.data_ptr()) : nullptr, dp.defined() ? dp.data_ptr() : nullptr,
-                             ws == nullptr ? nullptr : ws->data_ptr(), ws == nullptr ? 0 : (size_t)ws->numel(), stream),
-          "ssm_conv1d_bwd");
+    const at::Tensor ws = workspace(api.ssm_conv1d_bwd_workspace_bytes(&p), x, stream);
+    call("ssm_conv1d_bwd", [&] {
+        return api.ssm_conv1d_bwd(&p, px, pw, pb, pp, pg, dx.data_ptr(), static_cast<float*>(dw.data_ptr()),
+        db.defined() ? static_cast<float*>(db.data_ptr()) : nullptr, dp.defined() ? dp.data_ptr() : nullptr,
+        ws.defined() ? ws.data_ptr() : nullptr, ws.defined() ? (size_t)ws.numel() : 0, stream);
+      });
     Py_INCREF(o);
     return o;
   });

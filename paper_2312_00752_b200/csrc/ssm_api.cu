@@ -107,7 +107,7 @@ bool lane_bwd(const ssm_problem_t& p) {
   plan_lane_bwd(p, kLaneWarps, &pl, &lane);
   return 1037.f * lane + 20e3f < tuned;
 }
-// Time segments of a lane launch.  A chain already spreads over up to 64 warps of a cluster, so the launch itself is
+// Time segments of a lane launch.  A chain already spreads over up to 32 warps of a cluster, so the launch itself is
 // split (summary pass, carry, full pass) only for a handful of chains and then into segments of at least 2048 steps.
 static int lane_segments(const ssm_problem_t& p) {
   const long long chains = (long long)p.batch * ((p.D + 31) / 32);
