@@ -22,9 +22,11 @@ namespace {
 
 constexpr int kConvThreads = 64;
 constexpr int kConvMinSteps = 32;   // time steps per thread and chunk: chosen per launch between these two so that the
-constexpr int kConvMaxSteps = 128;  // grid fills the GPU a whole number of times (see choose_steps)
+constexpr int kConvMaxSteps = 512;  // grid fills the GPU a whole number of times (see choose_steps)
+constexpr int kConvFixed = 24;
 constexpr int kConvAheadFwd = 8;    // rows loaded before the first of them is used
-constexpr int kConvAheadBwd = 8;    // (two tensors per row in the backward kernel; 2, 4, 8, 16 measured: 78, 64, 60, 83 us)
+constexpr int kConvAheadBwd = 8;    // (two tensors per row in the backward kernel; 2, 4, 8, 16 measured: 78, 64, 60, 83 us;
+                                    // a row requested as soon as the one A before it is used, instead of A at once: 76)
 
 struct ConvParams {
   const void* x;
@@ -275,25 +277,20 @@ __device__ __forceinline__ void store4(float* __restrict__ p, const float2 (&v)[
   *reinterpret_cast<float4*>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
 }
 
-// sigmoid of a pair.  FAST: 1/2 + 1/2 tanh(v/2) with the hardware tanh (one special-function operation instead of two;
-// relative error about 2^-11, used for bf16 io only, whose own rounding is 2^-9); otherwise ex2 + reciprocal.
-template <bool FAST>
-__device__ __forceinline__ float2 sigmoid2(float2 v) {
-  if (FAST) {
-    const float2 h = f2mul(v, f2dup(0.5f));
-    return f2fma(make_float2(tanh_approx(h.x), tanh_approx(h.y)), f2dup(0.5f), f2dup(0.5f));
-  }
-  return make_float2(sigmoid_fast(v.x), sigmoid_fast(v.y));
-}
+// sigmoid of a pair, by ex2 and reciprocal (float io).  bf16 io takes sigma(v) = 1/2 + 1/2 tanh(v/2) with the hardware
+// tanh (one special-function operation instead of two; relative error about 2^-11, the io's own rounding is 2^-9), and
+// its kernels hold half the taps, so that the sum over the taps is v/2 itself.
+__device__ __forceinline__ float2 sigmoid2(float2 v) { return make_float2(sigmoid_fast(v.x), sigmoid_fast(v.y)); }
+__device__ __forceinline__ float2 tanh2(float2 v) { return make_float2(tanh_approx(v.x), tanh_approx(v.y)); }
 
 template <typename IO, int W>
-__device__ __forceinline__ void load_taps4(const ConvParams& p, int c0, float2 (&wv)[W][2], float2 (&bv)[2]) {
+__device__ __forceinline__ void load_taps4(const ConvParams& p, int c0, float scale, float2 (&wv)[W][2], float2 (&bv)[2]) {
   float wq[4][W], bq[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    bq[q] = p.bias != nullptr ? p.bias[c0 + q] : 0.f;
+    bq[q] = p.bias != nullptr ? scale * p.bias[c0 + q] : 0.f;
 #pragma unroll
-    for (int k = 0; k < W; ++k) wq[q][k] = p.w[(size_t)(c0 + q) * W + k];
+    for (int k = 0; k < W; ++k) wq[q][k] = scale * p.w[(size_t)(c0 + q) * W + k];
   }
   bv[0] = make_float2(bq[0], bq[1]);
   bv[1] = make_float2(bq[2], bq[3]);
@@ -324,9 +321,10 @@ __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_fwd_vec4_kernel(const
   const int t1 = min(p.L, t0 + p.steps);
   constexpr int H = W > 1 ? W - 1 : 1;
   constexpr int A = kConvAheadFwd;
+  constexpr bool HALF = SILU && FAST;   // taps and bias scaled by 1/2 (exact)
 
   float2 wv[W][2], bv[2], win[H][2];
-  load_taps4<IO, W>(p, c0, wv, bv);
+  load_taps4<IO, W>(p, c0, HALF ? 0.5f : 1.f, wv, bv);
 #pragma unroll
   for (int i = 0; i < W - 1; ++i) load_input_row4<IO, W>(p, b, t0 - (W - 1) + i, c0, win[i]);
 
@@ -357,7 +355,8 @@ __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_fwd_vec4_kernel(const
           float2 pre = f2fma(wv[W - 1][h], cur[h], bv[h]);
 #pragma unroll
           for (int k = 0; k < W - 1; ++k) pre = f2fma(wv[k][h], win[k][h], pre);
-          o[h] = SILU ? f2mul(pre, sigmoid2<FAST>(pre)) : pre;
+          if (!SILU) o[h] = pre;
+          else o[h] = HALF ? f2fma(pre, tanh2(pre), pre) : f2mul(pre, sigmoid2(pre));
 #pragma unroll
           for (int k = 0; k + 1 < W - 1; ++k) win[k][h] = win[k + 1][h];
           if (W > 1) win[H - 1][h] = cur[h];
@@ -382,12 +381,15 @@ __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_bwd_vec4_kernel(const
   const int t0 = blockIdx.y * p.steps;
   const int t1 = min(p.L, t0 + p.steps);
   constexpr int A = kConvAheadBwd;
+  // taps and bias scaled by -1/2: pre is then -v/2 for the true pre-activation v, dpre twice the true one (the signs make
+  // every term of 2 silu'(v) = 1 + tanh(v/2) + v/2 (1 - tanh^2(v/2)) one multiply-add); all exact
+  constexpr bool HALF = SILU && FAST;
 
   float2 wv[W][2], bv[2];
   float2 xw[W][2];    // xw[i] = x[t - (W-1) + i]
   float2 dp[W][2];    // dp[i] = dpre[t - (W-1) + i]; values before this chunk are never used and start as zero
   float2 dwa[W][2], dba[2];
-  load_taps4<IO, W>(p, c0, wv, bv);
+  load_taps4<IO, W>(p, c0, HALF ? -0.5f : 1.f, wv, bv);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     dba[h] = make_float2(0.f, 0.f);
@@ -443,22 +445,25 @@ __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_bwd_vec4_kernel(const
 #pragma unroll
           for (int k = 0; k < W; ++k) pre = f2fma(wv[k][h], xw[k][h], pre);
           float2 dpre = g2[h];
-          if (SILU) {
-            const float2 sg = sigmoid2<FAST>(pre);
+          if constexpr (HALF) {
+            const float2 th = tanh2(pre);
+            const float2 u2 = f2fma(th, th, f2dup(-1.f)), om = f2fma(th, f2dup(-1.f), f2dup(1.f));
+            dpre = f2mul(dpre, f2fma(pre, u2, om));
+          } else if constexpr (SILU) {
+            const float2 sg = sigmoid2(pre);
             const float2 om = f2fma(sg, f2dup(-1.f), f2dup(1.f));
             dpre = f2mul(dpre, f2mul(sg, f2fma(pre, om, f2dup(1.f))));
           }
           dp[W - 1][h] = dpre;
           if (own) {
-            dba[h].x += dpre.x;
-            dba[h].y += dpre.y;
+            dba[h] = __fadd2_rn(dba[h], dpre);
 #pragma unroll
             for (int k = 0; k < W; ++k) dwa[k][h] = f2fma(dpre, xw[k][h], dwa[k][h]);
           }
           float2 acc = f2mul(wv[0][h], dp[W - 1][h]);
 #pragma unroll
           for (int k = 1; k < W; ++k) acc = f2fma(wv[k][h], dp[W - 1 - k][h], acc);   // dpre[s + (W-1) - k] = dpre[tt - k]
-          o[h] = acc;
+          o[h] = HALF ? make_float2(-acc.x, -acc.y) : acc;
 #pragma unroll
           for (int k = 0; k + 1 < W; ++k) {
             xw[k][h] = xw[k + 1][h];
@@ -479,16 +484,17 @@ __global__ void __launch_bounds__(kConvThreads) ssm_conv1d_bwd_vec4_kernel(const
   for (; t + A <= t1; t += A) batch(t, std::true_type{});
   for (; t < t_stop; t += A) batch(t, std::false_type{});
 
+  const float half = HALF ? 0.5f : 1.f;
   float* part = p.part + ((size_t)(b * gridDim.y + blockIdx.y) * p.D + c0) * (W + 1);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
 #pragma unroll
     for (int k = 0; k < W; ++k) {
-      part[(2 * h) * (W + 1) + k] = dwa[k][h].x;
-      part[(2 * h + 1) * (W + 1) + k] = dwa[k][h].y;
+      part[(2 * h) * (W + 1) + k] = half * dwa[k][h].x;
+      part[(2 * h + 1) * (W + 1) + k] = half * dwa[k][h].y;
     }
-    part[(2 * h) * (W + 1) + W] = dba[h].x;
-    part[(2 * h + 1) * (W + 1) + W] = dba[h].y;
+    part[(2 * h) * (W + 1) + W] = half * dba[h].x;
+    part[(2 * h + 1) * (W + 1) + W] = half * dba[h].y;
   }
 }
 
@@ -523,17 +529,19 @@ __global__ void __launch_bounds__(kRedOutputs* kRedSlices) ssm_conv1d_reduce_ker
   }
 }
 
-// Steps per chunk.  Every block costs about (steps + W - 1) row visits and the blocks run in
-// ceil(blocks / resident blocks) rounds, so the run time goes like rounds * (steps + W - 1): pick the chunk length in
-// [kConvMinSteps, kConvMaxSteps] that minimises it (a grid that fills the GPU a whole number of times; for small
-// problems the shortest chunk, i.e. the most parallelism), longer chunks winning ties (fewer halo rows).
+// Steps per chunk.  A block costs about steps + W - 1 row visits plus what it takes until its first rows have arrived
+// and its partial sums are out (kConvFixed, in steps), and the blocks run in ceil(blocks / resident blocks) rounds:
+// pick the chunk length in [kConvMinSteps, kConvMaxSteps] with the smallest rounds * cost (a grid that fills the GPU a
+// whole number of times; for small problems the shortest chunk, i.e. the most parallelism), longer chunks winning ties
+// (fewer halo rows and partial sums).  One round of long chunks beats two of half the length: backward with its
+// reduction, bf16 W = 4, (4, 2048, 5120): 94 steps 61.6 us, 187 steps 53.2; (8, 4096, 2048): 92.9 -> 81.8.
 int choose_steps(long long blocks_per_chunk, int L, int W, long long resident) {
   int best = kConvMinSteps;
   long long best_cost = -1;
   for (int steps = kConvMinSteps; steps <= kConvMaxSteps; ++steps) {
     const long long chunks = (L + steps - 1) / steps;
     const long long rounds = (blocks_per_chunk * chunks + resident - 1) / resident;
-    const long long cost = rounds * (steps + W - 1);
+    const long long cost = rounds * (steps + W - 1 + kConvFixed);
     if (best_cost < 0 || cost <= best_cost) {
       best_cost = cost;
       best = steps;
