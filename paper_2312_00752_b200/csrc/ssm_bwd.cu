@@ -351,44 +351,96 @@ __global__ void __launch_bounds__(BwdGeom<N>::THREADS) ssm_bwd_local_kernel(cons
 
 // Second stage of the deterministic reductions: sums the per-block dB/dC partials over channel groups and the
 // per-(batch, segment) dA/dD partials, in ascending order, and rounds dB/dC to the io dtype.
-template <typename IO>
-__global__ void __launch_bounds__(256) ssm_bwd_reduce_kernel(const ReduceParams p) {
+// dB / dC: a block owns kRedLanes * V adjacent values of one of them (V = 4 per load where the rows are aligned); its
+// slices of threads each add a contiguous range of the channel groups in ascending order, in whole batches of loads, and
+// the range sums are added in ascending order through shared memory.  HBM-bound: 168 MB of partial sums at
+// (4, 2048, 5120), more than the L2 holds.  A thread per value that walked all the groups kept too little in flight:
+// 34.6 -> 27.2 us there (4.8 -> 6.2 TB/s), 9.6 -> 7.3 us at float32 (2, 2048, 1536); 4 or 8 slices, or 16 loads per
+// batch, are within 5 % on large problems and slower on the others.
+// Behind those blocks: dA, dD and what else is summed over (batch, segment), a thread per value.
+constexpr int kRedSlices = 2, kRedLanes = 64, kRedBatch = 8;
+template <typename IO, int V>
+__global__ void __launch_bounds__(kRedLanes * kRedSlices) ssm_bwd_reduce_kernel(const ReduceParams p, const unsigned bc_blocks) {
+  __shared__ float s_sum[kRedSlices][V][kRedLanes];
   dependency_wait();
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < p.bln) {
-    float sb = 0.f, sc = 0.f;
-    for (int g = 0; g < p.groups; ++g) {
-      sb += p.dBC_part[((size_t)g * 2 + 0) * p.bln + i];
-      sc += p.dBC_part[((size_t)g * 2 + 1) * p.bln + i];
+  if (blockIdx.x < bc_blocks) {
+    const int lane = threadIdx.x % kRedLanes, slice = threadIdx.x / kRedLanes, which = blockIdx.x & 1;
+    const long long i = ((long long)(blockIdx.x >> 1) * kRedLanes + lane) * V;
+    IO* const out = static_cast<IO*>(which == 0 ? p.dB : p.dC);
+    if (out == nullptr) return;
+    const int per = (p.groups + kRedSlices - 1) / kRedSlices;
+    const int g0 = min(p.groups, slice * per), g1 = min(p.groups, g0 + per);
+    float acc[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) acc[k] = 0.f;
+    if (i < p.bln) {
+      const float* __restrict__ part = p.dBC_part + ((size_t)g0 * 2 + which) * p.bln + i;
+      // (whole batches of loads, so that a short range is not a chain of round trips to memory)
+      for (int g = g0; g < g1; g += kRedBatch, part += (size_t)kRedBatch * 2 * p.bln) {
+        float v[kRedBatch][V];
+#pragma unroll
+        for (int u = 0; u < kRedBatch; ++u) {
+          const float* const at = part + (size_t)(g + u < g1 ? u : 0) * 2 * p.bln;
+          if constexpr (V == 4) {
+            const float4 q = __ldcs(reinterpret_cast<const float4*>(at));
+            v[u][0] = q.x;
+            v[u][1] = q.y;
+            v[u][2] = q.z;
+            v[u][3] = q.w;
+          } else {
+            v[u][0] = __ldcs(at);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kRedBatch; ++u) {
+#pragma unroll
+          for (int k = 0; k < V; ++k) acc[k] += g + u < g1 ? v[u][k] : 0.f;
+        }
+      }
     }
-    if (p.dB != nullptr) static_cast<IO*>(p.dB)[i] = float_to_io<IO>(sb);
-    if (p.dC != nullptr) static_cast<IO*>(p.dC)[i] = float_to_io<IO>(sc);
+#pragma unroll
+    for (int k = 0; k < V; ++k) s_sum[slice][k][lane] = acc[k];
+    __syncthreads();
+    if (slice != 0 || i >= p.bln) return;
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+#pragma unroll
+      for (int r = 1; r < kRedSlices; ++r) acc[k] += s_sum[r][k][lane];
+    }
+    if constexpr (V == 4) {
+      if constexpr (sizeof(IO) == 4) {
+        *reinterpret_cast<float4*>(out + i) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      } else {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(acc[0], acc[1]), hi = __floats2bfloat162_rn(acc[2], acc[3]);
+        *reinterpret_cast<uint2*>(out + i) =
+            make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+      }
+    } else {
+      out[i] = float_to_io<IO>(acc[0]);
+    }
+    return;
   }
+  const long long i = (long long)(blockIdx.x - bc_blocks) * blockDim.x + threadIdx.x;
   const long long dn = (long long)p.D * p.N;
+  auto sum = [&](const float* __restrict__ part, long long n) {
+    float v = 0.f;
+    for (int q = 0; q < p.parts; q += kRedBatch) {
+      float w[kRedBatch];
+#pragma unroll
+      for (int u = 0; u < kRedBatch; ++u) w[u] = part[(size_t)(q + u < p.parts ? q + u : q) * n + i];
+#pragma unroll
+      for (int u = 0; u < kRedBatch; ++u) v += q + u < p.parts ? w[u] : 0.f;
+    }
+    return v;
+  };
   if (i < dn) {
-    float sa = 0.f;
-    for (int q = 0; q < p.parts; ++q) sa += p.dA_part[(size_t)q * dn + i];
-    p.dA[i] = sa;
-    if (p.dBs != nullptr) {
-      float v = 0.f;
-      for (int q = 0; q < p.parts; ++q) v += p.dBs_part[(size_t)q * dn + i];
-      p.dBs[i] = v;
-    }
-    if (p.dCs != nullptr) {
-      float v = 0.f;
-      for (int q = 0; q < p.parts; ++q) v += p.dCs_part[(size_t)q * dn + i];
-      p.dCs[i] = v;
-    }
+    p.dA[i] = sum(p.dA_part, dn);
+    if (p.dBs != nullptr) p.dBs[i] = sum(p.dBs_part, dn);
+    if (p.dCs != nullptr) p.dCs[i] = sum(p.dCs_part, dn);
   }
-  if (p.dD != nullptr && i < p.D) {
-    float sd = 0.f;
-    for (int q = 0; q < p.parts; ++q) sd += p.dD_part[(size_t)q * p.D + i];
-    p.dD[i] = sd;
-  }
-  if (p.dbias != nullptr && i < p.D) {
-    float sb = 0.f;
-    for (int q = 0; q < p.parts; ++q) sb += p.dbias_part[(size_t)q * p.D + i];
-    p.dbias[i] = sb;
+  if (i < p.D) {
+    if (p.dD != nullptr) p.dD[i] = sum(p.dD_part, p.D);
+    if (p.dbias != nullptr) p.dbias[i] = sum(p.dbias_part, p.D);
   }
 }
 
@@ -441,11 +493,18 @@ cudaError_t launch_bwd(const ssm_problem_t& prob, const Plan& plan, const BwdPar
   return launch_bwd_io<float>(prob, plan, p, mode, s);
 }
 
+template <typename IO>
+static cudaError_t launch_reduce_io(const ReduceParams& p, cudaStream_t s) {
+  constexpr int kThreads = kRedLanes * kRedSlices;
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p.dB) | reinterpret_cast<uintptr_t>(p.dC);
+  const int V = p.bln % 4 == 0 && at % (4 * sizeof(IO)) == 0 ? 4 : 1;
+  const unsigned bc = 2 * (unsigned)((p.bln + kRedLanes * V - 1) / (kRedLanes * V));
+  const unsigned rest = (unsigned)(((long long)p.D * p.N + kThreads - 1) / kThreads);   // (D N >= D)
+  return V == 4 ? launch_dependent(ssm_bwd_reduce_kernel<IO, 4>, bc + rest, kThreads, 0, 1, s, p, bc)
+                : launch_dependent(ssm_bwd_reduce_kernel<IO, 1>, bc + rest, kThreads, 0, 1, s, p, bc);
+}
 cudaError_t launch_bwd_reduce(const ssm_problem_t& prob, const ReduceParams& p, cudaStream_t s) {
-  const long long work = p.bln > (long long)p.D * p.N ? p.bln : (long long)p.D * p.N;
-  const unsigned blocks = (unsigned)((work + 255) / 256);
-  if (prob.io_dtype == SSM_BF16) return launch_dependent(ssm_bwd_reduce_kernel<__nv_bfloat16>, blocks, 256, 0, 1, s, p);
-  return launch_dependent(ssm_bwd_reduce_kernel<float>, blocks, 256, 0, 1, s, p);
+  return prob.io_dtype == SSM_BF16 ? launch_reduce_io<__nv_bfloat16>(p, s) : launch_reduce_io<float>(p, s);
 }
 
 }  // namespace ssm
