@@ -343,6 +343,14 @@ static cudaError_t attach_fwd_sched(const ssm_problem_t& p, const Plan& pl, char
   return cudaMemsetAsync(ws + w.flags, 0, (size_t)(w.max_workers + 1) * sizeof(int), s);
 }
 
+// Pieces a segment of the tuned kernels is cut into for the adjoint pre-pass.  The segments give the main kernel one to
+// two warps per sub-partition; the pre-pass has room for three and waits for its own latencies with less, so they are
+// halved ((4, 2048, 5120), two segments: 75 -> 62 us and 4 us of carry; half a million steps at width 1536: 1.98 -> 1.85 ms;
+// thirds are no faster).
+static int prepass_split(const ssm_problem_t& p, const Plan& pl) {
+  return tuned_shape(p) && pl.nseg > 1 && !lane_bwd(p) ? 2 : 1;
+}
+
 struct BwdWorkspace {
   size_t dBC_part, dA_part, dD_part, dbias_part, ckpt, seg_local, seg_dsum, mu_in, fwd, flags, handoff, total;
   size_t dBs_part, dCs_part;   // static B / C
@@ -372,9 +380,10 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
   if (pl.nseg > 1) {
     // (the lane kernels keep whole groups of 32 channels and of 16 states)
     const size_t d32 = (size_t)((p.D + 31) / 32) * 32, n16 = (size_t)((p.N + 15) / 16) * 16;
-    w.seg_local = take(segs * d32 * n16 * sizeof(float));
-    if (!lane_bwd(p)) w.mu_in = take(segs * p.D * p.N * sizeof(float));
-    w.seg_dsum = take(segs * d32 * sizeof(float));
+    const size_t pieces = segs * prepass_split(p, pl);
+    w.seg_local = take(pieces * d32 * n16 * sizeof(float));
+    if (!lane_bwd(p)) w.mu_in = take(pieces * p.D * p.N * sizeof(float));
+    w.seg_dsum = take(pieces * d32 * sizeof(float));
   }
   w.fwd = take(fwd_layout(p, pl_fwd).total);   // the forward sweep that rebuilds checkpoints uses the forward split
   w.handoff = take((size_t)(w.max_workers + 1) *
@@ -824,19 +833,17 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   BwdParams carried = bp;
   if (pl.nseg > 1) carried.mu_in = nullptr;   // (the main kernel's inflow is then in the workspace)
   const bool lane = bwd_lane_applicable(bp) && (lane_bwd(*p) || !bwd_fast_applicable(*p, carried));
+  bp.local_split = 1;
+  bp.local_steps = pl.seg_steps;
+  if (!lane && pl.nseg > 1 && bwd_fast_applicable(*p, carried) && bwd_local_fast_applicable(*p, bp)) {
+    bp.local_split = prepass_split(*p, pl);
+    bp.local_steps = ((pl.seg_steps + bp.local_split - 1) / bp.local_split + kSegAlign - 1) / kSegAlign * kSegAlign;
+  }
   if (lane && pl.nseg > 1) {
     // the lane kernel folds the segments' results itself
     bp.seg_local = reinterpret_cast<float*>(ws + w.seg_local);
     bp.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum);
     if (launch_bwd_lane(*p, pl, bp, kBwdLocal, s) != cudaSuccess) return SSM_ERR_CUDA;
-  } else if (pl.nseg == 2 && dh_last == nullptr && (bp.seg_local = reinterpret_cast<float*>(ws + w.mu_in),
-                                              bp.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum),
-                                              bwd_local_fast_applicable(*p, bp))) {
-    // two segments and nothing flowing in from outside: the adjoint leaving segment 1 IS the inflow of segment 0, so
-    // the tuned pre-pass writes it there and the carry scan is skipped
-    bp.local_as_inflow = 1;
-    if (launch_bwd(*p, pl, bp, kBwdLocal, s) != cudaSuccess) return SSM_ERR_CUDA;
-    bp.mu_in = bp.seg_local;
   } else if (pl.nseg > 1) {
     bp.seg_local = reinterpret_cast<float*>(ws + w.seg_local);
     bp.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum);
@@ -847,7 +854,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
     cp.A = A;
     cp.carried = reinterpret_cast<float*>(ws + w.mu_in);
     cp.batch = p->batch;
-    cp.nseg = pl.nseg;
+    cp.nseg = pl.nseg * bp.local_split;
     cp.D = p->D;
     cp.N = p->N;
     cp.reverse = 1;

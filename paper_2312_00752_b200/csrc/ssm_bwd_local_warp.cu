@@ -6,9 +6,14 @@
 // Only this lambda / mu recurrence is needed here: no states, no x, no B.  Segment 0 has no earlier segment to hand its
 // adjoint to and is not computed.
 //
+// Bound by latency and, with one exponential per state, the special-function unit (19 operations = 152 cycles per warp
+// and step), so warps per sub-partition count: segments are halved (ssm_api.cu) and the ring is as short as the copies allow.
+// With a third stage a block took half of an SM's shared memory (all of what fits with the fused step size): general A
+// and fused step size, (8, 2048, 1536): 152 -> 108 us.
+//
 // Same construction as the tuned forward kernel (ssm_fwd_warp.cu) run backwards in time: one warp owns 32 adjacent
 // channels of one segment, lane l holds all 16 states of channel l as packed float2 pairs (no exchanges between lanes),
-// stages delta, z, dout and C with 16-byte cp.async copies into a three-stage ring of 32-step tiles private to the warp
+// stages delta, z, dout and C with 16-byte cp.async copies into a two-stage ring of 32-step tiles private to the warp
 // (walked from the last tile of the segment to the first), widens C to float once per tile and turns dout and z into ds
 // once per element.  The (chain, tile) space is cut into equal ranges, one per resident warp (WarpSched in
 // ssm_common.cuh); a chain that two warps share hands mu and the partial sum of delta over once, through L2, behind a
@@ -24,7 +29,7 @@ int warp_workers(int chains, int sms, int per_sm, int max_workers);
 namespace {
 
 constexpr int kLT = 32;          // steps per tile
-constexpr int kLStages = 3;      // ring stages
+constexpr int kLStages = 2;      // ring stages (a tile of 32 steps takes longer than a trip to memory; a third stage costs a block per SM)
 constexpr int kLWarps = 4;       // warps per block
 constexpr int kLocalHandoffVec = 5;   // float4 per lane: 16 adjoint values, sum of delta
 
@@ -38,8 +43,6 @@ struct LocalWarpSmem {
   float fC[SC ? 1 : kLT][20];               // C of the current tile widened to float (padded likewise)
   float dF[SP ? kLT : 1][32];      // SP: step sizes after bias and softplus
 };
-
-__device__ __forceinline__ void cp_async_wait_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 }  // namespace
 
@@ -66,17 +69,18 @@ __global__ void __launch_bounds__(kLWarps * 32) ssm_bwd_local_warp_kernel(const 
   };
 
   const int groups = (D + 31) / 32;
-  const int nsegs = p.nseg - 1;   // segments 1 .. nseg - 1
+  const int split = p.local_split, nsegs = (p.nseg - 1) * split;   // pieces of segments 1 .. nseg - 1
   const WorkList wl = make_worklist(sc, worker);
   for (int pi = 0; pi < wl.count; ++pi) {
     int chain, from, to;
     get_piece(wl, sc.tiles, pi, chain, from, to);
     const int grp = chain % groups;
     const int bs = chain / groups;
-    const int seg = 1 + bs % nsegs, b = bs / nsegs;
+    const int seg = split + bs % nsegs, b = bs / nsegs;   // (number of the piece)
     const int d_w = grp * 32;
-    const int t_seg0 = seg * p.seg_steps;
-    const int t_seg_end = min(p.L, t_seg0 + p.seg_steps);
+    const int whole = seg / split;
+    const int t_seg0 = whole * p.seg_steps + (seg - whole * split) * p.local_steps;
+    const int t_seg_end = min(min(p.L, (whole + 1) * p.seg_steps), t_seg0 + p.local_steps);   // (may be before t_seg0)
     const int live_tiles = (t_seg_end - t_seg0 + kLT - 1) / kLT;
     // positions [from, to) of the chain in processing order are tiles tile_hi down to tile_lo (time runs backwards)
     const int tile_lo = sc.tiles - to;
@@ -115,7 +119,6 @@ __global__ void __launch_bounds__(kLWarps * 32) ssm_bwd_local_warp_kernel(const 
       cp_async_commit();
     };
     issue_tile(0);
-    issue_tile(1);
 
     // ---- per-thread constants and the carried adjoint
     const int c_own = d_w + lane;
@@ -222,9 +225,9 @@ __global__ void __launch_bounds__(kLWarps * 32) ssm_bwd_local_warp_kernel(const 
     };
 
     for (int i = 0; i < ntiles; ++i) {
-      cp_async_wait_but_one();
+      cp_async_wait_all();
       __syncwarp();             // tile i landed for all lanes; all lanes are done with tile i - 1
-      issue_tile(i + 2);        // into the stage tile i - 1 used
+      issue_tile(i + 1);        // into the stage tile i - 1 used
       const int st = i % kLStages;
       const int t0 = t_seg0 + (tile_hi - i) * kLT;
       {
@@ -266,17 +269,12 @@ __global__ void __launch_bounds__(kLWarps * 32) ssm_bwd_local_warp_kernel(const 
       __stcg(hb + 4, make_float4(dsum, 0.f, 0.f, 0.f));
       publish_handoff(sc, worker, lane);
     } else if (valid) {
-      const size_t sg = (size_t)b * p.nseg + seg;
-      // (as inflow: what leaves segment 1 enters segment 0, and nothing enters segment 1)
-      const size_t so = p.local_as_inflow ? sg - 1 : sg;
+      const size_t sg = (size_t)b * p.nseg * split + seg;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        *reinterpret_cast<float4*>(p.seg_local + (so * D + c_own) * 16 + 4 * k) =
+      for (int k = 0; k < 4; ++k)
+        *reinterpret_cast<float4*>(p.seg_local + (sg * D + c_own) * 16 + 4 * k) =
             make_float4(mu[2 * k].x, mu[2 * k].y, mu[2 * k + 1].x, mu[2 * k + 1].y);
-        if (p.local_as_inflow)
-          *reinterpret_cast<float4*>(p.seg_local + (sg * D + c_own) * 16 + 4 * k) = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-      if (!p.local_as_inflow) p.seg_dsum[sg * D + c_own] = dsum;
+      p.seg_dsum[sg * D + c_own] = dsum;
     }
   }
 }
@@ -284,7 +282,7 @@ __global__ void __launch_bounds__(kLWarps * 32) ssm_bwd_local_warp_kernel(const 
 bool bwd_local_fast_applicable(const ssm_problem_t& prob, const BwdParams& p) {
   auto al16 = [](const void* q) { return q == nullptr || (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
   return prob.io_dtype == SSM_BF16 && prob.N == 16 && prob.D % 8 == 0 && p.seg_steps % kLT == 0 && al16(p.delta) &&
-         al16(p.z) && al16(p.dout) && al16(p.C) && al16(p.A) && al16(p.seg_local) && al16(p.handoff);
+         al16(p.z) && al16(p.dout) && al16(p.C) && al16(p.A) && al16(p.seg_local) && al16(p.handoff) && p.local_steps % kLT == 0;
 }
 
 namespace {
@@ -297,8 +295,8 @@ cudaError_t launch_local(const Plan& plan, const BwdParams& p, cudaStream_t s) {
   cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), kLWarps * 32, smem, &lim);
   if (e != cudaSuccess) return e;
   WarpSched sc{};
-  sc.chains = p.batch * (plan.nseg - 1) * ((p.D + 31) / 32);
-  sc.tiles = (plan.seg_steps + kLT - 1) / kLT;
+  sc.chains = p.batch * (plan.nseg - 1) * p.local_split * ((p.D + 31) / 32);
+  sc.tiles = (p.local_steps + kLT - 1) / kLT;
   const bool can_share = p.abort != nullptr && p.flags != nullptr && p.handoff != nullptr && p.max_workers > 0;
   sc.workers = warp_workers(sc.chains, lim.sms, lim.per_sm * kLWarps, can_share ? p.max_workers : 0);
   const long long total = (long long)sc.chains * sc.tiles;

@@ -704,7 +704,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
         for (int k = 0; k < S / 4; ++k) {
           float4 m4 = make_float4(0.f, 0.f, 0.f, 0.f);
           if (valid && p.mu_in != nullptr)
-            m4 = *reinterpret_cast<const float4*>(p.mu_in + (((size_t)b * p.nseg + seg) * D + chan(q)) * 16 + S * j + 4 * k);
+            m4 = *reinterpret_cast<const float4*>(p.mu_in + ((((size_t)b * p.nseg + seg + 1) * p.local_split - 1) * D + chan(q)) * 16 + S * j + 4 * k);
           cr.mu[q][2 * k] = make_float2(m4.x, m4.y);
           cr.mu[q][2 * k + 1] = make_float2(m4.z, m4.w);
           cr.dA[q][2 * k] = cr.dA[q][2 * k + 1] = make_float2(0.f, 0.f);

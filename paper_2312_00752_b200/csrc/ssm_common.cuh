@@ -120,11 +120,11 @@ struct BwdParams {
   const void* dout;
   const float* ckpt;      // checkpoint states (layout: ckpt_offset below)
   int ckpt_tiled;         // 1: the tiled layout
-  const float* mu_in;     // [batch][nseg][D][N] adjoint inflow of each segment; null: zero
+  const float* mu_in;     // [batch][nseg * local_split][D][N] adjoint inflow of each piece of a segment; null: zero
   float* seg_local;       // LOCAL mode: [batch][nseg][D][N] adjoint leaving each segment with zero inflow
-  int local_as_inflow;    // tuned LOCAL kernel, two segments, no outside adjoint: write the result of segment 1 as the
-                          // inflow of segment 0 and zero as the inflow of segment 1 (the layout of mu_in), so that the
-                          // carry scan over two segments is not needed
+  int local_split, local_steps;  // tuned kernels: pieces a segment is cut into for the adjoint pre-pass, their length (a
+                          // multiple of a tile; the last may be shorter); the arrays of per-segment values have one
+                          // entry per piece, and the inflow of a segment is that of its last piece
   float* seg_dsum;        // LOCAL mode: [batch][nseg][D]
   void* dx;
   void* ddelta;
