@@ -749,12 +749,14 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
 
-  // the status word, and the hand-off flags of the tuned kernels (the lane kernel clears the status word itself)
-  bool clear = true;
-#ifndef SSM_DEBUG_BOUNDS
-  clear = !lane_bwd(*p);
+  // The status word, and the hand-off flags of the tuned kernels.  The lane kernel zeroes the word itself, which saves a
+  // memset, but only where nothing runs before it that reads or raises the word: a rebuild of the checkpoints may run the
+  // tuned forward, whose waits give up at once when they find the word set, and whose time-out must not be erased.
+  bool lane_clears = lane_bwd(*p) && saved_states != nullptr;
+#ifdef SSM_DEBUG_BOUNDS
+  lane_clears = false;   // (any kernel may raise it)
 #endif
-  if (clear && cudaMemsetAsync(ws, 0, w.flags + (size_t)2 * (w.max_workers + 1) * sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
+  if (!lane_clears && cudaMemsetAsync(ws, 0, w.flags + (size_t)2 * (w.max_workers + 1) * sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
   // checkpoint states: the caller's, or rebuilt here with one more forward sweep
   const float* ckpt = static_cast<const float*>(saved_states);
   if (ckpt == nullptr) {
@@ -826,6 +828,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   bp.mu_in = dh_last;  // one segment: [batch][1][D][N] is the layout of the caller's adjoint
   bp.dbias_part = ddelta_bias != nullptr ? reinterpret_cast<float*>(ws + w.dbias_part) : nullptr;
   bp.abort = reinterpret_cast<int*>(ws);
+  bp.clear_abort = lane_clears ? 1 : 0;
   bp.flags = reinterpret_cast<int*>(ws + w.flags);
   bp.handoff = reinterpret_cast<float4*>(ws + w.handoff);
   bp.max_workers = w.max_workers;

@@ -230,7 +230,9 @@ cudaError_t complex_bwd(const ssm_problem_t& prob, const void* x, const void* de
   p.groups = pl.bwd_groups;
   p.seg_local = reinterpret_cast<float*>(ws + w.seg_local);
   p.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum);
+  p.clear_abort = 1;   // (the rebuild above is a lane kernel too: it neither reads nor raises the word)
 #ifdef SSM_DEBUG_BOUNDS
+  p.clear_abort = 0;   // (any kernel may raise it)
   if ((e = cudaMemsetAsync(ws, 0, 256, s)) != cudaSuccess) return e;
 #endif
   if (pl.nseg > 1 && (e = launch_bwd_lane(prob, pl, p, kBwdLocal, s)) != cudaSuccess) return e;
