@@ -83,6 +83,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   const bool split = W * CL > 1;
   const bool bvec = (reinterpret_cast<uintptr_t>(p.B) & (4 * sizeof(IO) - 1)) == 0;
   const bool cvec = (reinterpret_cast<uintptr_t>(p.C) & (4 * sizeof(IO) - 1)) == 0;
+  // (the caller's buffer has any float's alignment; off the 16-byte grid the launch takes the variant without VEC)
+  const bool ck_vec = VEC || (reinterpret_cast<uintptr_t>(p.ckpt) & 15) == 0;
   const bool has_z = full && gz != nullptr;
   const int cols = min(32, D - grp * 32);
   const int NC = lane_ckpt_rows<CPLX>(N);
@@ -221,9 +223,19 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
             if (NC >= 4) {   // (lanes past the last channel fill the padding of the tiled layout)
               float* dst = p.ckpt + ckpt_offset(1, b, p.nck, kc, D, NC, c_own, 16 * g);
 #pragma unroll
-              for (int k = 0; k < 4; ++k)
-                if (16 * g + 4 * k < NC)
-                  *reinterpret_cast<float4*>(dst + 128 * k) = make_float4(h[2 * k].x, h[2 * k].y, h[2 * k + 1].x, h[2 * k + 1].y);
+              for (int k = 0; k < 4; ++k) {
+                if (16 * g + 4 * k < NC) {
+                  const float4 q = make_float4(h[2 * k].x, h[2 * k].y, h[2 * k + 1].x, h[2 * k + 1].y);
+                  if (ck_vec) {
+                    *reinterpret_cast<float4*>(dst + 128 * k) = q;
+                  } else {
+                    dst[128 * k] = q.x;
+                    dst[128 * k + 1] = q.y;
+                    dst[128 * k + 2] = q.z;
+                    dst[128 * k + 3] = q.w;
+                  }
+                }
+              }
             } else if (valid) {
               float* dst = p.ckpt + ckpt_offset(0, b, p.nck, kc, D, N, c_own, 0);
               dst[0] = h[0].x;
@@ -493,9 +505,10 @@ cudaError_t launch_fwd_lane_n(const Plan& plan, const FwdParams& p, int N, int m
 
 template <typename IO, int NG, bool CPLX>
 cudaError_t launch_fwd_lane_vec(const Plan& plan, const FwdParams& p, int N, int mode, cudaStream_t s) {
-  // 16-byte row pieces need aligned rows and at least one whole vector of channels
+  // 16-byte row pieces need aligned rows and at least one whole vector of channels; checkpoints that are not aligned go
+  // with rows that are not, so that the common variant carries no test (it cost 1 % at bf16 (1, 2048, 5120), N = 64)
   bool vec = (size_t)p.D * sizeof(IO) % 16 == 0;
-  for (const void* q : {p.x, p.delta, p.z, (const void*)p.out}) vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
+  for (const void* q : {p.x, p.delta, p.z, (const void*)p.out, (const void*)p.ckpt}) vec = vec && (reinterpret_cast<uintptr_t>(q) & 15) == 0;
   return vec ? launch_fwd_lane_n<IO, NG, true, CPLX>(plan, p, N, mode, s) : launch_fwd_lane_n<IO, NG, false, CPLX>(plan, p, N, mode, s);
 }
 
