@@ -749,14 +749,14 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   char* ws = static_cast<char*>(workspace);
 
-  // The status word, and the hand-off flags of the tuned kernels.  The lane kernel zeroes the word itself, which saves a
-  // memset, but only where nothing runs before it that reads or raises the word: a rebuild of the checkpoints may run the
-  // tuned forward, whose waits give up at once when they find the word set, and whose time-out must not be erased.
-  bool lane_clears = lane_bwd(*p) && saved_states != nullptr;
+  // The status word, and the hand-off flags of the tuned kernels.  On the lane kernels the reduction behind them zeroes the
+  // word, which saves a memset, but only where no kernel of the call reads or raises it: a rebuild of the checkpoints may
+  // run the tuned forward, whose waits give up at once when they find the word set, and whose time-out must not be erased.
+  bool clear_late = lane_bwd(*p) && saved_states != nullptr;
 #ifdef SSM_DEBUG_BOUNDS
-  lane_clears = false;   // (any kernel may raise it)
+  clear_late = false;   // (any kernel may raise it)
 #endif
-  if (!lane_clears && cudaMemsetAsync(ws, 0, w.flags + (size_t)2 * (w.max_workers + 1) * sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
+  if (!clear_late && cudaMemsetAsync(ws, 0, w.flags + (size_t)2 * (w.max_workers + 1) * sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
   // checkpoint states: the caller's, or rebuilt here with one more forward sweep
   const float* ckpt = static_cast<const float*>(saved_states);
   if (ckpt == nullptr) {
@@ -828,7 +828,6 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   bp.mu_in = dh_last;  // one segment: [batch][1][D][N] is the layout of the caller's adjoint
   bp.dbias_part = ddelta_bias != nullptr ? reinterpret_cast<float*>(ws + w.dbias_part) : nullptr;
   bp.abort = reinterpret_cast<int*>(ws);
-  bp.clear_abort = lane_clears ? 1 : 0;
   bp.flags = reinterpret_cast<int*>(ws + w.flags);
   bp.handoff = reinterpret_cast<float4*>(ws + w.handoff);
   bp.max_workers = w.max_workers;
@@ -888,6 +887,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   rp.parts = p->batch * pl.nseg * pl.split.cluster;
   rp.D = p->D;
   rp.N = p->N;
+  rp.clear = clear_late ? bp.abort : nullptr;
   if (launch_bwd_reduce(*p, rp, s) != cudaSuccess) return SSM_ERR_CUDA;
   return SSM_OK;
 }

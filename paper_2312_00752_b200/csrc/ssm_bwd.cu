@@ -422,6 +422,7 @@ __global__ void __launch_bounds__(kRedLanes * kRedSlices) ssm_bwd_reduce_kernel(
   }
   const long long i = (long long)(blockIdx.x - bc_blocks) * blockDim.x + threadIdx.x;
   const long long dn = (long long)p.D * p.N;
+  if (i == 0 && p.clear != nullptr) *p.clear = 0;
   auto sum = [&](const float* __restrict__ part, long long n) {
     float v = 0.f;
     for (int q = 0; q < p.parts; q += kRedBatch) {

@@ -631,7 +631,6 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   const bool cvec = N >= 4 && (reinterpret_cast<uintptr_t>(p.C) & (4 * sizeof(IO) - 1)) == 0;
   const size_t row_b = (size_t)b * p.L;
   const int t_last = live_piece ? t_begin + (t_end - t_begin - 1) / kLB * kLB : t_begin;   // first step of the last block
-  if (p.clear_abort && blockIdx.x == 0 && threadIdx.x == 0) *p.abort = 0;   // (nothing here can give up)
   auto team_sync = [&] {
     if constexpr (NG == 1) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * NG) : "memory");

@@ -145,7 +145,6 @@ struct BwdParams {
   float* dCs_part;        // static C: same for dC
   int test_withhold;      // test hook: never publish hand-off flags, poll only 1000 times
   int* abort;             // status word of the workspace (non-zero: a bounded wait gave up)
-  int clear_abort;        // lane kernel: 1: it zeroes the status word (nothing before it in the call reads or raises it)
   int* flags;             // tuned kernel: [max_workers + 1] hand-off flags, zero before the launch
   float4* handoff;        // tuned kernel: carried values of a chain that two workers share
   int max_workers;        // tuned kernel: workers the hand-off slots allow (0: no chain may be shared)
@@ -167,6 +166,7 @@ struct ReduceParams {
   const float* dCs_part;
   float* dBs;             // static B: float32 [D][N] (then dB above is null)
   float* dCs;
+  int* clear;             // status word to zero, of a call none of whose kernels reads or raises it; null: none
 };
 
 // SMs of the current device and blocks of a kernel that fit one of them, with `smem` bytes of dynamic shared memory, which

@@ -230,10 +230,8 @@ cudaError_t complex_bwd(const ssm_problem_t& prob, const void* x, const void* de
   p.groups = pl.bwd_groups;
   p.seg_local = reinterpret_cast<float*>(ws + w.seg_local);
   p.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum);
-  p.clear_abort = 1;   // (the rebuild above is a lane kernel too: it neither reads nor raises the word)
 #ifdef SSM_DEBUG_BOUNDS
-  p.clear_abort = 0;   // (any kernel may raise it)
-  if ((e = cudaMemsetAsync(ws, 0, 256, s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(ws, 0, 256, s)) != cudaSuccess) return e;   // (any kernel may raise the status word)
 #endif
   if (pl.nseg > 1 && (e = launch_bwd_lane(prob, pl, p, kBwdLocal, s)) != cudaSuccess) return e;
   if ((e = launch_bwd_lane(prob, pl, p, kBwdFull, s)) != cudaSuccess) return e;
@@ -251,6 +249,9 @@ cudaError_t complex_bwd(const ssm_problem_t& prob, const void* x, const void* de
   rp.parts = prob.batch * pl.nseg * pl.split.cluster;
   rp.D = prob.D;
   rp.N = prob.N * 2;
+#ifndef SSM_DEBUG_BOUNDS
+  rp.clear = p.abort;   // (no kernel of this path reads or raises the word)
+#endif
   return launch_bwd_reduce(prob, rp, s);
 }
 
