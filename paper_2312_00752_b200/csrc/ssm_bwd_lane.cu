@@ -182,7 +182,7 @@ __device__ __forceinline__ float lane_dot_a(const float2 (&w)[4], const float2 (
   // part: the sum over pairs 0, 1 (real parts) on entry
   if constexpr (CPLX) {
     const float2 im = f2fma(w[3], A2[3], f2mul(w[2], A2[2]));
-    return fmaf(im.x + im.y, kTurn / kLn2, part.x + part.y);
+    return fmaf(im.x + im.y, 1.f / kLn2, part.x + part.y);
   } else {
     const float2 all = f2fma(w[3], A2[3], f2fma(w[2], A2[2], part));
     return all.x + all.y;
@@ -420,6 +420,7 @@ __device__ __forceinline__ void adjoint_sweep(const BwdParams& p, int N, int gi,
   auto run = [&](auto ap_tag) {
     constexpr bool AP = decltype(ap_tag)::value;
     int buf = 0;
+    float dlost = 0.f;
 #pragma unroll 1
     for (int t0 = t_last; t0 >= t_begin; t0 -= kLB, buf ^= 1) {
       float* const tb = tiles + buf * 1024;
@@ -457,8 +458,7 @@ __device__ __forceinline__ void adjoint_sweep(const BwdParams& p, int N, int gi,
           ds[t] = t < t_end - t0 ? ds[t] : 0.f;
         }
       }
-#pragma unroll
-      for (int t = 0; t < kLB; ++t) dsum += dt[t];
+      add_steps<CPLX>(dt, dsum, dlost);
       // decays and C ds of a step are prepared one step ahead of the recurrence that consumes them
       float2 aN[2][8], cN[2][8];
       auto front = [&](int t, float2 (&a)[8], float2 (&cd)[8]) {

@@ -41,16 +41,10 @@ struct CplxStepParams {
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
-// exp(dt * A) for A = (re, im)
+// exp(dt A) for A = (re, im), as in the scan (cexp_pair)
 __device__ __forceinline__ float2 cexp_step(float dt, float2 A) {
-  const float mag = ex2_approx(dt * A.x * kLog2e);
-  const float ang = dt * A.y;
-  const float k = rintf(ang * 0.15915494309189535f);
-  float r = fmaf(-k, 6.2831854820251465f, ang);     // 2 pi split in two floats
-  r = fmaf(-k, -1.7484555e-7f, r);
-  float sn, cs;
-  __sincosf(r, &sn, &cs);
-  return make_float2(mag * cs, mag * sn);
+  const float mag = ex2_approx(dt * (A.x * kLog2e)), r = reduce_angle(dt, A.y);
+  return make_float2(mag * __cosf(r), mag * __sinf(r));
 }
 
 template <typename IO>

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   const float bias = p.delta_bias != nullptr ? p.delta_bias[c_ld] : 0.f;
   const float Dk = (full && p.Dskip != nullptr) ? p.Dskip[c_ld] : 0.f;
   const float gate_off = has_z ? 0.f : 1.f;
-  float dsum = 0.f;
+  float dsum = 0.f, dlost = 0.f;
 
   auto load_h = [&](int g) {
 #pragma unroll
@@ -209,10 +209,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
         for (int t = 0; t < kLB; ++t) dt[t] = t < live ? dt[t] : 0.f;
       }
-      if (!READ) {
-#pragma unroll
-        for (int t = 0; t < kLB; ++t) dsum += dt[t];
-      }
+      if constexpr (!READ) add_steps<CPLX>(dt, dsum, dlost);
 
 #pragma unroll 1
       for (int g = 0; g < NG; ++g) {

@@ -211,11 +211,10 @@ __device__ __forceinline__ int lane_col(int n) {
 // rows (and columns) of a channel's checkpoint
 template <bool CPLX>
 __host__ __device__ __forceinline__ int lane_ckpt_rows(int N) { return CPLX && N < 8 ? 8 : N; }
-constexpr float kTurn = 6.2831853071795865f;   // 2 pi
-constexpr float kInvTurn = 0.15915494309189534f;
-// what a row of A is multiplied with when it is staged: real parts for ex2, imaginary parts in turns
+// what a row of A is multiplied with when it is staged: real parts for ex2, imaginary parts stay in radians (scaled to turns
+// they would carry a rounding of their own, the same in every step of a channel)
 template <bool CPLX>
-__device__ __forceinline__ float lane_a_scale(int n) { return CPLX && (n & 4) ? kInvTurn : kLog2e; }
+__device__ __forceinline__ float lane_a_scale(int n) { return CPLX && (n & 4) ? 1.f : kLog2e; }
 // Four columns of B or C (quad v of a batch of rows of 16 NG) into the staged rows; im_sign: of imaginary parts
 template <bool CPLX>
 __device__ __forceinline__ void put_quad(float* rows, int v, float4 q, float im_sign) {
@@ -229,14 +228,22 @@ __device__ __forceinline__ void put_quad(float* rows, int v, float4 q, float im_
   }
 }
 
-// exp(dt A) for a pair of complex states: magnitude by ex2, phase by sin and cos of the angle reduced to half a turn (the
-// reduction is one multiply-add of the unrounded product)
+// Angles are reduced to half a turn the way of Cody and Waite: k whole turns off the unrounded product dt Im A, 2 pi as the
+// sum of a number of 8 bits (so that k times it is exact up to k = 2^16) and a rest.
+constexpr float kInvTurn = 0.15915494309189534f, kTurnHi = 6.28125f, kTurnLo = 0.0019353071795864769f;
+__device__ __forceinline__ float reduce_angle(float s, float aim) {
+  const float k = rintf(s * aim * kInvTurn);
+  return fmaf(k, -kTurnLo, fmaf(s, aim, k * -kTurnHi));
+}
+// exp(dt A) for a pair of complex states: magnitude by ex2, phase by sin and cos of the reduced angle.  (Six packed operations
+// for the reduction.  With Im A staged in turns, which takes six as well, the state of float32 (8, 512, 2400), N = 8, Re A = 0
+// turned by 560 rad was off by 7.0e-5, against 6.3e-5 this way and with each product rounded.)
 __device__ __forceinline__ void cexp_pair(float dt, float2 are, float2 aim, float2& ar, float2& ai) {
-  const float2 e = f2mul(f2dup(dt), are);
+  const float2 d = f2dup(dt), e = f2mul(d, are);
   const float2 m = make_float2(ex2_approx(e.x), ex2_approx(e.y));
   constexpr float kRound = 12582912.f;   // 1.5 * 2^23: adding it rounds to a whole number
-  const float2 k = __fadd2_rn(__fadd2_rn(f2mul(f2dup(dt), aim), f2dup(kRound)), f2dup(-kRound));
-  const float2 r = f2mul(f2fma(f2dup(dt), aim, f2mul(k, f2dup(-1.f))), f2dup(kTurn));
+  const float2 k = __fadd2_rn(f2fma(f2mul(d, aim), f2dup(kInvTurn), f2dup(kRound)), f2dup(-kRound));
+  const float2 r = f2fma(k, f2dup(-kTurnLo), f2fma(d, aim, f2mul(k, f2dup(-kTurnHi))));
   ar = f2mul(m, make_float2(__cosf(r.x), __cosf(r.y)));
   ai = f2mul(m, make_float2(__sinf(r.x), __sinf(r.y)));
 }
@@ -244,9 +251,24 @@ __device__ __forceinline__ float2 f2neg(float2 v) { return make_float2(-v.x, -v.
 // (re, im) <- exp(s A) (re, im) (conjugate: exp(s conj A)), A as staged
 template <bool CONJ>
 __device__ __forceinline__ float2 cexp_apply(float s, float are, float aim, float2 v) {
-  const float m = ex2_approx(s * are), t = s * aim, r = fmaf(s, aim, -rintf(t)) * kTurn;
+  const float m = ex2_approx(s * are), r = reduce_angle(s, aim);
   const float c = m * __cosf(r), n = (CONJ ? -m : m) * __sinf(r);
   return make_float2(fmaf(c, v.x, -n * v.y), fmaf(c, v.y, n * v.x));
+}
+
+// sum += the step sizes of a batch.  Complex: the sum turns the state of a whole piece at once, so its rounding counts as
+// often as the piece has radians; it is kept to one rounding by Kahan's compensation (`lost`: what the last addition dropped).
+template <bool CPLX>
+__device__ __forceinline__ void add_steps(const float (&dt)[kLB], float& sum, float& lost) {
+  if constexpr (CPLX) {
+    const float batch = ((dt[0] + dt[1]) + (dt[2] + dt[3])) + ((dt[4] + dt[5]) + (dt[6] + dt[7]));
+    const float y = batch - lost, t = sum + y;
+    lost = (t - sum) - y;
+    sum = t;
+  } else {
+#pragma unroll
+    for (int t = 0; t < kLB; ++t) sum += dt[t];
+  }
 }
 
 // 16 floats of a shared-memory row as packed pairs

@@ -164,3 +164,35 @@ def test_options_that_do_not_combine_are_refused():
     args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
     with pytest.raises(K.SsmScanError):
         K.ssm_scan_fwd(*args, zoh=True, complex_state=True)
+
+
+@pytest.mark.parametrize("batch,L,D,im,split", [
+    (8, 512, 2400, 5000.0, False),   # 600 chains: the forward does not split time; a step turns the state up to 90 times
+    (1, 2048, 64, 50.0, True),       # two chains of 32 pieces of 64 steps: the fold turns it by whole pieces
+])
+def test_the_phase_of_an_undamped_state(batch, L, D, im, split):
+    """Re A = 0, no input: h_last = exp(A sum delta) h0 and dh0 = exp(conj(A) sum delta) dh_last.  A step is off by the
+    sine's and cosine's absolute error, at most 2^-21.2 each (CUDA's table of intrinsics, angles within half a turn), hence
+    sqrt(2) times that and the number of steps if the errors all had one sign; where time is split, a state goes through
+    the steps of one piece and then through sums of step sizes, each rounded once, which counts 2^-25 with the radians
+    that the sum stands for.  No rounding of A or of a product delta A may come on top: in the first case the state turns
+    by some 1e5 rad, so that 2^-25 of those would be 3e-3."""
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    g = torch.Generator("cuda").manual_seed(3)
+    n = lambda *s: torch.randn(*s, generator=g, device="cuda")
+    u = lambda *s: torch.rand(*s, generator=g, device="cuda")
+    x = torch.zeros(batch, L, D, device="cuda")
+    delta = (u(D) * np.log(10.0) + np.log(0.01)).exp() * (1 + 0.2 * u(batch, L, D))
+    A = torch.stack((torch.zeros(D, 8, device="cuda"), im * u(D, 8)), -1).contiguous()
+    B, C, h0, dh = n(batch, L, 8, 2), n(batch, L, 8, 2), n(batch, D, 8, 2), n(batch, D, 8, 2)
+    h_last = torch.empty_like(h0)
+    K.ssm_scan_fwd(x, delta, A, B, C, complex_state=True, h0=h0, h_last=h_last)
+    dh0 = K.ssm_scan_bwd(x, delta, A, B, C, None, None, x, None, complex_state=True, h0=h0, dh_last=dh, want_dh0=True)["dh0"]
+    angle = A[..., 1].double() * delta.double().sum(1)[:, :, None]
+    turn = torch.polar(torch.ones_like(angle), angle)
+    c = lambda v: torch.view_as_complex(v.double())
+    err = lambda v, ref: float((c(v) - ref).norm() / ref.norm())
+    step, sums = 2 ** 0.5 * 2 ** -21.2, float(angle.pow(2).mean().sqrt()) * 2 ** -25
+    assert err(h_last, turn * c(h0)) <= (64 * step + sums if split else L * step)
+    assert err(dh0, turn.conj() * c(dh)) <= (64 if split else L) * step + sums
