@@ -8,6 +8,7 @@
 #include <dlfcn.h>
 
 #include <map>
+#include <mutex>
 #include <string>
 #include <utility>
 
@@ -107,15 +108,27 @@ void* stream_of(PyObject* stream, const at::Tensor& x) {
   return s;
 }
 
-// Grow-only scratch buffer per (device, stream): calls on different streams never share scratch memory.  (Guarded by the
-// interpreter lock; never destroyed, because the allocator may be gone by the time statics are.)
-std::map<std::pair<int, void*>, at::Tensor>& workspaces() {
-  static auto* m = new std::map<std::pair<int, void*>, at::Tensor>();
+// Scratch of one (device, stream): a buffer that only grows (calls on different streams never share scratch memory), and a lock
+// that a call on it holds while it enqueues.  A call is several launches that hand results to each other through the buffer,
+// and the interpreter lock is not held meanwhile: without this one the launches of two threads on one stream would mix.
+// (The table is guarded by the interpreter lock; never destroyed, because the allocator may be gone by the time statics are.)
+struct Scratch {
+  at::Tensor buffer;
+  std::mutex enqueue;
+};
+std::map<std::pair<int, void*>, Scratch>& workspaces() {
+  static auto* m = new std::map<std::pair<int, void*>, Scratch>();
   return *m;
 }
-at::Tensor workspace(size_t bytes, const at::Tensor& x, void* stream) {
+// What a call uses of it: a reference to the buffer of its own (another thread may put a larger one in its place), and the lock.
+struct Workspace {
+  at::Tensor buffer;
+  std::mutex* enqueue = nullptr;
+};
+Workspace workspace(size_t bytes, const at::Tensor& x, void* stream) {
   if (bytes == 0) return {};
-  at::Tensor& ws = workspaces()[{x.device().index(), stream}];
+  Scratch& scratch = workspaces()[{x.device().index(), stream}];
+  at::Tensor& ws = scratch.buffer;
   if (!ws.defined() || (size_t)ws.numel() < bytes) {
     if (ws.defined()) {
       // kernels already enqueued on that stream may still use the old buffer: the caching allocator must not hand its
@@ -125,14 +138,20 @@ at::Tensor workspace(size_t bytes, const at::Tensor& x, void* stream) {
     }
     ws = empty({(int64_t)bytes}, at::kByte, x);
   }
-  return ws;   // (a reference of the caller's own: another thread may put a larger one in its place)
+  return {ws, &scratch.enqueue};
 }
 
 // Calls a function of the library with the interpreter lock released (a full launch queue blocks), raises its error.
+// `enqueue`: the lock of the scratch the call works in, if it does; taken without the interpreter lock, so that a thread
+// that waits for the one never holds the other.
 template <typename F>
-void call(const char* what, F&& f) {
+void call(const char* what, std::mutex* enqueue, F&& f) {
   PyThreadState* const t = PyEval_SaveThread();
-  const ssm_status_t st = f();
+  ssm_status_t st;
+  {
+    const auto hold = enqueue != nullptr ? std::unique_lock<std::mutex>(*enqueue) : std::unique_lock<std::mutex>();
+    st = f();
+  }
   PyEval_RestoreThread(t);
   if (st != SSM_OK) raise(std::string(what) + ": " + api.ssm_status_string(st));
 }
@@ -231,9 +250,9 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor saved;
     if (save) saved = sgiven != nullptr ? *sgiven : empty({(int64_t)(api.ssm_scan_saved_state_bytes(&pr.p) / 4)}, at::kFloat, x);
     const at::Tensor* ws = tensor(a[12], "workspace");
-    at::Tensor own;
+    Workspace own;
     if (ws == nullptr && entry != 2) own = workspace(api.ssm_scan_fwd_workspace_bytes(&pr.p), x, stream);
-    if (own.defined()) ws = &own;
+    if (own.buffer.defined()) ws = &own.buffer;
     void* wp = pointer(ws, "workspace");
     const size_t wbytes = ws == nullptr ? 0 : (size_t)ws->numel() * ws->element_size();
     void* px = pointer(&x, "x", pr.rows, pr.io);
@@ -248,16 +267,16 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     auto* pl = static_cast<float*>(pointer(a[10], "h_last", pr.h, at::kFloat));
     void* ps = save ? pointer(&saved, "saved_states") : nullptr;
     if (entry == 2) {
-      call("ssm_scan_fwd_static", [&] {
+      call("ssm_scan_fwd_static", nullptr, [&] {
         return api.ssm_scan_fwd_static(&pr.p, px, pd, pA, pB, pC, pD, pz, po, ps, stream);
       });
     } else if (entry == 1) {
       auto* pb = static_cast<float*>(pointer(a[2], "delta_bias", {D}, at::kFloat));
-      call("ssm_scan_fwd_fused_dt", [&] {
+      call("ssm_scan_fwd_fused_dt", own.enqueue, [&] {
         return api.ssm_scan_fwd_fused_dt(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, ph, po, pl, ps, wp, wbytes, stream);
       });
     } else {
-      call("ssm_scan_fwd_state", [&] {
+      call("ssm_scan_fwd_state", own.enqueue, [&] {
         return api.ssm_scan_fwd_state(&pr.p, px, pd, pA, pB, pC, pD, pz, ph, po, pl, ps, wp, wbytes, stream);
       });
     }
@@ -308,9 +327,9 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     PyObject* o = a[14];
     void* stream = stream_of(a[13], x);
     const at::Tensor* ws = tensor(a[12], "workspace");
-    at::Tensor own;
+    Workspace own;
     if (ws == nullptr) own = workspace(api.ssm_scan_bwd_workspace_bytes(&pr.p), x, stream);
-    if (own.defined()) ws = &own;
+    if (own.buffer.defined()) ws = &own.buffer;
     void* wp = pointer(ws, "workspace");
     const size_t wbytes = ws == nullptr ? 0 : (size_t)ws->numel() * ws->element_size();
     void* px = pointer(&x, "x", pr.rows, pr.io);
@@ -338,22 +357,22 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (fused) {
       auto* pb = static_cast<float*>(pointer(a[2], "delta_bias", {D}, at::kFloat));
       if (state)
-        call("ssm_scan_bwd_fused_dt_state", [&] {
+        call("ssm_scan_bwd_fused_dt_state", own.enqueue, [&] {
         return api.ssm_scan_bwd_fused_dt_state(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, pg, ph, pm, ps, data(dx), data(dd), fdata(dbias),
         fdata(dA), data(dB), data(dC), fdata(dD), data(dz), fdata(dh0), wp, wbytes, stream);
       });
       else
-        call("ssm_scan_bwd_fused_dt", [&] {
+        call("ssm_scan_bwd_fused_dt", own.enqueue, [&] {
         return api.ssm_scan_bwd_fused_dt(&pr.p, px, pd, pb, pA, pB, pC, pD, pz, pg, ps, data(dx), data(dd), fdata(dbias), fdata(dA),
         data(dB), data(dC), fdata(dD), data(dz), wp, wbytes, stream);
       });
     } else if (state) {
-      call("ssm_scan_bwd_state", [&] {
+      call("ssm_scan_bwd_state", own.enqueue, [&] {
         return api.ssm_scan_bwd_state(&pr.p, px, pd, pA, pB, pC, pD, pz, pg, ph, pm, ps, data(dx), data(dd), fdata(dA), data(dB), data(dC),
         fdata(dD), data(dz), fdata(dh0), wp, wbytes, stream);
       });
     } else {
-      call("ssm_scan_bwd", [&] {
+      call("ssm_scan_bwd", own.enqueue, [&] {
         return api.ssm_scan_bwd(&pr.p, px, pd, pA, pB, pC, pD, pz, pg, ps, data(dx), data(dd), fdata(dA), data(dB), data(dC), fdata(dD),
         data(dz), wp, wbytes, stream);
       });
@@ -384,7 +403,7 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor out = given != nullptr ? *given : empty(pr.rows, pr.io, x);
     void* po = pointer(&out, "out", pr.rows, pr.io);
     void* stream = stream_of(a[9], x);
-    call("ssm_step", [&] {
+    call("ssm_step", nullptr, [&] {
         return api.ssm_step(&pr.p, px, pd, pA, pB, pC, pD, pz, ph, po, stream);
       });
     return wrap(out);
@@ -417,7 +436,7 @@ PyObject* conv_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     at::Tensor y = given != nullptr ? *given : empty(x.sizes(), io, x);
     void* py = pointer(&y, "y", x.sizes(), io);
     void* stream = stream_of(a[5], x);
-    call("ssm_conv1d_fwd", [&] {
+    call("ssm_conv1d_fwd", nullptr, [&] {
         return api.ssm_conv1d_fwd(&p, px, pw, pb, pp, py, stream);
       });
     return wrap(y);
@@ -446,8 +465,9 @@ PyObject* conv_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (pb != nullptr) db = output(o, "dbias", {D}, at::kFloat, x);
     else no_output(o, "dbias");
     if (truth(a[8]) && W > 1) dp = output(o, "dx_prev", {(int64_t)p.batch, W - 1, D}, io, x);
-    const at::Tensor ws = workspace(api.ssm_conv1d_bwd_workspace_bytes(&p), x, stream);
-    call("ssm_conv1d_bwd", [&] {
+    const Workspace own = workspace(api.ssm_conv1d_bwd_workspace_bytes(&p), x, stream);
+    const at::Tensor& ws = own.buffer;
+    call("ssm_conv1d_bwd", own.enqueue, [&] {
         return api.ssm_conv1d_bwd(&p, px, pw, pb, pp, pg, dx.data_ptr(), static_cast<float*>(dw.data_ptr()),
         db.defined() ? static_cast<float*>(db.data_ptr()) : nullptr, dp.defined() ? dp.data_ptr() : nullptr,
         ws.defined() ? ws.data_ptr() : nullptr, ws.defined() ? (size_t)ws.numel() : 0, stream);
@@ -465,8 +485,8 @@ PyObject* cached_workspace(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void* s = PyLong_AsVoidPtr(a[1]);
     if (PyErr_Occurred()) throw Raised{};
     auto it = workspaces().find({dev, s});
-    if (it == workspaces().end() || !it->second.defined()) Py_RETURN_NONE;
-    return wrap(it->second);
+    if (it == workspaces().end() || !it->second.buffer.defined()) Py_RETURN_NONE;
+    return wrap(it->second.buffer);
   });
 }
 
