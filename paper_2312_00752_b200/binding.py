@@ -8,6 +8,7 @@ host buffers, go through ctypes.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 import shutil
 
@@ -172,11 +173,14 @@ def _native():
         load_library()
         if _build.marshal_is_stale() and shutil.which(os.environ.get("CXX", "g++")):
             _build.build_marshal()
-        if not os.path.exists(_build.MARSHAL_PATH):
-            raise SsmScanError(f"{_build.MARSHAL_PATH} is missing and there is no compiler to build it; there is no fallback path")
-        from . import _marshal
-        _marshal.init(_library_path, SsmScanError, torch.OutOfMemoryError)
-        _marshal_module = _marshal
+        path = _build.marshal_path()
+        if not os.path.exists(path):
+            raise SsmScanError(f"{path} is missing and there is no compiler to build it; there is no fallback path")
+        spec = importlib.util.spec_from_file_location(__package__ + "._marshal", path)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        module.init(_library_path, SsmScanError, torch.OutOfMemoryError)
+        _marshal_module = module
     return _marshal_module
 
 

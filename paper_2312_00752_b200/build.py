@@ -1,5 +1,5 @@
 """Compiles the CUDA sources in csrc/ into libssm_scan.so next to this file (sm_100a only, in-tree), and the binding's
-argument marshalling (csrc/marshal.cpp, against torch's headers) into _marshal.so."""
+argument marshalling (csrc/marshal.cpp, against torch's headers) into _marshal-<torch>-<python>.so."""
 from __future__ import annotations
 
 import glob
@@ -20,7 +20,6 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "--use_fast_math", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden", "-cudart", "static"]
 
 MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
-MARSHAL_PATH = os.path.join(_HERE, "_marshal.so")
 
 
 def sources():
@@ -73,21 +72,31 @@ if __name__ == "__main__":
     print(build_library(force=True, verbose="-v" in sys.argv))
 
 
+def marshal_path() -> str:
+    """Where the marshalling module for the torch and the interpreter in use lies.  It is C++ against torch's headers and
+    fits no other build of torch, which file dates do not show, so both are in its name."""
+    import torch
+    tag = f"torch{torch.__version__}.{(torch.version.git_version or '')[:8]}-{sysconfig.get_config_var('SOABI')}"
+    return os.path.join(_HERE, f"_marshal-{tag}.so")
+
+
 def marshal_is_stale() -> bool:
-    if not os.path.exists(MARSHAL_PATH):
+    path = marshal_path()
+    if not os.path.exists(path):
         return True
-    t = os.path.getmtime(MARSHAL_PATH)
+    t = os.path.getmtime(path)
     return any(os.path.getmtime(d) > t for d in [MARSHAL_SOURCE, *glob.glob(os.path.join(INCLUDE, "*.h"))])
 
 
 def build_marshal(force: bool = False) -> str:
     """g++ -shared of the marshalling module; returns its path.  Raises if the compiler fails."""
+    path = marshal_path()
     if not force and not marshal_is_stale():
-        return MARSHAL_PATH
+        return path
     torch_dir = importlib.util.find_spec("torch").submodule_search_locations[0]
     include = os.path.join(torch_dir, "include")
     cuda = os.path.dirname(os.path.dirname(shutil.which(os.environ.get("NVCC", "nvcc")) or "/usr/local/cuda/bin/nvcc"))
-    tmp = MARSHAL_PATH + f".tmp{os.getpid()}"
+    tmp = path + f".tmp{os.getpid()}"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I", INCLUDE,
            "-I", include, "-I", os.path.join(include, "torch", "csrc", "api", "include"),
            "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"), MARSHAL_SOURCE, "-o", tmp,
@@ -96,5 +105,5 @@ def build_marshal(force: bool = False) -> str:
     if pr.returncode != 0:
         print(pr.stdout)
         raise RuntimeError(f"{cmd[0]} failed on {MARSHAL_SOURCE}")
-    os.replace(tmp, MARSHAL_PATH)
-    return MARSHAL_PATH
+    os.replace(tmp, path)
+    return path
