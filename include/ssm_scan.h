@@ -63,8 +63,8 @@ typedef enum {
   SSM_ERR_WORKSPACE = 3,    /* workspace null / misaligned / smaller than the query reports                     */
   SSM_ERR_CUDA = 4,         /* a CUDA runtime call or a kernel launch failed                                    */
   SSM_ERR_TIMEOUT = 5,      /* a bounded device-side wait gave up (reported by ssm_scan_check_status)           */
-  SSM_ERR_BOUNDS = 6        /* bounds-checking build only: a tuned kernel computed a tile row or a global row /
-                               channel outside its range; the access was clamped or skipped, nothing faulted
+  SSM_ERR_BOUNDS = 6        /* bounds-checking build only: a tuned or lane kernel computed a tile row or a global
+                               address outside its range; the access was clamped or skipped, nothing faulted
                                (reported by ssm_scan_check_status)                                              */
 } ssm_status_t;
 
@@ -237,8 +237,9 @@ SSM_API ssm_status_t ssm_scan_bwd_state(const ssm_problem_t* p, const void* x, c
  * (the first word of every non-empty workspace) is set.  This call synchronises `stream`, copies that word to the host
  * and returns SSM_ERR_TIMEOUT if it is set (the results of that call are then incomplete), SSM_OK otherwise.  `p` and
  * `workspace` must be those of the call.  A library built with -DSSM_DEBUG_BOUNDS (the stand-in for a memory checker:
- * every tile row index and every global row / channel offset of the tuned kernels is range-checked, a bad one is
- * clamped or its access skipped, nothing traps) reports a violation here as SSM_ERR_BOUNDS.
+ * every tile row index and every global row / channel offset of the tuned kernels and the global accesses and shared
+ * memory of the lane kernels are range-checked, a bad one is clamped or its access skipped, nothing traps) reports a
+ * violation here as SSM_ERR_BOUNDS; in that build every call needs a workspace, if only for the status word.
  */
 SSM_API ssm_status_t ssm_scan_check_status(const ssm_problem_t* p, const void* workspace, void* stream /* cudaStream_t */);
 

@@ -14,7 +14,7 @@ size_t complex_bwd_workspace_bytes(const ssm_problem_t& p);
 size_t complex_saved_state_bytes(const ssm_problem_t& p);
 cudaError_t complex_fwd(const ssm_problem_t& prob, const void* x, const void* delta, const float* A, const void* B,
                         const void* C, const float* D_skip, const void* z, const float* h0, void* out, float* h_last,
-                        void* saved_states, cudaStream_t s);
+                        void* saved_states, int* status, cudaStream_t s);
 cudaError_t complex_bwd(const ssm_problem_t& prob, const void* x, const void* delta, const float* A, const void* B,
                         const void* C, const float* D_skip, const void* z, const void* dout, const float* h0,
                         const float* dh_last, const void* saved_states, void* dx, void* ddelta, float* dA, void* dB,
@@ -303,7 +303,12 @@ static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
   FwdWorkspace w{};
   const int cw = fwd_fast_channels_per_warp();
   w.max_workers = tuned_shape(p) && !lane_fwd(p) ? shared_workers((long long)p.batch * pl.nseg * ((p.D + cw - 1) / cw)) : 0;
-  if (pl.nseg == 1 && w.max_workers == 0) return w;
+  if (pl.nseg == 1 && w.max_workers == 0) {
+#ifdef SSM_DEBUG_BOUNDS
+    w.total = kStatusBytes;   // (a place for the status word)
+#endif
+    return w;
+  }
   size_t off = kStatusBytes;
   auto take = [&](size_t bytes) {
     const size_t at = off;
@@ -540,8 +545,14 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
     if (q && !aligned_to(q, 4)) return SSM_ERR_INVALID_ARG;
   if (p->flags & SSM_FLAG_COMPLEX) {
     if (delta_bias != nullptr) return SSM_ERR_UNSUPPORTED;
+    int* status = nullptr;
+#ifdef SSM_DEBUG_BOUNDS
+    if ((st = check_ws(workspace, workspace_bytes, kStatusBytes)) != SSM_OK) return st;
+    status = static_cast<int*>(workspace);
+    if (cudaMemsetAsync(status, 0, kStatusBytes, static_cast<cudaStream_t>(stream)) != cudaSuccess) return SSM_ERR_CUDA;
+#endif
     return complex_fwd(*p, x, delta, A, B, C, has_d ? D_skip : nullptr, has_z ? z : nullptr, h0, out, h_last,
-                       save ? saved_states : nullptr, static_cast<cudaStream_t>(stream)) == cudaSuccess
+                       save ? saved_states : nullptr, status, static_cast<cudaStream_t>(stream)) == cudaSuccess
                ? SSM_OK
                : SSM_ERR_CUDA;
   }

@@ -45,7 +45,7 @@ struct BwdLaneSmem {
   static constexpr int kRed = 4 * 32 * 4 * 16;
   static constexpr int kWarp = 2 * kLB * 16 * 4 + 2 * 4 * 32 * 16 + kRed + (NG > 1 ? kLB * 32 * 16 : 0);
   static constexpr int kChain = NP * 128 + 128 + kTeams * 128;
-  static constexpr int bytes(int chains) { return kTeams * kTeam + kLaneWarps * kWarp + chains * kChain + kLaneWarps * 256; }
+  static __host__ __device__ constexpr int bytes(int chains) { return kTeams * kTeam + kLaneWarps * kWarp + chains * kChain + kLaneWarps * 256; }
 };
 
 __device__ __forceinline__ void cp_async4(void* dst, const void* src, int bytes) {
@@ -94,11 +94,14 @@ struct RawRows {
       }
     }
   }
-  __device__ __forceinline__ void issue(unsigned char* tile, const IO* base, int D, int lane, int cols, int live) const {
+  __device__ __forceinline__ void issue(unsigned char* tile, const IO* base, int D, int lane, int cols, int live
+                                        SSM_DEBUG_ARGS(const IO* tensor, size_t count, int* status)) const {
     if constexpr (ROWS == kElements) {
 #pragma unroll 1
-      for (int t = 0; t < live; ++t)
+      for (int t = 0; t < live; ++t) {
+        SSM_GUARD_SPAN(base + (size_t)t * D, cols, tensor, count, status, return)
         if (lane < cols) reinterpret_cast<IO*>(tile + t * kPitch)[lane] = base[(size_t)t * D + lane];
+      }
       return;
     }
     const IO* const from = reinterpret_cast<const IO*>(reinterpret_cast<const char*>(base) - kBack);
@@ -106,6 +109,9 @@ struct RawRows {
     for (int i = 0; i < kCopies; ++i) {
       if ((int)(dst[i] >> 16) < live) {
         unsigned char* const to = tile + (dst[i] & 0xfffu);
+        SSM_GUARD((dst[i] & 0xfffu) + (VEC ? 16 : 4) <= (BwdLaneSmem<IO, 1, VEC>::kRaw), status, continue)
+        SSM_GUARD_SPAN(reinterpret_cast<const char*>(at_bytes(from, off[i])), VEC ? 16 : 4 - (int)(dst[i] >> 11 & 2u), tensor,
+                       count * sizeof(IO), status, continue)
         if constexpr (VEC) cp_async16(to, at_bytes(from, off[i]), true);
         else cp_async4(to, at_bytes(from, off[i]), 4 - (int)(dst[i] >> 11 & 2u));
       }
@@ -213,7 +219,8 @@ __device__ __forceinline__ float3 finish_step(LaneChain& lc, float4 v1, float4 v
 template <bool AP, bool CPLX, typename Emit>
 __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, const float4* t2, const float* fB, const float* fC,
                                            const float4* ck, float4* red, float* part_dB, float* part_dC, int N, int n_live,
-                                           int live, int lane, Emit&& emit) {
+                                           int live, int lane, Emit&& emit
+                                           SSM_DEBUG_ARGS(const float* parts, size_t part_count, int* status)) {
   const int j = lane & 1;
   float2 hist[kLB / 2][2][4];
   {
@@ -375,6 +382,7 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
       const int row = 2 * m + s;
       if (row < live && n0 < n_live) {
         float* dst = (which ? part_dC : part_dB) + (size_t)row * N + n0;
+        SSM_GUARD_SPAN(dst, min(n_live - n0, 4), parts, part_count, status, dst = const_cast<float*>(parts))
         if (n_live - n0 >= 4) {   // (then N is a multiple of 4)
           *reinterpret_cast<float4*>(dst) = acc;
         } else {
@@ -406,6 +414,7 @@ __device__ __forceinline__ void adjoint_sweep(const BwdParams& p, int N, int gi,
   auto fetch = [&](int t0) {
     const size_t base = (row_b + t0) * D + c0;
     const int last = t_end - 1 - t0, r = lane >> 2, n = 16 * gi + 4 * (lane & 3);
+    SSM_GUARD((lane_rows_exist<IO, VEC>((int)(row_b / p.L), p.batch, t0, last, p.L, c0, cols, D)), p.abort, return)
     rd.load(gd + base, D, lane, last, cols);
     if (has_z) rz.load(gz + base, D, lane, last, cols);
     rg.load(gg + base, D, lane, last, cols);
@@ -558,6 +567,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, sizeof(IO) == 4 ? 3 : 4) ssm_
   adjoint_sweep<IO, VEC, CPLX>(p, N, gi, (size_t)b * p.L, t_begin, t_end, grp * 32, lane, sA, ap, bias, cvec, s_tiles[bwarp], mu, dsum);
   // [batch][segment][channel group][row][32], rows as in shared memory
   const size_t at = ((size_t)b * p.nseg + seg) * groups + grp;
+  SSM_GUARD(at < (size_t)p.batch * p.nseg * groups && gi < ng, p.abort, return)
   float* const dst = p.seg_local + (at * ng + gi) * 512 + lane;
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
@@ -580,6 +590,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   const int team = bwarp / NG, gi = bwarp % NG; // gi: this warp's group of 16 states
   const int sub = div_pow2(team, W), tw = team - sub * W;      // which chain of the block, which of its pieces here
   const int per_block = div_pow2(kTeams, W);
+  SSM_GUARD(W * per_block == kTeams && SM::bytes(per_block) <= dynamic_smem_bytes() && cluster_rank() < CL, p.abort, return)
   unsigned char* const sTeam = smem + team * SM::kTeam;
   unsigned char* const rX = sTeam;
   unsigned char* const rD = rX + SM::kRaw;
@@ -644,6 +655,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   // four of the 16 states of row lane / 4 of a block of B or C; rows past the end are zero
   auto quad = [&](LaneQuad<IO>& q, const IO* src, int t0, bool vec) {
     const int r = lane >> 2, n = 16 * gi + 4 * (lane & 3);
+    SSM_GUARD(t0 + r >= t_end || n >= N || (row_b + t0 + r) * N + n + min(N - n, 4) <= (size_t)p.batch * p.L * N, p.abort, return)
     q.load(src + (row_b + t0 + r) * N + n, t0 + r < t_end ? N - n : 0, vec);
   };
   __syncthreads();
@@ -676,10 +688,10 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   auto issue_rows = [&](int t0) {
     const size_t base = (row_b + t0) * D + grp * 32;
     const int live = min(kLB, t_end - t0);
-    if (0 % NG == gi) rr.issue(rX, gx + base, D, lane, cols, live);
-    if (1 % NG == gi) rr.issue(rD, gd + base, D, lane, cols, live);
-    if (2 % NG == gi && has_z) rr.issue(rZ, gz + base, D, lane, cols, live);
-    if (3 % NG == gi) rr.issue(rG, gg + base, D, lane, cols, live);
+    if (0 % NG == gi) rr.issue(rX, gx + base, D, lane, cols, live SSM_DEBUG_ARGS(gx, (size_t)p.batch * p.L * D, p.abort));
+    if (1 % NG == gi) rr.issue(rD, gd + base, D, lane, cols, live SSM_DEBUG_ARGS(gd, (size_t)p.batch * p.L * D, p.abort));
+    if (2 % NG == gi && has_z) rr.issue(rZ, gz + base, D, lane, cols, live SSM_DEBUG_ARGS(gz, (size_t)p.batch * p.L * D, p.abort));
+    if (3 % NG == gi) rr.issue(rG, gg + base, D, lane, cols, live SSM_DEBUG_ARGS(gg, (size_t)p.batch * p.L * D, p.abort));
   };
   // the states before a block, for the lane's two channels and 8 states: vectors [2 q + k][lane]
   const bool ck_vec = p.ckpt_tiled && (reinterpret_cast<uintptr_t>(p.ckpt) & 15) == 0;
@@ -700,6 +712,10 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         float4* at = dst + (2 * q + k) * 32 + lane;
+        SSM_GUARD(!ck_bytes[q][k] || ckpt_offset(p.ckpt_tiled, b, p.nck, kc, D, NC, grp * 32 + (lane ^ q), n_own + 4 * k) + min(4, NC) <=
+                                         (size_t)p.batch * p.nck * ckpt_floats_per_step(p.ckpt_tiled, D, NC), p.abort, continue)
+        SSM_GUARD(!ck_vec || src + k * 128 + (lane ^ q) * 4 == p.ckpt + ckpt_offset(1, b, p.nck, kc, D, NC, grp * 32 + (lane ^ q), n_own + 4 * k),
+                  p.abort, continue)
         if (ck_vec) {
           cp_async16_bytes(at, ck_bytes[q][k] ? src + k * 128 + (lane ^ q) * 4 : p.ckpt, ck_bytes[q][k]);
         } else {
@@ -933,7 +949,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
                      [&](int t, float y, float lb, float wa, float4 v1, float4 v2) {
                        if constexpr (NG == 1) put(t, finish_step(lc, v1, v2, y, lb, wa, t < live));
                        else ex[t * 32 + lane] = make_float4(y, lb, wa, 0.f);
-                     });
+                     } SSM_DEBUG_ARGS(p.dBC_part, (size_t)groups * 2 * bln, p.abort));
       if constexpr (NG > 1) {
         team_sync();
 #pragma unroll
@@ -960,6 +976,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
         for (int i = 0; i < kFlush; ++i) {
           if ((int)(fl_slot[i] >> 16) < min(live, kLB)) {
             const float4* const from = t2 + (fl_slot[i] & 0xfff8u);
+            SSM_GUARD((fl_slot[i] & 0xfff8u) + 8 <= kLB * 32, p.abort, continue)
+            SSM_GUARD_SPAN(at_bytes(ox + base, fl_off[i]), R::EPV, ox, (size_t)p.batch * p.L * D, p.abort, continue)
             const int x = fl_slot[i] & 7;
             __align__(16) IO vx[R::EPV], vd[R::EPV], vz[R::EPV];
 #pragma unroll
@@ -980,6 +998,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
         for (int i = 0; i < kLB / NG; ++i, at += (unsigned)D * (unsigned)sizeof(IO)) {
           const int t = gi * (kLB / NG) + i;
           if (t >= live) break;
+          SSM_GUARD_SPAN(at_bytes(ox + base, at), 1, ox, (size_t)p.batch * p.L * D, p.abort, break)
           const float4 v = t2[t * 32 + out_slot(t, lane)];
           *at_bytes(ox + base, at) = float_to_io<IO>(v.x);
           *at_bytes(od + base, at) = float_to_io<IO>(v.y);
@@ -1025,6 +1044,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   __syncthreads();
   if (valid && chain_id < chains) {
     const size_t part = ((size_t)b * p.nseg + seg) * CL + rank;
+    SSM_GUARD(part < (size_t)p.batch * p.nseg * CL, p.abort, return)
     for (int n = tw * NG + gi; n < NP; n += W * NG) {
       const int col = lane_col<CPLX>(n);
       float v = 0.f;

@@ -232,15 +232,27 @@ enum BwdMode { kBwdFull = 0, kBwdLocal = 1 };
 #ifdef __CUDACC__
 // Bounds-checking build (-DSSM_DEBUG_BOUNDS; a memory checker is not available on the GPUs this is developed on): the
 // tuned kernels range-check every tile row index (clamped to row 0 on violation) and every global row / channel offset
-// they store to (the store is skipped), and record a violation as the value 2 in the status word of the workspace.
+// they store to (the store is skipped), the lane kernels the shared memory they were launched with and every global
+// access but those to per-channel arrays at the lane's own channel (the access is skipped); a violation is recorded as the
+// value 2 in the status word of the workspace.
 // Nothing traps or asserts, so a bad index can be found on a small case without losing the context.
+// SSM_GUARD(cond, status, act) does `act` (return, continue, ...) where cond does not hold, SSM_GUARD_SPAN where the n elements
+// from `at` are not among the `count` from `base`; SSM_DEBUG_ARGS are arguments that only these need.  All three leave
+// nothing behind in the ordinary build (a condition that is always true cost the lane backward up to 0.9 %).
 #ifdef SSM_DEBUG_BOUNDS
 #define SSM_TILE_ROW(r, limit, status) \
   (((unsigned)(r) < (unsigned)(limit)) ? (r) : (((status) != nullptr ? atomicExch((status), 2) : 0), 0))
 #define SSM_IN_RANGE(cond, status) ((cond) ? true : (((status) != nullptr ? atomicExch((status), 2) : 0), false))
+#define SSM_GUARD(cond, status, act) if (!SSM_IN_RANGE(cond, status)) act;
+#define SSM_GUARD_SPAN(at, n, base, count, status, act) \
+  SSM_GUARD((uintptr_t)(at) >= (uintptr_t)(base) && (uintptr_t)((at) + (n)) <= (uintptr_t)(base) + (count) * sizeof(*(at)), status, act)
+#define SSM_DEBUG_ARGS(...) , __VA_ARGS__
 #else
 #define SSM_TILE_ROW(r, limit, status) (r)
 #define SSM_IN_RANGE(cond, status) true
+#define SSM_GUARD(cond, status, act)
+#define SSM_GUARD_SPAN(at, n, base, count, status, act)
+#define SSM_DEBUG_ARGS(...)
 #endif
 
 __device__ __forceinline__ float ex2_approx(float v) {

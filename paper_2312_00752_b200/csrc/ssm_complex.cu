@@ -142,9 +142,10 @@ size_t complex_saved_state_bytes(const ssm_problem_t& p) {
 
 cudaError_t complex_fwd(const ssm_problem_t& prob, const void* x, const void* delta, const float* A, const void* B,
                         const void* C, const float* D_skip, const void* z, const float* h0, void* out, float* h_last,
-                        void* saved_states, cudaStream_t s) {
+                        void* saved_states, int* status, cudaStream_t s) {
   const Plan pl = cplx_fwd_plan(prob);
   FwdParams p{};
+  p.abort = status;
   p.x = x;
   p.delta = delta;
   p.z = z;
@@ -174,6 +175,9 @@ cudaError_t complex_bwd(const ssm_problem_t& prob, const void* x, const void* de
   const CplxWorkspace w = cplx_layout(prob, pl);
   char* ws = static_cast<char*>(workspace);
   cudaError_t e;
+#ifdef SSM_DEBUG_BOUNDS
+  if ((e = cudaMemsetAsync(ws, 0, 256, s)) != cudaSuccess) return e;   // (any kernel may raise the status word)
+#endif
   const float* ckpt = static_cast<const float*>(saved_states);
   if (ckpt == nullptr) {
     // rebuild the checkpoint states with one more forward sweep
@@ -186,6 +190,7 @@ cudaError_t complex_bwd(const ssm_problem_t& prob, const void* x, const void* de
     f.h_start = h0;
     f.ckpt = reinterpret_cast<float*>(ws + w.ckpt);
     f.ckpt_tiled = 1;
+    f.abort = reinterpret_cast<int*>(ws);
     f.batch = prob.batch;
     f.L = prob.L;
     f.D = prob.D;
@@ -224,9 +229,6 @@ cudaError_t complex_bwd(const ssm_problem_t& prob, const void* x, const void* de
   p.groups = pl.bwd_groups;
   p.seg_local = reinterpret_cast<float*>(ws + w.seg_local);
   p.seg_dsum = reinterpret_cast<float*>(ws + w.seg_dsum);
-#ifdef SSM_DEBUG_BOUNDS
-  if ((e = cudaMemsetAsync(ws, 0, 256, s)) != cudaSuccess) return e;   // (any kernel may raise the status word)
-#endif
   if (pl.nseg > 1 && (e = launch_bwd_lane(prob, pl, p, kBwdLocal, s)) != cudaSuccess) return e;
   if ((e = launch_bwd_lane(prob, pl, p, kBwdFull, s)) != cudaSuccess) return e;
   // the fixed-order second stage is the real path's, on rows of 2 N columns

@@ -32,7 +32,7 @@ struct FwdLaneSmem {
   static constexpr int kIO = 2 * kBuf + kTile;    // floats per warp
   static constexpr int kState = NP * 32;          // floats per warp
   static constexpr int kChain = 2 * kState + 32;  // floats per chain
-  static constexpr size_t bytes(int warps, int chains) {
+  static __host__ __device__ constexpr size_t bytes(int warps, int chains) {
     return sizeof(float) * ((size_t)warps * (kIO + kState + 32) + (size_t)chains * kChain);
   }
 };
@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   const int bwarp = uniform_warp(), lane = threadIdx.x & 31;
   const int W = sp.warps, CL = sp.cluster;
   constexpr int nwarps = kLaneWarps;
+  SSM_GUARD(W * (nwarps / W) == nwarps && SM::bytes(nwarps, nwarps / W) <= dynamic_smem_bytes() && cluster_rank() < CL, p.abort, return)
   const int sub = div_pow2(bwarp, W), warp = bwarp - sub * W;   // sub: which chain of the block
   float* const sIO = smem + (size_t)bwarp * SM::kIO;
   float* const sE = smem + (size_t)nwarps * SM::kIO + (size_t)sub * W * SM::kState;         // [W][NP][32]
@@ -97,6 +98,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   auto prefetch = [&](int t0, bool read) {
     const size_t base = (row_b + t0) * D + grp * 32, baseBC = (row_b + t0) * N;
     const int last = t_end - 1 - t0;
+    SSM_GUARD((lane_rows_exist<IO, VEC>(b, p.batch, t0, last, p.L, grp * 32, cols, D)), p.abort, return)
     rd.load(gd + base, D, lane, last, cols);
     rx.load(gx + base, D, lane, last, cols);
     if (read && has_z) rz.load(gz + base, D, lane, last, cols);
@@ -222,6 +224,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
                 if (16 * g + 4 * k < NC) {
+                  SSM_GUARD_SPAN(dst + 128 * k, 4, p.ckpt, (size_t)p.batch * p.nck * ckpt_floats_per_step(1, D, NC), p.abort, continue)
                   const float4 q = make_float4(h[2 * k].x, h[2 * k].y, h[2 * k + 1].x, h[2 * k + 1].y);
                   if (ck_vec) {
                     *reinterpret_cast<float4*>(dst + 128 * k) = q;
@@ -235,6 +238,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
               }
             } else if (valid) {
               float* dst = p.ckpt + ckpt_offset(0, b, p.nck, kc, D, N, c_own, 0);
+              SSM_GUARD_SPAN(dst, N, p.ckpt, (size_t)p.batch * p.nck * ckpt_floats_per_step(0, D, N), p.abort, return)
               dst[0] = h[0].x;
               if (N > 1) dst[1] = h[0].y;
             }
@@ -347,6 +351,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
       }
       if constexpr (READ) {
         IO* const bo = gout + (row_b + t0) * D + grp * 32;
+        SSM_GUARD_SPAN(bo + (size_t)(min(live, kLB) - 1) * D, cols, gout, (size_t)p.batch * p.L * D, p.abort, return)
 #pragma unroll
         for (int t = 0; t < kLB; ++t) {
           // without z its rows are zero: silu(0) = 0, and gate_off = 1 takes its place

@@ -159,6 +159,12 @@ struct LaneRows {
     else return LaneRaw<IO>::widen(r[t]);
   }
 };
+// (bounds-checking build) whether a batch from row t0 with `last` as in LaneRows::load, and `cols` channels from c0, exist
+template <typename IO, bool VEC>
+__device__ __forceinline__ bool lane_rows_exist(int b, int batch, int t0, int last, int L, int c0, int cols, int D) {
+  return b >= 0 && b < batch && t0 >= 0 && last >= 0 && t0 + min(last, kLB - 1) < L && c0 >= 0 &&
+         cols >= (VEC ? LaneRows<IO, VEC>::EPV : 1) && c0 + cols <= D;
+}
 // The way back: results of a batch, collected in a tile (VEC) and written with 16-byte stores, or written one by one.
 template <typename IO, bool VEC>
 struct LaneOut {
@@ -197,6 +203,11 @@ __device__ __forceinline__ int cluster_rank() {
   unsigned v;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(v));
   return (int)v;
+}
+__device__ __forceinline__ unsigned dynamic_smem_bytes() {
+  unsigned v;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(v));
+  return v;
 }
 // x / w for w = 1, 2 or 4
 __device__ __forceinline__ int div_pow2(int x, int w) { return x >> (w >> 1); }

@@ -36,6 +36,19 @@ def to_host(t) -> np.ndarray:
     return t.detach().to(torch.float32).cpu().numpy()
 
 
+def kernels(run) -> set:
+    """Names of the library's kernels that `run()` launches (the profiler's record, template arguments cut off)."""
+    import re
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
+        run()
+        torch.cuda.synchronize()
+    found = (re.search(r"\bssm_\w+_kernel\b", e.key) for e in prof.key_averages())
+    return {m.group(0) for m in found if m}
+
+
 def gpu_fwd_bwd(dev: dict, use_saved=True, general_A=False):
     """Runs the CUDA forward (+ saved states) and backward through the binding; returns host float arrays."""
     from paper_2312_00752_b200 import binding as K

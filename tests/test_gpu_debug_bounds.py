@@ -1,6 +1,7 @@
-"""The tuned kernels under the bounds-checking build of the library (-DSSM_DEBUG_BOUNDS): every tile row index and every
-global row / channel offset they store to is range-checked on the device, a violation is clamped or skipped and reported
-by ssm_scan_check_status as SSM_ERR_BOUNDS.  Nothing traps, so this is safe to run on a shared GPU; it stands in for a
+"""The tuned and the lane kernels under the bounds-checking build of the library (-DSSM_DEBUG_BOUNDS): tile row indices and
+the global rows / channels the tuned kernels store to, the global accesses and the shared memory of the lane kernels are
+range-checked on the device, a violation is clamped or skipped and reported by ssm_scan_check_status as SSM_ERR_BOUNDS.
+Nothing traps, so this is safe to run on a shared GPU; it stands in for a
 memory checker on small shapes with ragged tiles, partial channel groups and time splits."""
 import os
 import subprocess
