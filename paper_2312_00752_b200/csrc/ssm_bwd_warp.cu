@@ -4,12 +4,9 @@
 // One warp is one worker, as in the tuned forward kernel (ssm_fwd_warp.cu): it owns CW adjacent channels of one batch
 // entry, walks its part of the sequence backwards in tiles of 8 steps, stages its own tiles with cp.async and shares
 // nothing with the other warps of its block.  A thread holds S states of CPT channels as packed float2 pairs; the
-// LPC = 16 / S lanes of a group cover the 16 states of the group's channels.  With CPT = LPC (16 recurrences per thread,
-// CW = 32) local channel q of lane j (j = lane % LPC) is channel j ^ q of the group, so the sums over n are
-// reduce-scattered with xor-shuffles and every lane finishes exactly one channel per step (channel `lane`).  With
-// S = 8, CPT = 1 (8 recurrences per thread, CW = 16) the two lanes of a group share one channel, the sums are completed
-// in both, and lane j finishes the steps of parity j; this mapping needs half the registers, so twice as many warps are
-// resident, and a problem has twice as many chains to give them.
+// LPC = 16 / S = 2 lanes of a group cover the 16 states of the group's CPT = 2 channels (16 recurrences per thread,
+// CW = 32).  Local channel q of lane j (j = lane % LPC) is channel j ^ q of the group, so the sums over n are
+// reduce-scattered with xor-shuffles and every lane finishes exactly one channel per step (channel `lane`).
 //
 // Recomputation.  The forward pass left the state at the start of every block of 8 steps, so a sub-block of 8 steps is
 // rebuilt directly from its checkpoint: a forward sweep keeps the states after the odd steps in registers (64
@@ -24,7 +21,6 @@
 //
 // Schedule.  As in the forward kernel (WarpSched in ssm_common.cuh), in reverse time: a chain that two workers share
 // hands the adjoint mu and the dA / dD accumulators from one to the other once, through L2, behind a bounded wait.
-#include <cstdlib>
 #include <type_traits>
 
 #include "ssm_common.cuh"
@@ -72,52 +68,24 @@ template <int S, int CPT_>
 struct Lane {
   static constexpr int LPC = 16 / S, CPT = CPT_, H = S / 2, V = S / 2;   // V: float4 of dB / dC terms per thread and step
   static constexpr int CW = (32 / LPC) * CPT;       // channels per warp
-  static constexpr bool OWN = (CPT == LPC);          // every lane finishes its own channel (else: parity of the step)
-  static_assert(OWN || (CPT == 1 && LPC == 2), "supported mappings");
-  int lane, j, g, co;    // co: the channel (within the warp) this lane finishes
+  static_assert(LPC == 2 && CPT == 2, "the mapping: a lane pair shares 2 channels, every lane finishes its own");
+  int lane, j, g;
   uint32_t sel0, sel1;
   __device__ __forceinline__ explicit Lane(int l) : lane(l), j(l % LPC), g(l / LPC) {
-    co = OWN ? lane : g;
     sel0 = (j & 1) ? 0x3244u : 0x1044u;
     sel1 = (j & 1) ? 0x1044u : 0x3244u;
   }
   // the CPT values of a tile row (CW channels as bf16 pairs) that belong to this thread, by local channel
   __device__ __forceinline__ void unpack_row(const uint32_t* row, float (&v)[CPT]) const {
-    if constexpr (!OWN) {
-      v[0] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(row)[g] << 16);
-    } else if constexpr (CPT == 1) {
-      v[0] = __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(row)[lane] << 16);
-    } else if constexpr (CPT == 2) {
-      const uint32_t w = row[g];
-      v[0] = bf16sel(w, sel0);
-      v[1] = bf16sel(w, sel1);
-    } else {
-      const uint2 w = *reinterpret_cast<const uint2*>(row + 2 * g);
-      const uint32_t wa = (j & 2) ? w.y : w.x, wb = (j & 2) ? w.x : w.y;
-      v[0] = bf16sel(wa, sel0);
-      v[1] = bf16sel(wa, sel1);
-      v[2] = bf16sel(wb, sel0);
-      v[3] = bf16sel(wb, sel1);
-    }
+    const uint32_t w = row[g];
+    v[0] = bf16sel(w, sel0);
+    v[1] = bf16sel(w, sel1);
   }
   // the same from a row of CW floats
   __device__ __forceinline__ void pick_row(const float* row, float (&v)[CPT]) const {
-    if constexpr (!OWN) {
-      v[0] = row[g];
-    } else if constexpr (CPT == 1) {
-      v[0] = row[lane];
-    } else if constexpr (CPT == 2) {
-      const float2 f = *reinterpret_cast<const float2*>(row + 2 * g);
-      v[0] = (j & 1) ? f.y : f.x;
-      v[1] = (j & 1) ? f.x : f.y;
-    } else {
-      const float4 f = *reinterpret_cast<const float4*>(row + 4 * g);
-      const float a0 = (j & 2) ? f.z : f.x, a1 = (j & 2) ? f.w : f.y, b0 = (j & 2) ? f.x : f.z, b1 = (j & 2) ? f.y : f.w;
-      v[0] = (j & 1) ? a1 : a0;
-      v[1] = (j & 1) ? a0 : a1;
-      v[2] = (j & 1) ? b1 : b0;
-      v[3] = (j & 1) ? b0 : b1;
-    }
+    const float2 f = *reinterpret_cast<const float2*>(row + 2 * g);
+    v[0] = (j & 1) ? f.y : f.x;
+    v[1] = (j & 1) ? f.x : f.y;
   }
   // this thread's S states of a row of 16 floats
   __device__ __forceinline__ void load_states_f(const float* row, float2 (&v)[H]) const {
@@ -126,24 +94,6 @@ struct Lane {
       const float4 a = *reinterpret_cast<const float4*>(row + S * j + 4 * k);
       v[2 * k] = make_float2(a.x, a.y);
       v[2 * k + 1] = make_float2(a.z, a.w);
-    }
-  }
-  // this thread's S states of a packed B or C row (16 states as 8 bf16 pairs), widened
-  __device__ __forceinline__ void load_states(const uint32_t* row, float2 (&v)[H]) const {
-    if constexpr (H == 8) {
-      const uint4 a = *reinterpret_cast<const uint4*>(row), b = *reinterpret_cast<const uint4*>(row + 4);
-      const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = make_float2(bf16lo(w[k]), bf16hi(w[k]));
-    } else if constexpr (H == 4) {
-      const uint4 a = *reinterpret_cast<const uint4*>(row + 4 * j);
-      const uint32_t w[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-      for (int k = 0; k < 4; ++k) v[k] = make_float2(bf16lo(w[k]), bf16hi(w[k]));
-    } else {
-      const uint2 a = *reinterpret_cast<const uint2*>(row + 2 * j);
-      v[0] = make_float2(bf16lo(a.x), bf16hi(a.x));
-      v[1] = make_float2(bf16lo(a.y), bf16hi(a.y));
     }
   }
 };
@@ -204,7 +154,6 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
                                           float* part_dB, float* part_dC, int* abort_word) {
   using LN = Lane<S, CPT>;
   constexpr int LPC = LN::LPC, H = LN::H, V = LN::V, CW = LN::CW, WPR = CW / 2;
-  constexpr bool OWN = LN::OWN;
   constexpr bool SB = BC & 1, SC = BC & 2;
   const int lane = ln.lane;
   // B / C of a (step, channel, state pair): the staged row, or the channel's parameter
@@ -272,7 +221,7 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
     else ln.unpack_row(td + r1 * WPR, dt1);
     ln.unpack_row(tx + r1 * WPR, u1);
     ln.pick_row(tds + r1 * CW, ds1);
-    const float gp1 = tgp[r1 * CW + ln.co];
+    const float gp1 = tgp[r1 * CW + lane];
     float y1[CPT], lb1[CPT], mb1[ZOH ? CPT : 1];   // mb: sum mu B (ZOH: the step-size gradient through E)
     {
       float2 Bv[H], Cv[H];
@@ -324,21 +273,15 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
           rrow[(V / 2 + v) ^ swz] = make_float4(dCt[2 * v].x, dCt[2 * v].y, dCt[2 * v + 1].x, dCt[2 * v + 1].y);
       }
     }
-    if constexpr (OWN) {
 #pragma unroll
-      for (int mm = 1; mm < LPC; mm <<= 1) {
+    for (int mm = 1; mm < LPC; mm <<= 1) {
 #pragma unroll
-        for (int q = 0; q < CPT; ++q)
-          if ((q & (2 * mm - 1)) == 0) {
-            y1[q] += __shfl_xor_sync(0xffffffffu, y1[q + mm], mm);
-            lb1[q] += __shfl_xor_sync(0xffffffffu, lb1[q + mm], mm);
-            if constexpr (ZOH) mb1[q] += __shfl_xor_sync(0xffffffffu, mb1[q + mm], mm);
-          }
-      }
-    } else {
-      y1[0] += __shfl_xor_sync(0xffffffffu, y1[0], 1);
-      lb1[0] += __shfl_xor_sync(0xffffffffu, lb1[0], 1);
-      if constexpr (ZOH) mb1[0] += __shfl_xor_sync(0xffffffffu, mb1[0], 1);
+      for (int q = 0; q < CPT; ++q)
+        if ((q & (2 * mm - 1)) == 0) {
+          y1[q] += __shfl_xor_sync(0xffffffffu, y1[q + mm], mm);
+          lb1[q] += __shfl_xor_sync(0xffffffffu, lb1[q + mm], mm);
+          if constexpr (ZOH) mb1[q] += __shfl_xor_sync(0xffffffffu, mb1[q + mm], mm);
+        }
     }
 
     // ======== even step t0 = 2m: its state is rebuilt from the one before it
@@ -348,7 +291,7 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
     else ln.unpack_row(td + r0e * WPR, dt0);
     ln.unpack_row(tx + r0e * WPR, u0);
     ln.pick_row(tds + r0e * CW, ds0);
-    const float gp0 = tgp[r0e * CW + ln.co];
+    const float gp0 = tgp[r0e * CW + lane];
     float y0[CPT], lb0[CPT], wa0[CPT], wa1[CPT], mb0[ZOH ? CPT : 1];
     {
       float2 Bv[H], Cv[H];
@@ -412,66 +355,41 @@ __device__ __forceinline__ void sub_block(const Lane<S, CPT>& ln, ChainRegs<S, C
           rrow[(V / 2 + v) ^ swz] = make_float4(dCt[2 * v].x, dCt[2 * v].y, dCt[2 * v + 1].x, dCt[2 * v + 1].y);
       }
     }
-    if constexpr (OWN) {
 #pragma unroll
-      for (int mm = 1; mm < LPC; mm <<= 1) {
+    for (int mm = 1; mm < LPC; mm <<= 1) {
 #pragma unroll
-        for (int q = 0; q < CPT; ++q)
-          if ((q & (2 * mm - 1)) == 0) {
-            y0[q] += __shfl_xor_sync(0xffffffffu, y0[q + mm], mm);
-            lb0[q] += __shfl_xor_sync(0xffffffffu, lb0[q + mm], mm);
-            wa0[q] += __shfl_xor_sync(0xffffffffu, wa0[q + mm], mm);
-            wa1[q] += __shfl_xor_sync(0xffffffffu, wa1[q + mm], mm);
-            if constexpr (ZOH) mb0[q] += __shfl_xor_sync(0xffffffffu, mb0[q + mm], mm);
-          }
-      }
-      // ---- finish both steps of the pair for this lane's own channel
-      const float dz1 = gp1 * fmaf(cr.Dk, u1[0], y1[0]);
-      // default rule: dx = delta sum lam B, ddelta = x sum lam B + sum w A; ZOH: dx = sum lam E B, ddelta = x sum mu B + sum w A
-      const float dx1 = ZOH ? fmaf(ds1[0], cr.Dk, lb1[0]) : fmaf(dt1[0], lb1[0], ds1[0] * cr.Dk);
-      const float dz0 = gp0 * fmaf(cr.Dk, u0[0], y0[0]);
-      const float dx0 = ZOH ? fmaf(ds0[0], cr.Dk, lb0[0]) : fmaf(dt0[0], lb0[0], ds0[0] * cr.Dk);
-      cr.dD = fmaf(ds1[0], u1[0], cr.dD);
-      cr.dD = fmaf(ds0[0], u0[0], cr.dD);
-      float dd1 = fmaf(u1[0], ZOH ? mb1[0] : lb1[0], wa1[0] * kInvLog2e);
-      float dd0 = fmaf(u0[0], ZOH ? mb0[0] : lb0[0], wa0[0] * kInvLog2e);
-      if constexpr (SP) {
-        // the gradient goes to the pre-activation v: d softplus(v) / dv = sigmoid(v); the bias gets the sum over time
-        dd1 *= tdS[r1 * CW + lane];
-        dd0 *= tdS[r0e * CW + lane];
-        if (r0 + 2 * m + 1 < nlive) cr.dbias += dd1;
-        if (r0 + 2 * m < nlive) cr.dbias += dd0;
-      }
-      reinterpret_cast<__nv_bfloat16*>(tox + r1 * WPR)[lane] = __float2bfloat16_rn(dx1);
-      reinterpret_cast<__nv_bfloat16*>(tod + r1 * WPR)[lane] = __float2bfloat16_rn(dd1);
-      reinterpret_cast<__nv_bfloat16*>(toz + r1 * WPR)[lane] = __float2bfloat16_rn(dz1 * gate_on);
-      reinterpret_cast<__nv_bfloat16*>(tox + r0e * WPR)[lane] = __float2bfloat16_rn(dx0);
-      reinterpret_cast<__nv_bfloat16*>(tod + r0e * WPR)[lane] = __float2bfloat16_rn(dd0);
-      reinterpret_cast<__nv_bfloat16*>(toz + r0e * WPR)[lane] = __float2bfloat16_rn(dz0 * gate_on);
-    } else {
-      // both lanes of the group complete the sums; lane 1 finishes the odd step of the pair, lane 0 the even one
-      y0[0] += __shfl_xor_sync(0xffffffffu, y0[0], 1);
-      lb0[0] += __shfl_xor_sync(0xffffffffu, lb0[0], 1);
-      wa0[0] += __shfl_xor_sync(0xffffffffu, wa0[0], 1);
-      wa1[0] += __shfl_xor_sync(0xffffffffu, wa1[0], 1);
-      if constexpr (ZOH) mb0[0] += __shfl_xor_sync(0xffffffffu, mb0[0], 1);
-      const bool odd = ln.j != 0;
-      const float ym = odd ? y1[0] : y0[0], lbm = odd ? lb1[0] : lb0[0], wam = odd ? wa1[0] : wa0[0];
-      const float um = odd ? u1[0] : u0[0], dtm = odd ? dt1[0] : dt0[0], dsm = odd ? ds1[0] : ds0[0];
-      const float gpm = odd ? gp1 : gp0;
-      const int rm = odd ? r1 : r0e;
-      const float dzm = gpm * fmaf(cr.Dk, um, ym);
-      const float dxm = ZOH ? fmaf(dsm, cr.Dk, lbm) : fmaf(dtm, lbm, dsm * cr.Dk);
-      cr.dD = fmaf(dsm, um, cr.dD);
-      float ddm = fmaf(um, ZOH ? (odd ? mb1[0] : mb0[0]) : lbm, wam * kInvLog2e);
-      if constexpr (SP) {
-        ddm *= tdS[rm * CW + ln.co];
-        if (r0 + 2 * m + (odd ? 1 : 0) < nlive) cr.dbias += ddm;
-      }
-      reinterpret_cast<__nv_bfloat16*>(tox + rm * WPR)[ln.co] = __float2bfloat16_rn(dxm);
-      reinterpret_cast<__nv_bfloat16*>(tod + rm * WPR)[ln.co] = __float2bfloat16_rn(ddm);
-      reinterpret_cast<__nv_bfloat16*>(toz + rm * WPR)[ln.co] = __float2bfloat16_rn(dzm * gate_on);
+      for (int q = 0; q < CPT; ++q)
+        if ((q & (2 * mm - 1)) == 0) {
+          y0[q] += __shfl_xor_sync(0xffffffffu, y0[q + mm], mm);
+          lb0[q] += __shfl_xor_sync(0xffffffffu, lb0[q + mm], mm);
+          wa0[q] += __shfl_xor_sync(0xffffffffu, wa0[q + mm], mm);
+          wa1[q] += __shfl_xor_sync(0xffffffffu, wa1[q + mm], mm);
+          if constexpr (ZOH) mb0[q] += __shfl_xor_sync(0xffffffffu, mb0[q + mm], mm);
+        }
     }
+    // ---- finish both steps of the pair for this lane's own channel
+    const float dz1 = gp1 * fmaf(cr.Dk, u1[0], y1[0]);
+    // default rule: dx = delta sum lam B, ddelta = x sum lam B + sum w A; ZOH: dx = sum lam E B, ddelta = x sum mu B + sum w A
+    const float dx1 = ZOH ? fmaf(ds1[0], cr.Dk, lb1[0]) : fmaf(dt1[0], lb1[0], ds1[0] * cr.Dk);
+    const float dz0 = gp0 * fmaf(cr.Dk, u0[0], y0[0]);
+    const float dx0 = ZOH ? fmaf(ds0[0], cr.Dk, lb0[0]) : fmaf(dt0[0], lb0[0], ds0[0] * cr.Dk);
+    cr.dD = fmaf(ds1[0], u1[0], cr.dD);
+    cr.dD = fmaf(ds0[0], u0[0], cr.dD);
+    float dd1 = fmaf(u1[0], ZOH ? mb1[0] : lb1[0], wa1[0] * kInvLog2e);
+    float dd0 = fmaf(u0[0], ZOH ? mb0[0] : lb0[0], wa0[0] * kInvLog2e);
+    if constexpr (SP) {
+      // the gradient goes to the pre-activation v: d softplus(v) / dv = sigmoid(v); the bias gets the sum over time
+      dd1 *= tdS[r1 * CW + lane];
+      dd0 *= tdS[r0e * CW + lane];
+      if (r0 + 2 * m + 1 < nlive) cr.dbias += dd1;
+      if (r0 + 2 * m < nlive) cr.dbias += dd0;
+    }
+    reinterpret_cast<__nv_bfloat16*>(tox + r1 * WPR)[lane] = __float2bfloat16_rn(dx1);
+    reinterpret_cast<__nv_bfloat16*>(tod + r1 * WPR)[lane] = __float2bfloat16_rn(dd1);
+    reinterpret_cast<__nv_bfloat16*>(toz + r1 * WPR)[lane] = __float2bfloat16_rn(dz1 * gate_on);
+    reinterpret_cast<__nv_bfloat16*>(tox + r0e * WPR)[lane] = __float2bfloat16_rn(dx0);
+    reinterpret_cast<__nv_bfloat16*>(tod + r0e * WPR)[lane] = __float2bfloat16_rn(dd0);
+    reinterpret_cast<__nv_bfloat16*>(toz + r0e * WPR)[lane] = __float2bfloat16_rn(dz0 * gate_on);
 
     if (BC != 3 && (2 * m) % kRB == 0) {
       // dB / dC of steps 2m .. 2m + 3: every lane sums one float4 of one step over the lane groups, ascending
@@ -511,7 +429,6 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
   constexpr int HV = bwd_handoff_vec(BC);
   using LN = Lane<S, CPT>;
   constexpr int H = S / 2, CW = LN::CW, WPR = CW / 2, NV = CPT * S / 4;   // NV: float4 of a thread's states
-  constexpr bool OWN = LN::OWN;
   using Smem = BwdWarpSmem<S, CPT, SP>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   dependency_wait();
@@ -557,7 +474,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
     constexpr int XCH = kBT * CPR;              // chunks per tensor and tile
     const int c_grp = d_w + g * CPT;            // first channel of this lane group
     const bool valid = WHOLE || c_grp < D;      // (CPT channels: all valid or none, D is a multiple of 8)
-    auto chan = [&](int q) { return OWN ? c_grp + (j ^ q) : c_grp; };
+    auto chan = [&](int q) { return c_grp + (j ^ q); };
     auto issue_tile = [&](int tile, int st) {
       if (tile >= tile_lo && tile >= 0) {
         const int t0 = t_seg0 + tile * kBT;
@@ -651,7 +568,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
       }
     }
     ap = __all_sync(0xffffffffu, ap);
-    const int c_own = d_w + ln.co;
+    const int c_own = d_w + lane;
     const float gate_off = has_z ? 0.f : 1.f;
     // (with 32 channels per warp an element's channel is this lane's own; with 16 it is lane % 16)
     const int c_el = d_w + lane % CW;
@@ -858,11 +775,6 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
       publish_handoff(sc, worker, lane);
     } else {
       // first step in time done: the chain is complete
-      float dD_tot = cr.dD, dbias_tot = cr.dbias;
-      if constexpr (!OWN) {   // the two lanes of a group summed the steps of one parity each
-        dD_tot += __shfl_xor_sync(0xffffffffu, dD_tot, 1);
-        dbias_tot += __shfl_xor_sync(0xffffffffu, dbias_tot, 1);
-      }
       if (valid) {
         const size_t part = (size_t)b * p.nseg + seg;
 #pragma unroll
@@ -881,10 +793,8 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
               *reinterpret_cast<float4*>(p.dh0 + ((size_t)b * D + chan(q)) * 16 + S * j + 4 * k) =
                   make_float4(cr.mu[q][2 * k].x, cr.mu[q][2 * k].y, cr.mu[q][2 * k + 1].x, cr.mu[q][2 * k + 1].y);
           }
-        if (OWN || j == 0) {
-          p.dD_part[part * D + c_own] = dD_tot;
-          if (SP && p.dbias_part != nullptr) p.dbias_part[part * D + c_own] = dbias_tot;
-        }
+        p.dD_part[part * D + c_own] = cr.dD;
+        if (SP && p.dbias_part != nullptr) p.dbias_part[part * D + c_own] = cr.dbias;
       }
     }
   }

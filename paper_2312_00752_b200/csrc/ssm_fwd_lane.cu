@@ -248,7 +248,6 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
         // recurrence that consumes them.
         auto run = [&](auto ap_tag) {
           constexpr bool AP = decltype(ap_tag)::value;
-          constexpr int GB = kLB;
           float a0s = 0.f, rs = 0.f;
           if constexpr (AP) {
             a0s = sA[(16 * g) * 32 + lane];
@@ -258,87 +257,82 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
             for (int k = 0; k < 8; ++k)
               A2[k] = make_float2(sA[(16 * g + 2 * k) * 32 + lane], sA[(16 * g + 2 * k + 1) * 32 + lane]);
           }
+          float e0[AP ? kLB : 1], e1[AP ? kLB : 1];
 #pragma unroll
-          for (int gb = 0; gb < kLB / GB; ++gb) {
-            float e0[AP ? GB : 1], e1[AP ? GB : 1];
-#pragma unroll
-            for (int t = 0; t < GB; ++t) {
-              const float dtt = dt[gb * GB + t];
-              if constexpr (AP) {
-                e0[t] = ex2_approx(dtt * a0s);
-                e1[t] = ex2_approx(dtt * rs);
-              }
+          for (int t = 0; t < kLB; ++t) {
+            if constexpr (AP) {
+              e0[t] = ex2_approx(dt[t] * a0s);
+              e1[t] = ex2_approx(dt[t] * rs);
             }
-            // general A: the exponentials of a step are taken AH steps ahead of its recurrence, between the multiply-adds of
-            // the steps before it (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1, 4, 5): a batch of
-            // exponentials ahead of a batch of recurrences left the FMA pipe idle during the one and the special-function
-            // unit during the other (bf16 (1, 2048, 5120), N = 64: 394 -> 348 us; complex is fastest two steps ahead)
-            constexpr int AH = CPLX ? 2 : 1, NA = AH + 1;
-            float2 aN[NA][8], bxN[2][8], CvN[2][READ ? 8 : 1];
-            auto exps = [&](int t, float2 (&a)[8]) {
-              const float dtt = dt[gb * GB + t];
-              if constexpr (CPLX) {
+          }
+          // general A: the exponentials of a step are taken AH steps ahead of its recurrence, between the multiply-adds of
+          // the steps before it (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1, 4, 5): a batch of
+          // exponentials ahead of a batch of recurrences left the FMA pipe idle during the one and the special-function
+          // unit during the other (bf16 (1, 2048, 5120), N = 64: 394 -> 348 us; complex is fastest two steps ahead)
+          constexpr int AH = CPLX ? 2 : 1, NA = AH + 1;
+          float2 aN[NA][8], bxN[2][8], CvN[2][READ ? 8 : 1];
+          auto exps = [&](int t, float2 (&a)[8]) {
+            const float dtt = dt[t];
+            if constexpr (CPLX) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                  const int k = (kk & 1) + 4 * (kk >> 1);
-                  cexp_pair(dtt, A2[k], A2[k + 2], a[k], a[k + 2]);
-                }
-              } else {
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                  const float2 e = f2mul(f2dup(dtt), A2[k]);
-                  a[k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
-                }
+              for (int kk = 0; kk < 4; ++kk) {
+                const int k = (kk & 1) + 4 * (kk >> 1);
+                cexp_pair(dtt, A2[k], A2[k + 2], a[k], a[k + 2]);
               }
-            };
-            if constexpr (!AP) {
-#pragma unroll
-              for (int t = 0; t < AH; ++t) exps(t, aN[t]);
-            }
-            auto front = [&](int t, float2 (&a)[8], float2 (&bx)[8], float2 (&Cv)[READ ? 8 : 1]) {
-              const int ts = gb * GB + t;
-              load16(fB + ts * NP + 16 * g, bx);
-              if constexpr (READ) load16(fC + ts * NP + 16 * g, Cv);
-              if constexpr (AP) {
-                const float a0 = e0[t], rr = e1[t], r2 = rr * rr, r4 = r2 * r2, r8 = r4 * r4;
-                a[0] = make_float2(a0, a0 * rr);
-                a[1] = f2mul(a[0], f2dup(r2));
-                a[2] = f2mul(a[0], f2dup(r4));
-                a[3] = f2mul(a[1], f2dup(r4));
-#pragma unroll
-                for (int k = 0; k < 4; ++k) a[4 + k] = f2mul(a[k], f2dup(r8));
-              }
-              const float2 du2 = f2dup(dt[ts] * u[ts]);
-#pragma unroll
-              for (int k = 0; k < 8; ++k) bx[k] = f2mul(du2, bx[k]);
-            };
-            front(0, aN[0], bxN[0], CvN[0]);
-#pragma unroll
-            for (int t = 0; t < GB; ++t) {
-              if constexpr (!AP) {
-                if (t + AH < GB) exps(t + AH, aN[(t + AH) % NA]);
-              }
-              if (t + 1 < GB) front(t + 1, aN[(t + 1) % NA], bxN[(t + 1) & 1], CvN[(t + 1) & 1]);
-              float2 yv = make_float2(0.f, 0.f), yw = yv;
-              if constexpr (CPLX) {
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                  const int k = (kk & 1) + 4 * (kk >> 1);
-                  const float2 ar = aN[t % NA][k], ai = aN[t % NA][k + 2], hr = h[k], hi = h[k + 2];
-                  h[k] = f2fma(f2neg(ai), hi, f2fma(ar, hr, bxN[t & 1][k]));
-                  h[k + 2] = f2fma(ai, hr, f2fma(ar, hi, bxN[t & 1][k + 2]));
-                }
-              }
+            } else {
 #pragma unroll
               for (int k = 0; k < 8; ++k) {
-                if constexpr (!CPLX) h[k] = f2fma(aN[t % NA][k], h[k], bxN[t & 1][k]);
-                if constexpr (READ) {
-                  if (k & 1) yw = f2fma(CvN[t & 1][k], h[k], yw);
-                  else yv = f2fma(CvN[t & 1][k], h[k], yv);
-                }
+                const float2 e = f2mul(f2dup(dtt), A2[k]);
+                a[k] = make_float2(ex2_approx(e.x), ex2_approx(e.y));
               }
-              if constexpr (READ) y[gb * GB + t] += (yv.x + yw.x) + (yv.y + yw.y);
             }
+          };
+          if constexpr (!AP) {
+#pragma unroll
+            for (int t = 0; t < AH; ++t) exps(t, aN[t]);
+          }
+          auto front = [&](int t, float2 (&a)[8], float2 (&bx)[8], float2 (&Cv)[READ ? 8 : 1]) {
+            load16(fB + t * NP + 16 * g, bx);
+            if constexpr (READ) load16(fC + t * NP + 16 * g, Cv);
+            if constexpr (AP) {
+              const float a0 = e0[t], rr = e1[t], r2 = rr * rr, r4 = r2 * r2, r8 = r4 * r4;
+              a[0] = make_float2(a0, a0 * rr);
+              a[1] = f2mul(a[0], f2dup(r2));
+              a[2] = f2mul(a[0], f2dup(r4));
+              a[3] = f2mul(a[1], f2dup(r4));
+#pragma unroll
+              for (int k = 0; k < 4; ++k) a[4 + k] = f2mul(a[k], f2dup(r8));
+            }
+            const float2 du2 = f2dup(dt[t] * u[t]);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) bx[k] = f2mul(du2, bx[k]);
+          };
+          front(0, aN[0], bxN[0], CvN[0]);
+#pragma unroll
+          for (int t = 0; t < kLB; ++t) {
+            if constexpr (!AP) {
+              if (t + AH < kLB) exps(t + AH, aN[(t + AH) % NA]);
+            }
+            if (t + 1 < kLB) front(t + 1, aN[(t + 1) % NA], bxN[(t + 1) & 1], CvN[(t + 1) & 1]);
+            float2 yv = make_float2(0.f, 0.f), yw = yv;
+            if constexpr (CPLX) {
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk) {
+                const int k = (kk & 1) + 4 * (kk >> 1);
+                const float2 ar = aN[t % NA][k], ai = aN[t % NA][k + 2], hr = h[k], hi = h[k + 2];
+                h[k] = f2fma(f2neg(ai), hi, f2fma(ar, hr, bxN[t & 1][k]));
+                h[k + 2] = f2fma(ai, hr, f2fma(ar, hi, bxN[t & 1][k + 2]));
+              }
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              if constexpr (!CPLX) h[k] = f2fma(aN[t % NA][k], h[k], bxN[t & 1][k]);
+              if constexpr (READ) {
+                if (k & 1) yw = f2fma(CvN[t & 1][k], h[k], yw);
+                else yv = f2fma(CvN[t & 1][k], h[k], yv);
+              }
+            }
+            if constexpr (READ) y[t] += (yv.x + yw.x) + (yv.y + yw.y);
           }
         };
         if constexpr (sizeof(IO) == 2 && !CPLX) {
@@ -550,7 +544,7 @@ LaneSplit choose_lane_split(long long chains, int steps, float extra, float fixe
   return best;
 }
 
-bool fwd_lane_applicable(const ssm_problem_t& prob, const FwdParams& p) {
+bool fwd_lane_applicable(const FwdParams& p) {
   return !p.zoh && !p.static_B && !p.static_C;
 }
 
