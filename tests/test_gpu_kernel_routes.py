@@ -1,0 +1,143 @@
+"""Which kernels a problem runs, and their results: the tuned kernels want bf16, N = 16 (or fewer, widened), aligned
+pointers and at least 296 chains of 32 channels (or the zero-order-hold rule); small problems of the same kind run the
+lane kernels, so what is to be tested of the tuned ones is wide here.  Every case asserts the route."""
+import numpy as np
+import pytest
+
+from paper_2312_00752_b200 import synth
+from tests import _gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+TUNED = ("ssm_fwd_warp_kernel", "ssm_bwd_warp_kernel")
+LANE = ("ssm_fwd_lane_kernel", "ssm_bwd_lane_kernel")
+GENERIC = ("ssm_fwd_kernel", "ssm_bwd_kernel")
+
+
+def _shifted(t):
+    """The same values at an address 8 bytes past a 16-byte boundary."""
+    import torch
+    buf = torch.empty(t.numel() + 8, dtype=t.dtype, device=t.device)
+    off = 8 // t.element_size()
+    v = buf[off:off + t.numel()].view(t.shape)
+    v.copy_(t)
+    assert v.data_ptr() % 16 == 8
+    return v
+
+
+def _check(batch, L, D, N=16, io="bf16", *, fwd=TUNED[0], bwd=TUNED[1], more=(), gate=True, skip=True, zoh=False, fused=False,
+           carry=False, saved=True, perturb_A=0.0, A=None, off=()):
+    import torch
+    from oracle import ssm_oracle as O
+    from paper_2312_00752_b200 import binding as K
+    inp = synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, io, 1e-3, 1e-1), seed=L, perturb_A=perturb_A)
+    rng = np.random.default_rng(L + N)
+    if A is not None:
+        inp["A"] = np.tile(np.asarray(A, dtype=np.float32), (D, 1))
+    if not gate:
+        inp["z"] = None
+    if not skip:
+        inp["D_skip"] = None
+    kw, okw, bias = dict(zoh=zoh), dict(zoh=zoh), None
+    if fused:
+        inp["delta"] = synth.round_to_io(0.1 * rng.standard_normal((batch, L, D)), io)
+        bias = (0.5 * rng.standard_normal(D) - 4.0).astype(np.float32)
+        okw.update(delta_softplus=True, delta_bias=bias)
+    state = (batch, D, N)
+    h0, dh = (rng.standard_normal(state).astype(np.float32) for _ in range(2)) if carry else (None, None)
+    t = lambda a: None if a is None else torch.from_numpy(a).cuda()
+    dev = U.to_device(inp, io)
+    x_fwd, x_bwd = (_shifted(dev["x"]) if k in off else dev["x"] for k in ("fwd", "bwd"))
+    h_last = torch.empty(state, device="cuda")
+    bkw = dict(h0=t(h0), dh_last=t(dh), want_dh0=True, **kw)
+    fkw = dict(save_states=True, h0=t(h0), h_last=h_last, **kw)
+    got = {}
+
+    def run():
+        rest = (dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+        if fused:
+            f = lambda x: (x, dev["delta"], t(bias), *rest)
+            out, sv = K.ssm_scan_fwd_fused_dt(*f(x_fwd), **fkw)
+            g = K.ssm_scan_bwd_fused_dt(*f(x_bwd), dev["dout"], sv if saved else None, **bkw)
+        else:
+            f = lambda x: (x, dev["delta"], *rest)
+            out, sv = K.ssm_scan_fwd(*f(x_fwd), **fkw)
+            g = K.ssm_scan_bwd(*f(x_bwd), dev["dout"], sv if saved else None, **bkw)
+        got.update(out=out, **g)
+    ran = U.kernels(run)
+    K.check_status(K.make_problem(dev["x"], dev["B"], gate, skip, zoh=zoh), K.last_bwd_workspace("cuda"))
+    assert {k for k in ran if k in TUNED + LANE + GENERIC} == {fwd, bwd}, ran
+    assert all(any(k.startswith(m) for k in ran) for m in more), ran
+    a = (inp["x"], inp["delta"], inp["A"], inp["B"], inp["C"])
+    out, h = O.scan_fwd(*a, D_skip=inp["D_skip"], z=inp["z"], h0=h0, return_h_last=True, **okw)
+    ref = dict(O.scan_bwd(*a, inp["D_skip"], inp["z"], inp["dout"], h0=h0, dh_last=dh, **okw), out=out)
+    host = {k: U.to_host(v) for k, v in got.items() if v is not None}
+    assert U.rel_err(U.to_host(h_last), h) <= (1e-5 if io == "f32" else 1e-4)
+    U.assert_parity(host, {k: v for k, v in ref.items() if k in host}, io, "route")
+    if io == "bf16":
+        U.assert_elementwise(host, ref, io, "route")
+
+
+@pytest.mark.parametrize("batch,L,D", [
+    (1, 1, 9480),       # a single step; 296 whole groups of 32 channels and one of 8
+    (2, 31, 4744),      # one step short of a tile
+    (1, 33, 9544),      # one step past one, a last group of 8
+    (4, 64, 2560),      # whole tiles and groups: the instantiations without range tests
+    (2, 512, 4736),     # ... with the backward in two segments
+    (1, 600, 9480),     # two ragged segments
+    (2, 96, 9984),      # 624 chains for 592 warps in the first round: some are shared
+])
+@pytest.mark.parametrize("fused", [False, True])
+def test_tuned_kernels_at_the_edges_of_tiles_groups_and_segments(batch, L, D, fused):
+    more = ("ssm_bwd_local_warp_kernel", "ssm_carry") if L >= 512 else ()
+    _check(batch, L, D, fused=fused, carry=fused, more=more)
+
+
+@pytest.mark.parametrize("options", [
+    dict(gate=False), dict(skip=False), dict(gate=False, skip=False), dict(carry=True), dict(carry=True, saved=False),
+    dict(perturb_A=0.05), dict(perturb_A=0.05, fused=True, saved=False), dict(fused=True, gate=False, carry=True),
+], ids=lambda o: "-".join(f"{k}={v}" for k, v in o.items()))
+@pytest.mark.parametrize("batch,L,D", [(1, 150, 9480), (4, 64, 2560)])   # ragged; whole
+def test_options_on_the_tuned_kernels(batch, L, D, options):
+    _check(batch, L, D, **options)
+
+
+@pytest.mark.parametrize("N", [1, 2, 4, 8])
+@pytest.mark.parametrize("saved", [True, False])
+def test_small_states_widened_for_the_tuned_kernels(N, saved):
+    _check(1, 70, 9480, N, carry=True, saved=saved, more=("ssm_repack_kernel",))
+
+
+@pytest.mark.parametrize("A", [(-4.0, -3.0, -2.0, -1.0), (-16.0, -15.0, -14.0, -13.0), (-0.7, -0.7, -0.7, -0.7), (-0.3, -2.0, -0.9, -4.0)])
+def test_rows_of_A_widened_for_the_tuned_kernels(A):
+    # a progression that would turn positive, one that only just would, step 0, no progression
+    _check(1, 40, 9480, 4, A=A, more=("ssm_repack_kernel",))
+
+
+@pytest.mark.parametrize("off,fwd,bwd", [
+    (("fwd",), LANE[0], TUNED[1]), (("bwd",), TUNED[0], LANE[1]), (("fwd", "bwd"), *LANE),
+])
+def test_pointers_off_the_16_byte_grid_and_states_passed_between_the_families(off, fwd, bwd):
+    _check(2, 150, 4744, fwd=fwd, bwd=bwd, off=off)
+
+
+def test_states_rebuilt_off_the_16_byte_grid():
+    _check(2, 150, 4744, fwd=LANE[0], bwd=LANE[1], off=("fwd", "bwd"), saved=False)
+
+
+@pytest.mark.parametrize("batch,L,D,N,io,more", [
+    (2, 1237, 1001, 16, "bf16", ("ssm_bwd_lane_local_kernel",)),   # odd width, the backward in segments with a pre-pass
+    (1, 2000, 1500, 16, "f32", ("ssm_bwd_lane_local_kernel",)),
+    (1, 900, 1300, 64, "bf16", ("ssm_bwd_lane_local_kernel",)),
+    (1, 4133, 20, 16, "f32", ("ssm_carry",)),                      # the launch split in time
+    (2, 100, 40, 16, "bf16", ()),                                  # a tuned shape with few channels
+])
+def test_lane_kernels(batch, L, D, N, io, more):
+    _check(batch, L, D, N, io, fwd=LANE[0], bwd=LANE[1], more=more)
+
+
+@pytest.mark.parametrize("D,io,fwd,bwd,off", [
+    (40, "bf16", *TUNED, ()), (41, "bf16", *GENERIC, ()), (40, "f32", *GENERIC, ()), (40, "bf16", *GENERIC, ("fwd", "bwd")),
+])
+def test_zero_order_hold_keeps_to_the_tuned_and_generic_kernels(D, io, fwd, bwd, off):
+    _check(2, 150, D, 16, io, zoh=True, fwd=fwd, bwd=bwd, off=off)

@@ -24,7 +24,7 @@ pytestmark = pytest.mark.gpu
     (5, 40, 2048, 16, "f32"),      # more chains than SM sub-partitions: several chains per block, no split
     (1, 4133, 20, 16, "f32"),      # the launch itself split in time (summary and carry)
     (1, 4100, 33, 64, "bf16"),
-    (2, 707, 1001, 16, "bf16"),    # backward split into segments with a pre-pass: odd rows, ragged last segment
+    (2, 707, 1001, 16, "bf16"),    # odd rows, several pieces per chain (segments with a pre-pass: test_gpu_kernel_routes.py)
     (1, 650, 1300, 32, "f32"),
 ])
 def test_edges(batch, L, D, N, io):
@@ -82,8 +82,9 @@ def test_few_channels_of_the_tuned_shapes(batch, L, D, N):
     (1, 63, 36, 1, "f32"),         # 16-byte rows, one step short of 8 pieces of 8
     (2, 65, 31, 8, "f32"),         # one group of 16 columns, rows at odd addresses
     (1, 520, 17, 32, "bf16"),      # four groups of 16 columns
-    (1, 4133, 20, 16, "f32"),      # the launch split in time
-    (2, 707, 1001, 8, "bf16"),     # backward split into segments with a pre-pass
+    (1, 4133, 20, 16, "f32"),      # forward cut inside clusters, backward into segments
+    (2, 707, 1001, 8, "bf16"),     # odd rows, several pieces per chain
+    (2, 1237, 1001, 8, "bf16"),    # backward split into segments with a pre-pass, ragged last segment
 ])
 def test_complex_edges(batch, L, D, N, io):
     from oracle import ssm_oracle_complex as OC

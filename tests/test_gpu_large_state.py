@@ -1,5 +1,5 @@
-"""State sizes above the ones the paper ablates (N = 32, 64) on the generic kernels against the oracle: forward and
-backward, both io dtypes, both B-bar rules, saved or rebuilt checkpoints, a time split, the carried state with the
+"""State sizes above the ones the paper ablates (N = 32, 64) against the oracle, on the lane kernels and, with the
+zero-order-hold rule, on the generic ones: forward and backward, both io dtypes, both B-bar rules, saved or rebuilt checkpoints, a time split, the carried state with the
 single recurrent step, and the backward in two pieces."""
 import numpy as np
 import pytest

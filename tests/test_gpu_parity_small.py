@@ -38,9 +38,9 @@ def test_config0_tiny_f32():
     (1, 130, 33, 2, "f32"),
     (2, 64, 70, 1, "bf16"),       # N = 1 (the setting of the gating theorem)
     (1, 333, 129, 16, "f32"),     # channels straddle several blocks
-    (1, 1, 8, 16, "bf16"),        # tuned kernels: a single step in a single partial channel block
-    (2, 31, 16, 16, "bf16"),      # tuned kernels: one step short of a tile
-    (1, 33, 72, 16, "bf16"),      # tuned kernels: one step past a tile, channel blocks 32 + 32 + 8
+    (1, 1, 8, 16, "bf16"),        # few channels: the lane kernels; a single step, a partial channel group
+    (2, 31, 16, 16, "bf16"),      # ... one step short of a tile of the tuned kernels
+    (1, 33, 72, 16, "bf16"),      # ... one step past one, channel groups 32 + 32 + 8
 ])
 def test_shapes_and_state_sizes(batch, L, D, N, io):
     cfg, inp = _case(batch, L, D, N, io)
@@ -48,7 +48,7 @@ def test_shapes_and_state_sizes(batch, L, D, N, io):
     U.assert_parity(got, U.oracle_fwd_bwd(inp), io, f"{(batch, L, D, N, io)}")
 
 
-@pytest.mark.parametrize("io", ["f32", "bf16"])     # generic and tuned kernels
+@pytest.mark.parametrize("io", ["f32", "bf16"])     # (lane kernels; the tuned ones: test_gpu_kernel_routes.py)
 @pytest.mark.parametrize("gate,skip", [(False, True), (True, False), (False, False)])
 def test_optional_gate_and_skip(gate, skip, io):
     cfg, inp = _case(2, 150, 48, 16, io)
@@ -154,7 +154,8 @@ def test_smoke_entry_point_runs():
 
 
 def test_pointers_off_the_16_byte_grid_take_the_generic_kernels():
-    # bf16 / N = 16 tensors whose addresses are only 8-byte aligned: the tuned kernels do not apply, the results must
+    # bf16 / N = 16 tensors whose addresses are only 8-byte aligned: no 16-byte rows (a problem of this size runs the lane
+    # kernels either way; from the tuned ones to them: test_gpu_kernel_routes.py); the results must
     # be the same within tolerance (and the call must not fault on a misaligned 16-byte access)
     import torch
     cfg, inp = _case(2, 100, 40, 16, "bf16")
@@ -174,8 +175,9 @@ def test_pointers_off_the_16_byte_grid_take_the_generic_kernels():
 
 @pytest.mark.parametrize("fwd_generic", [False, True])
 def test_saved_states_pass_between_tuned_and_generic_kernels(fwd_generic):
-    # the forward and the backward of one problem may take different kernels (the tuned ones need 16-byte aligned
-    # pointers): the checkpoint states one of them saves must be the ones the other reads.  D = 72 leaves the third
+    # the forward and the backward of one problem may take different kernels: the checkpoint states one of them saves must
+    # be the ones the other reads (here the lane kernels with and without 16-byte rows; tuned and lane kernels:
+    # test_gpu_kernel_routes.py).  D = 72 leaves the third
     # group of 32 channels ragged.
     import torch
     from paper_2312_00752_b200 import binding as K

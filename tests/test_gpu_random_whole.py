@@ -1,5 +1,6 @@
-"""Seeded sweep over problems whose tiles and channel groups are all whole (L a multiple of 32, D a multiple of 32): these
-take the instantiations of the tuned kernels that carry no range tests.  Same options as the other sweeps (gate / skip,
+"""Seeded sweep over problems whose tiles and channel groups are all whole (L a multiple of 32, D a multiple of 32): with the
+zero-order-hold rule these take the instantiations of the tuned kernels that carry no range tests, with the default rule
+the lane kernels (wide problems on the tuned ones: test_gpu_kernel_routes.py, test_gpu_random_wide.py).  Same options as the other sweeps (gate / skip,
 both B-bar rules, arithmetic-progression or general A, saved or rebuilt checkpoints, carried state and adjoint, every
 state size up to 16, both io dtypes), several time-split lengths among them."""
 import numpy as np

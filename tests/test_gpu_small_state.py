@@ -1,5 +1,6 @@
-"""bf16 problems with fewer than 16 states per channel (the state sizes of Table 10) run on the tuned 16-state kernels
-with A, B, C and the state arrays widened by columns that stay zero.  Checked here against the oracle at the problem's
+"""bf16 problems with fewer than 16 states per channel (the state sizes of Table 10): with many channels, non-selective B / C
+or the zero-order-hold rule they run on the tuned 16-state kernels with A, B, C and the state arrays widened by columns
+that stay zero, with few channels on the lane kernels as they are (wide ones: test_gpu_kernel_routes.py).  Checked here against the oracle at the problem's
 own N: every N below 16, the options that touch a widened array (carried state and adjoint, non-selective B / C, both
 B-bar rules, the fused step size), A rows that are and are not arithmetic progressions (the widening of A continues a
 progression only while it stays non-positive), and a wide shape where neighbouring warps share chains."""
@@ -30,7 +31,7 @@ def test_the_widened_route_is_taken_and_matches_the_oracle(N):
     dhl = rng.standard_normal(shape).astype(np.float32)
     dev = U.to_device(inp, "bf16")
     prob = K.make_problem(dev["x"], dev["B"], True, True)
-    assert prob.N == N and K.plan(prob)["states_per_thread"] == 16          # the plan of the 16-state problem
+    assert prob.N == N and K.plan(prob)["states_per_thread"] == 16          # (on the lane kernels too, which take a problem this small)
     args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
     t = lambda a: torch.from_numpy(a).cuda()
     h_last = torch.empty(shape, dtype=torch.float32, device="cuda")

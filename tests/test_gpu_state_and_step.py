@@ -21,8 +21,8 @@ def _oracle(inp, h0=None):
 
 
 @pytest.mark.parametrize("batch,L,D,N,io,cut", [
-    (2, 300, 40, 16, "bf16", 130),      # tuned kernels
-    (1, 200, 24, 8, "f32", 77),         # generic kernels
+    (2, 300, 40, 16, "bf16", 130),      # lane kernels (tuned ones: test_gpu_kernel_routes.py)
+    (1, 200, 24, 8, "f32", 77),         # lane kernels, float32
     (1, 6000, 64, 16, "bf16", 2048),    # both pieces split time into segments
 ])
 def test_two_pieces_equal_one_sequence(batch, L, D, N, io, cut):
@@ -109,9 +109,9 @@ def test_saved_states_carry_h0_into_backward():
 
 
 @pytest.mark.parametrize("batch,L,D,N,io,cut,saved", [
-    (2, 300, 40, 16, "bf16", 130, True),       # tuned kernels
+    (2, 300, 40, 16, "bf16", 130, True),       # lane kernels (tuned ones: test_gpu_kernel_routes.py)
     (2, 300, 40, 16, "bf16", 130, False),      # ... with the checkpoints rebuilt from h0
-    (1, 200, 24, 8, "f32", 77, True),          # generic kernels
+    (1, 200, 24, 8, "f32", 77, True),          # lane kernels, float32
     (1, 200, 24, 8, "f32", 77, False),
     (1, 6000, 64, 16, "bf16", 2048, True),     # both pieces split time: dh_last enters the reverse carry
 ])
