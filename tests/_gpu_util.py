@@ -37,16 +37,24 @@ def to_host(t) -> np.ndarray:
 
 
 def kernels(run) -> set:
-    """Names of the library's kernels that `run()` launches (the profiler's record, template arguments cut off)."""
+    """Names of the library's kernels that `run()` launches (template arguments cut off).  It is captured into a graph and
+    not executed; call it once before, so that nothing is set up for the first time."""
+    import os
     import re
+    import tempfile
+    import warnings
     import torch
-    from torch.profiler import ProfilerActivity, profile
-    torch.cuda.synchronize()
-    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as prof:
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    graph.enable_debug_mode()
+    with torch.cuda.graph(graph):
         run()
-        torch.cuda.synchronize()
-    found = (re.search(r"\bssm_\w+_kernel\b", e.key) for e in prof.key_averages())
-    return {m.group(0) for m in found if m}
+    with tempfile.TemporaryDirectory() as d:
+        path = os.path.join(d, "graph.dot")
+        with warnings.catch_warnings():
+            warnings.simplefilter("ignore")
+            graph.debug_dump(path)
+        with open(path) as f:   # (mangled names; a kernel in an anonymous namespace has its file's before its own)
+            return {m[m.rindex("ssm_"):] for m in re.findall(r"ssm_\w+?_kernel", f.read())}
 
 
 def gpu_fwd_bwd(dev: dict, use_saved=True, general_A=False):

@@ -51,21 +51,20 @@ def _check(batch, L, D, N=16, io="bf16", *, fwd=TUNED[0], bwd=TUNED[1], more=(),
     h_last = torch.empty(state, device="cuda")
     bkw = dict(h0=t(h0), dh_last=t(dh), want_dh0=True, **kw)
     fkw = dict(save_states=True, h0=t(h0), h_last=h_last, **kw)
-    got = {}
+    rest = (dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    tb = t(bias)
 
     def run():
-        rest = (dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
         if fused:
-            f = lambda x: (x, dev["delta"], t(bias), *rest)
+            f = lambda x: (x, dev["delta"], tb, *rest)
             out, sv = K.ssm_scan_fwd_fused_dt(*f(x_fwd), **fkw)
-            g = K.ssm_scan_bwd_fused_dt(*f(x_bwd), dev["dout"], sv if saved else None, **bkw)
-        else:
-            f = lambda x: (x, dev["delta"], *rest)
-            out, sv = K.ssm_scan_fwd(*f(x_fwd), **fkw)
-            g = K.ssm_scan_bwd(*f(x_bwd), dev["dout"], sv if saved else None, **bkw)
-        got.update(out=out, **g)
-    ran = U.kernels(run)
+            return dict(K.ssm_scan_bwd_fused_dt(*f(x_bwd), dev["dout"], sv if saved else None, **bkw), out=out)
+        f = lambda x: (x, dev["delta"], *rest)
+        out, sv = K.ssm_scan_fwd(*f(x_fwd), **fkw)
+        return dict(K.ssm_scan_bwd(*f(x_bwd), dev["dout"], sv if saved else None, **bkw), out=out)
+    got = run()
     K.check_status(K.make_problem(dev["x"], dev["B"], gate, skip, zoh=zoh), K.last_bwd_workspace("cuda"))
+    ran = U.kernels(run)
     assert {k for k in ran if k in TUNED + LANE + GENERIC} == {fwd, bwd}, ran
     assert all(any(k.startswith(m) for k in ran) for m in more), ran
     a = (inp["x"], inp["delta"], inp["A"], inp["B"], inp["C"])
