@@ -75,7 +75,7 @@ enum {
   SSM_FLAG_HAS_DSKIP = 2u,    /* D_skip is given; otherwise the skip term is absent and dD is not produced      */
   SSM_FLAG_SAVE_STATES = 4u,  /* forward: also write the checkpoint states that backward starts its recomputation
                                  from (the scan states Appendix D keeps between chunks)                          */
-  SSM_FLAG_GENERAL_A = 8u,    /* do not use the fast path for rows of A that are arithmetic progressions in n   */
+  SSM_FLAG_GENERAL_A = 8u,    /* do not use the fast path for rows of A that are falling arithmetic progressions in n */
   SSM_FLAG_DELTA_SOFTPLUS = 32u, /* ssm_scan_*_fused_dt: the step size is softplus(delta_pre + delta_bias[d])         */
   SSM_FLAG_ZOH_BBAR = 64u,    /* B-bar = (exp(delta A) - 1) / A * B, the zero-order hold of Eq. 4 (delta * B at A = 0),
                                  instead of the default delta * B; honoured by every call                        */

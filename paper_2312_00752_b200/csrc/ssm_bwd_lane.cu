@@ -531,6 +531,7 @@ __device__ __forceinline__ bool lane_progression(const float* a_log2, int N, int
   bool ap = sizeof(IO) == 2 && !general_A && N - 16 * gi >= 16;
   const float* a = a_log2 + lane;
   const float a0 = a[0], step = a[32] - a0, tol = 1e-6f * fabsf(a[32 * 15]);
+  ap = ap && step <= 0.f;   // (as in ssm_fwd_lane.cu)
 #pragma unroll
   for (int k = 2; k < 16; ++k) ap = ap && fabsf(a[32 * k] - (a0 + (float)k * step)) <= tol;
   return __all_sync(0xffffffffu, ap);

@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(kLWarps * 32) ssm_bwd_local_warp_kernel(const 
       }
       const float step = av[1] - av[0];
       const float tol = 1e-6f * fabsf(av[15]);
+      ap = ap && step <= 0.f;   // (as in ssm_fwd_warp.cu)
 #pragma unroll
       for (int k = 2; k < 16; ++k) ap = ap && fabsf(av[k] - (av[0] + (float)k * step)) <= tol;
 #pragma unroll

@@ -530,6 +530,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, (CPT == 16 / S) ? 2 : 3)
       }
       const float step = av[1] - av[0];
       const float tol = 1e-6f * fabsf(av[S - 1]);
+      ap = ap && step <= 0.f;   // (as in ssm_fwd_warp.cu)
 #pragma unroll
       for (int k = 2; k < S; ++k) ap = ap && fabsf(av[k] - (av[0] + (float)k * step)) <= tol;
       if (ZOH && valid) {

@@ -123,7 +123,8 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
   __syncthreads();
   float2 A2[8];
   float2 h[8];
-  // which groups of 16 have their A in arithmetic progression (padded states continue it as long as they decay)
+  // which groups of 16 have their A in arithmetic progression (falling only: a rising one starts from its smallest decay,
+  // which underflows for large steps, and padded states, which continue it, would come to grow)
   unsigned ap_mask = 0;
   if (sizeof(IO) == 2 && !CPLX && !p.general_A) {
 #pragma unroll 1
@@ -132,7 +133,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
       const int live = min(16, N - 16 * g);
       const float a0 = a[0], step = live > 1 ? a[32] - a0 : 0.f;
       const float tol = 1e-6f * fabsf(a[32 * (live - 1)]);
-      bool ok = live == 16 || step <= 0.f;
+      bool ok = step <= 0.f;
 #pragma unroll
       for (int k = 2; k < 16; ++k) ok = ok && (k >= live || fabsf(a[32 * k] - (a0 + (float)k * step)) <= tol);
       if (__all_sync(0xffffffffu, ok)) ap_mask |= 1u << g;

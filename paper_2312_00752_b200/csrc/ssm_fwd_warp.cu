@@ -198,6 +198,9 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MODE == kFwdFull ? 1 : 3)
       }
       const float step = av[1] - av[0];
       const float tol = 1e-6f * fabsf(av[S - 1]);
+      // (falling only: a rising one starts from its smallest decay, which underflows for large steps, while the powers of the
+      // ratio that should lead back up from it overflow)
+      ap = ap && step <= 0.f;
 #pragma unroll
       for (int k = 2; k < S; ++k) ap = ap && fabsf(av[k] - (av[0] + (float)k * step)) <= tol;
       if (ZOH && valid) {

@@ -26,11 +26,11 @@ def _shifted(t):
 
 
 def _check(batch, L, D, N=16, io="bf16", *, fwd=TUNED[0], bwd=TUNED[1], more=(), gate=True, skip=True, zoh=False, fused=False,
-           carry=False, saved=True, perturb_A=0.0, A=None, off=()):
+           carry=False, saved=True, perturb_A=0.0, A=None, dt=(1e-3, 1e-1), off=()):
     import torch
     from oracle import ssm_oracle as O
     from paper_2312_00752_b200 import binding as K
-    inp = synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, io, 1e-3, 1e-1), seed=L, perturb_A=perturb_A)
+    inp = synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, io, *dt), seed=L, perturb_A=perturb_A)
     rng = np.random.default_rng(L + N)
     if A is not None:
         inp["A"] = np.tile(np.asarray(A, dtype=np.float32), (D, 1))
@@ -111,6 +111,14 @@ def test_small_states_widened_for_the_tuned_kernels(N, saved):
 def test_rows_of_A_widened_for_the_tuned_kernels(A):
     # a progression that would turn positive, one that only just would, step 0, no progression
     _check(1, 40, 9480, 4, A=A, more=("ssm_repack_kernel",))
+
+
+@pytest.mark.parametrize("D,N,route", [(9480, 16, TUNED), (40, 16, (TUNED[0], LANE[1])), (41, 16, LANE), (41, 32, LANE)])
+@pytest.mark.parametrize("saved", [True, False])
+def test_rising_rows_of_A_with_large_steps(D, N, route, saved):
+    # exp(delta A) of the first state is below the smallest float32, that of the last one is not
+    _check(1, 40, D, N, A=np.arange(-16.0, 0.0).tolist() * (N // 16), dt=(8.0, 20.0), carry=True, saved=saved,
+           fwd=route[0], bwd=route[1])
 
 
 @pytest.mark.parametrize("off,fwd,bwd", [
