@@ -127,14 +127,20 @@ struct Workspace {
 };
 Workspace workspace(size_t bytes, const at::Tensor& x, void* stream) {
   if (bytes == 0) return {};
-  Scratch& scratch = workspaces()[{x.device().index(), stream}];
+  const c10::DeviceIndex dev = x.device().index();
+  // A call that is being captured gets a buffer of its own, from the graph's memory: the graph keeps its address, while the
+  // buffer kept here may be given back when a larger one takes its place.
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &capture) != cudaSuccess) (void)cudaGetLastError();
+  if (capture != cudaStreamCaptureStatusNone) return {empty({(int64_t)bytes}, at::kByte, x), nullptr};
+  Scratch& scratch = workspaces()[{dev, stream}];
   at::Tensor& ws = scratch.buffer;
   if (!ws.defined() || (size_t)ws.numel() < bytes) {
     if (ws.defined()) {
       // kernels already enqueued on that stream may still use the old buffer: the caching allocator must not hand its
       // memory to other work before they are done
       c10::cuda::CUDACachingAllocator::recordStream(
-          ws.storage().data_ptr(), c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), x.device().index()));
+          ws.storage().data_ptr(), c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), dev));
     }
     ws = empty({(int64_t)bytes}, at::kByte, x);
   }

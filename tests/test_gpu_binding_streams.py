@@ -1,0 +1,43 @@
+"""The binding's scratch memory beside graphs and streams."""
+import pytest
+
+from paper_2312_00752_b200 import synth
+from tests import _gpu_util as U
+
+pytestmark = pytest.mark.gpu
+
+
+def _call(L, D=64):
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("streams", 30, 1, L, D, 16, "bf16", 1e-3, 1e-1), seed=L), "bf16")
+    args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    return lambda **kw: K.ssm_scan_bwd(*args, dev["dout"], None, **kw)
+
+
+def test_a_captured_call_does_not_use_the_buffer_that_is_kept_for_its_stream():
+    # (that buffer is given back when a larger call comes along, the graph would go on writing to it)
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    run, larger = _call(300), _call(3000)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ref = run()
+    kept = K.last_bwd_workspace("cuda", s)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        got = run()
+    torch.cuda.synchronize()
+    kept.fill_(0x5a)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert bool((kept == 0x5a).all())
+    assert all(torch.equal(got[k], ref[k]) for k in ref)
+    with torch.cuda.stream(s):
+        larger()
+    assert K.last_bwd_workspace("cuda", s).numel() > kept.numel()
+    for v in got.values():
+        v.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(got[k], ref[k]) for k in ref)
