@@ -14,7 +14,7 @@
 
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
-#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
@@ -108,6 +108,14 @@ void* stream_of(PyObject* stream, const at::Tensor& x) {
   return s;
 }
 
+// A buffer for work on `stream`, which need not be the current one: a block of that stream's own, so that the allocator takes
+// it from nobody whose work on another stream still uses it, and gives it back to nobody else.
+at::Tensor scratch_buffer(size_t bytes, const at::Tensor& x, void* stream) {
+  const auto s = c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), x.device().index());
+  const c10::cuda::CUDAStreamGuard on(s);
+  return empty({(int64_t)bytes}, at::kByte, x);
+}
+
 // Scratch of one (device, stream): a buffer that only grows (calls on different streams never share scratch memory), and a lock
 // that a call on it holds while it enqueues.  A call is several launches that hand results to each other through the buffer,
 // and the interpreter lock is not held meanwhile: without this one the launches of two threads on one stream would mix.
@@ -127,23 +135,15 @@ struct Workspace {
 };
 Workspace workspace(size_t bytes, const at::Tensor& x, void* stream) {
   if (bytes == 0) return {};
-  const c10::DeviceIndex dev = x.device().index();
   // A call that is being captured gets a buffer of its own, from the graph's memory: the graph keeps its address, while the
   // buffer kept here may be given back when a larger one takes its place.
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &capture) != cudaSuccess) (void)cudaGetLastError();
-  if (capture != cudaStreamCaptureStatusNone) return {empty({(int64_t)bytes}, at::kByte, x), nullptr};
-  Scratch& scratch = workspaces()[{dev, stream}];
+  if (capture != cudaStreamCaptureStatusNone) return {scratch_buffer(bytes, x, stream), nullptr};
+  Scratch& scratch = workspaces()[{x.device().index(), stream}];
   at::Tensor& ws = scratch.buffer;
-  if (!ws.defined() || (size_t)ws.numel() < bytes) {
-    if (ws.defined()) {
-      // kernels already enqueued on that stream may still use the old buffer: the caching allocator must not hand its
-      // memory to other work before they are done
-      c10::cuda::CUDACachingAllocator::recordStream(
-          ws.storage().data_ptr(), c10::cuda::getStreamFromExternal(static_cast<cudaStream_t>(stream), dev));
-    }
-    ws = empty({(int64_t)bytes}, at::kByte, x);
-  }
+  // (the old buffer is a block of the same stream: whoever gets its memory is enqueued behind the kernels that use it)
+  if (!ws.defined() || (size_t)ws.numel() < bytes) ws = scratch_buffer(bytes, x, stream);
   return {ws, &scratch.enqueue};
 }
 

@@ -41,3 +41,19 @@ def test_a_captured_call_does_not_use_the_buffer_that_is_kept_for_its_stream():
     graph.replay()
     torch.cuda.synchronize()
     assert all(torch.equal(got[k], ref[k]) for k in ref)
+
+
+def test_the_buffer_of_a_stream_is_a_block_of_that_stream():
+    # (`stream` is not the current one: a block of the current stream may still be in use by its pending work, and would be
+    # given back to it)
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    s = torch.cuda.Stream()
+    run, ref = _call(400), _call(400)()
+    torch.cuda.synchronize()
+    got = run(stream=s)
+    s.synchronize()
+    assert all(torch.equal(got[k], ref[k]) for k in ref)
+    at = K.last_bwd_workspace("cuda", s).data_ptr()
+    owner = [seg["stream"] for seg in torch.cuda.memory_snapshot() if seg["address"] <= at < seg["address"] + seg["total_size"]]
+    assert owner == [s.cuda_stream]
