@@ -14,6 +14,7 @@
 
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -106,6 +107,17 @@ void* stream_of(PyObject* stream, const at::Tensor& x) {
   Py_DECREF(v);
   if (s == nullptr && PyErr_Occurred()) throw Raised{};
   return s;
+}
+
+// A new result of a call on `stream`.  It is a block of the current stream; where that is another one the allocator is told, so
+// that a result that is dropped early is not given to other tensors while the call still writes to it.
+at::Tensor result(at::IntArrayRef shape, at::ScalarType dtype, const at::Tensor& like, void* stream) {
+  at::Tensor t = empty(shape, dtype, like);
+  const auto s = static_cast<cudaStream_t>(stream);
+  const c10::DeviceIndex dev = like.device().index();
+  if (c10::cuda::getCurrentCUDAStream(dev).stream() != s)
+    c10::cuda::CUDACachingAllocator::recordStream(t.storage().data_ptr(), c10::cuda::getStreamFromExternal(s, dev));
+  return t;
 }
 
 // A buffer for work on `stream`, which need not be the current one: a block of that stream's own, so that the allocator takes
@@ -251,10 +263,10 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t D = pr.p.D;
     void* stream = stream_of(a[13], x);
     const at::Tensor* given = tensor(a[9], "out");
-    at::Tensor out = given != nullptr ? *given : empty(pr.rows, pr.io, x);
+    at::Tensor out = given != nullptr ? *given : result(pr.rows, pr.io, x, stream);
     const at::Tensor* sgiven = save ? tensor(a[11], "saved_states") : nullptr;
     at::Tensor saved;
-    if (save) saved = sgiven != nullptr ? *sgiven : empty({(int64_t)(api.ssm_scan_saved_state_bytes(&pr.p) / 4)}, at::kFloat, x);
+    if (save) saved = sgiven != nullptr ? *sgiven : result({(int64_t)(api.ssm_scan_saved_state_bytes(&pr.p) / 4)}, at::kFloat, x, stream);
     const at::Tensor* ws = tensor(a[12], "workspace");
     Workspace own;
     if (ws == nullptr && entry != 2) own = workspace(api.ssm_scan_fwd_workspace_bytes(&pr.p), x, stream);
@@ -297,14 +309,15 @@ PyObject* fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
 }
 
 // an output of a backward call: the tensor of `outputs` under that name, or a new one, which is put there
-at::Tensor output(PyObject* outputs, const char* name, at::IntArrayRef shape, at::ScalarType dtype, const at::Tensor& like) {
+at::Tensor output(PyObject* outputs, const char* name, at::IntArrayRef shape, at::ScalarType dtype, const at::Tensor& like,
+                  void* stream) {
   PyObject* have = PyDict_GetItemString(outputs, name);
   if (have != nullptr && have != Py_None) {
     const at::Tensor* t = tensor(have, name);
     pointer(t, name, shape, dtype);
     return *t;
   }
-  at::Tensor t = empty(shape, dtype, like);
+  at::Tensor t = result(shape, dtype, like, stream);
   PyObject* o = wrap(t);
   const int rc = PyDict_SetItemString(outputs, name, o);
   Py_DECREF(o);
@@ -349,15 +362,15 @@ PyObject* bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void* ps = pointer(tensor(a[9], "saved_states"), "saved_states");
     auto* ph = static_cast<float*>(pointer(a[10], "h0", pr.h, at::kFloat));
     auto* pm = static_cast<float*>(pointer(a[11], "dh_last", pr.h, at::kFloat));
-    at::Tensor dx = output(o, "dx", pr.rows, pr.io, x), dd = output(o, "ddelta", pr.rows, pr.io, x);
-    at::Tensor dA = output(o, "dA", pr.a, at::kFloat, x), dB = output(o, "dB", pr.b, pr.bt, x), dC = output(o, "dC", pr.c, pr.ct, x);
+    at::Tensor dx = output(o, "dx", pr.rows, pr.io, x, stream), dd = output(o, "ddelta", pr.rows, pr.io, x, stream);
+    at::Tensor dA = output(o, "dA", pr.a, at::kFloat, x, stream), dB = output(o, "dB", pr.b, pr.bt, x, stream), dC = output(o, "dC", pr.c, pr.ct, x, stream);
     at::Tensor dD, dz, dbias, dh0;
-    if (pD != nullptr) dD = output(o, "dD", {D}, at::kFloat, x);
+    if (pD != nullptr) dD = output(o, "dD", {D}, at::kFloat, x, stream);
     else no_output(o, "dD");
-    if (pz != nullptr) dz = output(o, "dz", pr.rows, pr.io, x);
+    if (pz != nullptr) dz = output(o, "dz", pr.rows, pr.io, x, stream);
     else no_output(o, "dz");
-    if (fused) dbias = output(o, "ddelta_bias", {D}, at::kFloat, x);
-    if (want_dh0) dh0 = output(o, "dh0", pr.h, at::kFloat, x);
+    if (fused) dbias = output(o, "ddelta_bias", {D}, at::kFloat, x, stream);
+    if (want_dh0) dh0 = output(o, "dh0", pr.h, at::kFloat, x, stream);
     auto data = [](const at::Tensor& t) { return t.defined() ? t.data_ptr() : nullptr; };
     auto fdata = [](const at::Tensor& t) { return t.defined() ? static_cast<float*>(t.data_ptr()) : nullptr; };
     if (fused) {
@@ -406,9 +419,9 @@ PyObject* step(PyObject*, PyObject* const* a, Py_ssize_t n) {
     auto* pD = static_cast<float*>(pointer(a[5], "D_skip", {(int64_t)pr.p.D}, at::kFloat));
     void* pz = pointer(a[6], "z", pr.rows, pr.io);
     auto* ph = static_cast<float*>(pointer(a[7], "h", pr.h, at::kFloat));
-    at::Tensor out = given != nullptr ? *given : empty(pr.rows, pr.io, x);
-    void* po = pointer(&out, "out", pr.rows, pr.io);
     void* stream = stream_of(a[9], x);
+    at::Tensor out = given != nullptr ? *given : result(pr.rows, pr.io, x, stream);
+    void* po = pointer(&out, "out", pr.rows, pr.io);
     call("ssm_step", nullptr, [&] {
         return api.ssm_step(&pr.p, px, pd, pA, pB, pC, pD, pz, ph, po, stream);
       });
@@ -439,9 +452,9 @@ PyObject* conv_fwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     auto* pb = static_cast<float*>(pointer(a[2], "bias", {D}, at::kFloat));
     void* pp = pointer(a[3], "x_prev", {(int64_t)p.batch, W - 1, D}, io);
     const at::Tensor* given = tensor(a[4], "y");
-    at::Tensor y = given != nullptr ? *given : empty(x.sizes(), io, x);
-    void* py = pointer(&y, "y", x.sizes(), io);
     void* stream = stream_of(a[5], x);
+    at::Tensor y = given != nullptr ? *given : result(x.sizes(), io, x, stream);
+    void* py = pointer(&y, "y", x.sizes(), io);
     call("ssm_conv1d_fwd", nullptr, [&] {
         return api.ssm_conv1d_fwd(&p, px, pw, pb, pp, py, stream);
       });
@@ -467,10 +480,10 @@ PyObject* conv_bwd(PyObject*, PyObject* const* a, Py_ssize_t n) {
     auto* pb = static_cast<float*>(pointer(a[2], "bias", {D}, at::kFloat));
     void* pp = pointer(a[3], "x_prev", {(int64_t)p.batch, W - 1, D}, io);
     void* pg = pointer(a[4], "dy", x.sizes(), io);
-    at::Tensor dx = output(o, "dx", x.sizes(), io, x), dw = output(o, "dw", {D, W}, at::kFloat, x), db, dp;
-    if (pb != nullptr) db = output(o, "dbias", {D}, at::kFloat, x);
+    at::Tensor dx = output(o, "dx", x.sizes(), io, x, stream), dw = output(o, "dw", {D, W}, at::kFloat, x, stream), db, dp;
+    if (pb != nullptr) db = output(o, "dbias", {D}, at::kFloat, x, stream);
     else no_output(o, "dbias");
-    if (truth(a[8]) && W > 1) dp = output(o, "dx_prev", {(int64_t)p.batch, W - 1, D}, io, x);
+    if (truth(a[8]) && W > 1) dp = output(o, "dx_prev", {(int64_t)p.batch, W - 1, D}, io, x, stream);
     const Workspace own = workspace(api.ssm_conv1d_bwd_workspace_bytes(&p), x, stream);
     const at::Tensor& ws = own.buffer;
     call("ssm_conv1d_bwd", own.enqueue, [&] {

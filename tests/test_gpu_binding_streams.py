@@ -57,3 +57,26 @@ def test_the_buffer_of_a_stream_is_a_block_of_that_stream():
     at = K.last_bwd_workspace("cuda", s).data_ptr()
     owner = [seg["stream"] for seg in torch.cuda.memory_snapshot() if seg["address"] <= at < seg["address"] + seg["total_size"]]
     assert owner == [s.cuda_stream]
+
+
+def test_a_result_that_is_dropped_is_not_handed_on_while_the_call_still_writes_to_it():
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    x = torch.randn(2, 500, 64, device="cuda")
+    w = torch.randn(64, 4, device="cuda")
+    s = torch.cuda.Stream()
+    K.ssm_conv1d_fwd(x, w, stream=s)                 # (everything set up)
+    run = _call(500)
+    run(stream=s)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(200_000_000)               # the calls below wait behind this, a tenth of a second
+    y = K.ssm_conv1d_fwd(x, w, stream=s)
+    g = run(stream=s)
+    gone = {t.data_ptr() for t in (y, *g.values()) if t is not None}
+    shapes = [(t.shape, t.dtype) for t in (y, *g.values()) if t is not None]
+    assert not s.query()
+    del y, g
+    new = [torch.empty(shape, dtype=dtype, device="cuda") for shape, dtype in shapes]
+    assert not s.query() and not {t.data_ptr() for t in new} & gone
+    torch.cuda.synchronize()
