@@ -177,6 +177,12 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
       float* const fB = sBuf + 3 * SM::kTile;
       float* const fC = fB + kLB * NP;
       const int live = t_end - t0;
+      if (live < kLB) {   // rows past the end are identity steps (below), and zero times infinity is not zero
+#pragma unroll
+        for (int i = 0; i < NG; ++i)
+          if ((lane + 32 * i) / (4 * NG) >= live) qB[i].zero();
+        rx.zero_from(live, lane);
+      }
       rd.put(td, lane);
       rx.put(tx, lane);
       if constexpr (READ) rz.put(tz, lane);
@@ -208,7 +214,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
         for (int t = 0; t < kLB; ++t) dt[t] = lane_softplus<IO>(dt[t]);
       }
-      if (live < kLB) {   // rows past the end are identity steps
+      if (live < kLB) {
 #pragma unroll
         for (int t = 0; t < kLB; ++t) dt[t] = t < live ? dt[t] : 0.f;
       }

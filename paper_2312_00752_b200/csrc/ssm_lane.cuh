@@ -64,6 +64,7 @@ struct LaneQuad;
 template <>
 struct LaneQuad<float> {
   float4 v;
+  __device__ __forceinline__ void zero() { v = make_float4(0.f, 0.f, 0.f, 0.f); }
   __device__ __forceinline__ void load(const float* p, int n, bool vec) {
     v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (n >= 4 && vec) {
@@ -80,6 +81,7 @@ struct LaneQuad<float> {
 template <>
 struct LaneQuad<__nv_bfloat16> {
   uint2 v;
+  __device__ __forceinline__ void zero() { v = make_uint2(0u, 0u); }
   __device__ __forceinline__ void load(const __nv_bfloat16* p, int n, bool vec) {
     v = make_uint2(0u, 0u);
     if (n >= 4 && vec) {
@@ -144,6 +146,18 @@ struct LaneRows {
     } else {
 #pragma unroll
       for (int t = 0; t < kLB; ++t) r[t] = RawT(0);
+    }
+  }
+  // rows `live` .. of the batch
+  __device__ __forceinline__ void zero_from(int live, int lane) {
+    if constexpr (VEC) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+        if ((lane + 32 * i) / VPR >= live) v[i] = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+#pragma unroll
+      for (int t = 0; t < kLB; ++t)
+        if (t >= live) r[t] = RawT(0);
     }
   }
   // into the tile [kLB][32] (VEC only)

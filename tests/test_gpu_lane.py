@@ -103,3 +103,28 @@ def test_complex_edges(batch, L, D, N, io):
             assert U.rel_err(U.to_host(g[k]), ref[k]) <= U.TOL[io]["grad"], (k, sv is None)
         for k in ("dA", "dB", "dC"):
             assert _cerr(_c(g[k]), ref[k]) <= U.TOL[io]["grad"], (k, sv is None)
+
+
+@pytest.mark.parametrize("which", ["x", "B"])
+@pytest.mark.parametrize("batch,L,D,N,io", [
+    (1, 33, 40, 16, "f32"),        # one step in the last batch of 8
+    (1, 33, 41, 16, "bf16"),       # odd width
+    (2, 61, 17, 64, "bf16"),       # four groups of states
+    (1, 299, 24, 4, "f32"),        # cut in time
+    (1, 33, 9480, 16, "bf16"),     # the tuned kernels
+])
+def test_an_infinite_input_of_the_last_step_stays_infinite(batch, L, D, N, io, which):
+    """Rows past the end of a ragged batch are identity steps: zero times what they hold must not make NaN of the state."""
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("inf", 31, batch, L, D, N, io, 1e-3, 1e-1), seed=L), io)
+    dev["x"][:, -1].abs_().clamp_(min=0.5)
+    dev["B"][:, -1].abs_().clamp_(min=0.5)
+    args = lambda: (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    h_last = torch.empty(batch, D, N, device="cuda")
+    before = K.ssm_scan_fwd(*args())
+    dev[which] = dev[which].clone()
+    dev[which][:, -1] = float("inf")
+    out = K.ssm_scan_fwd(*args(), h_last=h_last)
+    assert bool((h_last == float("inf")).all())
+    assert torch.equal(out[:, :-1], before[:, :-1])
