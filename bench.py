@@ -152,13 +152,22 @@ def job_value(elements_per_rank: int, world: int, ms_per_step: float) -> float:
     return world * elements_per_rank / (ms_per_step * 1e-3)
 
 
-def kernels_per_step(plan_info: dict, bwd_plan_info: dict) -> int:
-    """Kernel launches of one fwd (saving states) + bwd (given saved states) pass; each direction splits the sequence
-    in time on its own terms."""
-    fwd = 1 if plan_info["n_segments"] == 1 else 3        # [summary, carry,] forward
-    # [adjoint pre-pass, carry (not with two segments: the pre-pass writes the inflow itself),] backward, reduction
-    bwd = {1: 2, 2: 3}.get(bwd_plan_info["n_segments"], 4)
-    return fwd + bwd
+def kernels_per_step(torch, step) -> int:
+    """Launches of the library's kernels in one step, counted: the step is captured into a graph (and not run) and the
+    graph's kernel nodes are listed."""
+    import tempfile
+    import warnings
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    graph.enable_debug_mode()
+    with torch.cuda.graph(graph):
+        step()
+    with tempfile.TemporaryDirectory() as d:
+        path = os.path.join(d, "graph.dot")
+        with warnings.catch_warnings():
+            warnings.simplefilter("ignore")
+            graph.debug_dump(path)
+        with open(path) as f:
+            return sum("ssm_" in row and "_kernel" in row for row in f)
 
 
 def workload_name(cfg) -> str:
@@ -290,7 +299,7 @@ def time_shape(K, torch, dev, stream, cfg, peak, general_A=False, reps=None, zoh
     res = {"workload": f"config {cfg.cfg_id}: batch {cfg.batch}, L {cfg.L}, D {cfg.D}, N {cfg.N}, {cfg.io} io" +
                        (", A perturbed (no arithmetic progression: one exponential per state)" if general_A else "") +
                        (", zero-order-hold B-bar (SSM_FLAG_ZOH_BBAR)" if zoh else "") +
-                       (", complex state with S4D-Lin A (SSM_FLAG_COMPLEX; plain kernels)" if complex_state else "") +
+                       (", complex state with S4D-Lin A (SSM_FLAG_COMPLEX)" if complex_state else "") +
                        (", B and C as parameters (SSM_FLAG_STATIC_B | SSM_FLAG_STATIC_C)" if static_bc else ""),
            "fwd_ms": f, "bwd_ms": b, "fwd_elements_per_s": cfg.elements / (f * 1e-3),
            "bwd_elements_per_s": cfg.elements / (b * 1e-3), "step_elements_per_s": cfg.elements / ((f + b) * 1e-3),
@@ -338,13 +347,13 @@ def run_ours(args, cfg):
              "dA": torch.empty_like(d0["A"]), "dD": torch.empty_like(d0["D_skip"])}
     stream = torch.cuda.current_stream(dev)
 
-    def fwd(s):
+    def fwd(s, on=stream):
         K.ssm_scan_fwd(s["x"], s["delta"], s["A"], s["B"], s["C"], s["D_skip"], s["z"], save_states=True, out=out,
-                       saved_states=saved, stream=stream)
+                       saved_states=saved, stream=on)
 
-    def bwd(s):
+    def bwd(s, on=stream):
         K.ssm_scan_bwd(s["x"], s["delta"], s["A"], s["B"], s["C"], s["D_skip"], s["z"], s["dout"], saved,
-                       outputs=grads, stream=stream)
+                       outputs=grads, stream=on)
 
     def barrier():
         if world > 1:
@@ -437,7 +446,7 @@ def run_ours(args, cfg):
                    "plan": plan_info, "bwd_plan": bwd_plan_info,
                    "parallelism": "replicas" if world > 1 else "single"},
         "clocks": clocks,
-        "gpu_launches": kernels_per_step(plan_info, bwd_plan_info) * args.steps,
+        "gpu_launches": kernels_per_step(torch, lambda: (fwd(d0, None), bwd(d0, None))) * args.steps,
         "fwd": {"ms": f_ms, "elements_per_s": cfg.elements / (f_ms * 1e-3), "algorithmic_bytes": fwd_bytes,
                 "achieved_gbs": fwd_gbs, "frac_of_hbm_peak": fwd_gbs / peak, **alu_fracs("fwd", f_ms),
                 "traffic": NCU_TRAFFIC_BYTES_FWD.get(cfg.cfg_id) if not args.general_A else None},
@@ -445,7 +454,7 @@ def run_ours(args, cfg):
                 "achieved_gbs": bwd_gbs, "frac_of_hbm_peak": bwd_gbs / peak, **alu_fracs("bwd", b_ms)},
         "roofline": {"bound": "hbm", "binding_bound": "alu (FP32 lanes; see roofline_alu)",
                      "kernel": "ssm_scan_bwd call (ssm_bwd_warp_kernel, the dominant kernel, timed together with the "
-                               "adjoint pre-pass and reduction kernels of the same call)",
+                               "adjoint pre-pass, carry and reduction kernels of the same call)",
                      "achieved": bwd_gbs, "peak": peak, "peak_kind": f"{peak_kind} copy bandwidth",
                      "unit": "GB/s", "frac": bwd_gbs / peak,
                      "traffic": NCU_TRAFFIC_BYTES.get(cfg.cfg_id) if not args.general_A else None,
@@ -568,7 +577,7 @@ def run_ours(args, cfg):
             except Exception as exc:
                 line["variants"][name] = {"error": str(exc)}
         # other state sizes at the same (batch, L, D): N = 8 (bf16: the 16-state kernels on a widened problem) and
-        # N = 64 at a quarter of the batch (generic kernels)
+        # N = 64 at a quarter of the batch (lane kernels)
         for name, small in (("state_8", cfg.scaled(N=8)), ("state_64_batch_1", cfg.scaled(N=64, batch=1))):
             try:
                 line["variants"][name] = time_shape(K, torch, dev, stream, small, peak, reps=5)
