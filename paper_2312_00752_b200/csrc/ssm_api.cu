@@ -11,6 +11,7 @@ int fwd_channels_per_block(int N);
 int bwd_channels_per_block(int N);
 bool complex_supported(const ssm_problem_t& p);
 size_t complex_bwd_workspace_bytes(const ssm_problem_t& p);
+Plan complex_bwd_plan(const ssm_problem_t& p);
 size_t complex_saved_state_bytes(const ssm_problem_t& p);
 cudaError_t complex_fwd(const ssm_problem_t& prob, const void* x, const void* delta, const float* A, const void* B,
                         const void* C, const float* D_skip, const void* z, const float* h0, void* out, float* h_last,
@@ -200,7 +201,7 @@ Plan make_plan(const ssm_problem_t& p) {
   const long long sub_partitions = 4LL * kNumSMs;
   int nseg = 1;
   if (p.flags & SSM_FLAG_COMPLEX) {
-    // the complex path does not split time
+    // (forward: cut inside clusters only)
   } else if (lane_fwd(p)) {
     nseg = lane_segments(p);
   } else if (tuned_shape(p)) {
@@ -275,9 +276,7 @@ Plan make_bwd_plan(const ssm_problem_t& p) {
   const long long chains = (long long)p.batch * pl.bwd_groups;
   const long long resident = 4LL * kNumSMs;
   int nseg = 1;
-  if (p.flags & SSM_FLAG_COMPLEX) {
-    // the complex path does not split time
-  } else if (tuned_shape(p)) {
+  if (tuned_shape(p)) {
     nseg = tuned_bwd_segments(p);
   } else if (chains * generic_bwd_warps(p.N) < 4 * resident) {
     // generic kernel: latency-bound warps, so aim for 8 per sub-partition (measured against 2: 1.1 to 1.5 times faster)
@@ -509,7 +508,7 @@ ssm_status_t ssm_scan_plan(const ssm_problem_t* p, int32_t* n_segments, int32_t*
   if (n_segments) *n_segments = pl.nseg;
   if (segment_steps) *segment_steps = pl.seg_steps;
   if (channels_per_block) *channels_per_block = pl.fwd_ch;
-  if (states_per_thread) *states_per_thread = lane_fwd(*p) ? 16 : tuned_shape(*p) ? fwd_states_per_thread() : (p->N < 4 ? p->N : 4);
+  if (states_per_thread) *states_per_thread = lane_fwd(*p) ? 16 : (p->flags & SSM_FLAG_COMPLEX) ? 8 : tuned_shape(*p) ? fwd_states_per_thread() : (p->N < 4 ? p->N : 4);
   return SSM_OK;
 }
 
@@ -519,7 +518,7 @@ ssm_status_t ssm_scan_bwd_plan(const ssm_problem_t* p, int32_t* n_segments, int3
   if (st != SSM_OK) return st;
   ssm_problem_t wide;
   if (widen_route(*p, &wide)) return ssm_scan_bwd_plan(&wide, n_segments, segment_steps, channels_per_group);
-  const Plan pl = make_bwd_plan(*p);
+  const Plan pl = (p->flags & SSM_FLAG_COMPLEX) ? complex_bwd_plan(*p) : make_bwd_plan(*p);
   if (n_segments) *n_segments = pl.nseg;
   if (segment_steps) *segment_steps = pl.seg_steps;
   if (channels_per_group) *channels_per_group = pl.bwd_ch;

@@ -134,6 +134,8 @@ bool complex_supported(const ssm_problem_t& p) {
   return p.N <= 32 && (p.flags & not_with) == 0;
 }
 
+Plan complex_bwd_plan(const ssm_problem_t& p) { return cplx_bwd_plan(p); }
+
 size_t complex_bwd_workspace_bytes(const ssm_problem_t& p) { return cplx_layout(p, cplx_bwd_plan(p)).total; }
 
 size_t complex_saved_state_bytes(const ssm_problem_t& p) {

@@ -72,6 +72,16 @@ def test_complex_state_queries_and_refused_combinations():
     assert lib.ssm_scan_plan(ctypes.byref(_prob(2, 100, 64, N=64, flags=3 | K.SSM_FLAG_COMPLEX)), None, None, None, None) == 2
 
 
+def test_the_backward_plan_of_a_complex_state_is_the_one_that_runs():
+    p = _prob(2, 1237, 1001, N=8, flags=3 | K.SSM_FLAG_COMPLEX)
+    pl, wide = K.bwd_plan(p), K.bwd_plan(_prob(2, 1237, 1001, N=16))     # (8 complex states are 16 columns)
+    assert pl == wide and pl["n_segments"] > 1 and pl["n_segments"] * pl["segment_steps"] >= 1237
+    one = _prob(2, 64, 1001, N=8, flags=3 | K.SSM_FLAG_COMPLEX)
+    assert K.bwd_plan(one)["n_segments"] == 1
+    # what leaves a segment (16 rows and a sum of step sizes for 32 groups of 32 channels) lies in the workspace
+    assert K.bwd_workspace_bytes(p) > 2 * pl["n_segments"] * 32 * 32 * 17 * 4
+
+
 def test_null_misaligned_and_workspace_errors_before_launch():
     lib = K.load_library()
     p = _prob()
