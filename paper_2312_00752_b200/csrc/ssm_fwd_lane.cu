@@ -181,10 +181,17 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
 #pragma unroll
         for (int i = 0; i < NG; ++i)
           if ((lane + 32 * i) / (4 * NG) >= live) qB[i].zero();
-        rx.zero_from(live, lane);
+        if constexpr (!VEC) rx.zero_from(live);
       }
       rd.put(td, lane);
       rx.put(tx, lane);
+      if constexpr (VEC) {
+        if (live < kLB) {
+          __syncwarp();
+#pragma unroll 1
+          for (int t = live; t < kLB; ++t) tx[t * 32 + lane] = float_to_io<IO>(0.f);
+        }
+      }
       if constexpr (READ) rz.put(tz, lane);
 #pragma unroll
       for (int i = 0; i < NG; ++i) {

@@ -148,17 +148,11 @@ struct LaneRows {
       for (int t = 0; t < kLB; ++t) r[t] = RawT(0);
     }
   }
-  // rows `live` .. of the batch
-  __device__ __forceinline__ void zero_from(int live, int lane) {
-    if constexpr (VEC) {
+  // rows `live` .. of the batch (not VEC: they are zeroed in the tile there)
+  __device__ __forceinline__ void zero_from(int live) {
 #pragma unroll
-      for (int i = 0; i < NV; ++i)
-        if ((lane + 32 * i) / VPR >= live) v[i] = make_uint4(0u, 0u, 0u, 0u);
-    } else {
-#pragma unroll
-      for (int t = 0; t < kLB; ++t)
-        if (t >= live) r[t] = RawT(0);
-    }
+    for (int t = 0; t < kLB; ++t)
+      if (t >= live) r[t] = RawT(0);
   }
   // into the tile [kLB][32] (VEC only)
   __device__ __forceinline__ void put(IO* tile, int lane) const {
