@@ -75,7 +75,7 @@ static int tuned_bwd_segments(const ssm_problem_t& p) {
 // with so few chains that the split inside a cluster is faster: below, both sides' run times are estimated in cycles (a
 // lone tuned warp takes 178 cycles per forward step, a lone lane warp about 205; 890 and 1037 backward; the rest is measured
 // launch and fold overhead).  Measured at batch 1, D = 1536, L = 333, forward, A trained and step size fused: 56 us with
-// the tuned kernel (one warp walks the 333 steps of each chain), 17 us with the lane kernel; the lines meet near
+// the tuned kernel (one warp walks the 333 steps of each chain), 16 us with the lane kernel; the lines meet near
 // chains * L = 2^18 .. 2^20.
 static bool lane_shape(const ssm_problem_t& p) {
   if (p.flags & (SSM_FLAG_COMPLEX | SSM_FLAG_ZOH_BBAR | SSM_FLAG_STATIC_B | SSM_FLAG_STATIC_C)) return false;

@@ -15,11 +15,13 @@
 // piece to the first.  That is for little work (one launch); with more, the launch is cut into segments that fill whole
 // waves and the first sweep is a kernel of its own at four warps per sub-partition instead of two (plan_lane_bwd).
 //
-// Bound: instruction issue and latency at two warps per sub-partition (255 registers; 315 warp instructions per warp and
-// step with one exponential per state, 0.43 issued per cycle), and the instruction cache: a block's body is near its size
-// (at 340 instructions per step the time was a fifth longer), hence rolled loops around it.  Measured against the generic
-// kernel, backward call: float32 (2, 2048, 1536), N = 16: 485 -> 193 us; bf16 (3, 1237, 1001): 430 -> 134 us; bf16
-// (1, 2048, 5120), N = 64: 3003 -> 860 us; float32 (1, 256, 64): 207 -> 16 us.
+// Bound (counters): latency at two warps per sub-partition (255 registers).  Issue slots 40 to 44 % in use, FMA pipe 31 to
+// 46 %, special-function unit 11 to 35 %; per issued instruction a warp waits 1.0 to 1.2 cycles for fixed latencies, 0.6 to
+// 0.9 for shared memory and special functions and, a block's body being near the size of the instruction cache, 0.2
+// (float32, N = 64) to 0.7 (bf16 rows at odd addresses, complex states) for instructions, hence rolled loops around it;
+// 315 warp instructions per warp and step at float32 (2, 2048, 1536).  Measured against the generic
+// kernel, backward call: float32 (2, 2048, 1536), N = 16: 485 -> 177 us; bf16 (3, 1237, 1001): 430 -> 127 us; bf16
+// (1, 2048, 5120), N = 64: 3003 -> 831 us; float32 (1, 256, 64): 207 -> 16 us.
 #include <type_traits>
 
 #include "ssm_lane.cuh"

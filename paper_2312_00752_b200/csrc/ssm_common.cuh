@@ -29,7 +29,7 @@ struct LaneSplit {
 };
 struct Plan {
   int nseg;        // time segments per sequence (1: a thread sweeps the whole sequence)
-  int seg_steps;   // steps per segment (multiple of kSegAlign; the last segment may be shorter)
+  int seg_steps;   // steps per segment (multiple of kSegAlign, lane backward of kCkptSteps; the last segment may be shorter)
   int nck;         // checkpoints per sequence = ceil(L / kCkptSteps)
   int fwd_cpt;     // channels per thread, forward
   int fwd_ch;      // channels per block, forward
@@ -180,7 +180,7 @@ cudaError_t kernel_limits(const void* kernel, int threads, size_t smem, KernelLi
 // Programmatic dependent launch: a kernel launched by launch_dependent is set up while the kernel before it in the stream is
 // still running; dependency_wait, the first thing such a kernel does, waits until that one has completed and its writes are
 // visible.  That takes the launch gap out: a decoding step of 64 sequences at D = 5120 (7.9 us on the GPU) 10.2 -> 7.4 us a
-// call, training of a float32 (1, 256, 64) problem (three kernels) 29.7 -> 24.7, the convolution both ways 95.5 -> 88.
+// call, training of a float32 (1, 256, 64) problem (three kernels) 29.7 -> 24.7, the convolution both ways 95.5 -> 92.
 // (Letting the next kernel's blocks in before the last ones here are done, with griddepcontrol.launch_dependents, was
 // slower: they take the places that fall free first, and the grid ends up unevenly spread over the SMs; float32
 // (2, 2048, 1536) 265 -> 295 us against 255 without.)

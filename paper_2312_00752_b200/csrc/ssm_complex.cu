@@ -17,9 +17,12 @@
 //
 // Forward and backward run in the lane kernels (ssm_fwd_lane.cu, ssm_bwd_lane.cu): the arrays are those of a real problem
 // with 2 N columns, and what differs is the arithmetic on a pair.  The forward splits a chain in time inside a cluster only,
-// the backward also into segments.  The bound is the special-function unit: an ex2, a sine and a cosine per state and step are 24 cycles of a
-// warp, 384 at N = 16, in every sweep.  Measured at bf16 (2, 2048, 1536), N = 16, against kernels with a thread per 4
-// states and no time split: forward 784 -> 226 us, backward call 1970 -> 510 us.  Here: the calls, and the kernel of the single step.
+// the backward also into segments.  The bound is the special-function unit in the forward and the adjoint pre-pass (68 and
+// 72 % busy: an ex2, a sine and a cosine per state and step are 24 cycles of a warp, 384 at N = 16, in every sweep), latency
+// and the instruction cache in the main kernel of the backward (35 %).  Measured at bf16 (2, 2048, 1536), N = 16, against
+// kernels with a thread per 4 states and no time split: forward 784 -> 222 us, backward call 1970 -> 513 us (the main kernel
+// takes 383 to 409 us from build to build, its body lying at the edge of the instruction cache).  Here: the calls, and the
+// kernel of the single step.
 #include "ssm_common.cuh"
 #include "ssm_lane.cuh"
 

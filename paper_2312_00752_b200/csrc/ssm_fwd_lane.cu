@@ -5,12 +5,14 @@
 // thread.  With N > 16 the groups of 16 states of a batch run one after the other, their state parked in shared memory;
 // everything that belongs to the channel (step size, input, gate, rounding) is done once.
 //
-// Bound: instruction issue (80 warp instructions per warp and step, 0.4 issued per cycle by a lone warp of a
-// sub-partition) and, with one exponential per state, the special-function unit (16 ex2 = 128 cycles per warp and step),
-// so the registers are capped for three warps per sub-partition and a chain is split in time until they are there.
-// Measured against the generic kernel with its summary and carry launches: float32 (2, 2048, 1536), N = 16: 262 -> 76 us;
-// bf16 (3, 1237, 1001), N = 16: 268 -> 51 us; bf16 (1, 2048, 5120), N = 64: 1204 -> 348 us; float32 (1, 256, 64):
-// 126 -> 7 us.
+// Bound (counters): with one exponential per state the special-function unit, 70 % busy at float32 (2, 2048, 1536), 66 %
+// at bf16 (3, 1237, 1001), 68 % with complex states at (2, 2048, 1536); with two per group of 16 (bf16 (1, 2048, 5120),
+// N = 64) latency: FMA pipe and issue slots 49 %, special-function unit 15 %, a warp waits 1.1 cycles per instruction
+// for fixed latencies.  The issue slots are 43 to 49 % in use.  So the registers are capped for three warps per
+// sub-partition and a chain is split in time until they are there.
+// Measured against the generic kernel with its summary and carry launches: float32 (2, 2048, 1536), N = 16: 262 -> 75 us;
+// bf16 (3, 1237, 1001), N = 16: 268 -> 49 us; bf16 (1, 2048, 5120), N = 64: 1204 -> 347 us (472 us with A off the
+// progression); float32 (1, 256, 64): 126 -> 7.6 us.
 #include <type_traits>
 
 #include "ssm_lane.cuh"
@@ -280,9 +282,10 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 3) ssm_fwd_lane_kernel(const 
             }
           }
           // general A: the exponentials of a step are taken AH steps ahead of its recurrence, between the multiply-adds of
-          // the steps before it (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1, 4, 5): a batch of
-          // exponentials ahead of a batch of recurrences left the FMA pipe idle during the one and the special-function
-          // unit during the other (bf16 (1, 2048, 5120), N = 64: 394 -> 348 us; complex is fastest two steps ahead)
+          // the steps before it (complex: pairs k and k + 2 are real and imaginary parts, k = 0, 1, 4, 5).  Four steps'
+          // exponentials ahead of four recurrences are no slower, since the other warps of the sub-partition fill in
+          // (float32 (2, 2048, 1536) 73.8 us against 74.7, bf16 (1, 2048, 5120), N = 64, trained A 476.7 against 473.6); two
+          // steps ahead are worth 1 % in complex states (222.8 -> 220.5 us) and nothing elsewhere
           constexpr int AH = CPLX ? 2 : 1, NA = AH + 1;
           float2 aN[NA][8], bxN[2][8], CvN[2][READ ? 8 : 1];
           auto exps = [&](int t, float2 (&a)[8]) {
