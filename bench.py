@@ -29,10 +29,9 @@ if ROOT not in sys.path:
 METRIC = "selective-scan fwd+bwd elements/s (elements = batch*L*D); achieved HBM GB/s as % of measured B200 peak"
 FALLBACK_HBM_GBS = 6650.0
 # DRAM bytes (read + write) of one launch of the dominant kernel of each direction from ncu captures at the bench
-# workload itself (profiles/ssm_bwd_warp_kernel_mamba2p8b_layer.md, profiles/ssm_fwd_warp_kernel_mamba2p8b_layer.md);
-# None where no capture exists.
-NCU_TRAFFIC_BYTES = {3: 705.4e6 + 395.6e6}
-NCU_TRAFFIC_BYTES_FWD = {3: 265.7e6 + 368.4e6}
+# workload's shape (profiles/kernel_counters_by_case.md); None where no capture exists.
+NCU_TRAFFIC_BYTES = {3: 704.7e6 + 396.1e6}
+NCU_TRAFFIC_BYTES_FWD = {3: 264.6e6 + 366.7e6}
 
 
 def parse_args():
