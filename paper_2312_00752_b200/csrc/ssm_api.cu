@@ -53,12 +53,21 @@ static bool tuned_shape(const ssm_problem_t& p) {
 }
 // Checkpoint states are tiled by groups of 32 channels whenever a channel's states are whole 16-byte quads.
 static bool ckpt_tiled(const ssm_problem_t& p) { return p.N % 4 == 0 && !(p.flags & SSM_FLAG_COMPLEX); }
-// Time segments of the tuned forward: one warp per chain of 32 channels; a split costs half a forward sweep more, so only
-// when fewer than half of the sub-partitions would have a warp, and then into two rounds of chains.
+// Time segments of the tuned forward: one warp per chain of 32 channels.  A split costs a summary sweep over all segments but
+// the last, so only where the chains alone leave much of the GPU empty: below half of the sub-partitions into two rounds of
+// chains; above, into four segments, which fill every sub-partition with two warps, when that is estimated shorter (in steps
+// of a lone warp: 1.31 times the share of the sub-partitions that have a chain and 290 for three more launches, 1.24 and 150
+// with the fused step size).  Measured, whole calls, D = 1536, batch 8 (share 0.65): L = 2048 167 -> 158 us, with A trained
+// 228 -> 218, and the step size fused 306 -> 270; L = 1024 would go 87 -> 91, 116 -> 122, 157 -> 150; D = 960, batch 10
+// (0.51), L = 2048: 168 -> 142, 228 -> 197, 307 -> 245.
 static int tuned_fwd_segments(const ssm_problem_t& p) {
   const int cw = fwd_fast_channels_per_warp();
   const long long chains = (long long)p.batch * ((p.D + cw - 1) / cw), sub_partitions = 4LL * kNumSMs;
-  if (2 * chains >= sub_partitions) return 1;
+  if (2 * chains >= sub_partitions) {
+    const bool fused = p.flags & SSM_FLAG_DELTA_SOFTPLUS;
+    const float share = (float)chains / (float)sub_partitions, steps = (float)p.L;
+    return share * steps * (fused ? 1.24f : 1.31f) + (fused ? 150.f : 290.f) < steps ? 4 : 1;
+  }
   const long long want = (2 * sub_partitions + chains - 1) / chains;
   return (int)std::min<long long>(std::min<long long>(want, std::max(1, p.L / 256)), 65535);
 }

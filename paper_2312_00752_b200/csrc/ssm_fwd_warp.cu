@@ -117,7 +117,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MODE == kFwdFull ? 1 : 3)
     const int groups = (D + CW - 1) / CW;
     const int grp = chain % groups;
     const int bs = chain / groups;
-    const int seg = bs % p.nseg, b = bs / p.nseg;
+    const int segs = SUMMARY ? p.nseg - 1 : p.nseg;   // (nobody wants what leaves the last segment)
+    const int seg = bs % segs, b = bs / segs;
     const int d_w = grp * CW;
     const int t_seg0 = seg * p.seg_steps;
     const int t_seg_end = min(p.L, t_seg0 + p.seg_steps);
@@ -549,7 +550,7 @@ cudaError_t launch_variant_w(const Plan& plan, const FwdParams& p, cudaStream_t 
   cudaError_t e;
   if ((e = fwd_occupancy<S, MODE, SP, ZOH, BC, 3>(&sms, &per_sm, &smem)) != cudaSuccess) return e;
   WarpSched sc{};
-  sc.chains = p.batch * plan.nseg * ((p.D + CW - 1) / CW);
+  sc.chains = p.batch * (MODE == kFwdSummary ? plan.nseg - 1 : plan.nseg) * ((p.D + CW - 1) / CW);
   sc.tiles = (plan.seg_steps + kWT - 1) / kWT;
   const bool can_share = p.abort != nullptr && p.flags != nullptr && p.handoff != nullptr;
   const int max_workers = can_share ? p.max_workers : 0;

@@ -92,6 +92,17 @@ def test_tuned_kernels_at_the_edges_of_tiles_groups_and_segments(batch, L, D, fu
     _check(batch, L, D, fused=fused, carry=fused, more=more)
 
 
+@pytest.mark.parametrize("batch,L,D,options", [
+    (2, 1024, 4736, {}),                                  # whole tiles and segments
+    (2, 1030, 4744, dict(carry=True, perturb_A=0.05)),    # ragged tile, group and last segment
+    (2, 1030, 4744, dict(saved=False)),                   # the states rebuilt by the split forward
+    (2, 409, 4744, dict(fused=True, carry=True)),         # a last segment of 25 steps, less than a tile
+    (2, 416, 4736, dict(fused=True, saved=False)),        # ... of one tile
+])
+def test_tuned_forward_split_in_time_with_more_than_half_the_sub_partitions(batch, L, D, options):
+    _check(batch, L, D, more=("ssm_carry",), **options)
+
+
 @pytest.mark.parametrize("options", [
     dict(gate=False), dict(skip=False), dict(gate=False, skip=False), dict(carry=True), dict(carry=True, saved=False),
     dict(perturb_A=0.05), dict(perturb_A=0.05, fused=True, saved=False), dict(fused=True, gate=False, carry=True),
