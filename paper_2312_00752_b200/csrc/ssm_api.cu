@@ -117,6 +117,23 @@ bool lane_bwd(const ssm_problem_t& p) {
   plan_lane_bwd(p, kLaneWarps, &pl, &lane);
   return 1037.f * lane + 20e3f < tuned;
 }
+// The team kernel (ssm_fwd_team.cu) runs a chain of 32 or 64 states in one sweep with N / 16 warps; the lane kernel cuts it in
+// time, sweeps twice, and runs the groups of 16 states one after the other.  So the lane kernel keeps the problems whose
+// teams would leave most of the GPU empty for long, and those without one whole group of 32 channels.  Both sides in steps of the lane estimate: the team takes 0.26 (N = 64)
+// or 0.5 of one per step, whatever the chains, up to a team per SM (two for N = 32), and more in proportion from there.
+// Measured, lane / team, us, N = 64: (1, 2048, 5120) 332 / 201, with A off the progression 460 / 271; (1, 2048, 2560)
+// 201 / 175, (2, 2048, 1024) 139 / 174, (1, 512, 2560) 73 / 47, (1, 1024, 1280) 83 / 89, (1, 300, 1280) 39 / 30, (1, 64, 256)
+// 20 / 12; N = 32: (2, 2048, 5120) 313 / 217, (1, 2048, 5120) 177 / 190, (2, 300, 2560) 38 / 33, (1, 128, 256) 12 / 16.
+static int team_size(const ssm_problem_t& p) { return p.N / 16; }
+bool team_fwd(const ssm_problem_t& p) {
+  if (!lane_shape(p) || p.io_dtype != SSM_BF16 || (p.N != 32 && p.N != 64) || p.D % 8 != 0 || p.D < kLaneChannels) return false;
+  const long long chains = (long long)p.batch * ((p.D + kLaneChannels - 1) / kLaneChannels), slots = 4LL * kNumSMs / team_size(p);
+  const float share = (float)chains / (float)slots;
+  float lane = 0.f;
+  choose_lane_split(chains, p.L, 0.75f, 25.f, p.N > 32 ? 2 : 3, kLaneWarps, &lane);
+  const float steps = (float)p.L * std::max(1.f, share);
+  return lane > (p.N == 64 ? 0.26f * steps : 0.5f * steps + 30.f);
+}
 // Time segments of a lane launch.  A chain already spreads over up to 32 warps of a cluster, so the launch itself is
 // split (summary pass, carry, full pass) only for a handful of chains and then into segments of at least 2048 steps.
 static int lane_segments(const ssm_problem_t& p) {
@@ -211,6 +228,8 @@ Plan make_plan(const ssm_problem_t& p) {
   int nseg = 1;
   if (p.flags & SSM_FLAG_COMPLEX) {
     // (forward: cut inside clusters only)
+  } else if (team_fwd(p)) {
+    // (one sweep)
   } else if (lane_fwd(p)) {
     nseg = lane_segments(p);
   } else if (tuned_shape(p)) {
@@ -310,7 +329,9 @@ struct FwdWorkspace {
 static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
   FwdWorkspace w{};
   const int cw = fwd_fast_channels_per_warp();
-  w.max_workers = tuned_shape(p) && !lane_fwd(p) ? shared_workers((long long)p.batch * pl.nseg * ((p.D + cw - 1) / cw)) : 0;
+  const long long groups = (long long)p.batch * ((p.D + cw - 1) / cw);
+  w.max_workers = tuned_shape(p) && !lane_fwd(p) ? shared_workers(groups * pl.nseg) : 0;
+  if (team_fwd(p) && groups * team_size(p) > 4 * kNumSMs) w.max_workers = 4 * kNumSMs;   // (a hand-off per warp of a team)
   if (pl.nseg == 1 && w.max_workers == 0) {
 #ifdef SSM_DEBUG_BOUNDS
     w.total = kStatusBytes;   // (a place for the status word)

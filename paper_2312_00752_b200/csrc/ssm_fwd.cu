@@ -251,11 +251,15 @@ int fwd_channels_per_block(int N) {
 bool fwd_fast_applicable(const ssm_problem_t& prob, const FwdParams& p);
 cudaError_t launch_fwd_fast(const Plan& plan, const FwdParams& p, int mode, cudaStream_t s);
 bool lane_fwd(const ssm_problem_t& p);
+bool team_fwd(const ssm_problem_t& p);
+bool fwd_team_applicable(const FwdParams& p);
+cudaError_t launch_fwd_team(const ssm_problem_t& prob, const FwdParams& p, cudaStream_t s);
 bool fwd_lane_applicable(const FwdParams& p);
 cudaError_t launch_fwd_lane(const ssm_problem_t& prob, const Plan& plan, const FwdParams& p, int mode, cudaStream_t s);
 
 cudaError_t launch_fwd(const ssm_problem_t& prob, const Plan& plan, const FwdParams& p, int mode, cudaStream_t s) {
   if (!lane_fwd(prob) && fwd_fast_applicable(prob, p)) return launch_fwd_fast(plan, p, mode, s);
+  if (mode != kFwdSummary && team_fwd(prob) && fwd_team_applicable(p)) return launch_fwd_team(prob, p, s);
   if (fwd_lane_applicable(p)) return launch_fwd_lane(prob, plan, p, mode, s);
   if (prob.io_dtype == SSM_BF16) return launch_fwd_io<__nv_bfloat16>(prob, plan, p, mode, s);
   return launch_fwd_io<float>(prob, plan, p, mode, s);

@@ -6,6 +6,7 @@ import sys
 import numpy as np
 
 FWD, BWD, LOCAL, CARRY = "ssm_fwd_warp_kernel", "ssm_bwd_warp_kernel", "ssm_bwd_local_warp_kernel", "ssm_carry"
+TEAM_FWD = "ssm_fwd_team_kernel"
 LANE_FWD, LANE_BWD, LANE_LOCAL = "ssm_fwd_lane_kernel", "ssm_bwd_lane_kernel", "ssm_bwd_lane_local_kernel"
 
 CASES = [  # batch, L, D, N, io, ZOH, the kernels that have to run
@@ -37,6 +38,10 @@ CASES = [  # batch, L, D, N, io, ZOH, the kernels that have to run
     (2, 1237, 1001, 16, "bf16", False, (LANE_FWD, LANE_BWD, LANE_LOCAL)),
     (1, 650, 1300, 32, "f32", False, (LANE_FWD, LANE_BWD, LANE_LOCAL)),
     (1, 90, 24, 64, "bf16", False, (LANE_FWD, LANE_BWD)),
+    # teams of warps: ragged tile and group, chains shared between teams
+    (1, 70, 2568, 64, "bf16", False, (TEAM_FWD, LANE_BWD)),
+    (2, 40, 2568, 64, "bf16", False, (TEAM_FWD, LANE_BWD)),
+    (2, 96, 5128, 32, "bf16", False, (TEAM_FWD, LANE_BWD)),
 ]
 COMPLEX = [  # batch, L, D, N, io, the kernels that have to run
     (1, 63, 36, 1, "f32", (LANE_FWD, LANE_BWD)),

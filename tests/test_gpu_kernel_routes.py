@@ -12,6 +12,7 @@ pytestmark = pytest.mark.gpu
 TUNED = ("ssm_fwd_warp_kernel", "ssm_bwd_warp_kernel")
 LANE = ("ssm_fwd_lane_kernel", "ssm_bwd_lane_kernel")
 GENERIC = ("ssm_fwd_kernel", "ssm_bwd_kernel")
+TEAM = "ssm_fwd_team_kernel"   # forward of 32 or 64 states
 
 
 def _shifted(t):
@@ -65,7 +66,7 @@ def _check(batch, L, D, N=16, io="bf16", *, fwd=TUNED[0], bwd=TUNED[1], more=(),
     got = run()
     K.check_status(K.make_problem(dev["x"], dev["B"], gate, skip, zoh=zoh), K.last_bwd_workspace("cuda"))
     ran = U.kernels(run)
-    assert {k for k in ran if k in TUNED + LANE + GENERIC} == {fwd, bwd}, ran
+    assert {k for k in ran if k in (*TUNED, *LANE, *GENERIC, TEAM)} == {fwd, bwd}, ran
     assert all(any(k.startswith(m) for k in ran) for m in more), ran
     a = (inp["x"], inp["delta"], inp["A"], inp["B"], inp["C"])
     out, h = O.scan_fwd(*a, D_skip=inp["D_skip"], z=inp["z"], h0=h0, return_h_last=True, **okw)
@@ -110,6 +111,27 @@ def test_tuned_forward_split_in_time_with_more_than_half_the_sub_partitions(batc
 @pytest.mark.parametrize("batch,L,D", [(1, 150, 9480), (4, 64, 2560)])   # ragged; whole
 def test_options_on_the_tuned_kernels(batch, L, D, options):
     _check(batch, L, D, **options)
+
+
+@pytest.mark.parametrize("batch,L,D,N,options", [
+    (1, 1, 2568, 64, {}),                                        # a single step; 80 whole groups of channels and one of 8
+    (1, 31, 2560, 64, dict(carry=True)),                         # one step short of a tile
+    (1, 33, 2568, 64, dict(perturb_A=0.05, gate=False)),         # one past it
+    (2, 64, 1280, 64, dict(fused=True, skip=False)),             # whole tiles
+    (2, 75, 2568, 64, dict(carry=True, fused=True)),             # 162 chains for 148 teams: some are shared, ragged tile
+    (2, 160, 2560, 64, dict(perturb_A=0.05, saved=False)),       # ... whole; states rebuilt by the team kernel
+    (3, 40, 2560, 64, dict(saved=False, carry=True)),
+    (2, 70, 2568, 32, dict(carry=True)),                         # 162 chains, two teams per block, a block with one
+    (2, 200, 5128, 32, dict(fused=True, carry=True, perturb_A=0.05)),   # 322 chains for 296 teams
+    (2, 128, 5120, 32, dict(saved=False, gate=False, skip=False)),
+])
+def test_teams_of_warps_for_large_states(batch, L, D, N, options):
+    _check(batch, L, D, N, fwd=TEAM, bwd=LANE[1], **options)
+
+
+def test_large_states_off_the_16_byte_grid_and_of_few_channels_keep_the_lane_kernel():
+    _check(1, 100, 2560, 64, fwd=LANE[0], bwd=LANE[1], off=("fwd",), carry=True)
+    _check(1, 300, 64, 32, fwd=LANE[0], bwd=LANE[1])
 
 
 @pytest.mark.parametrize("N", [1, 2, 4, 8])
