@@ -841,23 +841,34 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
       M[n] = p.mu_in != nullptr && col < N ? p.mu_in[((size_t)b * D + c_ld) * N + col] : 0.f;
     }
     const float* const a = sA + gi * 512 + lane;
+    // (the values of several segments requested before the first is used: one by one the fold took 7000 cycles of a block's
+    // 230000 at 12 segments)
+    constexpr int kAhead = CPLX ? 2 : 4;
 #pragma unroll 1
-    for (int sg = p.nseg - 1; sg > seg; --sg) {
-      const size_t at = ((size_t)b * p.nseg + sg) * groups + grp;
-      const float* const src = p.seg_local + (at * NG + gi) * 512 + lane;
-      const float ds = p.seg_dsum[at * 32 + lane];
-      float l[16];
+    for (int sg = p.nseg - 1; sg > seg; sg -= kAhead) {
+      float l[kAhead][16], ds[kAhead];
 #pragma unroll
-      for (int n = 0; n < 16; ++n) l[n] = src[32 * n];
+      for (int i = 0; i < kAhead; ++i) {
+        const size_t at = ((size_t)b * p.nseg + max(sg - i, seg + 1)) * groups + grp;
+        const float* const src = p.seg_local + (at * NG + gi) * 512 + lane;
+        ds[i] = p.seg_dsum[at * 32 + lane];
 #pragma unroll
-      for (int n = 0; n < 16; ++n) {
-        if constexpr (CPLX) {
-          if (n & 4) continue;
-          const float2 q = cexp_apply<true>(ds, a[32 * n], a[32 * n + 128], make_float2(M[n], M[n + 4]));
-          M[n] = q.x + l[n];
-          M[n + 4] = q.y + l[n + 4];
-        } else {
-          M[n] = fmaf(ex2_approx(a[32 * n] * ds), M[n], l[n]);
+        for (int n = 0; n < 16; ++n) l[i][n] = src[32 * n];
+      }
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) {
+        if (sg - i > seg) {
+#pragma unroll
+          for (int n = 0; n < 16; ++n) {
+            if constexpr (CPLX) {
+              if (n & 4) continue;
+              const float2 q = cexp_apply<true>(ds[i], a[32 * n], a[32 * n + 128], make_float2(M[n], M[n + 4]));
+              M[n] = q.x + l[i][n];
+              M[n + 4] = q.y + l[i][n + 4];
+            } else {
+              M[n] = fmaf(ex2_approx(a[32 * n] * ds[i]), M[n], l[i][n]);
+            }
+          }
         }
       }
     }
@@ -912,31 +923,58 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
       put_quad<CPLX>(fB, lane, qB.widen(), 1.f);
       put_quad<CPLX>(fC, lane, qC.widen(), -1.f);   // (complex: conj C)
       team_sync();   // the rows of all warps of the team have landed
-      // per-step values of the rows, each warp its share: step size, input, gate terms.  (Not unrolled further: the body of a
-      // block is near the size of the instruction cache.)
-#pragma unroll 2
-      for (int i = 0; i < kLB / NG; ++i) {
-        const int t = gi * (kLB / NG) + i;
-        const bool ok = valid && t < live;
-        const float dv = rr.get(rD, t, lane) + bias;
-        float dt = dv, step = 1.f;
-        if (p.softplus) {
-          dt = lane_softplus<IO>(dv);
-          step = sizeof(IO) == 4 ? 1.f / (1.f + __expf(-dv)) : sigmoid_from_softplus(dt);
+      // per-step values of the rows, each warp its share: step size, input, gate terms.  Two rows at a time, their loads and
+      // arithmetic before the first store, which no later load may pass (it was a fifth of a block's time, 2270 of 10700 cycles at
+      // float32 (2, 2048, 1536), with a row's stores before the next row's loads).  Not more, and with complex states one: the
+      // body of a block is near the size of the instruction cache or beyond it (main kernel at float32 (2, 2048, 1536) 133.0 us
+      // before, 130.4 with two rows, 131.0 with four, 133.0 with eight; complex (2, 2048, 1536) 406, 384 with one row, 410 with
+      // two; bf16 (3, 1237, 1001) 97.0, 95.3 with two).
+      constexpr int kOwn = kLB / NG, kAtOnce = CPLX ? 1 : 2;
+      static_assert(kOwn % kAtOnce == 0, "whole groups of rows");
+#pragma unroll 1
+      for (int i0 = 0; i0 < kOwn; i0 += kAtOnce) {
+        const int tb = gi * kOwn + i0;
+        float dt[kAtOnce], uu[kAtOnce], ds[kAtOnce], gp[kAtOnce], step[kAtOnce];
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+          dt[i] = rr.get(rD, tb + i, lane) + bias;
+          uu[i] = rr.get(rX, tb + i, lane);
+          ds[i] = rr.get(rG, tb + i, lane);
+          gp[i] = 0.f;
+          step[i] = 1.f;
         }
-        const float u = rr.get(rX, t, lane);
-        const float g = rr.get(rG, t, lane);
-        float ds = g, gp = 0.f;
         if (has_z) {
-          const float z = rr.get(rZ, t, lane), sg = sigmoid_fast(z);
-          ds = g * z * sg;
-          gp = g * sg * fmaf(z, 1.f - sg, 1.f);
+          float z[kAtOnce];
+#pragma unroll
+          for (int i = 0; i < kAtOnce; ++i) z[i] = rr.get(rZ, tb + i, lane);
+#pragma unroll
+          for (int i = 0; i < kAtOnce; ++i) {
+            const float g = ds[i], sg = sigmoid_fast(z[i]);
+            ds[i] = g * z[i] * sg;
+            gp[i] = g * sg * fmaf(z[i], 1.f - sg, 1.f);
+          }
         }
-        dt = ok ? dt : 0.f;
-        const float uu = ok ? u : 0.f;
-        ds = ok ? ds : 0.f;
-        t1[t * 32 + lane] = make_float4(dt, __shfl_xor_sync(0xffffffffu, dt, 1), uu, __shfl_xor_sync(0xffffffffu, uu, 1));
-        t2[t * 32 + lane] = make_float4(ds, __shfl_xor_sync(0xffffffffu, ds, 1), ok ? gp : 0.f, step);
+        if (p.softplus) {
+#pragma unroll
+          for (int i = 0; i < kAtOnce; ++i) {
+            const float dv = dt[i];
+            dt[i] = lane_softplus<IO>(dv);
+            step[i] = sizeof(IO) == 4 ? 1.f / (1.f + __expf(-dv)) : sigmoid_from_softplus(dt[i]);
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+          const bool ok = valid && tb + i < live;
+          dt[i] = ok ? dt[i] : 0.f;
+          uu[i] = ok ? uu[i] : 0.f;
+          ds[i] = ok ? ds[i] : 0.f;
+          gp[i] = ok ? gp[i] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+          t1[(tb + i) * 32 + lane] = make_float4(dt[i], __shfl_xor_sync(0xffffffffu, dt[i], 1), uu[i], __shfl_xor_sync(0xffffffffu, uu[i], 1));
+          t2[(tb + i) * 32 + lane] = make_float4(ds[i], __shfl_xor_sync(0xffffffffu, ds[i], 1), gp[i], step[i]);
+        }
       }
       team_sync();
       if (t0 > t_begin) {
