@@ -37,7 +37,7 @@ constexpr float kLn2 = 0.6931471805599453f;
 // Shared memory of a block, in bytes: per team the raw rows and the per-step values of a block of 8 steps; per warp B and
 // C of the block, two checkpoints, the transposing buffer (also: tiles of the first sweep, what leaves a piece, dA), the
 // sums over n (N > 16); per chain A * log2(e) and the sums of delta
-template <typename IO, int NG, bool VEC>
+template <typename IO, int NG, bool VEC, bool ROLLED = false>
 struct BwdLaneSmem {
   static constexpr int NP = 16 * NG, kTeams = kLaneWarps / NG;
   static constexpr int kPitch = (VEC || sizeof(IO) == 4) ? 32 * (int)sizeof(IO) : 80;   // bytes of a raw row
@@ -45,7 +45,7 @@ struct BwdLaneSmem {
   static constexpr int kTeam = 4 * kRaw + 2 * kLB * 32 * 16;
   static_assert(2 * kLB * 32 * 16 >= NP * 128, "the totals of a chain fit where the per-step values go");
   static constexpr int kRed = 4 * 32 * 4 * 16;
-  static constexpr int kWarp = 2 * kLB * 16 * 4 + 2 * 4 * 32 * 16 + kRed + (NG > 1 ? kLB * 32 * 16 : 0);
+  static constexpr int kWarp = 2 * kLB * 16 * 4 + 2 * 4 * 32 * 16 + kRed + (NG > 1 ? kLB * 32 * 16 : 0) + (ROLLED ? kLB / 2 * 4 * 32 * 16 : 0);
   static constexpr int kChain = NP * 128 + 128 + kTeams * 128;
   static __host__ __device__ constexpr int bytes(int chains) { return kTeams * kTeam + kLaneWarps * kWarp + chains * kChain + kLaneWarps * 256; }
 };
@@ -215,16 +215,18 @@ __device__ __forceinline__ float3 finish_step(LaneChain& lc, float4 v1, float4 v
   return make_float3(dx, dd, dz);
 }
 
-// One block of 8 steps of one group of 16 states.  t1 / t2: per-step values; fB / fC: rows of 16 states; ck: the states
+// One block of 8 steps of one group of 16 states.  ROLLED: loops over the steps, states after the odd steps in sh
+// [4][vectors as in ck][32] instead of registers.  t1 / t2: per-step values; fB / fC: rows of 16 states; ck: the states
 // before the block; part_dB / part_dC: first row of this block in the partial sums (stride N); emit(t, y, lb, wa, v1, v2)
 // takes the sums over the 16 states for the lane's own channel.
-template <bool AP, bool CPLX, typename Emit>
+template <bool AP, bool CPLX, bool ROLLED, typename Emit>
 __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, const float4* t2, const float* fB, const float* fC,
-                                           const float4* ck, float4* red, float* part_dB, float* part_dC, int N, int n_live,
+                                           const float4* ck, float4* sh, float4* red, float* part_dB, float* part_dC, int N, int n_live,
                                            int live, int lane, Emit&& emit
                                            SSM_DEBUG_ARGS(const float* parts, size_t part_count, int* status)) {
   const int j = lane & 1;
-  float2 hist[kLB / 2][2][4];
+  float2 hist[ROLLED ? 1 : kLB / 2][2][4];
+  constexpr int kUnroll = ROLLED ? 1 : kLB;
   {
     float2 h[2][4];
 #pragma unroll
@@ -235,7 +237,7 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
         h[q][2 * k] = make_float2(v.x, v.y);
         h[q][2 * k + 1] = make_float2(v.z, v.w);
       }
-#pragma unroll
+#pragma unroll kUnroll
     for (int t = 0; t < kLB; ++t) {
       const float4 v = t1[t * 32 + lane];
       float2 Bv[4];
@@ -253,13 +255,25 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           h[q][k] = hn[k];
-          if (t & 1) hist[t >> 1][q][k] = hn[k];
+          if (!ROLLED && (t & 1)) hist[ROLLED ? 0 : t >> 1][q][k] = hn[k];
+        }
+      }
+      if (ROLLED && (t & 1)) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 lo = h[i >> 1][2 * (i & 1)], hi = h[i >> 1][2 * (i & 1) + 1];
+          sh[(t >> 1) * 128 + i * 32 + lane] = make_float4(lo.x, lo.y, hi.x, hi.y);
         }
       }
     }
   }
-#pragma unroll
+#pragma unroll kUnroll
   for (int m = kLB / 2 - 1; m >= 0; --m) {
+    // pair k of channel q of a lane's states, as the checkpoint holds them
+    auto pair_of = [&](const float4* st, int q, int k) {
+      const float4 v = st[(2 * q + (k >> 1)) * 32 + lane];
+      return (k & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+    };
     // ---- odd step 2m + 1: its state is hist[m]; its w = mu h_{t-1} waits for the even step's state
     const int to = 2 * m + 1, te = 2 * m;
     const float4 v1o = t1[to * 32 + lane], v2o = t2[to * 32 + lane];
@@ -280,7 +294,7 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
         float2 yv = make_float2(0.f, 0.f), lb = yv, lam[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const float2 hc = hist[m][q][k];
+          const float2 hc = ROLLED ? pair_of(sh + m * 128, q, k) : hist[ROLLED ? 0 : m][q][k];
           lam[k] = f2fma(Cv[k], ds2, lc.mu[q][k]);
           dCt[k] = q == 0 ? f2mul(ds2, hc) : f2fma(ds2, hc, dCt[k]);
           dBt[k] = q == 0 ? f2mul(lam[k], du2) : f2fma(lam[k], du2, dBt[k]);
@@ -317,12 +331,9 @@ __device__ __forceinline__ void lane_block(LaneChain& lc, const float4* t1, cons
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           // the state before the even step: the history entry before, or the checkpoint
-          if (m > 0) {
-            hpp[k] = hist[m > 0 ? m - 1 : 0][q][k];
-          } else {
-            const float4 v = ck[(2 * q + (k >> 1)) * 32 + lane];
-            hpp[k] = (k & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
-          }
+          if (ROLLED) hpp[k] = pair_of(m > 0 ? sh + (m - 1) * 128 : ck, q, k);
+          else if (m > 0) hpp[k] = hist[!ROLLED && m > 0 ? m - 1 : 0][q][k];
+          else hpp[k] = pair_of(ck, q, k);
           bx[k] = f2mul(du2, Bv[k]);
         }
         lane_mul_add<CPLX>(a, hpp, bx, he);
@@ -581,10 +592,10 @@ __global__ void __launch_bounds__(kLaneWarps * 32, sizeof(IO) == 4 ? 3 : 4) ssm_
 }
 
 // CPLX: complex states, as in ssm_fwd_lane.cu
-template <typename IO, int NG, int ROWS, bool CPLX>
+template <typename IO, int NG, int ROWS, bool CPLX, bool ROLLED>
 __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const BwdParams p, const LaneSplit sp, const int N) {
   constexpr bool VEC = ROWS == kVectors;
-  using SM = BwdLaneSmem<IO, NG, VEC>;
+  using SM = BwdLaneSmem<IO, NG, VEC, ROLLED>;
   constexpr int NP = SM::NP, kTeams = SM::kTeams;
   extern __shared__ __align__(16) unsigned char smem[];
   dependency_wait();
@@ -608,6 +619,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   float4* const ck = reinterpret_cast<float4*>(fC + kLB * 16);   // [2][4][32]
   float4* const red = ck + 2 * 128;
   float4* const ex = red + 4 * 128;                              // NG > 1: [kLB][32]
+  float4* const sh = red + 4 * 128 + (NG > 1 ? kLB * 32 : 0);    // ROLLED: states after the odd steps of a block
   // what leaves piece w of this chain, states 16 gi .. of it: in the transposing buffer of its warp
   auto leaving = [&](int w, int n) {
     return warp_base((sub * W + w) * NG + (n >> 4)) + 2 * kLB * 16 + 2 * 128 * 4 + (n & 15) * 32;
@@ -986,7 +998,7 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
       cp_async_commit();
       auto put = [&](int t, float3 r) { t2[t * 32 + out_slot(t, lane)] = make_float4(r.x, r.y, r.z, 0.f); };
       float* const part_dB = p.dBC_part + (size_t)grp * 2 * bln + row0 * N + 16 * gi;
-      lane_block<AP, CPLX>(lc, t1, t2, fB, fC, ck + st * 128, red, part_dB, part_dB + bln, N, N - 16 * gi, live, lane,
+      lane_block<AP, CPLX, ROLLED>(lc, t1, t2, fB, fC, ck + st * 128, sh, red, part_dB, part_dB + bln, N, N - 16 * gi, live, lane,
                      [&](int t, float y, float lb, float wa, float4 v1, float4 v2) {
                        if constexpr (NG == 1) put(t, finish_step(lc, v1, v2, y, lb, wa, t < live));
                        else ex[t * 32 + lane] = make_float4(y, lb, wa, 0.f);
@@ -1104,16 +1116,10 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
   }
 }
 
-template <typename IO, int NG, int ROWS, bool CPLX>
-cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int mode, cudaStream_t s) {
-  constexpr bool VEC = ROWS == kVectors;
-  using SM = BwdLaneSmem<IO, NG, VEC>;
-  auto kern = ssm_bwd_lane_kernel<IO, NG, ROWS, CPLX>;
-  if (mode == kBwdLocal) {
-    const long long items = (long long)p.batch * (plan.nseg - 1) * ((p.D + 31) / 32) * NG;
-    if (items <= 0) return cudaSuccess;
-    return launch_dependent(ssm_bwd_lane_local_kernel<IO, VEC, CPLX>, (unsigned)((items + kLaneWarps - 1) / kLaneWarps), kLaneWarps * 32, 0, 1, s, p, N, NG);
-  }
+template <typename IO, int NG, int ROWS, bool CPLX, bool ROLLED>
+cudaError_t launch_bwd_lane_main(const Plan& plan, const BwdParams& p, int N, cudaStream_t s) {
+  using SM = BwdLaneSmem<IO, NG, ROWS == kVectors, ROLLED>;
+  auto kern = ssm_bwd_lane_kernel<IO, NG, ROWS, CPLX, ROLLED>;
   const long long chains = (long long)p.batch * plan.nseg * ((p.D + 31) / 32);
   const LaneSplit sp = plan.split;
   const int per_block = SM::kTeams / sp.warps;
@@ -1121,6 +1127,27 @@ cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int m
   const cudaError_t e = kernel_limits(reinterpret_cast<const void*>(kern), 32 * kLaneWarps, SM::bytes(SM::kTeams), &lim);
   if (e != cudaSuccess) return e;
   return launch_dependent(kern, (unsigned)((chains + per_block - 1) / per_block * sp.cluster), 32 * kLaneWarps, SM::bytes(per_block), sp.cluster, s, p, sp, N);
+}
+
+template <typename IO, int NG, int ROWS, bool CPLX>
+cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int mode, cudaStream_t s) {
+  if (mode == kBwdLocal) {
+    const long long items = (long long)p.batch * (plan.nseg - 1) * ((p.D + 31) / 32) * NG;
+    if (items <= 0) return cudaSuccess;
+    return launch_dependent(ssm_bwd_lane_local_kernel<IO, ROWS == kVectors, CPLX>, (unsigned)((items + kLaneWarps - 1) / kLaneWarps), kLaneWarps * 32, 0, 1, s, p, N, NG);
+  }
+  // A piece of one block runs the block's code once, so its time is that of fetching the code: with loops over the steps, and
+  // the states after the odd steps in shared memory instead of registers, that is a quarter of it (float32 (1, 256, 64): main
+  // kernel 13.6 -> 12.0 us; with two blocks per piece the loops cost what they save).  Its shared memory leaves room for one
+  // block per SM, so only for grids that then still run at once (float32 (2, 256, 256), 16 clusters of 8: 25.5 -> 34.6 us a
+  // pass): eight clusters of 8, smaller clusters on three quarters of the SMs, or a block per SM.
+  if constexpr (NG == 1 && !CPLX) {
+    const LaneSplit sp = plan.split;
+    const int per_block = kLaneWarps / sp.warps, most = sp.cluster == 8 ? 64 : sp.cluster > 1 ? 112 : kNumSMs;
+    const long long chains = (long long)p.batch * ((p.D + 31) / 32), blocks = (chains + per_block - 1) / per_block * sp.cluster;
+    if (plan.nseg == 1 && sp.piece <= kLB && blocks <= most) return launch_bwd_lane_main<IO, NG, ROWS, CPLX, true>(plan, p, N, s);
+  }
+  return launch_bwd_lane_main<IO, NG, ROWS, CPLX, false>(plan, p, N, s);
 }
 
 template <typename IO, int NG, bool CPLX>

@@ -113,6 +113,20 @@ def test_options_on_the_tuned_kernels(batch, L, D, options):
     _check(batch, L, D, **options)
 
 
+@pytest.mark.parametrize("batch,L,D,N,io,options", [   # (backward in pieces of one block of 8 steps: up to 32 pieces per chain)
+    (1, 1, 40, 16, "f32", dict(carry=True)),
+    (1, 8, 31, 16, "bf16", {}),
+    (1, 9, 64, 4, "f32", dict(saved=False)),
+    (1, 255, 33, 16, "f32", dict(carry=True, perturb_A=0.05)),
+    (1, 256, 64, 16, "f32", {}),
+    (2, 249, 32, 16, "bf16", dict(carry=True, fused=True)),
+    (1, 64, 100, 8, "f32", dict(gate=False, skip=False)),
+    (2, 31, 47, 16, "bf16", dict(perturb_A=0.05, saved=False)),
+])
+def test_lane_kernels_in_pieces_of_one_block(batch, L, D, N, io, options):
+    _check(batch, L, D, N, io, fwd=LANE[0], bwd=LANE[1], **options)
+
+
 @pytest.mark.parametrize("batch,L,D,N,options", [
     (1, 1, 2568, 64, {}),                                        # a single step; 80 whole groups of channels and one of 8
     (1, 31, 2560, 64, dict(carry=True)),                         # one step short of a tile
