@@ -60,10 +60,12 @@ static bool ckpt_tiled(const ssm_problem_t& p) { return p.N % 4 == 0 && !(p.flag
 // with the fused step size).  Measured, whole calls, D = 1536, batch 8 (share 0.65): L = 2048 167 -> 158 us, with A trained
 // 228 -> 218, and the step size fused 306 -> 270; L = 1024 would go 87 -> 91, 116 -> 122, 157 -> 150; D = 960, batch 10
 // (0.51), L = 2048: 168 -> 142, 228 -> 197, 307 -> 245.
-static int tuned_fwd_segments(const ssm_problem_t& p) {
+// optional_split: the split above half of the sub-partitions may be taken (it needs workspace that the problem does not).
+static int tuned_fwd_segments(const ssm_problem_t& p, bool optional_split = true) {
   const int cw = fwd_fast_channels_per_warp();
   const long long chains = (long long)p.batch * ((p.D + cw - 1) / cw), sub_partitions = 4LL * kNumSMs;
   if (2 * chains >= sub_partitions) {
+    if (!optional_split) return 1;
     const bool fused = p.flags & SSM_FLAG_DELTA_SOFTPLUS;
     const float share = (float)chains / (float)sub_partitions, steps = (float)p.L;
     return share * steps * (fused ? 1.24f : 1.31f) + (fused ? 150.f : 290.f) < steps ? 4 : 1;
@@ -214,7 +216,7 @@ static ssm_status_t validate_problem(const ssm_problem_t* p) {
 
 // The sequence is split in time only when (batch, channel, state) parallelism alone would leave most of the GPU
 // idle: every time segment but the first costs one extra sweep of the recurrence.
-Plan make_plan(const ssm_problem_t& p) {
+static Plan plan_fwd(const ssm_problem_t& p, bool optional_split) {
   Plan pl{};
   pl.nck = (p.L + kCkptSteps - 1) / kCkptSteps;
   pl.fwd_cpt = 2;
@@ -233,7 +235,7 @@ Plan make_plan(const ssm_problem_t& p) {
   } else if (lane_fwd(p)) {
     nseg = lane_segments(p);
   } else if (tuned_shape(p)) {
-    nseg = tuned_fwd_segments(p);
+    nseg = tuned_fwd_segments(p, optional_split);
   } else if (warps < sub_partitions * 3) {
     // generic kernels: a warp is latency-bound, so aim for 6 warps per sub-partition although a split costs half a
     // sweep more (measured 2 to 2.5 times faster than one or two warps per sub-partition)
@@ -248,6 +250,8 @@ Plan make_plan(const ssm_problem_t& p) {
   pl.split = LaneSplit{1, 1, seg_steps};
   return pl;
 }
+
+Plan make_plan(const ssm_problem_t& p) { return plan_fwd(p, true); }
 
 // Time split of the lane backward kernel: inside clusters (one launch, for little work) or into segments of the launch
 // with a pre-pass of its own (which runs at twice the occupancy).  Costs in steps of a lone warp of the main kernel:
@@ -358,6 +362,14 @@ static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
   w.total = off;
   return w;
 }
+// Bytes of workspace of a forward call with and without the optional split.  A call that is given less than the first takes
+// the unsplit plan, so whoever has that much (or the fixed scratch of ssm_scan_fwd_static) is not refused.
+static size_t fwd_workspace(const ssm_problem_t& p, bool optional_split) {
+  ssm_problem_t wide;
+  if (widen_route(p, &wide)) return widen_layout(p, fwd_workspace(wide, optional_split), false).total;
+  return fwd_layout(p, plan_fwd(p, optional_split)).total;
+}
+size_t fwd_workspace_least(const ssm_problem_t& p) { return std::min(fwd_workspace(p, true), fwd_workspace(p, false)); }
 // Points the forward parameters at the scheduling words of a forward workspace and clears them; a status word at the head
 // of that workspace is cleared with them.
 static cudaError_t attach_fwd_sched(const ssm_problem_t& p, const Plan& pl, char* ws, int* abort_word, FwdParams& fp,
@@ -478,11 +490,10 @@ using namespace ssm;
 extern "C" {
 
 size_t ssm_scan_fwd_workspace_bytes(const ssm_problem_t* p) {
-  if (validate_problem(p) != SSM_OK) return 0;
-  ssm_problem_t wide;
-  if (widen_route(*p, &wide)) return widen_layout(*p, ssm_scan_fwd_workspace_bytes(&wide), false).total;
-  return fwd_layout(*p, make_plan(*p)).total;
+  return validate_problem(p) == SSM_OK ? fwd_workspace(*p, true) : 0;
 }
+// The least a forward call of the problem can do with (0 for an invalid one).
+size_t ssm_fwd_workspace_least(const ssm_problem_t* p) { return validate_problem(p) == SSM_OK ? fwd_workspace_least(*p) : 0; }
 
 size_t ssm_scan_bwd_workspace_bytes(const ssm_problem_t* p) {
   if (validate_problem(p) != SSM_OK) return 0;
@@ -587,7 +598,7 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   }
   ssm_problem_t wide;
   if (widen_route(*p, &wide)) {
-    const size_t inner = ssm_scan_fwd_workspace_bytes(&wide);
+    const size_t inner = fwd_workspace(wide, workspace_bytes >= fwd_workspace(*p, true));
     const WidenLayout wl = widen_layout(*p, inner, false);
     st = check_ws(workspace, workspace_bytes, wl.total);
     if (st != SSM_OK) return st;
@@ -610,7 +621,7 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
     repack_add(outj, h_last ? ws + wl.h_last : nullptr, h_last, rows_s, kWideN, p->N, kRepackF32);
     return repack_run(outj, s) == cudaSuccess ? SSM_OK : SSM_ERR_CUDA;
   }
-  const Plan pl = make_plan(*p);
+  const Plan pl = plan_fwd(*p, workspace_bytes >= fwd_workspace(*p, true));
   st = check_ws(workspace, workspace_bytes, fwd_layout(*p, pl).total);
   if (st != SSM_OK) return st;
 

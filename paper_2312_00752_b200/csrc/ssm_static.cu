@@ -15,6 +15,8 @@
 
 #include "ssm_scan.h"
 
+extern "C" size_t ssm_fwd_workspace_least(const ssm_problem_t* p);   // ssm_api.cu, not exported
+
 namespace {
 
 static __device__ __align__(256) unsigned char g_static_scratch[SSM_STATIC_SCRATCH_BYTES];
@@ -49,7 +51,7 @@ extern "C" ssm_status_t ssm_scan_fwd_static(const ssm_problem_t* p, const void* 
                                             void* saved_states, void* stream) {
   // Size check first: a problem whose scratch does not fit the fixed array is refused before anything else happens.
   // (An invalid problem reports 0 bytes here and is then rejected by the regular argument checks below.)
-  const size_t need = ssm_scan_fwd_workspace_bytes(p);
+  const size_t need = ssm_fwd_workspace_least(p);
   if (need > (size_t)SSM_STATIC_SCRATCH_BYTES) return SSM_ERR_WORKSPACE;
   void* scratch = nullptr;
   if (static_scratch_on_current_device(&scratch) != cudaSuccess) return SSM_ERR_CUDA;

@@ -113,6 +113,23 @@ def test_options_on_the_tuned_kernels(batch, L, D, options):
     _check(batch, L, D, **options)
 
 
+def test_tuned_forward_takes_the_unsplit_plan_where_the_split_one_has_no_room():
+    # the fixed scratch of the static entry holds nothing of this split (8 MB), and the problem needs none without it
+    import torch
+    from oracle import ssm_oracle as O
+    from paper_2312_00752_b200 import binding as K
+    inp = synth.make_inputs(synth.ScanConfig("routes", 29, 2, 1024, 4736, 16, "bf16", 1e-3, 1e-1), seed=5)
+    dev = U.to_device(inp, "bf16")
+    args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    assert K.fwd_workspace_bytes(K.make_problem(dev["x"], dev["B"], True, True)) > 4 << 20
+    out = torch.empty_like(dev["x"])
+    got = K.ssm_scan_fwd_static(*args, out=out)
+    got = got[0] if isinstance(got, tuple) else got
+    ref = {"out": O.scan_fwd(inp["x"], inp["delta"], inp["A"], inp["B"], inp["C"], D_skip=inp["D_skip"], z=inp["z"])}
+    U.assert_elementwise({"out": U.to_host(got)}, ref, "bf16", "static scratch")
+    assert U.kernels(lambda: K.ssm_scan_fwd_static(*args, out=out)) == {TUNED[0]}
+
+
 @pytest.mark.parametrize("batch,L,D,N,io,options", [   # (backward in pieces of one block of 8 steps: up to 32 pieces per chain)
     (1, 1, 40, 16, "f32", dict(carry=True)),
     (1, 8, 31, 16, "bf16", {}),
