@@ -20,8 +20,8 @@
 // 0.9 for shared memory and special functions and, a block's body being near the size of the instruction cache, 0.2
 // (float32, N = 64) to 0.7 (bf16 rows at odd addresses, complex states) for instructions, hence rolled loops around it;
 // 315 warp instructions per warp and step at float32 (2, 2048, 1536).  Measured against the generic
-// kernel, backward call: float32 (2, 2048, 1536), N = 16: 485 -> 177 us; bf16 (3, 1237, 1001): 430 -> 127 us; bf16
-// (1, 2048, 5120), N = 64: 3003 -> 831 us; float32 (1, 256, 64): 207 -> 16 us.
+// kernel, backward call: float32 (2, 2048, 1536), N = 16: 485 -> 174 us; bf16 (3, 1237, 1001): 430 -> 125 us; bf16
+// (1, 2048, 5120), N = 64: 3003 -> 824 us; float32 (1, 256, 64): 207 -> 14 us.
 #include <type_traits>
 
 #include "ssm_lane.cuh"

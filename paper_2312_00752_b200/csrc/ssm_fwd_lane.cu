@@ -7,7 +7,7 @@
 //
 // Bound (counters): with one exponential per state the special-function unit, 70 % busy at float32 (2, 2048, 1536), 66 %
 // at bf16 (3, 1237, 1001), 68 % with complex states at (2, 2048, 1536); with two per group of 16 (bf16 (1, 2048, 5120),
-// N = 64) latency: FMA pipe and issue slots 49 %, special-function unit 15 %, a warp waits 1.1 cycles per instruction
+// N = 64, which ssm_fwd_team.cu takes now) latency: FMA pipe and issue slots 49 %, special-function unit 15 %, a warp waits 1.1 cycles per instruction
 // for fixed latencies.  The issue slots are 43 to 49 % in use.  So the registers are capped for three warps per
 // sub-partition and a chain is split in time until they are there.
 // Measured against the generic kernel with its summary and carry launches: float32 (2, 2048, 1536), N = 16: 262 -> 75 us;
