@@ -35,9 +35,10 @@
  *     of its own; larger bf16 problems with N < 16 and D % 8 == 0 run on them too, with A, B, C and the state arrays
  *     widened inside the workspace by columns that stay zero.)  All io pointers must be aligned to the element size;
  *     16-byte aligned pointers together with rows that are multiples of 16 bytes select the vector path.
- *   - Results are bitwise reproducible for fixed inputs, shape, flags and library build: every reduction (over n,
- *     over channels for dB/dC, over batch and time for dA/dD) has a fixed order and no floating-point atomics
- *     are used.
+ *   - Results are bitwise reproducible for fixed inputs, shape, flags and library build (and, for the forward calls
+ *     named at ssm_scan_fwd_workspace_bytes, a workspace that holds the queried size or one that does not): every
+ *     reduction (over n, over channels for dB/dC, over batch and time for dA/dD) has a fixed order and no
+ *     floating-point atomics are used.
  *   - NaN and Inf propagate; signs are not validated (A < 0 and delta > 0 are expected).
  */
 #ifndef SSM_SCAN_H_
@@ -60,7 +61,8 @@ typedef enum {
   SSM_OK = 0,
   SSM_ERR_INVALID_ARG = 1,  /* null required pointer, non-positive dimension, misaligned pointer, bad flag      */
   SSM_ERR_UNSUPPORTED = 2,  /* N or dtype outside the supported set                                             */
-  SSM_ERR_WORKSPACE = 3,    /* workspace null / misaligned / smaller than the query reports                     */
+  SSM_ERR_WORKSPACE = 3,    /* workspace null / misaligned / smaller than the call can do with (that is what the
+                               query reports, but for the forward calls named at ssm_scan_fwd_workspace_bytes)  */
   SSM_ERR_CUDA = 4,         /* a CUDA runtime call or a kernel launch failed                                    */
   SSM_ERR_TIMEOUT = 5,      /* a bounded device-side wait gave up (reported by ssm_scan_check_status)           */
   SSM_ERR_BOUNDS = 6        /* bounds-checking build only: a tuned or lane kernel computed a tile row or a global
@@ -103,8 +105,15 @@ typedef struct {
   uint32_t flags;           /* SSM_FLAG_* */
 } ssm_problem_t;
 
-/* Bytes of scratch memory ssm_scan_fwd / ssm_scan_bwd need for this problem (0 is possible).  Returns 0 for an
- * invalid problem; the call itself then reports the error. */
+/* Bytes of scratch memory ssm_scan_fwd / ssm_scan_bwd use for this problem (0 is possible).  Returns 0 for an
+ * invalid problem; the call itself then reports the error.  A call that is given less is refused with
+ * SSM_ERR_WORKSPACE, with one exception:
+ *   - Forward, bf16, N <= 16, D % 8 == 0 and 296 to about 450 groups of 32 channels in all batch entries together:
+ *     where it is estimated to be faster, ssm_scan_plan reports four time segments, which take scratch memory; a call
+ *     without it (too small, NULL or not 256-byte aligned) runs the sequence in one piece instead.  N = 16 then needs
+ *     none, smaller N the widened copies of A, B, C and the state arrays alone.  Its results are as accurate, but not
+ *     bit for bit those of the call that splits, since the states of a segment are summed in another order; they do not
+ *     depend on anything else about the workspace. */
 SSM_API size_t ssm_scan_fwd_workspace_bytes(const ssm_problem_t* p);
 SSM_API size_t ssm_scan_bwd_workspace_bytes(const ssm_problem_t* p);
 
@@ -124,7 +133,8 @@ SSM_API int32_t ssm_scan_checkpoint_steps(void);
  *   z                     in, io_dtype; required iff SSM_FLAG_HAS_Z
  *   out                   out, io_dtype [batch][L][D]
  *   saved_states          out, float32, ssm_scan_saved_state_bytes(p) bytes; required iff SSM_FLAG_SAVE_STATES
- *   workspace             scratch of at least ssm_scan_fwd_workspace_bytes(p) bytes (may be NULL if that is 0)
+ *   workspace             scratch of ssm_scan_fwd_workspace_bytes(p) bytes or more (may be NULL if that is 0; less is
+ *                         refused but for the exception named there)
  */
 SSM_API ssm_status_t ssm_scan_fwd(const ssm_problem_t* p, const void* x, const void* delta, const float* A, const void* B,
                           const void* C, const float* D_skip, const void* z, void* out, void* saved_states,
@@ -234,7 +244,8 @@ SSM_API ssm_status_t ssm_scan_bwd_state(const ssm_problem_t* p, const void* x, c
  * every resident warp an equal share of the (channel group, time) work; where a share ends inside a channel group, the
  * next warp continues that group and first waits (with a bounded number of polls) for the state or adjoint the warp
  * before it hands over through the workspace.  If such a wait ever gives up, the waiting warps stop and a status word
- * (the first word of every non-empty workspace) is set.  This call synchronises `stream`, copies that word to the host
+ * (the first word of every non-empty workspace) is set.  (A forward call that did without the workspace it was short of
+ * has no such waits and may not have touched that word.)  This call synchronises `stream`, copies that word to the host
  * and returns SSM_ERR_TIMEOUT if it is set (the results of that call are then incomplete), SSM_OK otherwise.  `p` and
  * `workspace` must be those of the call.  A library built with -DSSM_DEBUG_BOUNDS (the stand-in for a memory checker:
  * every tile row index and every global row / channel offset of the tuned kernels and the global accesses and shared
@@ -250,11 +261,13 @@ SSM_API ssm_status_t ssm_scan_check_status(const ssm_problem_t* p, const void* w
  * It is for callers that are not allowed to allocate device memory at the point where they call the scan -- for
  * example a layer plug-in that receives only its input and output buffers from a host framework and must not
  * allocate while enqueueing work, because a device allocation synchronises the GPU, or an application whose memory
- * budget is fixed at start-up.  Same arguments and results as ssm_scan_fwd, minus the workspace: the scratch memory
- * of the time-split forward path is a fixed array of SSM_STATIC_SCRATCH_BYTES bytes inside the library's device
- * image, present on every GPU that loads the library until the process exits.
- *   - A problem whose ssm_scan_fwd_workspace_bytes() exceeds SSM_STATIC_SCRATCH_BYTES is refused with
- *     SSM_ERR_WORKSPACE before anything is launched; use ssm_scan_fwd with your own workspace for those.
+ * budget is fixed at start-up.  Same arguments as ssm_scan_fwd, minus the workspace, and bit for bit the results of
+ * ssm_scan_fwd with a workspace of SSM_STATIC_SCRATCH_BYTES bytes: the scratch memory of the time-split forward path is a
+ * fixed array of that size inside the library's device image, present on every GPU that loads the library until the
+ * process exits.
+ *   - A problem that ssm_scan_fwd would refuse with a workspace of that size is refused with SSM_ERR_WORKSPACE before
+ *     anything is launched; use ssm_scan_fwd with your own workspace for those.  Where ssm_scan_fwd_workspace_bytes()
+ *     exceeds it only for the time segments that a call can do without (named there), the sequence runs in one piece.
  *   - The call allocates and frees nothing.  The first call on a device looks up the device address of the array
  *     (with that device current) and keeps it; make that first call outside any stream capture.
  *   - All calls on a device share the one array: two calls that can overlap on the GPU (different streams, no
@@ -298,7 +311,7 @@ SSM_API ssm_status_t ssm_scan_fwd_bwd_host(const ssm_problem_t* p, const void* x
 SSM_API const char* ssm_status_string(ssm_status_t s);
 
 /*
- * Describes how the library would run this problem: number of time segments the sequence is split into, steps per
+ * Describes how the library runs this problem, given a workspace of ssm_scan_fwd_workspace_bytes(): number of time segments the sequence is split into, steps per
  * segment, channels per thread block and states per thread of the forward kernel.  Any output pointer may be NULL.
  * Returns SSM_OK or the validation error.  Host-only; launches nothing.
  */

@@ -362,14 +362,20 @@ static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
   w.total = off;
   return w;
 }
-// Bytes of workspace of a forward call with and without the optional split.  A call that is given less than the first takes
-// the unsplit plan, so whoever has that much (or the fixed scratch of ssm_scan_fwd_static) is not refused.
+// Bytes of workspace of a forward call with and without the optional split.  A call whose workspace does not hold the first
+// (missing and misaligned ones hold nothing) takes the unsplit plan, so whoever has what that needs (or the fixed scratch of
+// ssm_scan_fwd_static) is not refused.  The results are then those of one sweep, in the last bits not those of the split
+// one: ssm_scan.h says so at ssm_scan_fwd_workspace_bytes.
 static size_t fwd_workspace(const ssm_problem_t& p, bool optional_split) {
   ssm_problem_t wide;
   if (widen_route(p, &wide)) return widen_layout(p, fwd_workspace(wide, optional_split), false).total;
   return fwd_layout(p, plan_fwd(p, optional_split)).total;
 }
 size_t fwd_workspace_least(const ssm_problem_t& p) { return std::min(fwd_workspace(p, true), fwd_workspace(p, false)); }
+static bool aligned_to(const void* ptr, size_t a) { return (reinterpret_cast<uintptr_t>(ptr) % a) == 0; }
+static bool has_room(const void* ws, size_t have, size_t need) {
+  return need == 0 || (ws != nullptr && aligned_to(ws, 256) && have >= need);
+}
 // Points the forward parameters at the scheduling words of a forward workspace and clears them; a status word at the head
 // of that workspace is cleared with them.
 static cudaError_t attach_fwd_sched(const ssm_problem_t& p, const Plan& pl, char* ws, int* abort_word, FwdParams& fp,
@@ -440,7 +446,6 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
   return w;
 }
 
-static bool aligned_to(const void* ptr, size_t a) { return (reinterpret_cast<uintptr_t>(ptr) % a) == 0; }
 // static B / C (and their gradients) are float32 whatever the io dtype
 static bool static_bc_aligned(const ssm_problem_t& p, const void* B, const void* C, const void* dB, const void* dC) {
   const bool sb = p.flags & SSM_FLAG_STATIC_B, sc = p.flags & SSM_FLAG_STATIC_C;
@@ -449,9 +454,7 @@ static bool static_bc_aligned(const ssm_problem_t& p, const void* B, const void*
 }
 
 static ssm_status_t check_ws(const void* ws, size_t have, size_t need) {
-  if (need == 0) return SSM_OK;
-  if (ws == nullptr || !aligned_to(ws, 256) || have < need) return SSM_ERR_WORKSPACE;
-  return SSM_OK;
+  return has_room(ws, have, need) ? SSM_OK : SSM_ERR_WORKSPACE;
 }
 
 // Runs the passes that establish the state at the start of every segment (nothing to do without a time split).
@@ -598,7 +601,7 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   }
   ssm_problem_t wide;
   if (widen_route(*p, &wide)) {
-    const size_t inner = fwd_workspace(wide, workspace_bytes >= fwd_workspace(*p, true));
+    const size_t inner = fwd_workspace(wide, has_room(workspace, workspace_bytes, fwd_workspace(*p, true)));
     const WidenLayout wl = widen_layout(*p, inner, false);
     st = check_ws(workspace, workspace_bytes, wl.total);
     if (st != SSM_OK) return st;
@@ -621,7 +624,7 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
     repack_add(outj, h_last ? ws + wl.h_last : nullptr, h_last, rows_s, kWideN, p->N, kRepackF32);
     return repack_run(outj, s) == cudaSuccess ? SSM_OK : SSM_ERR_CUDA;
   }
-  const Plan pl = plan_fwd(*p, workspace_bytes >= fwd_workspace(*p, true));
+  const Plan pl = plan_fwd(*p, has_room(workspace, workspace_bytes, fwd_workspace(*p, true)));
   st = check_ws(workspace, workspace_bytes, fwd_layout(*p, pl).total);
   if (st != SSM_OK) return st;
 

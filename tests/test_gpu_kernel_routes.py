@@ -130,6 +130,37 @@ def test_tuned_forward_takes_the_unsplit_plan_where_the_split_one_has_no_room():
     assert U.kernels(lambda: K.ssm_scan_fwd_static(*args, out=out)) == {TUNED[0]}
 
 
+@pytest.mark.parametrize("batch,L,D,N", [(2, 1024, 4736, 16), (2, 1030, 4744, 16), (2, 1024, 4736, 8)])
+def test_forward_results_depend_on_the_workspace_only_by_whether_the_split_has_room(batch, L, D, N):
+    # what include/ssm_scan.h says of it: short, missing and misaligned workspaces and the fixed scratch give one result, bit
+    # for bit, and one sweep; every workspace that has room gives another, bit for bit, and the split
+    import torch
+    from oracle import ssm_oracle as O
+    from paper_2312_00752_b200 import binding as K
+    inp = synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, "bf16", 1e-3, 1e-1), seed=L)
+    dev = U.to_device(inp, "bf16")
+    args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    prob = K.make_problem(dev["x"], dev["B"], True, True)
+    need = K.fwd_workspace_bytes(prob)
+    assert K.plan(prob)["n_segments"] == 4 and need > K.SSM_STATIC_SCRATCH_BYTES
+    big = torch.full((need + 256,), 255, dtype=torch.uint8, device="cuda")
+    split = K.ssm_scan_fwd(*args)
+    assert torch.equal(K.ssm_scan_fwd(*args, workspace=big[:need]), split)
+    assert torch.equal(K.ssm_scan_fwd(*args, workspace=big), split)
+    short = [big[:need - 1]]
+    if N == 16:   # (N = 8 needs a workspace in any case)
+        short += [big[:0], big[:256], big[128:]]
+        assert torch.equal(K.ssm_scan_fwd_static(*args), K.ssm_scan_fwd(*args, workspace=short[0]))
+    one = K.ssm_scan_fwd(*args, workspace=short[0])
+    for ws in short[1:]:
+        assert torch.equal(K.ssm_scan_fwd(*args, workspace=ws), one)
+    assert "ssm_carry_few_kernel" in U.kernels(lambda: K.ssm_scan_fwd(*args, workspace=big))
+    assert not any(k.startswith("ssm_carry") for k in U.kernels(lambda: K.ssm_scan_fwd(*args, workspace=short[0])))
+    ref = {"out": O.scan_fwd(inp["x"], inp["delta"], inp["A"], inp["B"], inp["C"], D_skip=inp["D_skip"], z=inp["z"])}
+    for out in (split, one):
+        U.assert_elementwise({"out": U.to_host(out)}, ref, "bf16", "workspace")
+
+
 @pytest.mark.parametrize("batch,L,D,N,io,options", [   # (backward in pieces of one block of 8 steps: up to 32 pieces per chain)
     (1, 1, 40, 16, "f32", dict(carry=True)),
     (1, 8, 31, 16, "bf16", {}),
