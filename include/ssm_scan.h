@@ -36,7 +36,7 @@
  *     widened inside the workspace by columns that stay zero.)  All io pointers must be aligned to the element size;
  *     16-byte aligned pointers together with rows that are multiples of 16 bytes select the vector path.
  *   - Results are bitwise reproducible for fixed inputs, shape, flags and library build (and, for the forward calls
- *     named at ssm_scan_fwd_workspace_bytes, a workspace that holds the queried size or one that does not): every
+ *     split in time by choice, see ssm_scan_fwd_workspace_bytes, a workspace that holds the queried size or one that does not): every
  *     reduction (over n, over channels for dB/dC, over batch and time for dA/dD) has a fixed order and no
  *     floating-point atomics are used.
  *   - NaN and Inf propagate; signs are not validated (A < 0 and delta > 0 are expected).
@@ -62,7 +62,7 @@ typedef enum {
   SSM_ERR_INVALID_ARG = 1,  /* null required pointer, non-positive dimension, misaligned pointer, bad flag      */
   SSM_ERR_UNSUPPORTED = 2,  /* N or dtype outside the supported set                                             */
   SSM_ERR_WORKSPACE = 3,    /* workspace null / misaligned / smaller than the call can do with (that is what the
-                               query reports, but for the forward calls named at ssm_scan_fwd_workspace_bytes)  */
+                               query reports, but for the exceptions named at ssm_scan_fwd_workspace_bytes)     */
   SSM_ERR_CUDA = 4,         /* a CUDA runtime call or a kernel launch failed                                    */
   SSM_ERR_TIMEOUT = 5,      /* a bounded device-side wait gave up (reported by ssm_scan_check_status)           */
   SSM_ERR_BOUNDS = 6        /* bounds-checking build only: a tuned or lane kernel computed a tile row or a global
@@ -107,13 +107,16 @@ typedef struct {
 
 /* Bytes of scratch memory ssm_scan_fwd / ssm_scan_bwd use for this problem (0 is possible).  Returns 0 for an
  * invalid problem; the call itself then reports the error.  A call that is given less is refused with
- * SSM_ERR_WORKSPACE, with one exception:
+ * SSM_ERR_WORKSPACE, with two exceptions:
  *   - Forward, bf16, N <= 16, D % 8 == 0 and 296 to about 450 groups of 32 channels in all batch entries together:
  *     where it is estimated to be faster, ssm_scan_plan reports four time segments, which take scratch memory; a call
  *     without it (too small, NULL or not 256-byte aligned) runs the sequence in one piece instead.  N = 16 then needs
  *     none, smaller N the widened copies of A, B, C and the state arrays alone.  Its results are as accurate, but not
  *     bit for bit those of the call that splits, since the states of a segment are summed in another order; they do not
- *     depend on anything else about the workspace. */
+ *     depend on anything else about the workspace.
+ *   - Forward, bf16, N = 32 or 64, D % 8 == 0: where the kernel for these shares groups of 32 channels between
+ *     neighbouring teams of warps, it passes their state through scratch memory; a call without it runs every group on
+ *     one team and needs none.  The results are the same bit for bit. */
 SSM_API size_t ssm_scan_fwd_workspace_bytes(const ssm_problem_t* p);
 SSM_API size_t ssm_scan_bwd_workspace_bytes(const ssm_problem_t* p);
 
@@ -134,7 +137,7 @@ SSM_API int32_t ssm_scan_checkpoint_steps(void);
  *   out                   out, io_dtype [batch][L][D]
  *   saved_states          out, float32, ssm_scan_saved_state_bytes(p) bytes; required iff SSM_FLAG_SAVE_STATES
  *   workspace             scratch of ssm_scan_fwd_workspace_bytes(p) bytes or more (may be NULL if that is 0; less is
- *                         refused but for the exception named there)
+ *                         refused but for the exceptions named there)
  */
 SSM_API ssm_status_t ssm_scan_fwd(const ssm_problem_t* p, const void* x, const void* delta, const float* A, const void* B,
                           const void* C, const float* D_skip, const void* z, void* out, void* saved_states,

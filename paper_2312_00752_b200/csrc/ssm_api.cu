@@ -216,8 +216,10 @@ static ssm_status_t validate_problem(const ssm_problem_t* p) {
 
 // The sequence is split in time only when (batch, channel, state) parallelism alone would leave most of the GPU
 // idle: every time segment but the first costs one extra sweep of the recurrence.
-static Plan plan_fwd(const ssm_problem_t& p, bool optional_split) {
+// spare_workspace: the call has the workspace that the plan could do without (tuned_fwd_segments, fwd_layout).
+static Plan plan_fwd(const ssm_problem_t& p, bool spare_workspace) {
   Plan pl{};
+  pl.spare_workspace = spare_workspace;
   pl.nck = (p.L + kCkptSteps - 1) / kCkptSteps;
   pl.fwd_cpt = 2;
   pl.fwd_ch = fwd_channels_per_block(p.N);
@@ -235,7 +237,7 @@ static Plan plan_fwd(const ssm_problem_t& p, bool optional_split) {
   } else if (lane_fwd(p)) {
     nseg = lane_segments(p);
   } else if (tuned_shape(p)) {
-    nseg = tuned_fwd_segments(p, optional_split);
+    nseg = tuned_fwd_segments(p, spare_workspace);
   } else if (warps < sub_partitions * 3) {
     // generic kernels: a warp is latency-bound, so aim for 6 warps per sub-partition although a split costs half a
     // sweep more (measured 2 to 2.5 times faster than one or two warps per sub-partition)
@@ -335,7 +337,9 @@ static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
   const int cw = fwd_fast_channels_per_warp();
   const long long groups = (long long)p.batch * ((p.D + cw - 1) / cw);
   w.max_workers = tuned_shape(p) && !lane_fwd(p) ? shared_workers(groups * pl.nseg) : 0;
-  if (team_fwd(p) && groups * team_size(p) > 4 * kNumSMs) w.max_workers = 4 * kNumSMs;   // (a hand-off per warp of a team)
+  // (a hand-off per warp of a team; without the slots every team runs whole chains, the last wave of them on part of the GPU:
+  // (1, 2048, 5120), N = 64: 199 -> 345 us)
+  if (team_fwd(p) && pl.spare_workspace && groups * team_size(p) > 4 * kNumSMs) w.max_workers = 4 * kNumSMs;
   if (pl.nseg == 1 && w.max_workers == 0) {
 #ifdef SSM_DEBUG_BOUNDS
     w.total = kStatusBytes;   // (a place for the status word)
@@ -362,14 +366,15 @@ static FwdWorkspace fwd_layout(const ssm_problem_t& p, const Plan& pl) {
   w.total = off;
   return w;
 }
-// Bytes of workspace of a forward call with and without the optional split.  A call whose workspace does not hold the first
-// (missing and misaligned ones hold nothing) takes the unsplit plan, so whoever has what that needs (or the fixed scratch of
-// ssm_scan_fwd_static) is not refused.  The results are then those of one sweep, in the last bits not those of the split
-// one: ssm_scan.h says so at ssm_scan_fwd_workspace_bytes.
-static size_t fwd_workspace(const ssm_problem_t& p, bool optional_split) {
+// Bytes of workspace of a forward call with and without what it can do without: the optional split, the hand-offs between
+// teams.  A call whose workspace does not hold the first (missing and misaligned ones hold nothing) takes the plan of the
+// second, so whoever has what that needs (or the fixed scratch of ssm_scan_fwd_static) is not refused.  Without the split the
+// results are those of one sweep, in the last bits not those of the split one: ssm_scan.h says so at
+// ssm_scan_fwd_workspace_bytes.  A hand-off changes no bit.
+static size_t fwd_workspace(const ssm_problem_t& p, bool spare_workspace) {
   ssm_problem_t wide;
-  if (widen_route(p, &wide)) return widen_layout(p, fwd_workspace(wide, optional_split), false).total;
-  return fwd_layout(p, plan_fwd(p, optional_split)).total;
+  if (widen_route(p, &wide)) return widen_layout(p, fwd_workspace(wide, spare_workspace), false).total;
+  return fwd_layout(p, plan_fwd(p, spare_workspace)).total;
 }
 size_t fwd_workspace_least(const ssm_problem_t& p) { return std::min(fwd_workspace(p, true), fwd_workspace(p, false)); }
 static bool aligned_to(const void* ptr, size_t a) { return (reinterpret_cast<uintptr_t>(ptr) % a) == 0; }

@@ -36,6 +36,7 @@ struct Plan {
   int bwd_ch;      // channels per block, backward (= channel-group size of the dB/dC partial sums)
   int bwd_groups;  // ceil(D / bwd_ch)
   LaneSplit split; // lane-per-channel kernels only (of the direction the plan is for)
+  bool spare_workspace;   // forward: the call has the workspace that it could do without
 };
 Plan make_plan(const ssm_problem_t& p);
 

@@ -1,6 +1,8 @@
 """Which kernels a problem runs, and their results: the tuned kernels want bf16, N = 16 (or fewer, widened), aligned
 pointers and at least 296 chains of 32 channels (or the zero-order-hold rule); small problems of the same kind run the
 lane kernels, so what is to be tested of the tuned ones is wide here.  Every case asserts the route."""
+import os
+
 import numpy as np
 import pytest
 
@@ -24,6 +26,11 @@ def _shifted(t):
     v.copy_(t)
     assert v.data_ptr() % 16 == 8
     return v
+
+
+def _no_workspace(buf):
+    """An empty and a misaligned piece of a buffer (the bounds-checking build wants a status word of every call)."""
+    return [] if os.environ.get("SSM_SCAN_LIBRARY", "").endswith("_debug.so") else [buf[:0], buf[128:]]
 
 
 def _check(batch, L, D, N=16, io="bf16", *, fwd=TUNED[0], bwd=TUNED[1], more=(), gate=True, skip=True, zoh=False, fused=False,
@@ -149,7 +156,7 @@ def test_forward_results_depend_on_the_workspace_only_by_whether_the_split_has_r
     assert torch.equal(K.ssm_scan_fwd(*args, workspace=big), split)
     short = [big[:need - 1]]
     if N == 16:   # (N = 8 needs a workspace in any case)
-        short += [big[:0], big[:256], big[128:]]
+        short += [big[:256], *_no_workspace(big)]
         assert torch.equal(K.ssm_scan_fwd_static(*args), K.ssm_scan_fwd(*args, workspace=short[0]))
     one = K.ssm_scan_fwd(*args, workspace=short[0])
     for ws in short[1:]:
@@ -189,6 +196,25 @@ def test_lane_kernels_in_pieces_of_one_block(batch, L, D, N, io, options):
 ])
 def test_teams_of_warps_for_large_states(batch, L, D, N, options):
     _check(batch, L, D, N, fwd=TEAM, bwd=LANE[1], **options)
+
+
+@pytest.mark.parametrize("batch,L,D,N", [(2, 75, 2568, 64), (2, 200, 5128, 32)])   # 162 chains for 148 teams, 322 for 296
+def test_teams_of_warps_without_room_for_their_hand_offs(batch, L, D, N):
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, "bf16", 1e-3, 1e-1), seed=L), "bf16")
+    args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    need = K.fwd_workspace_bytes(K.make_problem(dev["x"], dev["B"], True, True))
+    assert need > 0
+    big = torch.full((need + 256,), 255, dtype=torch.uint8, device="cuda")
+
+    def run(ws):
+        h_last = torch.empty(batch, D, N, device="cuda")
+        return (*K.ssm_scan_fwd(*args, save_states=True, h_last=h_last, workspace=ws), h_last)
+    shared = run(big[:need])
+    for ws in (big[:need - 1], big[:256], *_no_workspace(big)):
+        assert all(torch.equal(a, b) for a, b in zip(run(ws), shared))
+    assert all(TEAM in U.kernels(lambda: run(ws)) for ws in (big, big[:256]))
 
 
 def test_large_states_off_the_16_byte_grid_and_of_few_channels_keep_the_lane_kernel():
