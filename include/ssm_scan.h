@@ -116,7 +116,9 @@ typedef struct {
  *     depend on anything else about the workspace.
  *   - Forward, bf16, N = 32 or 64, D % 8 == 0: where the kernel for these shares groups of 32 channels between
  *     neighbouring teams of warps, it passes their state through scratch memory; a call without it runs every group on
- *     one team and needs none.  The results are the same bit for bit. */
+ *     one team and needs none.  The results are the same bit for bit.
+ * A backward call does likewise without what its sweep that rebuilds the states would use for these (and uses none of it
+ * when it is given saved_states). */
 SSM_API size_t ssm_scan_fwd_workspace_bytes(const ssm_problem_t* p);
 SSM_API size_t ssm_scan_bwd_workspace_bytes(const ssm_problem_t* p);
 
@@ -291,7 +293,8 @@ SSM_API ssm_status_t ssm_scan_fwd_static(const ssm_problem_t* p, const void* x, 
  *   x, delta, z, dout, B, C, A, D_skip      in, HOST pointers, layouts and dtypes as for ssm_scan_fwd / ssm_scan_bwd
  *   out, dx, ddelta, dz, dB, dC, dA, dD     out, HOST pointers, every element overwritten; dz / dD are required iff
  *                                           SSM_FLAG_HAS_Z / SSM_FLAG_HAS_DSKIP
- *   device_arena   DEVICE scratch of at least ssm_scan_host_arena_bytes(p) bytes, 256-byte aligned, caller-owned
+ *   device_arena   DEVICE scratch of ssm_scan_host_arena_bytes(p) bytes or more, 256-byte aligned, caller-owned (less is
+ *                  refused but for what the two calls can do without, see ssm_scan_fwd_workspace_bytes)
  *   stream         the call is ordered after everything already enqueued on it, and work enqueued on it afterwards
  *                  is ordered after every copy of this call; the call itself does not wait for the GPU
  * Host buffers should be page-locked: with pageable memory the results are the same but the copies do not overlap.

@@ -450,6 +450,14 @@ static BwdWorkspace bwd_layout(const ssm_problem_t& p, const Plan& pl, const Pla
   w.total = off;
   return w;
 }
+// Bytes of workspace of a backward call; spare_workspace as in fwd_workspace, for the sweep that rebuilds the checkpoints.
+static size_t bwd_workspace(const ssm_problem_t& p, bool spare_workspace) {
+  if (p.flags & SSM_FLAG_COMPLEX) return complex_bwd_workspace_bytes(p);
+  ssm_problem_t wide;
+  if (widen_route(p, &wide)) return widen_layout(p, bwd_workspace(wide, spare_workspace), true).total;
+  return bwd_layout(p, make_bwd_plan(p), plan_fwd(p, spare_workspace)).total;
+}
+size_t bwd_workspace_least(const ssm_problem_t& p) { return std::min(bwd_workspace(p, true), bwd_workspace(p, false)); }
 
 // static B / C (and their gradients) are float32 whatever the io dtype
 static bool static_bc_aligned(const ssm_problem_t& p, const void* B, const void* C, const void* dB, const void* dC) {
@@ -500,16 +508,13 @@ extern "C" {
 size_t ssm_scan_fwd_workspace_bytes(const ssm_problem_t* p) {
   return validate_problem(p) == SSM_OK ? fwd_workspace(*p, true) : 0;
 }
-// The least a forward call of the problem can do with (0 for an invalid one).
+// The least a forward and a backward call of the problem can do with (0 for an invalid one).
 size_t ssm_fwd_workspace_least(const ssm_problem_t* p) { return validate_problem(p) == SSM_OK ? fwd_workspace_least(*p) : 0; }
 
 size_t ssm_scan_bwd_workspace_bytes(const ssm_problem_t* p) {
-  if (validate_problem(p) != SSM_OK) return 0;
-  if (p->flags & SSM_FLAG_COMPLEX) return complex_bwd_workspace_bytes(*p);
-  ssm_problem_t wide;
-  if (widen_route(*p, &wide)) return widen_layout(*p, ssm_scan_bwd_workspace_bytes(&wide), true).total;
-  return bwd_layout(*p, make_bwd_plan(*p), make_plan(*p)).total;
+  return validate_problem(p) == SSM_OK ? bwd_workspace(*p, true) : 0;
 }
+size_t ssm_bwd_workspace_least(const ssm_problem_t* p) { return validate_problem(p) == SSM_OK ? bwd_workspace_least(*p) : 0; }
 
 size_t ssm_scan_saved_state_bytes(const ssm_problem_t* p) {
   if (validate_problem(p) != SSM_OK) return 0;
@@ -772,7 +777,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   }
   ssm_problem_t wide;
   if (widen_route(*p, &wide)) {
-    const size_t inner = ssm_scan_bwd_workspace_bytes(&wide);
+    const size_t inner = bwd_workspace(wide, has_room(workspace, workspace_bytes, bwd_workspace(*p, true)));
     const WidenLayout wl = widen_layout(*p, inner, true);
     st = check_ws(workspace, workspace_bytes, wl.total);
     if (st != SSM_OK) return st;
@@ -800,7 +805,7 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
     repack_add(outj, dh0 ? ws + wl.dh0 : nullptr, dh0, rows_s, kWideN, p->N, kRepackF32);
     return repack_run(outj, s) == cudaSuccess ? SSM_OK : SSM_ERR_CUDA;
   }
-  const Plan pl = make_bwd_plan(*p), pl_fwd = make_plan(*p);
+  const Plan pl = make_bwd_plan(*p), pl_fwd = plan_fwd(*p, has_room(workspace, workspace_bytes, bwd_workspace(*p, true)));
   const BwdWorkspace w = bwd_layout(*p, pl, pl_fwd);
   st = check_ws(workspace, workspace_bytes, w.total);
   if (st != SSM_OK) return st;

@@ -19,6 +19,9 @@
 
 #include "ssm_scan.h"
 
+extern "C" size_t ssm_fwd_workspace_least(const ssm_problem_t* p);   // ssm_api.cu, not exported
+extern "C" size_t ssm_bwd_workspace_least(const ssm_problem_t* p);
+
 namespace {
 
 constexpr int kMaxChunks = 8;
@@ -55,7 +58,7 @@ struct HostPlan {
   // arena offsets
   size_t in[2], out[2];              // double-buffered piece inputs (x, delta, z, dout, B, C) and outputs
   size_t A, Dskip, dA_part, dD_part, dA, dD, saved, ws;
-  size_t ws_bytes, total;
+  size_t ws_bytes, total, least;     // least: the arena with the least workspace that the two calls take
 };
 
 bool make_host_plan(const ssm_problem_t* p, HostPlan* hp) {
@@ -90,6 +93,7 @@ bool make_host_plan(const ssm_problem_t* p, HostPlan* hp) {
   h.ws_bytes = std::max(ssm_scan_fwd_workspace_bytes(&h.chunk), ssm_scan_bwd_workspace_bytes(&h.chunk));
   h.ws = take(h.ws_bytes);
   h.total = off;
+  h.least = h.ws + align_up(std::max(ssm_fwd_workspace_least(&h.chunk), ssm_bwd_workspace_least(&h.chunk)));
   *hp = h;
   return true;
 }
@@ -121,8 +125,9 @@ extern "C" ssm_status_t ssm_scan_fwd_bwd_host(const ssm_problem_t* p, const void
   const bool has_z = p->flags & SSM_FLAG_HAS_Z, has_d = p->flags & SSM_FLAG_HAS_DSKIP;
   if (!x || !delta || !A || !B || !C || !dout || !out || !dx || !ddelta || !dA || !dB || !dC) return SSM_ERR_INVALID_ARG;
   if ((has_z && (!z || !dz)) || (has_d && (!D_skip || !dD))) return SSM_ERR_INVALID_ARG;
-  if (device_arena == nullptr || (reinterpret_cast<uintptr_t>(device_arena) & 255) != 0 || arena_bytes < h.total)
+  if (device_arena == nullptr || (reinterpret_cast<uintptr_t>(device_arena) & 255) != 0 || arena_bytes < h.least)
     return SSM_ERR_WORKSPACE;
+  h.ws_bytes = std::min(h.ws_bytes, arena_bytes - h.ws);
 
   cudaStream_t s_run = static_cast<cudaStream_t>(stream), s_in = nullptr, s_out = nullptr;
   if (helper_streams(&s_in, &s_out) != cudaSuccess) return SSM_ERR_CUDA;

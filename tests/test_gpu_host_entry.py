@@ -75,6 +75,26 @@ def test_host_call_twice_on_one_arena_and_argument_errors():
                                 h1["dout"], device="cuda:0")
 
 
+def test_host_call_without_room_for_the_time_segments_taken_by_choice():
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    h = _host_tensors(synth.make_inputs(synth.ScanConfig("host", 15, 1, 848, 9472, 16, "bf16", 1e-3, 1e-1), seed=3), "bf16")
+    prob = K.make_problem(h["x"], h["B"], True, True)
+    assert K.plan(prob)["n_segments"] == 4
+    arena = torch.empty(K.host_arena_bytes(prob), dtype=torch.uint8, device="cuda:0")
+    least = arena.numel() - K.fwd_workspace_bytes(prob) + 256   # (256: the status word of the bounds-checking build)
+    call = lambda ws: K.ssm_scan_fwd_bwd_host(h["x"], h["delta"], h["A"], h["B"], h["C"], h["D_skip"], h["z"], h["dout"],
+                                              device="cuda:0", arena=ws)
+    full = call(arena)
+    torch.cuda.synchronize()
+    short = call(arena[:least])
+    torch.cuda.synchronize()
+    for k in full:
+        assert torch.equal(full[k], short[k]), k
+    with pytest.raises(K.SsmScanError):
+        call(arena[:least - 512])
+
+
 def test_host_call_honours_the_zoh_flag():
     import torch
     from paper_2312_00752_b200 import binding as K

@@ -168,6 +168,37 @@ def test_forward_results_depend_on_the_workspace_only_by_whether_the_split_has_r
         U.assert_elementwise({"out": U.to_host(out)}, ref, "bf16", "workspace")
 
 
+@pytest.mark.parametrize("batch,L,D,N", [(2, 1024, 4736, 16), (2, 1030, 4744, 8), (2, 75, 2568, 64)])
+def test_backward_without_room_for_what_its_rebuilding_sweep_can_do_without(batch, L, D, N):
+    # the time segments taken by choice (N <= 16), the hand-offs between teams: as the forward without them, bit for bit
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, "bf16", 1e-3, 1e-1), seed=L), "bf16")
+    args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    prob = K.make_problem(dev["x"], dev["B"], True, True)
+    need, need_fwd = K.bwd_workspace_bytes(prob), K.fwd_workspace_bytes(prob)
+    wide = K.ssm_problem_t(batch, L, D, max(N, 16), prob.io_dtype, prob.flags)
+    least = need - K.fwd_workspace_bytes(wide) + 256   # (256: the status word that the bounds-checking build wants)
+    big = torch.full((need,), 255, dtype=torch.uint8, device="cuda")
+    big_fwd = torch.full((need_fwd,), 255, dtype=torch.uint8, device="cuda")
+    assert least < need and need_fwd > 0
+
+    def bwd(saved, ws):
+        got = K.ssm_scan_bwd(*args, dev["dout"], saved, workspace=ws)
+        K.check_status(prob, ws)
+        return got
+
+    def equal(a, b):
+        assert all(torch.equal(a[k], b[k]) for k in U.GRADS)
+    split = K.ssm_scan_fwd(*args, save_states=True, workspace=big_fwd)[1]
+    whole = K.ssm_scan_fwd(*args, save_states=True, workspace=big_fwd[:need_fwd - 1])[1]
+    equal(bwd(split, big[:least]), bwd(split, big))
+    equal(bwd(None, big), bwd(split, big))
+    equal(bwd(None, big[:least]), bwd(whole, big))
+    with pytest.raises(K.SsmScanError):
+        bwd(None, big[:least - 512])
+
+
 @pytest.mark.parametrize("batch,L,D,N,io,options", [   # (backward in pieces of one block of 8 steps: up to 32 pieces per chain)
     (1, 1, 40, 16, "f32", dict(carry=True)),
     (1, 8, 31, 16, "bf16", {}),
