@@ -249,8 +249,8 @@ SSM_API ssm_status_t ssm_scan_bwd_state(const ssm_problem_t* p, const void* x, c
  * every resident warp an equal share of the (channel group, time) work; where a share ends inside a channel group, the
  * next warp continues that group and first waits (with a bounded number of polls) for the state or adjoint the warp
  * before it hands over through the workspace.  If such a wait ever gives up, the waiting warps stop and a status word
- * (the first word of every non-empty workspace) is set.  (A forward call that did without the workspace it was short of
- * has no such waits and may not have touched that word.)  This call synchronises `stream`, copies that word to the host
+ * (the first word of every non-empty workspace) is set.  (A forward call that does without the workspace it is short of
+ * has no such waits; it clears the word of what it is given, if that has room for one.)  This call synchronises `stream`, copies that word to the host
  * and returns SSM_ERR_TIMEOUT if it is set (the results of that call are then incomplete), SSM_OK otherwise.  `p` and
  * `workspace` must be those of the call.  A library built with -DSSM_DEBUG_BOUNDS (the stand-in for a memory checker:
  * every tile row index and every global row / channel offset of the tuned kernels and the global accesses and shared

@@ -634,7 +634,8 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
     repack_add(outj, h_last ? ws + wl.h_last : nullptr, h_last, rows_s, kWideN, p->N, kRepackF32);
     return repack_run(outj, s) == cudaSuccess ? SSM_OK : SSM_ERR_CUDA;
   }
-  const Plan pl = plan_fwd(*p, has_room(workspace, workspace_bytes, fwd_workspace(*p, true)));
+  const size_t full = fwd_workspace(*p, true);
+  const Plan pl = plan_fwd(*p, has_room(workspace, workspace_bytes, full));
   st = check_ws(workspace, workspace_bytes, fwd_layout(*p, pl).total);
   if (st != SSM_OK) return st;
 
@@ -660,9 +661,13 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.static_C = (p->flags & SSM_FLAG_STATIC_C) ? 1 : 0;
   fp.delta_bias = delta_bias;
   fp.softplus = (p->flags & SSM_FLAG_DELTA_SOFTPLUS) ? 1 : 0;
-  if (fwd_layout(*p, pl).total > 0 &&
-      attach_fwd_sched(*p, pl, static_cast<char*>(workspace), static_cast<int*>(workspace), fp, s, true) != cudaSuccess)
-    return SSM_ERR_CUDA;
+  if (fwd_layout(*p, pl).total > 0) {
+    if (attach_fwd_sched(*p, pl, static_cast<char*>(workspace), static_cast<int*>(workspace), fp, s, true) != cudaSuccess)
+      return SSM_ERR_CUDA;
+  } else if (full > 0 && workspace != nullptr && workspace_bytes >= sizeof(int)) {
+    // the call does without a workspace, but ssm_scan_check_status may be asked about the one it was given
+    if (cudaMemsetAsync(workspace, 0, sizeof(int), s) != cudaSuccess) return SSM_ERR_CUDA;
+  }
   const float* h_start = nullptr;
   if (run_segment_starts(*p, pl, fp, static_cast<char*>(workspace), h0, &h_start, s) != cudaSuccess) return SSM_ERR_CUDA;
   if (fp.max_workers > 0 && pl.nseg > 1) {

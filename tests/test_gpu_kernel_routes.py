@@ -168,6 +168,21 @@ def test_forward_results_depend_on_the_workspace_only_by_whether_the_split_has_r
         U.assert_elementwise({"out": U.to_host(out)}, ref, "bf16", "workspace")
 
 
+@pytest.mark.parametrize("batch,L,D,N", [(2, 1024, 4736, 16), (2, 1024, 4736, 8), (2, 75, 2568, 64)])
+def test_the_status_word_of_a_workspace_without_room_is_that_of_the_call(batch, L, D, N):
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, "bf16", 1e-3, 1e-1), seed=L), "bf16")
+    args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    prob = K.make_problem(dev["x"], dev["B"], True, True)
+    need = K.fwd_workspace_bytes(prob)
+    big = torch.full((need + 256,), 255, dtype=torch.uint8, device="cuda")
+    for ws in [big[:need - 1], *([] if N == 8 else [big[:256], *_no_workspace(big)[1:]])]:   # (N = 8 needs some in any case)
+        big.fill_(255)
+        K.ssm_scan_fwd(*args, workspace=ws)
+        K.check_status(prob, ws)
+
+
 @pytest.mark.parametrize("batch,L,D,N", [(2, 1024, 4736, 16), (2, 1030, 4744, 8), (2, 75, 2568, 64)])
 def test_backward_without_room_for_what_its_rebuilding_sweep_can_do_without(batch, L, D, N):
     # the time segments taken by choice (N <= 16), the hand-offs between teams: as the forward without them, bit for bit
