@@ -27,6 +27,8 @@ int fwd_states_per_thread();
 int fwd_fast_channels_per_warp();
 int bwd_fast_channels_per_warp();
 bool bwd_fast_applicable(const ssm_problem_t& prob, const BwdParams& p);
+bool fwd_fast_applicable(const ssm_problem_t& prob, const FwdParams& p);
+bool fwd_team_applicable(const FwdParams& p);
 bool bwd_lane_applicable(const BwdParams& p);
 // ssm_repack.cu
 enum { kRepackBf16 = 0, kRepackF32 = 1, kRepackA = 2 };
@@ -381,6 +383,9 @@ static bool aligned_to(const void* ptr, size_t a) { return (reinterpret_cast<uin
 static bool has_room(const void* ws, size_t have, size_t need) {
   return need == 0 || (ws != nullptr && aligned_to(ws, 256) && have >= need);
 }
+// Whether the kernel that the spare workspace is for takes the pointers of a call.  Off the 16-byte grid the lane (or generic)
+// kernel runs, which cuts a chain in time by itself.
+static bool uses_spare(const ssm_problem_t& p, const FwdParams& fp) { return team_fwd(p) ? fwd_team_applicable(fp) : fwd_fast_applicable(p, fp); }
 // Points the forward parameters at the scheduling words of a forward workspace and clears them; a status word at the head
 // of that workspace is cleared with them.
 static cudaError_t attach_fwd_sched(const ssm_problem_t& p, const Plan& pl, char* ws, int* abort_word, FwdParams& fp,
@@ -634,11 +639,6 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
     repack_add(outj, h_last ? ws + wl.h_last : nullptr, h_last, rows_s, kWideN, p->N, kRepackF32);
     return repack_run(outj, s) == cudaSuccess ? SSM_OK : SSM_ERR_CUDA;
   }
-  const size_t full = fwd_workspace(*p, true);
-  const Plan pl = plan_fwd(*p, has_room(workspace, workspace_bytes, full));
-  st = check_ws(workspace, workspace_bytes, fwd_layout(*p, pl).total);
-  if (st != SSM_OK) return st;
-
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   FwdParams fp{};
   fp.x = x;
@@ -649,6 +649,13 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.A = A;
   fp.Dskip = has_d ? D_skip : nullptr;
   fp.out = out;
+  fp.h_last = h_last;
+  fp.ckpt = save ? static_cast<float*>(saved_states) : nullptr;
+  fp.ckpt_tiled = ckpt_tiled(*p) ? 1 : 0;
+  const size_t full = fwd_workspace(*p, true);
+  const Plan pl = plan_fwd(*p, has_room(workspace, workspace_bytes, full) && uses_spare(*p, fp));
+  st = check_ws(workspace, workspace_bytes, fwd_layout(*p, pl).total);
+  if (st != SSM_OK) return st;
   fp.batch = p->batch;
   fp.L = p->L;
   fp.D = p->D;
@@ -676,9 +683,6 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
       return SSM_ERR_CUDA;
   }
   fp.h_start = h_start;
-  fp.h_last = h_last;
-  fp.ckpt = save ? static_cast<float*>(saved_states) : nullptr;
-  fp.ckpt_tiled = ckpt_tiled(*p) ? 1 : 0;
   if (launch_fwd(*p, pl, fp, kFwdFull, s) != cudaSuccess) return SSM_ERR_CUDA;
   return SSM_OK;
 }
@@ -810,7 +814,14 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
     repack_add(outj, dh0 ? ws + wl.dh0 : nullptr, dh0, rows_s, kWideN, p->N, kRepackF32);
     return repack_run(outj, s) == cudaSuccess ? SSM_OK : SSM_ERR_CUDA;
   }
-  const Plan pl = make_bwd_plan(*p), pl_fwd = plan_fwd(*p, has_room(workspace, workspace_bytes, bwd_workspace(*p, true)));
+  FwdParams fp{};   // of the forward sweep that rebuilds the checkpoints
+  fp.x = x;
+  fp.delta = delta;
+  fp.B = B;
+  fp.C = C;
+  fp.A = A;
+  const Plan pl = make_bwd_plan(*p);
+  const Plan pl_fwd = plan_fwd(*p, has_room(workspace, workspace_bytes, bwd_workspace(*p, true)) && uses_spare(*p, fp));
   const BwdWorkspace w = bwd_layout(*p, pl, pl_fwd);
   st = check_ws(workspace, workspace_bytes, w.total);
   if (st != SSM_OK) return st;
@@ -829,12 +840,6 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   // checkpoint states: the caller's, or rebuilt here with one more forward sweep
   const float* ckpt = static_cast<const float*>(saved_states);
   if (ckpt == nullptr) {
-    FwdParams fp{};
-    fp.x = x;
-    fp.delta = delta;
-    fp.B = B;
-    fp.C = C;
-    fp.A = A;
     fp.batch = p->batch;
     fp.L = p->L;
     fp.D = p->D;

@@ -295,6 +295,21 @@ def test_pointers_off_the_16_byte_grid_and_states_passed_between_the_families(of
     _check(2, 150, 4744, fwd=fwd, bwd=bwd, off=off)
 
 
+def test_no_time_segments_by_choice_off_the_16_byte_grid():
+    # the lane kernel runs these, which cuts a chain in time by itself
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("routes", 29, 2, 1030, 4744, 16, "bf16", 1e-3, 1e-1), seed=4), "bf16")
+    rest = (dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    x = _shifted(dev["x"])
+    assert K.plan(K.make_problem(x, dev["B"], True, True))["n_segments"] == 4
+    out = K.ssm_scan_fwd(x, *rest)
+    U.assert_elementwise({"out": U.to_host(out)}, {"out": U.to_host(K.ssm_scan_fwd(dev["x"], *rest))}, "bf16", "off the grid")
+    assert U.kernels(lambda: K.ssm_scan_fwd(x, *rest)) == {LANE[0]}
+    ran = U.kernels(lambda: K.ssm_scan_bwd(x, *rest, dev["dout"], None))
+    assert LANE[0] in ran and not any(k.startswith("ssm_carry") for k in ran), ran
+
+
 def test_states_rebuilt_off_the_16_byte_grid():
     _check(2, 150, 4744, fwd=LANE[0], bwd=LANE[1], off=("fwd", "bwd"), saved=False)
 
