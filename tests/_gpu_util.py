@@ -36,9 +36,10 @@ def to_host(t) -> np.ndarray:
     return t.detach().to(torch.float32).cpu().numpy()
 
 
-def kernels(run) -> set:
-    """Names of the library's kernels that `run()` launches (template arguments cut off).  It is captured into a graph and
-    not executed; call it once before, so that nothing is set up for the first time."""
+def kernels(run, arguments=False) -> set:
+    """Names of the library's kernels that `run()` launches, template arguments cut off or as they are in the mangled name
+    (ints and bools as Li16E, Lb1E).  It is captured into a graph and not executed; call it once before, so that nothing is set
+    up for the first time."""
     import os
     import re
     import tempfile
@@ -54,7 +55,9 @@ def kernels(run) -> set:
             warnings.simplefilter("ignore")
             graph.debug_dump(path)
         with open(path) as f:   # (mangled names; a kernel in an anonymous namespace has its file's before its own)
-            return {m[m.rindex("ssm_"):] for m in re.findall(r"ssm_\w+?_kernel", f.read())}
+            text = f.read()
+    names = re.findall(r"ssm_\w+?_kernel" + (r"\w*" if arguments else ""), text)
+    return {re.sub(r"^.*(?=ssm_\w+?_kernel)", "", m) for m in names}
 
 
 def gpu_fwd_bwd(dev: dict, use_saved=True, general_A=False):

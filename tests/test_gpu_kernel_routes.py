@@ -2,6 +2,7 @@
 pointers and at least 296 chains of 32 channels (or the zero-order-hold rule); small problems of the same kind run the
 lane kernels, so what is to be tested of the tuned ones is wide here.  Every case asserts the route."""
 import os
+import re
 
 import numpy as np
 import pytest
@@ -15,6 +16,9 @@ TUNED = ("ssm_fwd_warp_kernel", "ssm_bwd_warp_kernel")
 LANE = ("ssm_fwd_lane_kernel", "ssm_bwd_lane_kernel")
 GENERIC = ("ssm_fwd_kernel", "ssm_bwd_kernel")
 TEAM = "ssm_fwd_team_kernel"   # forward of 32 or 64 states
+# template arguments: summary pass of the tuned forward, its sweeps with output and with checkpoints only; rolled lane backward
+SUMMARY, FULL, CKPT = (r"ssm_fwd_warp_kernelILi16ELi%dE" % mode for mode in (1, 0, 2))
+ROLLED, UNROLLED = (r"ssm_bwd_lane_kernelI(f|13__nv_bfloat16)Li1ELi\dELb0ELb%dEE" % rolled for rolled in (1, 0))
 
 
 def _shifted(t):
@@ -34,7 +38,7 @@ def _no_workspace(buf):
 
 
 def _check(batch, L, D, N=16, io="bf16", *, fwd=TUNED[0], bwd=TUNED[1], more=(), gate=True, skip=True, zoh=False, fused=False,
-           carry=False, saved=True, perturb_A=0.0, A=None, dt=(1e-3, 1e-1), off=()):
+           carry=False, saved=True, perturb_A=0.0, A=None, dt=(1e-3, 1e-1), off=(), instances=()):
     import torch
     from oracle import ssm_oracle as O
     from paper_2312_00752_b200 import binding as K
@@ -75,6 +79,8 @@ def _check(batch, L, D, N=16, io="bf16", *, fwd=TUNED[0], bwd=TUNED[1], more=(),
     ran = U.kernels(run)
     assert {k for k in ran if k in (*TUNED, *LANE, *GENERIC, TEAM)} == {fwd, bwd}, ran
     assert all(any(k.startswith(m) for k in ran) for m in more), ran
+    ran = U.kernels(run, arguments=True)
+    assert all(any(re.match(m, k) for k in ran) for m in instances), ran
     a = (inp["x"], inp["delta"], inp["A"], inp["B"], inp["C"])
     out, h = O.scan_fwd(*a, D_skip=inp["D_skip"], z=inp["z"], h0=h0, return_h_last=True, **okw)
     ref = dict(O.scan_bwd(*a, inp["D_skip"], inp["z"], inp["dout"], h0=h0, dh_last=dh, **okw), out=out)
@@ -108,7 +114,8 @@ def test_tuned_kernels_at_the_edges_of_tiles_groups_and_segments(batch, L, D, fu
     (2, 416, 4736, dict(fused=True, saved=False)),        # ... of one tile
 ])
 def test_tuned_forward_split_in_time_with_more_than_half_the_sub_partitions(batch, L, D, options):
-    _check(batch, L, D, more=("ssm_carry",), **options)
+    instances = (SUMMARY, FULL) if options.get("saved", True) else (SUMMARY, FULL, CKPT)
+    _check(batch, L, D, more=("ssm_carry",), instances=instances, **options)
 
 
 @pytest.mark.parametrize("options", [
@@ -225,7 +232,17 @@ def test_backward_without_room_for_what_its_rebuilding_sweep_can_do_without(batc
     (2, 31, 47, 16, "bf16", dict(perturb_A=0.05, saved=False)),
 ])
 def test_lane_kernels_in_pieces_of_one_block(batch, L, D, N, io, options):
-    _check(batch, L, D, N, io, fwd=LANE[0], bwd=LANE[1], **options)
+    _check(batch, L, D, N, io, fwd=LANE[0], bwd=LANE[1], instances=(ROLLED,), **options)
+
+
+@pytest.mark.parametrize("L,D,rolled", [
+    (250, 256, True), (250, 288, False),     # clusters of 8: 8 and 9
+    (100, 896, True), (100, 928, False),     # of 4: 28 and 29
+    (64, 1792, True), (64, 1824, False),     # of 2: 56 and 57
+    (32, 4736, True), (32, 4768, False),     # a block per chain: 148 and 149
+])
+def test_rolled_lane_backward_only_where_its_blocks_run_at_once(L, D, rolled):
+    _check(1, L, D, 16, "f32", fwd=LANE[0], bwd=LANE[1], instances=(ROLLED if rolled else UNROLLED,))
 
 
 @pytest.mark.parametrize("batch,L,D,N,options", [
@@ -280,7 +297,8 @@ def test_rows_of_A_widened_for_the_tuned_kernels(A):
     _check(1, 40, 9480, 4, A=A, more=("ssm_repack_kernel",))
 
 
-@pytest.mark.parametrize("D,N,route", [(9480, 16, TUNED), (40, 16, (TUNED[0], LANE[1])), (41, 16, LANE), (41, 32, LANE)])
+@pytest.mark.parametrize("D,N,route", [(9480, 16, TUNED), (40, 16, (TUNED[0], LANE[1])), (41, 16, LANE), (41, 32, LANE),
+                                       (2568, 64, (TEAM, LANE[1]))])
 @pytest.mark.parametrize("saved", [True, False])
 def test_rising_rows_of_A_with_large_steps(D, N, route, saved):
     # exp(delta A) of the first state is below the smallest float32, that of the last one is not

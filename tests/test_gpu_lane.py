@@ -112,6 +112,8 @@ def test_complex_edges(batch, L, D, N, io):
     (2, 61, 17, 64, "bf16"),       # four groups of states
     (1, 299, 24, 4, "f32"),        # cut in time
     (1, 33, 9480, 16, "bf16"),     # the tuned kernels
+    (1, 33, 2568, 64, "bf16"),     # teams of warps
+    (2, 75, 2568, 64, "bf16"),     # ... that share chains
 ])
 def test_an_infinite_input_of_the_last_step_stays_infinite(batch, L, D, N, io, which):
     """Rows past the end of a ragged batch are identity steps: zero times what they hold must not make NaN of the state."""
