@@ -96,7 +96,8 @@ enum {
   SSM_FLAG_TEST_WITHHOLD = 16u /* test hook for the bounded waits: the tuned backward kernel shares channel groups
                                  between neighbouring warps whatever the shape, never publishes a hand-off flag and
                                  polls only 1000 times, so every warp that continues a group gives up and
-                                 ssm_scan_check_status reports SSM_ERR_TIMEOUT; the gradients are then undefined  */
+                                 ssm_scan_check_status reports SSM_ERR_TIMEOUT; the gradients are then undefined.
+                                 The same for a forward call of N = 32 or 64 that shares groups between teams     */
 };
 
 typedef struct {

@@ -668,6 +668,7 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.static_C = (p->flags & SSM_FLAG_STATIC_C) ? 1 : 0;
   fp.delta_bias = delta_bias;
   fp.softplus = (p->flags & SSM_FLAG_DELTA_SOFTPLUS) ? 1 : 0;
+  fp.test_withhold = (p->flags & SSM_FLAG_TEST_WITHHOLD) ? 1 : 0;
   if (fwd_layout(*p, pl).total > 0) {
     if (attach_fwd_sched(*p, pl, static_cast<char*>(workspace), static_cast<int*>(workspace), fp, s, true) != cudaSuccess)
       return SSM_ERR_CUDA;

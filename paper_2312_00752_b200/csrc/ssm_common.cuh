@@ -80,6 +80,7 @@ struct FwdParams {
   int* flags;            // tuned kernel: [max_workers + 1] hand-off flags, zero before the launch
   float4* handoff;       // tuned kernel: carried state of a chain that two workers share
   int max_workers;       // tuned kernel: workers the hand-off slots allow (0: no chain may be shared)
+  int test_withhold;     // team kernel, test hook: never publish hand-off flags, poll only 1000 times
 };
 
 // Work distribution of the warp-per-worker kernels.  The work is `chains` independent sequences of `tiles` tiles each

@@ -340,7 +340,8 @@ cudaError_t launch_team(const FwdParams& p, cudaStream_t s) {
   if (sc.chains > resident && lim.per_sm > 0 && p.handoff != nullptr && p.max_workers >= resident * T) sc.workers = resident;
   const long long total = (long long)sc.chains * sc.tiles;
   sc.quota = (int)((total + sc.workers - 1) / sc.workers);
-  sc.spin_limit = 1 << 22;
+  sc.spin_limit = p.test_withhold ? 1000 : 1 << 22;
+  sc.withhold = p.test_withhold;
   if (sc.workers < sc.chains) {
     sc.flags = p.flags;
     sc.abort = p.abort;

@@ -175,6 +175,31 @@ def test_forward_results_depend_on_the_workspace_only_by_whether_the_split_has_r
         U.assert_elementwise({"out": U.to_host(out)}, ref, "bf16", "workspace")
 
 
+@pytest.mark.parametrize("batch,L,D,N", [(2, 75, 2568, 64), (2, 200, 5128, 32)])   # 162 chains for 148 teams, 322 for 296
+def test_teams_of_warps_leave_together_when_a_hand_off_stays_away(batch, L, D, N):
+    # no flag is published: the teams that continue a chain give up after 1000 polls, which the host reads from the status
+    # word; the next call on that workspace is complete again
+    import ctypes
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, N, "bf16", 1e-3, 1e-1), seed=L), "bf16")
+    args = (dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"])
+    prob = K.make_problem(dev["x"], dev["B"], True, True)
+    ws = torch.empty(K.fwd_workspace_bytes(prob), dtype=torch.uint8, device="cuda")
+    good = K.ssm_scan_fwd(*args, workspace=ws)
+    K.check_status(prob, ws)
+    out = torch.empty_like(good)
+    prob.flags |= K.SSM_FLAG_TEST_WITHHOLD
+    code = K.load_library().ssm_scan_fwd(
+        ctypes.byref(prob), *[ctypes.c_void_p(t.data_ptr()) for t in (*args, out)], None, ctypes.c_void_p(ws.data_ptr()),
+        ctypes.c_size_t(ws.numel()), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert code == K.SSM_OK
+    with pytest.raises(K.SsmScanError, match="TIMEOUT"):
+        K.check_status(prob, ws)
+    assert torch.equal(K.ssm_scan_fwd(*args, workspace=ws), good)
+    K.check_status(prob, ws)
+
+
 @pytest.mark.parametrize("batch,L,D,N", [(2, 1024, 4736, 16), (2, 1024, 4736, 8), (2, 75, 2568, 64)])
 def test_the_status_word_of_a_workspace_without_room_is_that_of_the_call(batch, L, D, N):
     import torch
