@@ -57,11 +57,17 @@ static bool tuned_shape(const ssm_problem_t& p) {
 static bool ckpt_tiled(const ssm_problem_t& p) { return p.N % 4 == 0 && !(p.flags & SSM_FLAG_COMPLEX); }
 // Time segments of the tuned forward: one warp per chain of 32 channels.  A split costs a summary sweep over all segments but
 // the last, so only where the chains alone leave much of the GPU empty: below half of the sub-partitions into two rounds of
-// chains; above, into four segments, which fill every sub-partition with two warps, when that is estimated shorter (in steps
-// of a lone warp: 1.31 times the share of the sub-partitions that have a chain and 290 for three more launches, 1.24 and 150
-// with the fused step size).  Measured, whole calls, D = 1536, batch 8 (share 0.65): L = 2048 167 -> 158 us, with A trained
-// 228 -> 218, and the step size fused 306 -> 270; L = 1024 would go 87 -> 91, 116 -> 122, 157 -> 150; D = 960, batch 10
-// (0.51), L = 2048: 168 -> 142, 228 -> 197, 307 -> 245.
+// chains; above, into four segments, when that is estimated shorter (in steps of a lone warp: so many times the share of the
+// sub-partitions that have a chain, and so many for three more launches).  The split puts two warps on every sub-partition,
+// but the full sweep of the zero-order hold has shared memory for one, so it gains less; parameters B and C make the lone
+// warp's step shorter and the launches dearer.  Measured, whole calls, one piece / four segments, us, D = 1536, batch 8 (share
+// 0.65), L = 2048 unless stated:
+//   input-dependent B or C   172 / 163, A trained 232 / 222, step size fused 248 / 198; L = 1024 92 / 95, 122 / 127, 129 / 114;
+//                            D = 1664 (0.70) 173 / 177, 232 / 240, 249 / 214; D = 960, batch 10 (0.51) 172 / 146, 232 / 200, 248 / 177
+//   zero-order hold          287 / 292, 318 / 318, fused 402 / 402; D = 1440 (0.61) 286 / 280, 316 / 303, 399 / 382, and at
+//                            L = 1024 148 / 157, 164 / 171, 206 / 210; D = 1664, L = 4096 565 / 591, 627 / 644, 795 / 822
+//   parameters B and C       150 / 148, 210 / 210, fused 219 / 185; (10, 1024, 960) 80 / 83, 111 / 108, 115 / 99;
+//                            D = 1664, L = 4096 291 / 288, 410 / 419; fused with A trained D = 1792 584 / 595
 // optional_split: the split above half of the sub-partitions may be taken (it needs workspace that the problem does not).
 static int tuned_fwd_segments(const ssm_problem_t& p, bool optional_split = true) {
   const int cw = fwd_fast_channels_per_warp();
@@ -69,8 +75,16 @@ static int tuned_fwd_segments(const ssm_problem_t& p, bool optional_split = true
   if (2 * chains >= sub_partitions) {
     if (!optional_split) return 1;
     const bool fused = p.flags & SSM_FLAG_DELTA_SOFTPLUS;
+    float per_share = fused ? 1.24f : 1.31f, launches = fused ? 150.f : 290.f;
+    if (p.flags & SSM_FLAG_ZOH_BBAR) {
+      per_share = fused ? 1.45f : 1.42f;
+      launches = fused ? 140.f : 240.f;
+    } else if ((p.flags & SSM_FLAG_STATIC_B) && (p.flags & SSM_FLAG_STATIC_C)) {
+      per_share = fused ? 1.28f : 1.33f;
+      launches = fused ? 150.f : 350.f;
+    }
     const float share = (float)chains / (float)sub_partitions, steps = (float)p.L;
-    return share * steps * (fused ? 1.24f : 1.31f) + (fused ? 150.f : 290.f) < steps ? 4 : 1;
+    return share * steps * per_share + launches < steps ? 4 : 1;
   }
   const long long want = (2 * sub_partitions + chains - 1) / chains;
   return (int)std::min<long long>(std::min<long long>(want, std::max(1, p.L / 256)), 65535);

@@ -118,6 +118,34 @@ def test_tuned_forward_split_in_time_with_more_than_half_the_sub_partitions(batc
     _check(batch, L, D, more=("ssm_carry",), instances=instances, **options)
 
 
+@pytest.mark.parametrize("options", [dict(zoh=True), dict(static_B=True), dict(static_C=True), dict(static_B=True, static_C=True)])
+@pytest.mark.parametrize("fused", [False, True])
+def test_tuned_forward_split_in_time_by_the_other_rules(options, fused):
+    # the zero-order hold, parameters B and C: four segments (a ragged last one, from a carried state) against one piece on the
+    # generic kernel, which runs what is off the 16-byte grid
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    batch, L, D = 2, 1150, 4744
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("routes", 29, batch, L, D, 16, "bf16", 1e-3, 1e-1), seed=L, perturb_A=0.05), "bf16")
+    rng = torch.Generator(device="cuda").manual_seed(1)
+    for name in "BC":
+        if options.get("static_" + name):
+            dev[name] = torch.randn(D, 16, generator=rng, device="cuda")
+    h0 = torch.randn(batch, D, 16, generator=rng, device="cuda")
+    bias = (torch.full((D,), -4.0, device="cuda"),) if fused else ()
+    fwd = K.ssm_scan_fwd_fused_dt if fused else K.ssm_scan_fwd
+
+    def run(x):
+        h_last = torch.empty(batch, D, 16, device="cuda")
+        out = fwd(x, dev["delta"], *bias, dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"], h0=h0, h_last=h_last, **options)
+        return out, h_last
+    shifted = _shifted(dev["x"])
+    (out, h), (ref_out, ref_h) = run(dev["x"]), run(shifted)
+    assert "ssm_carry_few_kernel" in U.kernels(lambda: run(dev["x"])) and U.kernels(lambda: run(shifted)) == {GENERIC[0]}
+    U.assert_elementwise({"out": U.to_host(out)}, {"out": U.to_host(ref_out)}, "bf16", "segments")
+    assert U.rel_err(U.to_host(h), U.to_host(ref_h)) <= 1e-4
+
+
 @pytest.mark.parametrize("options", [
     dict(gate=False), dict(skip=False), dict(gate=False, skip=False), dict(carry=True), dict(carry=True, saved=False),
     dict(perturb_A=0.05), dict(perturb_A=0.05, fused=True, saved=False), dict(fused=True, gate=False, carry=True),

@@ -47,6 +47,20 @@ def test_queries_and_plan():
     assert K.fwd_workspace_bytes(long) >= 2 * pl["n_segments"] * 1536 * 16 * 4
 
 
+@pytest.mark.parametrize("flags,batch,L,D,split", [
+    # groups of 32 channels on 0.51 to 0.70 of the 592 sub-partitions; four segments only where they were measured shorter
+    (0, 8, 2048, 1536, True), (0, 8, 1024, 1536, False), (0, 8, 2048, 1664, False), (32, 8, 1024, 1536, True),
+    (64, 8, 2048, 1440, True), (64, 8, 2048, 1536, False), (64, 10, 1024, 960, True), (64, 8, 1024, 1344, False),
+    (64, 8, 4096, 1536, True), (64, 8, 4096, 1664, False), (64, 10, 768, 960, False),
+    (96, 8, 1024, 1344, True), (96, 8, 1024, 1440, False), (96, 8, 2048, 1536, False), (96, 8, 4096, 1792, False),
+    (256, 8, 2048, 1536, True), (512, 8, 2048, 1536, True),
+    (768, 8, 2048, 1440, True), (768, 10, 1024, 960, False), (768, 8, 4096, 1664, False), (800, 8, 1024, 1536, True), (800, 8, 4096, 1792, False),
+])
+def test_time_segments_of_the_tuned_forward_by_choice(flags, batch, L, D, split):
+    for save in (0, K.SSM_FLAG_SAVE_STATES):
+        assert K.plan(_prob(batch, L, D, flags=3 | flags | save))["n_segments"] == (4 if split else 1)
+
+
 @pytest.mark.parametrize("bad,code", [
     (dict(N=3), 2), (dict(N=128), 2), (dict(io=5), 2), (dict(L=0), 1), (dict(batch=-1), 1), (dict(flags=1 << 12), 1),
 ])
