@@ -24,7 +24,7 @@
 
 namespace ssm {
 
-int warp_workers(int chains, int sms, int per_sm, int max_workers);
+int warp_workers(int chains, int sms, int per_sm, int max_workers, bool nearly_whole);
 
 namespace {
 
@@ -299,7 +299,7 @@ cudaError_t launch_local(const Plan& plan, const BwdParams& p, cudaStream_t s) {
   sc.chains = p.batch * (plan.nseg - 1) * p.local_split * ((p.D + 31) / 32);
   sc.tiles = (p.local_steps + kLT - 1) / kLT;
   const bool can_share = p.abort != nullptr && p.flags != nullptr && p.handoff != nullptr && p.max_workers > 0;
-  sc.workers = warp_workers(sc.chains, lim.sms, lim.per_sm * kLWarps, can_share ? p.max_workers : 0);
+  sc.workers = warp_workers(sc.chains, lim.sms, lim.per_sm * kLWarps, can_share ? p.max_workers : 0, true);
   const long long total = (long long)sc.chains * sc.tiles;
   sc.quota = (int)((total + sc.workers - 1) / sc.workers);
   sc.spin_limit = 1 << 22;

@@ -27,7 +27,7 @@
 
 namespace ssm {
 
-int warp_workers(int chains, int sms, int per_sm, int max_workers);
+int warp_workers(int chains, int sms, int per_sm, int max_workers, bool nearly_whole);
 
 namespace {
 
@@ -816,7 +816,7 @@ cudaError_t launch_bwd_variant(const Plan& plan, const BwdParams& p, cudaStream_
   sc.chains = p.batch * plan.nseg * ((p.D + CW - 1) / CW);
   sc.tiles = (plan.seg_steps + kBT - 1) / kBT;
   const bool can_share = p.abort != nullptr && p.flags != nullptr && p.handoff != nullptr && p.max_workers > 0;
-  sc.workers = warp_workers(sc.chains, sms, per_sm * kBwdWarps, can_share ? p.max_workers : 0);
+  sc.workers = warp_workers(sc.chains, sms, per_sm * kBwdWarps, can_share ? p.max_workers : 0, true);
   if (p.test_withhold && can_share) {
     // test hook: make neighbouring workers share chains whatever the shape (all of them must be resident)
     sc.workers = p.max_workers < per_sm * kBwdWarps * sms ? p.max_workers : per_sm * kBwdWarps * sms;

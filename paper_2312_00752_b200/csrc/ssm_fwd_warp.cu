@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32, MODE == kFwdFull ? 1 : 3)
   }
 }
 
-int warp_workers(int chains, int sms, int per_sm, int max_workers);
+int warp_workers(int chains, int sms, int per_sm, int max_workers, bool nearly_whole);
 float warp_run_estimate(int chains, int sms, int per_sm, int max_workers);
 
 #ifdef SSM_FWD_LANE_PAIR
@@ -568,7 +568,7 @@ cudaError_t launch_variant_w(const Plan& plan, const FwdParams& p, cudaStream_t 
       smem = smem2;
     }
   }
-  sc.workers = warp_workers(sc.chains, sms, per_sm * kWarpsPerBlock, max_workers);
+  sc.workers = warp_workers(sc.chains, sms, per_sm * kWarpsPerBlock, max_workers, MODE == kFwdSummary || BC == 3);
   const long long total = (long long)sc.chains * sc.tiles;
   sc.quota = (int)((total + sc.workers - 1) / sc.workers);
   sc.spin_limit = 1 << 22;
@@ -655,15 +655,19 @@ static int warp_rounds(int chains, int sms, int per_sm, int max_workers, float* 
   return best;
 }
 
-int warp_workers(int chains, int sms, int per_sm, int max_workers) {
+int warp_workers(int chains, int sms, int per_sm, int max_workers, bool nearly_whole) {
   const int round = 4 * sms;
   if (max_workers <= 0 || chains <= round) return chains;
   float t;
   int workers = warp_rounds(chains, sms, per_sm, max_workers, &t) * round;
   if (workers > max_workers) workers = max_workers;
-  // With nearly a chain per worker the hand-offs cost more than the few warps that are left empty: 1152 chains of 20992 steps,
-  // 1184 warps, summary pass 1803 -> 1749 us; with 1024 chains sharing is the faster one (289 us against 309, L = 2048).
-  if (chains < workers && 20 * chains >= 19 * workers) workers = chains;
+  // With nearly a chain per worker (nearly_whole) the hand-offs of some kernels cost more than the few warps that are left
+  // empty.  Measured with chains on 96 or 97 % of the warps, us, shared / not: whole forward of (1, 524288, 1536), which has such
+  // a summary pass, 4734 / 4679; backward of (8, 400, 4544) 241 / 235, zero-order hold 403 / 363, parameters B and C 222 / 183;
+  // of (8, 700, 2304), which has such a pre-pass, 260 / 246; forward with parameters B and C, (8, 2048, 4544), 263 / 257, A
+  // trained 353 / 345.  The forward sweep with input-dependent B or C rather loses: 293 / 297, A trained 370 / 376, fused 350 /
+  // 350 (469 / 464 with A trained), B a parameter 282 / 289, C 276 / 277.  The line: backward with 92 % 230 / 234, with 95 % 243 / 234.
+  if (nearly_whole && chains < workers && 20 * chains >= 19 * workers) workers = chains;
   return workers;
 }
 

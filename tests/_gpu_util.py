@@ -38,8 +38,8 @@ def to_host(t) -> np.ndarray:
 
 def kernels(run, arguments=False) -> set:
     """Names of the library's kernels that `run()` launches, template arguments cut off or as they are in the mangled name
-    (ints and bools as Li16E, Lb1E).  It is captured into a graph and not executed; call it once before, so that nothing is set
-    up for the first time."""
+    (ints and bools as Li16E, Lb1E) with the x of the grid behind (<<<148).  It is captured into a graph and not executed; call it
+    once before, so that nothing is set up for the first time."""
     import os
     import re
     import tempfile
@@ -56,8 +56,8 @@ def kernels(run, arguments=False) -> set:
             graph.debug_dump(path)
         with open(path) as f:   # (mangled names; a kernel in an anonymous namespace has its file's before its own)
             text = f.read()
-    names = re.findall(r"ssm_\w+?_kernel" + (r"\w*" if arguments else ""), text)
-    return {re.sub(r"^.*(?=ssm_\w+?_kernel)", "", m) for m in names}
+    names = re.findall(r"ssm_\w+?_kernel" + (r"\w*(?:\\<\\<\\<\d+)?" if arguments else ""), text)
+    return {re.sub(r"^.*(?=ssm_\w+?_kernel)", "", m).replace("\\", "") for m in names}
 
 
 def gpu_fwd_bwd(dev: dict, use_saved=True, general_A=False):

@@ -118,6 +118,11 @@ def test_tuned_forward_split_in_time_with_more_than_half_the_sub_partitions(batc
     _check(batch, L, D, more=("ssm_carry",), instances=instances, **options)
 
 
+def test_chains_of_the_tuned_kernels_nearly_one_per_warp():
+    # 1136 chains for two rounds of 592 warps: the forward shares them among 1184, the backward leaves them whole
+    _check(8, 40, 4544, instances=(FULL + r"\w+<<<296", r"ssm_bwd_warp_kernel\w+<<<284"))
+
+
 @pytest.mark.parametrize("options", [dict(zoh=True), dict(static_B=True), dict(static_C=True), dict(static_B=True, static_C=True)])
 @pytest.mark.parametrize("fused", [False, True])
 def test_tuned_forward_split_in_time_by_the_other_rules(options, fused):
