@@ -89,11 +89,15 @@ bool make_host_plan(const ssm_problem_t* p, HostPlan* hp) {
   h.dD_part = take((size_t)h.nchunks * p->D * 4);
   h.dA = take((size_t)p->D * p->N * 4);
   h.dD = take((size_t)p->D * 4);
-  h.saved = take(ssm_scan_saved_state_bytes(&h.chunk));
-  h.ws_bytes = std::max(ssm_scan_fwd_workspace_bytes(&h.chunk), ssm_scan_bwd_workspace_bytes(&h.chunk));
+  // The last piece may be smaller, and a smaller problem may take a route that needs more (N < 16 widened for the tuned kernels)
+  ssm_problem_t last = h.chunk;
+  last.batch = p->batch - (h.nchunks - 1) * h.chunk_batch;
+  auto most = [&](size_t (*query)(const ssm_problem_t*)) { return std::max(query(&h.chunk), query(&last)); };
+  h.saved = take(most(ssm_scan_saved_state_bytes));
+  h.ws_bytes = std::max(most(ssm_scan_fwd_workspace_bytes), most(ssm_scan_bwd_workspace_bytes));
   h.ws = take(h.ws_bytes);
   h.total = off;
-  h.least = h.ws + align_up(std::max(ssm_fwd_workspace_least(&h.chunk), ssm_bwd_workspace_least(&h.chunk)));
+  h.least = h.ws + align_up(std::max(most(ssm_fwd_workspace_least), most(ssm_bwd_workspace_least)));
   *hp = h;
   return true;
 }

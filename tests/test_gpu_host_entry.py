@@ -95,6 +95,22 @@ def test_host_call_without_room_for_the_time_segments_taken_by_choice():
         call(arena[:least - 512])
 
 
+def test_host_call_whose_last_piece_is_widened_and_the_others_are_not():
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    batch, L, D, N = 9, 4402, 592, 2      # pieces of 2, 2, 2, 2 and 1
+    inp = synth.make_inputs(synth.ScanConfig("host", 15, batch, L, D, N, "bf16", 1e-3, 1e-1), seed=4)
+    h = _host_tensors(inp, "bf16")
+    res = K.ssm_scan_fwd_bwd_host(h["x"], h["delta"], h["A"], h["B"], h["C"], h["D_skip"], h["z"], h["dout"], device="cuda:0")
+    torch.cuda.synchronize()
+    dev = U.to_device(inp, "bf16")
+    for b0 in range(0, batch, 2):
+        part = {k: v if k in ("A", "D_skip") else v[b0:b0 + 2].contiguous() for k, v in dev.items()}
+        ref = U.gpu_fwd_bwd(part)
+        for k in ("out", "dx", "ddelta", "dz", "dB", "dC"):
+            assert np.array_equal(U.to_host(res[k][b0:b0 + 2]), ref[k]), (k, b0)
+
+
 def test_host_call_honours_the_zoh_flag():
     import torch
     from paper_2312_00752_b200 import binding as K

@@ -61,6 +61,16 @@ def test_time_segments_of_the_tuned_forward_by_choice(flags, batch, L, D, split)
         assert K.plan(_prob(batch, L, D, flags=3 | flags | save))["n_segments"] == (4 if split else 1)
 
 
+@pytest.mark.parametrize("batch,L,D,N", [(9, 4402, 592, 2), (17, 5238, 320, 2), (33, 4439, 200, 1), (2, 100, 64, 8)])
+def test_the_host_arena_holds_the_last_piece_where_it_needs_more(batch, L, D, N):
+    # pieces of 2, 3 and 5 batch entries and a last one of 1, 2 and 3, which is widened to 16 states where the others are not
+    piece = -(-batch // 8)
+    sizes = [_prob(b, L, D, N, flags=7) for b in {piece, batch - (-(-batch // piece) - 1) * piece}]
+    buffers = 4 * (4 * piece * L * D * 2 + 2 * piece * L * N * 2)      # inputs and outputs, both twice
+    arena = K.load_library().ssm_scan_host_arena_bytes(ctypes.byref(_prob(batch, L, D, N)))
+    assert arena >= buffers + max(map(K.saved_state_bytes, sizes)) + max(map(K.bwd_workspace_bytes, sizes))
+
+
 @pytest.mark.parametrize("bad,code", [
     (dict(N=3), 2), (dict(N=128), 2), (dict(io=5), 2), (dict(L=0), 1), (dict(batch=-1), 1), (dict(flags=1 << 12), 1),
 ])
