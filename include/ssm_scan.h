@@ -35,9 +35,9 @@
  *     of its own; larger bf16 problems with N < 16 and D % 8 == 0 run on them too, with A, B, C and the state arrays
  *     widened inside the workspace by columns that stay zero.)  All io pointers must be aligned to the element size;
  *     16-byte aligned pointers together with rows that are multiples of 16 bytes select the vector path.
- *   - Results are bitwise reproducible for fixed inputs, shape, flags and library build (and, for the forward calls
- *     split in time by choice, see ssm_scan_fwd_workspace_bytes, a workspace that holds the queried size or one that does not): every
- *     reduction (over n, over channels for dB/dC, over batch and time for dA/dD) has a fixed order and no
+ *   - Results are bitwise reproducible for fixed inputs, shape, flags, pointer alignment and library build (and, for the
+ *     calls split in time by choice, see ssm_scan_fwd_workspace_bytes, a workspace that holds the queried size or one that
+ *     does not): every reduction (over n, over channels for dB/dC, over batch and time for dA/dD) has a fixed order and no
  *     floating-point atomics are used.
  *   - NaN and Inf propagate; signs are not validated (A < 0 and delta > 0 are expected).
  */
@@ -111,7 +111,8 @@ typedef struct {
  * SSM_ERR_WORKSPACE, with two exceptions:
  *   - Forward, bf16, N <= 16, D % 8 == 0 and 296 to about 450 groups of 32 channels in all batch entries together:
  *     where it is estimated to be faster, ssm_scan_plan reports four time segments, which take scratch memory; a call
- *     without it (too small, NULL or not 256-byte aligned) runs the sequence in one piece instead.  N = 16 then needs
+ *     without it (too small, NULL or not 256-byte aligned) runs the sequence in one piece instead, as does one whose io
+ *     pointers are not 16-byte aligned.  N = 16 then needs
  *     none, smaller N the widened copies of A, B, C and the state arrays alone.  Its results are as accurate, but not
  *     bit for bit those of the call that splits, since the states of a segment are summed in another order; they do not
  *     depend on anything else about the workspace.
@@ -318,8 +319,9 @@ SSM_API ssm_status_t ssm_scan_fwd_bwd_host(const ssm_problem_t* p, const void* x
 SSM_API const char* ssm_status_string(ssm_status_t s);
 
 /*
- * Describes how the library runs this problem, given a workspace of ssm_scan_fwd_workspace_bytes(): number of time segments the sequence is split into, steps per
- * segment, channels per thread block and states per thread of the forward kernel.  Any output pointer may be NULL.
+ * Describes how the library runs this problem, given a workspace of ssm_scan_fwd_workspace_bytes() and pointers that are
+ * 16-byte aligned: number of time segments the sequence is split into, steps per segment, channels per thread block and
+ * states per thread of the forward kernel.  Any output pointer may be NULL.
  * Returns SSM_OK or the validation error.  Host-only; launches nothing.
  */
 SSM_API ssm_status_t ssm_scan_plan(const ssm_problem_t* p, int32_t* n_segments, int32_t* segment_steps,

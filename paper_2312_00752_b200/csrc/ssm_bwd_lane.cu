@@ -939,8 +939,9 @@ __global__ void __launch_bounds__(kLaneWarps * 32, 2) ssm_bwd_lane_kernel(const 
       // arithmetic before the first store, which no later load may pass (it was a fifth of a block's time, 2270 of 10700 cycles at
       // float32 (2, 2048, 1536), with a row's stores before the next row's loads).  Not more, and with complex states one: the
       // body of a block is near the size of the instruction cache or beyond it (main kernel at float32 (2, 2048, 1536) 133.0 us
-      // before, 130.4 with two rows, 131.0 with four, 133.0 with eight; complex (2, 2048, 1536) 406, 384 with one row, 410 with
-      // two; bf16 (3, 1237, 1001) 97.0, 95.3 with two).
+      // before, 130.4 with two rows, 131.0 with four, 133.0 with eight; bf16 (3, 1237, 1001) 97.0, 95.3 with two; complex, whole
+      // backward, the same within 1 % in two orders of the problems: bf16 (2, 2048, 1536) 489 before, 479 with one row, 497 with
+      // two, float32 (2, 2048, 1001) 360, 352, 363; small ones 1 to 2 % the other way, (2, 1000, 300) 101.1, 101.0, 99.4).
       constexpr int kOwn = kLB / NG, kAtOnce = CPLX ? 1 : 2;
       static_assert(kOwn % kAtOnce == 0, "whole groups of rows");
 #pragma unroll 1
@@ -1140,7 +1141,8 @@ cudaError_t launch_bwd_lane_n(const Plan& plan, const BwdParams& p, int N, int m
   // the states after the odd steps in shared memory instead of registers, that is a quarter of it (float32 (1, 256, 64): main
   // kernel 13.6 -> 12.0 us; with two blocks per piece the loops cost what they save).  Its shared memory leaves room for one
   // block per SM, so only for grids that then still run at once (float32 (2, 256, 256), 16 clusters of 8: 25.5 -> 34.6 us a
-  // pass): eight clusters of 8, smaller clusters on three quarters of the SMs, or a block per SM.
+  // pass): eight clusters of 8, smaller clusters on three quarters of the SMs, or a block per SM.  (The occupancy query
+  // gives 15 clusters of 8, 33 of 4 and 74 of 2 at once; between the lines and these nothing was timed.)
   if constexpr (NG == 1 && !CPLX) {
     const LaneSplit sp = plan.split;
     const int per_block = kLaneWarps / sp.warps, most = sp.cluster == 8 ? 64 : sp.cluster > 1 ? 112 : kNumSMs;

@@ -5,14 +5,13 @@
 // thread.  With N > 16 the groups of 16 states of a batch run one after the other, their state parked in shared memory;
 // everything that belongs to the channel (step size, input, gate, rounding) is done once.
 //
-// Bound (counters): with one exponential per state the special-function unit, 70 % busy at float32 (2, 2048, 1536), 66 %
-// at bf16 (3, 1237, 1001), 68 % with complex states at (2, 2048, 1536); with two per group of 16 (bf16 (1, 2048, 5120),
-// N = 64, which ssm_fwd_team.cu takes now) latency: FMA pipe and issue slots 49 %, special-function unit 15 %, a warp waits 1.1 cycles per instruction
-// for fixed latencies.  The issue slots are 43 to 49 % in use.  So the registers are capped for three warps per
-// sub-partition and a chain is split in time until they are there.
+// Bound (counters): the special-function unit with its one exponential per state, 70 % busy at float32 (2, 2048, 1536), 67 %
+// at bf16 (3, 1237, 1001), 68 % with complex states at (2, 2048, 1536), 62 % at float32 (1, 2048, 2560), N = 64 (two warps per
+// sub-partition: the states of four groups take the shared memory).  The issue slots are 35 to 50 % in use.  So the registers
+// are capped for three warps per sub-partition and a chain is split in time until they are there.
 // Measured against the generic kernel with its summary and carry launches: float32 (2, 2048, 1536), N = 16: 262 -> 75 us;
-// bf16 (3, 1237, 1001), N = 16: 268 -> 49 us; bf16 (1, 2048, 5120), N = 64: 1204 -> 347 us (472 us with A off the
-// progression); float32 (1, 256, 64): 126 -> 7.6 us.
+// bf16 (3, 1237, 1001), N = 16: 268 -> 49 us; float32 (1, 256, 64): 126 -> 7.6 us.  bf16 N = 32 and 64 with enough channels run
+// in ssm_fwd_team.cu.
 #include <type_traits>
 
 #include "ssm_lane.cuh"

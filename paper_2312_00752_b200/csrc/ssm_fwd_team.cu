@@ -3,14 +3,15 @@
 // team is such a warp for its own 16 states; only what belongs to the channel is shared.
 //
 // Time goes in tiles of 32 steps.  The warps of a team deal the rows of a tile among themselves: each copies its share
-// (16-byte cp.async, one tile ahead), turns its rows of the next tile into (step size, step size times input) pairs and
+// (16-byte cp.async, two tiles ahead), turns its rows of the next tile into (step size, step size times input) pairs and
 // finishes its rows of the tile before (sum of the team's partial readouts, skip term, gate, rounding).  Pairs and partial
 // readouts pass through shared memory, double-buffered, behind one barrier of the team per tile.
 //
 // Schedule: that of ssm_fwd_warp.cu (WarpSched) with a team in the place of a warp.
 //
 // Bound: as the tuned kernel, the arithmetic and the latencies of a lone warp per sub-partition (a block fills an SM's shared
-// memory); what a team adds to a step (pairs and readouts through shared memory, the barrier) is about what the gate saves.
+// memory; counters at (1, 2048, 5120), N = 64: issue slots 40 %, FMA pipe 42 %, fixed latencies 0.79 cycles per instruction; with
+// A off the progression the special-function unit 56 %, 1.38 cycles); what a team adds to a step (pairs and readouts through shared memory, the barrier) is about what the gate saves.
 // Tiles of 32 steps because the rows passes are chains of latencies that a tile pays once (with 8 steps per barrier 304 us at
 // (1, 2048, 5120), N = 64).  There: 201 us, 271 with A off the progression, against 332 and 460 for the lane kernel, which
 // sweeps each piece twice and parks the states of three groups in shared memory.  For 16 states split over two or four warps the
