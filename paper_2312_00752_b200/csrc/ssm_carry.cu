@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(kCarryCols* kCarryRanges) ssm_carry_kernel(con
     for (int i = i0; i < i1; ++i) {
       const size_t sg = (size_t)b * p.nseg + seg_of(i);
       p.carried[sg * DN + col] = carry;
-      carry = fmaf(ex2_approx(A2 * p.dsum[sg * p.D + d]), carry, p.local[sg * DN + col]);
+      carry = carry_over(ex2_approx(A2 * p.dsum[sg * p.D + d]), carry, p.local[sg * DN + col]);
     }
   }
 }
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256) ssm_carry_few_kernel(const CarryParams p)
       *reinterpret_cast<float4*>(p.carried + sg * DN + col) = make_float4(c[0], c[1], c[2], c[3]);
       const float l[4] = {e[i].x, e[i].y, e[i].z, e[i].w};
 #pragma unroll
-      for (int k = 0; k < 4; ++k) c[k] = fmaf(ex2_approx(a2[k] * ds[i]), c[k], l[k]);
+      for (int k = 0; k < 4; ++k) c[k] = carry_over(ex2_approx(a2[k] * ds[i]), c[k], l[k]);
     }
   }
 }

@@ -490,8 +490,13 @@ __device__ __forceinline__ float sigmoid_fast(float z) { return rcp_approx(1.0f 
 struct AffinePair {
   float a, b;
 };
+// decay h + e over a whole segment.  Its decay may underflow where that of no step does, and zero times an infinite state is NaN
+// where the steps one by one keep it infinite.
+__device__ __forceinline__ float carry_over(float decay, float h, float e) {
+  return fmaf(decay == 0.f && isinf(h) ? 1.f : decay, h, e);
+}
 __device__ __forceinline__ AffinePair combine(AffinePair first, AffinePair second) {
-  return {first.a * second.a, fmaf(second.a, first.b, second.b)};
+  return {first.a * second.a, carry_over(second.a, first.b, second.b)};
 }
 #endif
 

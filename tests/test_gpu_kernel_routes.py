@@ -118,6 +118,25 @@ def test_tuned_forward_split_in_time_with_more_than_half_the_sub_partitions(batc
     _check(batch, L, D, more=("ssm_carry",), instances=instances, **options)
 
 
+@pytest.mark.parametrize("batch,L,D,carry", [(2, 1024, 4736, "ssm_carry_few_kernel"), (1, 16384, 1536, "ssm_carry_kernel")])
+@pytest.mark.parametrize("which", ["x", "h0"])
+def test_an_infinite_state_stays_infinite_across_time_segments(batch, L, D, carry, which):
+    # the decay over a whole segment is zero in float32 for the fast states of many channels, that of a step is not
+    import torch
+    from paper_2312_00752_b200 import binding as K
+    dev = U.to_device(synth.make_inputs(synth.ScanConfig("inf", 31, batch, L, D, 16, "bf16", 1e-3, 1e-1), seed=L), "bf16")
+    h0, h_last = torch.zeros(batch, D, 16, device="cuda"), torch.empty(batch, D, 16, device="cuda")
+    if which == "x":
+        dev["x"][:, 100] = float("inf")
+        dev["B"][:, 100].abs_().clamp_(min=0.5)
+    else:
+        h0.fill_(float("-inf"))
+    run = lambda: K.ssm_scan_fwd(dev["x"], dev["delta"], dev["A"], dev["B"], dev["C"], dev["D_skip"], dev["z"], h0=h0, h_last=h_last)
+    run()
+    assert carry in U.kernels(run)
+    assert bool((h_last == float("inf" if which == "x" else "-inf")).all())
+
+
 def test_chains_of_the_tuned_kernels_nearly_one_per_warp():
     # 1136 chains for two rounds of 592 warps: the forward shares them among 1184, the backward leaves them whole
     _check(8, 40, 4544, instances=(FULL + r"\w+<<<296", r"ssm_bwd_warp_kernel\w+<<<284"))
