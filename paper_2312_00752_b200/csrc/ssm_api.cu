@@ -397,9 +397,11 @@ static bool aligned_to(const void* ptr, size_t a) { return (reinterpret_cast<uin
 static bool has_room(const void* ws, size_t have, size_t need) {
   return need == 0 || (ws != nullptr && aligned_to(ws, 256) && have >= need);
 }
-// Whether the kernel that the spare workspace is for takes the pointers of a call.  Off the 16-byte grid the lane (or generic)
-// kernel runs, which cuts a chain in time by itself.
-static bool uses_spare(const ssm_problem_t& p, const FwdParams& fp) { return team_fwd(p) ? fwd_team_applicable(fp) : fwd_fast_applicable(p, fp); }
+// Whether the kernel that spare workspace is for takes the pointers of a call (true where no kernel wants any).  Off the 16-byte
+// grid the lane (or generic) kernel runs, which cuts a chain in time by itself.
+static bool uses_spare(const ssm_problem_t& p, const FwdParams& fp) {
+  return team_fwd(p) ? fwd_team_applicable(fp) : !tuned_shape(p) || fwd_fast_applicable(p, fp);
+}
 // Points the forward parameters at the scheduling words of a forward workspace and clears them; a status word at the head
 // of that workspace is cleared with them.
 static cudaError_t attach_fwd_sched(const ssm_problem_t& p, const Plan& pl, char* ws, int* abort_word, FwdParams& fp,
@@ -630,7 +632,8 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   }
   ssm_problem_t wide;
   if (widen_route(*p, &wide)) {
-    const size_t inner = fwd_workspace(wide, has_room(workspace, workspace_bytes, fwd_workspace(*p, true)));
+    size_t inner = fwd_workspace(wide, true);
+    if (!has_room(workspace, workspace_bytes, widen_layout(*p, inner, false).total)) inner = fwd_workspace(wide, false);
     const WidenLayout wl = widen_layout(*p, inner, false);
     st = check_ws(workspace, workspace_bytes, wl.total);
     if (st != SSM_OK) return st;
@@ -666,9 +669,11 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.h_last = h_last;
   fp.ckpt = save ? static_cast<float*>(saved_states) : nullptr;
   fp.ckpt_tiled = ckpt_tiled(*p) ? 1 : 0;
-  const size_t full = fwd_workspace(*p, true);
-  const Plan pl = plan_fwd(*p, has_room(workspace, workspace_bytes, full) && uses_spare(*p, fp));
-  st = check_ws(workspace, workspace_bytes, fwd_layout(*p, pl).total);
+  Plan pl = plan_fwd(*p, true);
+  const size_t full = fwd_layout(*p, pl).total;
+  if (!has_room(workspace, workspace_bytes, full) || !uses_spare(*p, fp)) pl = plan_fwd(*p, false);
+  const size_t need = fwd_layout(*p, pl).total;
+  st = check_ws(workspace, workspace_bytes, need);
   if (st != SSM_OK) return st;
   fp.batch = p->batch;
   fp.L = p->L;
@@ -683,7 +688,7 @@ static ssm_status_t fwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.delta_bias = delta_bias;
   fp.softplus = (p->flags & SSM_FLAG_DELTA_SOFTPLUS) ? 1 : 0;
   fp.test_withhold = (p->flags & SSM_FLAG_TEST_WITHHOLD) ? 1 : 0;
-  if (fwd_layout(*p, pl).total > 0) {
+  if (need > 0) {
     if (attach_fwd_sched(*p, pl, static_cast<char*>(workspace), static_cast<int*>(workspace), fp, s, true) != cudaSuccess)
       return SSM_ERR_CUDA;
   } else if (full > 0 && workspace != nullptr && workspace_bytes >= sizeof(int)) {
@@ -801,7 +806,8 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   }
   ssm_problem_t wide;
   if (widen_route(*p, &wide)) {
-    const size_t inner = bwd_workspace(wide, has_room(workspace, workspace_bytes, bwd_workspace(*p, true)));
+    size_t inner = bwd_workspace(wide, true);
+    if (!has_room(workspace, workspace_bytes, widen_layout(*p, inner, true).total)) inner = bwd_workspace(wide, false);
     const WidenLayout wl = widen_layout(*p, inner, true);
     st = check_ws(workspace, workspace_bytes, wl.total);
     if (st != SSM_OK) return st;
@@ -836,8 +842,12 @@ static ssm_status_t bwd_impl(const ssm_problem_t* p, const void* x, const void* 
   fp.C = C;
   fp.A = A;
   const Plan pl = make_bwd_plan(*p);
-  const Plan pl_fwd = plan_fwd(*p, has_room(workspace, workspace_bytes, bwd_workspace(*p, true)) && uses_spare(*p, fp));
-  const BwdWorkspace w = bwd_layout(*p, pl, pl_fwd);
+  Plan pl_fwd = plan_fwd(*p, true);
+  BwdWorkspace w = bwd_layout(*p, pl, pl_fwd);
+  if (!has_room(workspace, workspace_bytes, w.total) || !uses_spare(*p, fp)) {
+    pl_fwd = plan_fwd(*p, false);
+    w = bwd_layout(*p, pl, pl_fwd);
+  }
   st = check_ws(workspace, workspace_bytes, w.total);
   if (st != SSM_OK) return st;
 
